@@ -2,17 +2,30 @@
 // (Sec. 6: the ARD lengthscales and outputscale are learned jointly by
 // maximising the marginal likelihood; all kernels in double precision).
 //
-// One block per (problem, objective, restart) runs the whole optimisation:
-// per Adam step it builds K = s2 M52(X, X) + noise I in fp64, factors it in
-// place (right-looking Cholesky), inverts the factor in place, forms K^-1 in
-// place, alpha = K^-1 y, the log likelihood and its gradient with respect to
+// One thread-block cluster per (problem, objective, restart) runs the whole
+// optimisation: per Adam step it builds K = s2 M52(X, X) + noise I in fp64,
+// factors it, inverts the factor and forms K^-1, alpha = K^-1 y, the log
+// likelihood (at the end) and its gradient with respect to
 // theta = (log l_1 .. log l_d, log s2, log noise),
 //   d log p / d theta_q = 1/2 sum_ij (alpha_i alpha_j - K^-1_ij) dK_ij / dtheta_q,
-// then takes a bias-corrected Adam ascent step and clamps theta to its
-// bounds. The lower triangle of the n x n workspace holds K, then L, then
-// L^-1, then K^-1; the upper triangle keeps exp(-sqrt5 r_ij) for the gradient.
-// The workspace is in shared memory when it fits, else in global memory
-// (one slice per block, L2-resident).
+// then takes a bias-corrected Adam ascent step and clamps theta to its bounds.
+//
+// What bounds it: fp64 issue. Measured here: one fp64 warp instruction every 19
+// clocks per SM whatever its active lanes, 110 clocks from a single warp, so
+// the work has to fill whole warps on as many SMs as possible, and what is
+// serial (a pivot's reciprocal, 350 clocks, per column) has to run beside the
+// rest. The matrices are therefore cut into 16 x 16 tiles (one entry per thread
+// of 256), spread over the cluster's CTAs, in a workspace in global memory that
+// stays in L2 (tile products take 2400 clocks of fp64 issue, their operands 6 KB).
+// The factorisation is right-looking over tile columns p, and the rows of
+// W = L^-1 and K^-1 = W^T W grow in the same loop:
+//   panel phase   L_ip = A_ip W_pp^T (i > p), W_pJ = W_pp B_pJ (J < p)
+//   update phase  A_ij -= L_ip L_jp^T, B_iJ -= L_ip W_pJ, K^-1_ij += W_pi^T W_pj:
+//                 nb (nb + 1) / 2 tile products for every p, beside which one
+//                 CTA updates, factors and inverts the next diagonal tile
+// with a cluster barrier (400 clocks) after each phase. n = 128, d = 12, six
+// restarts of 20 steps: 3.3 ms on clusters of 16 (one CTA per restart with the
+// matrix in shared memory and a barrier per column took 26.3 ms).
 #include <math.h>
 
 #include "internal.h"
@@ -21,9 +34,12 @@ namespace boute {
 
 namespace {
 
-constexpr int kLearnThreads = 256;
-constexpr int kLearnWarps = kLearnThreads / 32;
-constexpr int kLearnRows = 8;  // rows of K^-1 formed per pass
+constexpr int kT = 16;                // tile edge
+constexpr int kTE = kT * kT;          // entries of a tile, one per worker thread
+constexpr int kLearnWork = kTE;       // worker threads
+constexpr int kLearnThreads = kTE + 32;  // and one warp for the pivots' reciprocals
+constexpr int kTS = kT + 1;           // row stride of a tile in shared memory
+constexpr int kMaxCluster = 16;
 constexpr double kSqrt5d = 2.23606797749978969641;
 constexpr double kSqrt3d = 1.73205080756887729353;
 constexpr double kLog2Pi = 1.83787706640934548356;
@@ -34,13 +50,16 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   return v;
 }
 
-// Entry e of a lower triangle (diagonal included, row by row) -> (i, j).
-__device__ __forceinline__ void tri_index(int e, int &i, int &j) {
-  int r = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-  while (r * (r + 1) / 2 > e) --r;
-  while ((r + 1) * (r + 2) / 2 <= e) ++r;
+// Tile t of the lower triangle of tiles (row by row) -> (i, j).
+__device__ __forceinline__ void tri_index(int t, int &i, int &j) {
+  int r = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+  while (r * (r + 1) / 2 > t) --r;
+  while ((r + 1) * (r + 2) / 2 <= t) ++r;
   i = r;
-  j = e - r * (r + 1) / 2;
+  j = t - r * (r + 1) / 2;
+}
+__host__ __device__ __forceinline__ size_t tile_off(int i, int j) {
+  return ((size_t)i * (i + 1) / 2 + j) * kTE;
 }
 
 __device__ __forceinline__ double clamp_d(double v, double lo, double hi) {
@@ -57,15 +76,14 @@ __device__ __forceinline__ double clamp_param(int q, int d, double v) {
   return clamp_d(v, BOUTE_BETA_MIN, BOUTE_BETA_MAX);
 }
 
-// Row stride of the n x n workspace: odd, so that a column's 64-bit entries
-// fall in different shared-memory banks.
-__host__ __device__ inline int learn_ld(int n) { return n | 1; }
-
-// Doubles of one block's workspace: A (n x ld), X (n x d), y, alpha, tmp,
-// 1 / L_jj (n each), tmp2 (kLearnRows rows of K^-1), and for the composite
-// kernel <s, c_i> and w_i (n each).
-__host__ __device__ inline size_t learn_ws_doubles(int n, int d) {
-  return (size_t)n * learn_ld(n) + (size_t)n * d + 6 * (size_t)n + (size_t)kLearnRows * n;
+// Doubles of one cluster's workspace: the lower triangles of tiles of K (then
+// L, then K^-1), of B (then W = L^-1) and of two per-pair values kept for the
+// gradient (sqrt5 r and exp(-sqrt5 r); composite kernel: exp(-sqrt5 r_t) and
+// exp(-sqrt3 r_c)), alpha, the pivots, the CTAs' gradient sums, and a flag word.
+__host__ __device__ inline int learn_tiles(int n) { return (n + kT - 1) / kT; }
+__host__ __device__ inline size_t learn_ws_doubles(int n) {
+  const size_t nb = learn_tiles(n);
+  return 4 * (nb * (nb + 1) / 2) * kTE + 2 * nb * kT + (size_t)kMaxCluster * (BOUTE_MAX_D + 5) + 2;
 }
 
 constexpr int kMaxP = BOUTE_MAX_D + 5;  // parameters of the composite kernel
@@ -77,314 +95,437 @@ constexpr int kMaxP = BOUTE_MAX_D + 5;  // parameters of the composite kernel
 //               = 3 e^(-sqrt3 r_c) z_q^2 (s2_c w_i w_j + s2_x k52)        (deployment)
 //   dK/dlog s2_c = s2_c w_i w_j k32, dK/dlog s2_x = s2_x k52 k32,
 //   dK/dbeta = s2_c w_i w_j k32 (<s, c_i> + <s, c_j>).
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
+                   : "memory");
+}
+__device__ __forceinline__ int cluster_rank() {
+  int r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+
+using DTile = double[kT][kTS];
+
+// sum over the P rows of part (one double per worker thread each) into out
+__device__ __forceinline__ void reduce_rows(const double *part, int P, double *out) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int q = warp; q < P; q += kLearnThreads / 32) {
+    double v = 0.0;
+#pragma unroll
+    for (int e = 0; e < kLearnWork / 32; ++e) v += part[(size_t)q * kLearnWork + 32 * e + lane];
+    v = warp_sum_d(v);
+    if (lane == 0) __stcg(out + q, v);
+  }
+}
+
 template <bool COMP>
-__global__ void __launch_bounds__(kLearnThreads) learn_kernel(
-    const double *X, const double *Ys, int n, int d, int m, int R, const double *theta0,
+__global__ void __launch_bounds__(kLearnThreads, 1) learn_kernel(
+    const double *X, const double *Ys, int n, int d, int m, int R, int C, const double *theta0,
     int iters, double lr, double *theta_out, double *mll_out, double *grad_out, double *ws,
-    int use_smem, int dtau, const double *pref) {
-  extern __shared__ __align__(16) double lsm[];
-  __shared__ double th[kMaxP], m1[kMaxP], m2[kMaxP];
-  __shared__ double il[BOUTE_MAX_D], red[kLearnWarps][kMaxP];
-  __shared__ double logdet, mll_s;
-  __shared__ int bad;
+    int dtau, const double *pref) {
+  extern __shared__ __align__(16) double part[];  // P x kLearnWork gradient terms
+  __shared__ double th[kMaxP], m1[kMaxP], m2[kMaxP], gr[kMaxP];
+  __shared__ double il[kMaxP];  // 1 / l_q, then the scales
+  __shared__ DTile ta, tb;  // operand tiles of a product; the diagonal tile's columns
+  __shared__ double xi[kT][BOUTE_MAX_D + 1], xj[kT][BOUTE_MAX_D + 1];
+  __shared__ double pci[kT], pcj[kT], wvi[kT], wvj[kT], ai[kT], aj[kT];
+  __shared__ double inv_s;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int blk = blockIdx.x, bt = blk / R, b = bt / m, t = bt % m;
-  const int P = d + (COMP ? 5 : 2), ld = learn_ld(n), dc = d - dtau;
-  double *A = use_smem ? lsm : ws + (size_t)blk * learn_ws_doubles(n, d);
-  double *xs = A + (size_t)n * ld, *yv = xs + (size_t)n * d, *av = yv + n, *tmp = av + n, *dinv = tmp + n,
-         *tmp2 = dinv + n, *pc = tmp2 + (size_t)kLearnRows * n, *wv = pc + n;
-  for (int e = tid; e < n * d; e += kLearnThreads) xs[e] = X[(size_t)b * n * d + e];
-  for (int i = tid; i < n; i += kLearnThreads) yv[i] = Ys[((size_t)b * n + i) * m + t];
-  const double *th0 = theta0 + (size_t)blk * P;
+  const int rank = C > 1 ? cluster_rank() : 0;
+  const int blk = blockIdx.x / C, bt = blk / R, b = bt / m, t = bt % m;
+  const int P = d + (COMP ? 5 : 2), dc = d - dtau, nb = learn_tiles(n), nt = nb * (nb + 1) / 2;
+  const bool work = tid < kLearnWork;
+  const int r = tid / kT & (kT - 1), c = tid % kT;  // this thread's entry of a tile
+  double *KT = ws + (size_t)blk * learn_ws_doubles(n), *WT = KT + (size_t)nt * kTE;
+  double *E1 = WT + (size_t)nt * kTE, *E2 = E1 + (size_t)nt * kTE, *av = E2 + (size_t)nt * kTE;
+  double *piv = av + (size_t)nb * kT, *gpart = piv + (size_t)nb * kT;
+  volatile int *bad = (volatile int *)(gpart + (size_t)kMaxCluster * (BOUTE_MAX_D + 5));
+  const double *Xb = X + (size_t)b * n * d, *pb = COMP ? pref + (size_t)bt * dc : nullptr;
+  auto sync = [&]() {
+    if (C > 1) cluster_sync();
+    else __syncthreads();
+  };
+  // the rows of tiles i and j of X, zero past n (and <s, c>, w of the composite kernel)
+  auto load_x = [&](int i, int j) {
+    __syncthreads();  // the previous tile's are read
+    for (int e = tid; e < 2 * kT * d; e += kLearnThreads) {
+      const int h = e >= kT * d, f = h ? e - kT * d : e, row = f / d, q = f - row * d;
+      const int g = (h ? j : i) * kT + row;
+      (h ? xj : xi)[row][q] = g < n ? Xb[(size_t)g * d + q] : 0.0;
+    }
+    __syncthreads();
+    if (COMP) {
+      if (tid < 2 * kT) {
+        const int row = tid & (kT - 1);
+        const double *x = tid < kT ? xi[row] : xj[row];
+        double e = 0.0;
+        for (int k = 0; k < dc; ++k) e = fma(pb[k], x[dtau + k], e);
+        (tid < kT ? pci : pcj)[row] = e;
+        (tid < kT ? wvi : wvj)[row] = exp(th[d + 4] * e);
+      }
+      __syncthreads();
+    }
+  };
+  // operand tiles into ta and tb
+  auto load_ab = [&](const double *A, const double *B) {
+    double va = 0.0, vb = 0.0;
+    if (work) {
+      va = __ldcg(A + tid);
+      vb = __ldcg(B + tid);
+    }
+    __syncthreads();  // the previous product has read its operands
+    if (work) {
+      ta[r][c] = va;
+      tb[r][c] = vb;
+    }
+    __syncthreads();
+  };
   if (tid < P) {
-    th[tid] = clamp_param(tid, d, th0[tid]);
+    th[tid] = clamp_param(tid, d, theta0[(size_t)blk * P + tid]);
     m1[tid] = 0.0;
     m2[tid] = 0.0;
   }
-  if (COMP) {  // <s, c_i> of the training points (s fixed)
-    __syncthreads();
-    const double *pb = pref + (size_t)bt * dc;
-    for (int i = tid; i < n; i += kLearnThreads) {
-      double e = 0.0;
-      for (int k = 0; k < dc; ++k) e = fma(pb[k], xs[(size_t)i * d + dtau + k], e);
-      pc[i] = e;
-    }
-  }
+  if (rank == 0 && tid == 0) *bad = 0;
   double b1t = 1.0, b2t = 1.0;
+  bool failed = false;
   __syncthreads();
 
   for (int it = 0; it <= iters; ++it) {
     const bool last = it == iters;
-    const bool want_grad = !last || grad_out != nullptr;
-    // ---- K (lower) and exp(-sqrt5 r) (upper) at theta
-    if (tid < d) il[tid] = exp(-th[tid]);
-    if (tid == 0) bad = 0;
-    if (COMP)
-      for (int i = tid; i < n; i += kLearnThreads) wv[i] = exp(th[d + 4] * pc[i]);
+    // ---- K and the per-pair values, tile by tile (identity past n)
+    if (tid < P) il[tid] = exp(tid < d ? -th[tid] : th[tid]);
     __syncthreads();
-    const double s2 = exp(th[d]), nz = exp(th[d + 1]);
-    const double s2c = COMP ? exp(th[d + 2]) : 0.0, s2x = COMP ? exp(th[d + 3]) : 0.0;
-    const int npair = n * (n + 1) / 2;  // pairs i >= j, one thread each
-    for (int e = tid; e < npair; e += kLearnThreads) {
+    const double s2 = il[d], nz = il[d + 1];
+    const double s2c = COMP ? il[d + 2] : 0.0, s2x = COMP ? il[d + 3] : 0.0;
+    for (int e = rank; e < nt; e += C) {
       int i, j;
       tri_index(e, i, j);
-      if (COMP) {  // (the gradient recomputes the exponentials)
-        double rt2 = 0.0, rc2 = 0.0;
-        for (int q = 0; q < d; ++q) {
-          const double z = (xs[i * d + q] - xs[j * d + q]) * il[q];
-          if (q < dtau) rt2 = fma(z, z, rt2);
-          else rc2 = fma(z, z, rc2);
-        }
-        const double st = kSqrt5d * sqrt(rt2), sc = kSqrt3d * sqrt(rc2);
-        const double k52 = (1.0 + st + 5.0 * rt2 / 3.0) * exp(-st), k32 = (1.0 + sc) * exp(-sc);
-        A[(size_t)i * ld + j] =
-            s2 * k52 + s2c * wv[i] * wv[j] * k32 + s2x * k52 * k32 + (i == j ? nz : 0.0);
-        continue;
-      }
-      double r2 = 0.0;
+      load_x(i, j);
+      if (!work) continue;
+      const int gi = i * kT + r, gj = j * kT + c;
+      double rt2 = 0.0, rc2 = 0.0, v1, v2, k;
       for (int q = 0; q < d; ++q) {
-        const double z = (xs[i * d + q] - xs[j * d + q]) * il[q];
-        r2 = fma(z, z, r2);
+        const double z = (xi[r][q] - xj[c][q]) * il[q];
+        if (!COMP || q < dtau) rt2 = fma(z, z, rt2);
+        else rc2 = fma(z, z, rc2);
       }
-      const double rr = sqrt(r2), sr = kSqrt5d * rr, ex = exp(-sr);
-      A[(size_t)i * ld + j] = s2 * (1.0 + sr + 5.0 * r2 / 3.0) * ex + (i == j ? nz : 0.0);
-      if (i != j) A[(size_t)j * ld + i] = ex;
-    }
-    // ---- Cholesky in place (lower), column by column
-    for (int j = 0; j < n; ++j) {
-      __syncthreads();
-      const double djj = A[(size_t)j * ld + j];
-      if (!(djj > 0.0)) {  // not positive definite (every thread sees the same value)
-        if (tid == 0) bad = 1;
-        break;
+      if (COMP) {
+        const double st = kSqrt5d * sqrt(rt2), sc = kSqrt3d * sqrt(rc2);
+        v1 = exp(-st);
+        v2 = exp(-sc);
+        const double k52 = (1.0 + st + 5.0 * rt2 / 3.0) * v1, k32 = (1.0 + sc) * v2;
+        k = s2 * k52 + s2c * wvi[r] * wvj[c] * k32 + s2x * k52 * k32;
+      } else {
+        v1 = kSqrt5d * sqrt(rt2);
+        v2 = exp(-v1);
+        k = s2 * (1.0 + v1 + 5.0 * rt2 / 3.0) * v2;
       }
-      // one reciprocal square root on the column's critical path
-      const double inv = rsqrt(djj), Ljj = djj * inv;
-      for (int i = j + 1 + tid; i < n; i += kLearnThreads) A[(size_t)i * ld + j] *= inv;
-      __syncthreads();
-      // (the diagonal entry is replaced only now: every thread has read it)
-      if (tid == 0) A[(size_t)j * ld + j] = Ljj;
-      for (int i = j + 1 + warp; i < n; i += kLearnWarps) {
-        const double lij = A[(size_t)i * ld + j];
-        for (int k = j + 1 + lane; k <= i; k += 32)
-          A[(size_t)i * ld + k] = fma(-lij, A[(size_t)k * ld + j], A[(size_t)i * ld + k]);
-      }
+      if (gi == gj) k += nz;
+      if (gi >= n || gj >= n) k = gi == gj ? 1.0 : 0.0;
+      const size_t o = tile_off(i, j) + tid;
+      __stcg(KT + o, k);
+      __stcg(E1 + o, v1);
+      __stcg(E2 + o, v2);
     }
-    __syncthreads();
-    if (bad) break;  // keeps theta; the evaluation after the loop reports NaN
-    // log det K = 2 sum_j log L_jj (off the factorisation's critical path),
-    // and the reciprocals of the diagonal for the inversion
-    if (warp == 0) {
-      double s = 0.0;
-      for (int j = lane; j < n; j += 32) s += log(A[(size_t)j * ld + j]);
-      s = warp_sum_d(s);
-      if (lane == 0) logdet = s;
-    }
-    for (int j = tid; j < n; j += kLearnThreads) dinv[j] = 1.0 / A[(size_t)j * ld + j];
-    __syncthreads();
-    // ---- L^-1 in place by forward substitution of L X = I, right-looking:
-    // step k finishes row k of X (row k of B divided by L_kk) and subtracts
-    // L_ik times it from the rows i > k of B (B = I initially). Entry (i, c)
-    // holds L_ic until step c has used it, then B_ic, then X_ic.
-    for (int k = 0; k < n; ++k) {
-      const double ikk = dinv[k];
-      for (int i = k + 1 + tid; i < n; i += kLearnThreads) tmp[i] = A[(size_t)i * ld + k];
-      __syncthreads();  // column k of L saved; every thread has read L_kk
-      for (int c = tid; c <= k; c += kLearnThreads)
-        A[(size_t)k * ld + c] = c == k ? ikk : A[(size_t)k * ld + c] * ikk;
-      __syncthreads();
-      const int w = k + 1;  // entries per row to update: columns 0 .. k
-      for (int e = tid; e < (n - k - 1) * w; e += kLearnThreads) {
-        const int i = k + 1 + e / w, c = e - (e / w) * w;
-        const double xkc = A[(size_t)k * ld + c];
-        A[(size_t)i * ld + c] = c == k ? -tmp[i] * xkc : fma(-tmp[i], xkc, A[(size_t)i * ld + c]);
-      }
-      __syncthreads();  // tmp is rewritten by the next step
-    }
-    // ---- K^-1 = X^T X in place (X = L^-1 lower), kLearnRows rows at a time:
-    // entry (i, j <= i) is sum_{k >= i} X_ki X_kj, which needs only rows >= i
-    // of X, so a batch of rows is computed into tmp2 and written back after
-    __syncthreads();
-    for (int i0 = 0; i0 < n; i0 += kLearnRows) {
-      const int i1 = min(n, i0 + kLearnRows);
-      const int cnt = (i1 - i0) * i0 + (i1 - i0) * (i1 - i0 + 1) / 2;  // entries j <= i
-      for (int e = tid; e < cnt; e += kLearnThreads) {
-        // entry e -> (i, j): rows of i0 + 1, i0 + 2, ... entries
-        int i = i0, base = 0;
-        while (base + i + 1 <= e) {
-          base += i + 1;
-          ++i;
+    sync();
+    // ---- Cholesky, W = L^-1 and K^-1. diag(p): tile p's Schur complement (its
+    // entry in x) factored as L~ D L~^T and inverted in place: at step k the
+    // entries right of column k still hold A, those up to k hold the rows of
+    // L~^-1, and both take the same update x_rc -= (a_rk y_c) / a_kk, with y =
+    // column k of A (c > k) or row k of L~^-1 (c <= k), so that a thread has
+    // one product ready before the reciprocal and one fma after it.
+    auto diag = [&](int p, double x) {
+      double *col = &ta[0][0], *row = &tb[0][0];  // column k of A; row k of L~^-1
+      for (int k = 0; k < kT; ++k) {
+        if (work) {  // (rows and columns past k; row k of L~^-1)
+          if (c == k && r >= k) col[r] = x;
+          if (r == k) row[c] = c < k ? x : 1.0;
         }
-        const int j = e - base;
+        __syncthreads();
+        const double akk = col[k];
+        double y = 0.0;
+        const bool act = work && 2 * warp + 1 > k;  // (a warp holds two rows)
+        if (act) y = col[r] * (c > k ? col[c] : row[c]);
+        if (!work) {
+          const double iv = 1.0 / akk;
+          if (lane == 0) {
+            inv_s = iv;
+            __stcg(piv + p * kT + k, akk);
+            if (!(akk > 0.0)) *bad = 1;
+          }
+        }
+        __syncthreads();
+        if (act && r > k) x = fma(-y, inv_s, c == k ? 0.0 : x);
+      }
+      // W_pp = D^-1/2 L~^-1 (unit diagonal), zero above
+      if (work) {
+        if (c == r) x = 1.0;
+        const double dr = __ldcg(piv + p * kT + r);  // (written by this CTA before the barriers)
+        __stcg(WT + tile_off(p, p) + tid, c <= r ? x * rsqrt(dr) : 0.0);
+      }
+      __syncthreads();
+    };
+    if (rank == 0) diag(0, work ? __ldcg(KT + tile_off(0, 0) + tid) : 0.0);
+    sync();
+    failed = *bad != 0;
+    for (int p = 0; p < nb && !failed; ++p) {
+      // panel phase: tile p of nb is W_pp, done by diag
+      for (int e = rank; e < nb; e += C) {
+        if (e == p) continue;
         double s = 0.0;
-        for (int k = i; k < n; ++k) s = fma(A[(size_t)k * ld + i], A[(size_t)k * ld + j], s);
-        tmp2[e] = s;
-      }
-      __syncthreads();
-      for (int e = tid; e < cnt; e += kLearnThreads) {
-        int i = i0, base = 0;
-        while (base + i + 1 <= e) {
-          base += i + 1;
-          ++i;
+        if (e > p) {  // L_ep = A_ep W_pp^T
+          load_ab(KT + tile_off(e, p), WT + tile_off(p, p));
+          if (work) {
+#pragma unroll
+            for (int k = 0; k < kT; ++k) s = fma(ta[r][k], tb[c][k], s);
+            __stcg(KT + tile_off(e, p) + tid, s);
+          }
+        } else {  // W_pe = W_pp B_pe
+          load_ab(WT + tile_off(p, p), WT + tile_off(p, e));
+          if (work) {
+#pragma unroll
+            for (int k = 0; k < kT; ++k) s = fma(ta[r][k], tb[k][c], s);
+            __stcg(WT + tile_off(p, e) + tid, s);
+          }
         }
-        A[(size_t)i * ld + (e - base)] = tmp2[e];
       }
-      __syncthreads();
+      sync();
+      // update phase. The CTA of the next diagonal tile does only that (all of
+      // it with one CTA); tile (i, j) of the triangle is, by its row and column,
+      // a trailing tile (j > p), a tile of B (j <= p < i) or one of K^-1 (i <= p)
+      const int own = C > 1 && p + 1 < nb ? (p + 1) % C : -1;
+      if (p + 1 < nb && rank == (p + 1) % C) {
+        const double *L = KT + tile_off(p + 1, p);
+        load_ab(L, L);
+        double x = 0.0;
+        if (work) {
+          double s = 0.0;
+#pragma unroll
+          for (int k = 0; k < kT; ++k) s = fma(ta[r][k], tb[c][k], s);
+          x = __ldcg(KT + tile_off(p + 1, p + 1) + tid) - s;
+        }
+        __syncthreads();
+        diag(p + 1, x);
+      }
+      if (rank != own) {
+        const int nw = own >= 0 ? C - 1 : C, me = own >= 0 && rank > own ? rank - 1 : rank;
+        for (int e = me; e < nt; e += nw) {
+          int i, j;
+          tri_index(e, i, j);
+          if (i == p + 1 && j == p + 1) continue;
+          double *out = (j > p || i <= p ? KT : WT) + tile_off(i, j);
+          const bool fresh = j <= p && (i <= p ? i == p : j == p);  // its first term
+          const double old = work && !fresh ? __ldcg(out + tid) : 0.0;
+          double s = 0.0;
+          if (j > p) {
+            load_ab(KT + tile_off(i, p), KT + tile_off(j, p));
+            if (work) {
+#pragma unroll
+              for (int k = 0; k < kT; ++k) s = fma(ta[r][k], tb[c][k], s);
+              s = old - s;
+            }
+          } else if (i > p) {
+            load_ab(KT + tile_off(i, p), WT + tile_off(p, j));
+            if (work) {
+#pragma unroll
+              for (int k = 0; k < kT; ++k) s = fma(ta[r][k], tb[k][c], s);
+              s = old - s;
+            }
+          } else {
+            load_ab(WT + tile_off(p, i), WT + tile_off(p, j));
+            if (work) {
+#pragma unroll
+              for (int k = 0; k < kT; ++k) s = fma(ta[k][r], tb[k][c], s);
+              s = old + s;
+            }
+          }
+          if (work) __stcg(out + tid, s);
+        }
+      }
+      sync();
+      failed = *bad != 0;
     }
-    // ---- alpha = K^-1 y and the log likelihood
-    for (int i = warp; i < n; i += kLearnWarps) {
+    if (failed) break;  // (the same in every CTA) keeps theta
+    // ---- alpha = K^-1 y: a warp per row
+    for (int i = rank * (kLearnThreads / 32) + warp; i < n; i += C * (kLearnThreads / 32)) {
       double s = 0.0;
       for (int j = lane; j < n; j += 32) {
-        const double kij = j <= i ? A[(size_t)i * ld + j] : A[(size_t)j * ld + i];
-        s = fma(kij, yv[j], s);
+        const int hi = max(i, j), lo = min(i, j);
+        s = fma(__ldcg(KT + tile_off(hi / kT, lo / kT) + (hi % kT) * kT + lo % kT),
+                Ys[((size_t)b * n + j) * m + t], s);
       }
       s = warp_sum_d(s);
-      if (lane == 0) av[i] = s;
+      if (lane == 0) __stcg(av + i, s);
     }
-    __syncthreads();
-    if (tid < 32) {
-      double s = 0.0;
-      for (int i = lane; i < n; i += 32) s = fma(yv[i], av[i], s);
-      s = warp_sum_d(s);
-      if (lane == 0) mll_s = -0.5 * s - logdet - 0.5 * (double)n * kLog2Pi;
+    sync();
+    if (last) {
+      // log likelihood; log det K = sum_j log D_j
+      if (rank == 0 && warp == 0) {
+        double s = 0.0, l = 0.0;
+        for (int i = lane; i < n; i += 32) {
+          s = fma(Ys[((size_t)b * n + i) * m + t], __ldcg(av + i), s);
+          l += log(__ldcg(piv + i));
+        }
+        s = warp_sum_d(s);
+        l = warp_sum_d(l);
+        if (lane == 0) mll_out[blk] = -0.5 * s - 0.5 * l - 0.5 * (double)n * kLog2Pi;
+      }
+      if (!grad_out) break;
     }
-    if (!want_grad) break;
     // ---- gradient: pairs i >= j (an off-diagonal pair stands for two
     // entries); per pair f = s2 (5/3) (1 + sqrt5 r) e^(-sqrt5 r) multiplies
-    // (dx_q / l_q)^2 in the lengthscale terms
+    // (dx_q / l_q)^2 in the lengthscale terms, whose 1 / l_q^2 is left to the end
     double g[BOUTE_MAX_D], gs2 = 0.0, gnz = 0.0, gsc = 0.0, gsx = 0.0, gbe = 0.0;
 #pragma unroll
     for (int q = 0; q < BOUTE_MAX_D; ++q) g[q] = 0.0;
-    for (int e = tid; e < npair; e += kLearnThreads) {
+    for (int e = rank; e < nt; e += C) {
       int i, j;
       tri_index(e, i, j);
-      const double Q = (i == j ? 0.5 : 1.0) * (av[i] * av[j] - A[(size_t)i * ld + j]);
-      const double *xi = xs + (size_t)i * d, *xj = xs + (size_t)j * d;
+      load_x(i, j);
+      if (tid < 2 * kT) {
+        const int row = (tid < kT ? i : j) * kT + (tid & (kT - 1));
+        (tid < kT ? ai : aj)[tid & (kT - 1)] = row < n ? __ldcg(av + row) : 0.0;
+      }
+      __syncthreads();
+      const int gi = i * kT + r, gj = j * kT + c;
+      if (!work || gi >= n || gj > gi) continue;
+      const size_t o = tile_off(i, j) + tid;
+      const double Q = (gi == gj ? 0.5 : 1.0) * (ai[r] * aj[c] - __ldcg(KT + o));
+      const double v1 = __ldcg(E1 + o), v2 = __ldcg(E2 + o);
+      double ft, fc = 0.0;
       if (COMP) {
         double rt2 = 0.0, rc2 = 0.0;
         for (int q = 0; q < d; ++q) {
-          const double z = (xi[q] - xj[q]) * il[q];
+          const double z = (xi[r][q] - xj[c][q]) * il[q];
           if (q < dtau) rt2 = fma(z, z, rt2);
           else rc2 = fma(z, z, rc2);
         }
         const double st = kSqrt5d * sqrt(rt2), sc = kSqrt3d * sqrt(rc2);
-        const double e5 = exp(-st), e3 = exp(-sc);
-        const double k52 = (1.0 + st + 5.0 * rt2 / 3.0) * e5, k32 = (1.0 + sc) * e3;
-        const double ww = wv[i] * wv[j];
-        const double ft = Q * (5.0 / 3.0) * (1.0 + st) * e5 * (s2 + s2x * k32);
-        const double fc = Q * 3.0 * e3 * (s2c * ww + s2x * k52);
-#pragma unroll
-        for (int q = 0; q < BOUTE_MAX_D; ++q) {
-          if (q < d) {
-            const double z = (xi[q] - xj[q]) * il[q];
-            g[q] = fma(q < dtau ? ft : fc, z * z, g[q]);
-          }
-        }
+        const double k52 = (1.0 + st + 5.0 * rt2 / 3.0) * v1, k32 = (1.0 + sc) * v2;
+        const double ww = wvi[r] * wvj[c];
+        ft = Q * (5.0 / 3.0) * (1.0 + st) * v1 * (s2 + s2x * k32);
+        fc = Q * 3.0 * v2 * (s2c * ww + s2x * k52);
         gs2 = fma(Q, s2 * k52, gs2);
-        if (i == j) gnz = fma(Q, nz, gnz);
         const double tc = Q * s2c * ww * k32;
         gsc += tc;
         gsx = fma(Q, s2x * k52 * k32, gsx);
-        gbe = fma(tc, pc[i] + pc[j], gbe);
-        continue;
+        gbe = fma(tc, pci[r] + pcj[c], gbe);
+      } else {
+        const double qe = Q * s2 * v2;
+        ft = qe * (5.0 / 3.0) * (1.0 + v1);
+        gs2 = fma(qe, 1.0 + v1 + v1 * v1 / 3.0, gs2);  // (5/3 r^2 = (sqrt5 r)^2 / 3)
       }
-      double r2 = 0.0;
-      for (int q = 0; q < d; ++q) {
-        const double z = (xi[q] - xj[q]) * il[q];
-        r2 = fma(z, z, r2);
-      }
-      const double rr = sqrt(r2), sr = kSqrt5d * rr;
-      const double ex = i == j ? 1.0 : A[(size_t)j * ld + i];
-      const double Qf = Q * s2 * (5.0 / 3.0) * (1.0 + sr) * ex;
+      if (gi == gj) gnz = fma(Q, nz, gnz);
 #pragma unroll
       for (int q = 0; q < BOUTE_MAX_D; ++q) {
         if (q < d) {
-          const double z = (xi[q] - xj[q]) * il[q];
-          g[q] = fma(Qf, z * z, g[q]);
+          const double dx = xi[r][q] - xj[c][q];
+          g[q] = fma(COMP && q >= dtau ? fc : ft, dx * dx, g[q]);
         }
       }
-      gs2 = fma(Q, s2 * (1.0 + sr + 5.0 * r2 / 3.0) * ex, gs2);
-      if (i == j) gnz = fma(Q, nz, gnz);
     }
-    // block sums of the d + 2 components (the pair sums already carry the 1/2)
+    if (work) {
 #pragma unroll
-    for (int q = 0; q < BOUTE_MAX_D; ++q) {
-      if (q < d) {
-        const double v = warp_sum_d(g[q]);
-        if (lane == 0) red[warp][q] = v;
-      }
-    }
-    {
-      const double a = warp_sum_d(gs2), c = warp_sum_d(gnz);
-      if (lane == 0) {
-        red[warp][d] = a;
-        red[warp][d + 1] = c;
-      }
+      for (int q = 0; q < BOUTE_MAX_D; ++q)
+        if (q < d) part[(size_t)q * kLearnWork + tid] = g[q];
+      part[(size_t)d * kLearnWork + tid] = gs2;
+      part[(size_t)(d + 1) * kLearnWork + tid] = gnz;
       if (COMP) {
-        const double u = warp_sum_d(gsc), v2 = warp_sum_d(gsx), w2 = warp_sum_d(gbe);
-        if (lane == 0) {
-          red[warp][d + 2] = u;
-          red[warp][d + 3] = v2;
-          red[warp][d + 4] = w2;
-        }
+        part[(size_t)(d + 2) * kLearnWork + tid] = gsc;
+        part[(size_t)(d + 3) * kLearnWork + tid] = gsx;
+        part[(size_t)(d + 4) * kLearnWork + tid] = gbe;
       }
     }
     __syncthreads();
-    if (tid < P) {
-      double v = 0.0;
-      for (int w = 0; w < kLearnWarps; ++w) v += red[w][tid];
-      if (last) {
-        grad_out[(size_t)blk * P + tid] = v;
-      } else {
-        // Adam ascent step, bias-corrected moments, then the bounds
-        b1t *= BOUTE_ADAM_B1;
-        b2t *= BOUTE_ADAM_B2;
-        m1[tid] = BOUTE_ADAM_B1 * m1[tid] + (1.0 - BOUTE_ADAM_B1) * v;
-        m2[tid] = BOUTE_ADAM_B2 * m2[tid] + (1.0 - BOUTE_ADAM_B2) * v * v;
-        const double mh = m1[tid] / (1.0 - b1t), vh = m2[tid] / (1.0 - b2t);
-        th[tid] = clamp_param(tid, d, th[tid] + lr * mh / (sqrt(vh) + BOUTE_ADAM_EPS));
+    reduce_rows(part, P, gpart + (size_t)rank * P);
+    sync();
+    // ---- the CTAs' sums, then the Adam step, alike in every CTA
+    if (work) {
+      for (int q = tid / kMaxCluster; q < P; q += kLearnWork / kMaxCluster) {
+        double v = tid % kMaxCluster < C ? __ldcg(gpart + (size_t)(tid % kMaxCluster) * P + q) : 0.0;
+        const unsigned half = 0xffffu << (lane & 16);
+#pragma unroll
+        for (int o = kMaxCluster / 2; o > 0; o >>= 1) v += __shfl_xor_sync(half, v, o);
+        if (tid % kMaxCluster == 0) gr[q] = q < d ? v * (il[q] * il[q]) : v;
       }
+    }
+    __syncthreads();
+    if (last) {
+      if (rank == 0 && tid < P) grad_out[(size_t)blk * P + tid] = gr[tid];
+      break;
+    }
+    b1t *= BOUTE_ADAM_B1;
+    b2t *= BOUTE_ADAM_B2;
+    if (tid < P) {  // Adam ascent step, bias-corrected moments, then the bounds
+      const double v = gr[tid];
+      m1[tid] = BOUTE_ADAM_B1 * m1[tid] + (1.0 - BOUTE_ADAM_B1) * v;
+      m2[tid] = BOUTE_ADAM_B2 * m2[tid] + (1.0 - BOUTE_ADAM_B2) * v * v;
+      const double mh = m1[tid] / (1.0 - b1t), vh = m2[tid] / (1.0 - b2t);
+      th[tid] = clamp_param(tid, d, th[tid] + lr * mh / (sqrt(vh) + BOUTE_ADAM_EPS));
     }
     __syncthreads();
   }
-  __syncthreads();
-  if (tid < P) theta_out[(size_t)blk * P + tid] = th[tid];
-  if (tid == 0) mll_out[blk] = bad ? nan("") : mll_s;
-  if (bad && grad_out && tid < P) grad_out[(size_t)blk * P + tid] = nan("");
+  if (rank == 0) {
+    if (tid < P) theta_out[(size_t)blk * P + tid] = th[tid];
+    if (failed) {  // not positive definite
+      if (tid == 0) mll_out[blk] = nan("");
+      if (grad_out && tid < P) grad_out[(size_t)blk * P + tid] = nan("");
+    }
+  }
 }
 
 }  // namespace
-
-size_t learn_smem_limit() { return 200 * 1024; }
 
 // dtau, pref: the composite kernel (pref null: the Matern-5/2 kernel)
 int launch_learn(const double *X, const double *Ys, int B, int n, int d, int m,
                  const double *theta0, int R, int iters, double lr, double *theta, double *mll,
                  double *grad, int dtau, const double *pref, cudaStream_t s) {
-  const size_t per = learn_ws_doubles(n, d) * sizeof(double);
+  const size_t per = learn_ws_doubles(n) * sizeof(double);
   const int blocks = B * m * R;
-  const bool smem = per <= learn_smem_limit();
   double *ws = nullptr;
-  if (!smem && cudaMallocAsync((void **)&ws, per * blocks, s) != cudaSuccess) {
+  if (cudaMallocAsync((void **)&ws, per * blocks, s) != cudaSuccess) {
     cudaGetLastError();
     return BOUTE_ERR_OOM;
   }
+  // the largest cluster with which every restart still runs at once, and no
+  // more CTAs than the triangle has tiles
+  const int nb = learn_tiles(n), nt = nb * (nb + 1) / 2;
+  const long long sms = num_sms();
+  int C = kMaxCluster;
+  while (C > 1 && (C * (long long)blocks > sms || C > nt)) C /= 2;
+  const size_t smem = (size_t)(d + 5) * kLearnWork * sizeof(double);
+  int st = BOUTE_OK;
   auto go = [&](auto kern) {
-    if (smem) {
-      prefer_shared(kern);
-      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)per) !=
-          cudaSuccess)
-        return;
+    prefer_shared(kern);
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.blockDim = dim3(kLearnThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (C > 8)
+      cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    for (;; C /= 2) {  // (a partitioned device may not place the larger clusters)
+      attr[0].val.clusterDim.x = C;
+      cfg.gridDim = dim3((unsigned)(blocks * C));
+      int fit = 0;
+      if (C == 1 || (cudaOccupancyMaxActiveClusters(&fit, kern, &cfg) == cudaSuccess && fit > 0))
+        break;
+      cudaGetLastError();
     }
-    kern<<<blocks, kLearnThreads, smem ? per : 0, s>>>(X, Ys, n, d, m, R, theta0, iters, lr,
-                                                       theta, mll, grad, ws, smem ? 1 : 0, dtau,
-                                                       pref);
+    cudaLaunchKernelEx(&cfg, kern, X, Ys, n, d, m, R, C, theta0, iters, lr, theta, mll, grad, ws,
+                       dtau, pref);
   };
   if (pref) go(learn_kernel<true>);
   else go(learn_kernel<false>);
   count_launch();
-  const int st = last_launch_status();
-  if (ws) cudaFreeAsync(ws, s);
+  st = last_launch_status();
+  cudaFreeAsync(ws, s);
   return st;
 }
 

@@ -57,6 +57,21 @@ def test_likelihood_and_gradient_match_oracle(wi, B, n, R):
                                            atol=1e-9 * np.abs(g).max())
 
 
+@pytest.mark.parametrize("n,R", [(1, 1), (2, 3), (15, 1), (16, 2), (17, 5), (33, 20), (65, 40),
+                                 (96, 6), (161, 1)])
+def test_tile_edges_and_cluster_sizes_match_oracle(n, R):
+    """Tiles of 16: sizes at and around their edges, and restart counts that
+    take every cluster size (1 to 16 blocks a restart). fp64 on both sides:
+    rounding (1e-16) times a condition number below 1e6, with a margin of 10."""
+    w, X, Ys, theta0 = _problem(0, 1, n, R, seed=n)
+    theta, mll, grad = _gpu(X, Ys, theta0, 3, 0.05)
+    for t in range(w.m):
+        th_o, mll_o, g_o = oracle.gp_learn(X[0], Ys[0][:, t], theta0[0, t], 3, 0.05, grad=True)
+        np.testing.assert_allclose(theta[0, t], th_o, rtol=0, atol=1e-9)
+        np.testing.assert_allclose(mll[0, t], mll_o, rtol=1e-9, atol=1e-9)
+        np.testing.assert_allclose(grad[0, t], g_o, rtol=1e-7, atol=1e-9 * np.abs(g_o).max())
+
+
 @pytest.mark.parametrize("wi,B,n,R,iters", [(0, 1, 32, 4, 80), (1, 1, 128, 2, 40),
                                             (4, 1, 200, 1, 15)],
                          ids=["n32", "n128", "n200-global-workspace"])

@@ -390,9 +390,7 @@ int boute_select_topk(const float *acq, int B, long long N, int k, long long *id
  *   Set-up: the first call on a device, made with that device current, looks
  *   up the array's device address (once per device, under a lock); make that
  *   first call before any stream capture begins.
- *   The few words of the array that must start at zero (one counter per
- *   problem) are cleared by the call itself, on `stream`, before its kernel
- *   runs; every key is written before it is read.
+ *   Every word of the array is written before it is read.
  *   There is ONE array per device: calls that overlap in time on that device
  *   (on different streams, or from different threads) race on it and may
  *   return wrong results. Serialise them, e.g. by issuing them on one stream. */

@@ -633,11 +633,6 @@ int boute_engine_create(int B, int n, int d, int m, long long N, int mode, int S
   r |= dalloc(&e->idx, (size_t)B * k);
   r |= dalloc(&e->val, (size_t)B * k);
   r |= dalloc((unsigned char **)&e->scratch, topk_scratch_bytes(B, N, k));
-  // the top-k counters in the scratch start at zero; every step leaves them zero
-  if (r == BOUTE_OK && cudaMemset(e->scratch, 0, topk_scratch_bytes(B, N, k)) != cudaSuccess) {
-    cudaGetLastError();
-    r = BOUTE_ERR_CUDA;
-  }
   e->fuse_sel = engine_fuses_selection(e);
   if (r == BOUTE_OK && e->fuse_sel) {
     const size_t bytes = e->sel_bytes = mchvi2_select_scratch_bytes(B, N, 2 * n + 2);
@@ -786,7 +781,7 @@ static int engine_run(boute_engine *e, const double *X, const double *Y, const d
   }
   if (!e->fuse_sel || serial) {
     mark(ST_TOPK);
-    if ((r = launch_topk(e->acq, B, e->N, e->k, idx, val, e->scratch, s, true))) return r;
+    if ((r = launch_topk(e->acq, B, e->N, e->k, idx, val, e->scratch, s))) return r;
   }
   mark(ST_COUNT);
   e->launches = (int)(launch_count() - l0);
@@ -867,13 +862,12 @@ int boute_engine_step_async(boute_engine *e, const double *X, const double *Y,
                        (cudaStream_t)stream);
 }
 
-// After a failed step the cross-block counters of the kernels that select as
-// blocks finish may be left part-way: set them back to zero.
+// After a failed step the cross-block counters of the kernel that selects as
+// its blocks finish may be left part-way: set them back to zero.
 static void engine_reset_counters(boute_engine *e) {
   cudaDeviceSynchronize();
   cudaGetLastError();
   if (e->sel) cudaMemset(e->sel, 0, e->sel_bytes);
-  cudaMemset(e->scratch, 0, topk_scratch_bytes(e->B, e->N, e->k));
   cudaGetLastError();
 }
 

@@ -202,10 +202,7 @@ int launch_base_normals(unsigned long long seed, int B, long long N, int m, int 
 // a bounded device-side wait that runs out unless `complete` (selftest.cu)
 int launch_wait_selftest(int complete, unsigned long long limit_ns, int *status, cudaStream_t s);
 size_t topk_scratch_bytes(int B, long long N, int k);
-// counters_zeroed: the scratch's per-problem counters are known to be zero
-// (an engine's scratch: zeroed at creation, and every call leaves them zero);
-// otherwise the call clears them first.
 int launch_topk(const float *acq, int B, long long N, int k, long long *idx, float *val,
-                void *scratch, cudaStream_t s, bool counters_zeroed = false);
+                void *scratch, cudaStream_t s);
 
 }  // namespace boute

@@ -13,9 +13,7 @@ namespace boute {
 namespace {
 
 // Scratch of the levels after the first: two ping-pong arrays of 64-bit keys.
-// The only words that must start at zero (one counter per problem, on the
-// k <= 32 path) are cleared by every call before its kernel runs; every key
-// is written before it is read.
+// Every key is written before it is read.
 static __device__ __align__(256) unsigned char g_topk_scratch[BOUTE_TOPK_NOALLOC_SCRATCH_BYTES];
 
 constexpr int kMaxDevices = 64;
@@ -54,7 +52,7 @@ extern "C" int boute_select_topk_noalloc(const float *acq, int B, long long N, i
   if (!acq || !idx || !val || B < 1 || N < 1 || k < 1 || k > 1024 || k > N)
     return BOUTE_ERR_INVALID_ARG;
   if ((long long)B * N >= (1ll << 31)) return BOUTE_ERR_INVALID_ARG;
-  const long long nseg = (N + 2047) / 2048;  // first-level segments per problem
+  const long long nseg = (N + 2047) / 2048;  // the limit counts segments of 2048
   const unsigned long long need =
       nseg <= 1 ? 0ull
                 : 2ull * (unsigned long long)B * nseg * (k < 32 ? 32 : k) * sizeof(unsigned long long);

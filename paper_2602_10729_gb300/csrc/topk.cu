@@ -1,11 +1,20 @@
 // Deterministic top-k per problem. Values become 64-bit keys (order-preserving
 // float bits in the high word, the complement of the index in the low word), so
-// one unsigned comparison orders by value descending, then index ascending.
-// k <= 32 takes a warp-register path in one launch (below). Otherwise, level 1: every block sorts one segment of kSeg keys in shared memory
-// (bitonic) and keeps its k largest. Further levels apply the same segment
-// sort to the surviving keys until one segment per problem remains; the last
-// level writes indices and values. All levels are fully parallel across
-// blocks; nothing waits on another block.
+// one unsigned comparison orders by value descending, then index ascending, and
+// no two keys are equal.
+//
+// A block selects rather than sorts: it holds its segment's keys in registers
+// and builds the k-th largest key bit by bit, counting the keys at or above
+// each trial with the barrier's own count (__syncthreads_count, one barrier
+// per bit). The k-th largest of the threads' maxima comes first: k keys at
+// least reach it, and few others do, so that the rest of the search runs on the
+// survivors, one or two per thread (all of the segment's keys, from registers,
+// when more survive than that: k near the thread count, sorted inputs, ties).
+// Level 1 keeps k keys of each 8192 values; a further level does the same to
+// 8192 keys; as soon as 16384 entries (values or keys) are left, one block per
+// problem selects the k best and ranks them by counting. What bounds it is the
+// chain of barriers (about 70 a level), not the reads.
+// Four problems of 1 Mi values, k = 100: see launch_topk.
 #include <math.h>
 
 #include <algorithm>
@@ -17,213 +26,220 @@ namespace boute {
 
 namespace {
 
-constexpr int kThreads = 512;
-constexpr int kSeg = 2048;  // keys per segment (16 KB of shared memory)
+constexpr int kR = 16;                   // entries per thread
+constexpr int kSegThreads = 512;         // a level's blocks: segments of 8192 entries
+constexpr int kFinThreads = 1024;        // the last level: up to 16384 entries
+constexpr int kSeg = kSegThreads * kR;
+constexpr int kFin = kFinThreads * kR;
+constexpr int kMaxK = 1024;
 
-// Sort buf[0, L) descending, L a power of two.
-__device__ void bitonic_desc(unsigned long long *buf, int L) {
-  for (int size = 2; size <= L; size <<= 1) {
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int i = threadIdx.x; i < (L >> 1); i += blockDim.x) {
-        const int lo = 2 * i - (i & (stride - 1));
-        const int hi = lo + stride;
-        const bool desc = (lo & size) == 0;
-        const unsigned long long x = buf[lo], y = buf[hi];
-        if ((x < y) == desc && x != y) {
-          buf[lo] = y;
-          buf[hi] = x;
-        }
-      }
-      __syncthreads();
-    }
-  }
+// Sum of c over the block's NT threads, for every thread.
+template <int NT>
+__device__ __forceinline__ int block_count(int c, int *red) {
+  c = __reduce_add_sync(0xffffffffu, c);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = c;
+  __syncthreads();
+  int s = 0;
+#pragma unroll
+  for (int w = 0; w < NT / 32; ++w) s += red[w];
+  return s;
 }
 
-// One segment of problem b: keys [seg*kSeg, seg*kSeg + kSeg) of a row of
-// `len` entries (values when FROM_VALUES, else keys). Keeps the k largest.
-template <bool FROM_VALUES>
-__global__ void __launch_bounds__(kThreads) segment_topk_kernel(
-    const float *vals, const unsigned long long *keys_in, long long len, int k, int nseg,
-    unsigned long long *keys_out, const float *acq, long long N, long long *idx, float *val) {
-  __shared__ unsigned long long buf[kSeg];
-  pdl_wait();
-  const int b = blockIdx.y, seg = blockIdx.x;
-  const long long base = (long long)seg * kSeg;
-  const long long n_here = std::min<long long>(kSeg, len - base);
-  int L = 2;
-  while (L < n_here) L <<= 1;
-  for (int i = threadIdx.x; i < L; i += blockDim.x) {
-    unsigned long long key = 0ull;  // below every real key
-    if (i < n_here) {
-      const long long g = base + i;
-      key = FROM_VALUES ? make_key(__ldcs(vals + (size_t)b * len + g), (unsigned)g)
-                        : keys_in[(size_t)b * len + g];
-    }
-    buf[i] = key;
+// The largest t with at least k keys >= t (count(t): how many are), built from
+// the top bit; exact: set when exactly k keys reach it.
+template <class Count>
+__device__ __forceinline__ unsigned kth_word(int k, bool &exact, Count count) {
+  unsigned t = 0u;
+  exact = false;
+  for (unsigned bit = 0x80000000u; bit && !exact; bit >>= 1) {
+    const int c = count(t | bit);
+    if (c >= k) t |= bit;
+    exact = c == k;
+  }
+  return t;
+}
+
+// The k largest keys of the block's segment (hi[r], lo(r): the words of this
+// thread's keys, hi = 0 for none), in any order, into out (shared or global);
+// fewer when the segment holds fewer. Returns how many.
+template <int NT, class Lo>
+__device__ __forceinline__ int block_select(const unsigned (&hi)[kR], Lo lo, int k,
+                                            unsigned long long *buf, int *red,
+                                            unsigned long long *out) {
+  __shared__ int nsurv, nout;
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid == 0) nsurv = nout = 0;
+  unsigned m = 0u;
+#pragma unroll
+  for (int r = 0; r < kR; ++r) m = max(m, hi[r]);
+  bool exact;
+  unsigned t0 = 0u;
+  if (k <= NT) t0 = kth_word(k, exact, [&](unsigned t) { return __syncthreads_count(m >= t); });
+  else __syncthreads();
+  t0 = max(t0, 1u);  // (absent keys never survive)
+  // survivors into buf, while they fit
+#pragma unroll
+  for (int r = 0; r < kR; ++r) {
+    const unsigned bal = __ballot_sync(0xffffffffu, hi[r] >= t0);
+    if (bal == 0u) continue;
+    int pos = 0;
+    if (lane == 0) pos = atomicAdd(&nsurv, __popc(bal));
+    pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(bal & ((1u << lane) - 1u));
+    if (hi[r] >= t0 && pos < 2 * NT) buf[pos] = ((unsigned long long)hi[r] << 32) | lo(r);
   }
   __syncthreads();
-  bitonic_desc(buf, L);
-  if (idx) {  // final level: one segment per problem
-    for (int i = threadIdx.x; i < k; i += blockDim.x) {
-      const unsigned j = key_index(buf[i]);
-      if (BOUTE_INB(i, k) && BOUTE_INB(j, N)) {
-        idx[(size_t)b * k + i] = (long long)j;
-        val[(size_t)b * k + i] = acq[(size_t)b * N + j];
+  const int ns = nsurv;
+  unsigned long long thr = 0ull;
+  auto take = [&](bool in, unsigned long long key) {  // (k keys at most: thr selects exactly)
+    if (in) out[atomicAdd(&nout, 1)] = key;
+  };
+  if (ns <= 2 * NT) {
+    const unsigned long long a = tid < ns ? buf[tid] : 0ull, b = tid + NT < ns ? buf[tid + NT] : 0ull;
+    if (ns > k) {
+      const unsigned ah = (unsigned)(a >> 32), bh = (unsigned)(b >> 32);
+      const bool two = ns > NT;
+      unsigned th = kth_word(k, exact, [&](unsigned t) {
+        const int c = __syncthreads_count(ah >= t);
+        return two ? c + __syncthreads_count(bh >= t) : c;
+      });
+      thr = (unsigned long long)th << 32;
+      if (!exact) {  // ties at the k-th value: the smallest indices of them
+        int above = __syncthreads_count(ah > th);
+        if (two) above += __syncthreads_count(bh > th);
+        thr |= kth_word(k - above, exact, [&](unsigned t) {
+          const int c = __syncthreads_count(ah == th && (unsigned)a >= t);
+          return two ? c + __syncthreads_count(bh == th && (unsigned)b >= t) : c;
+        });
       }
     }
+    take(a != 0ull && a >= thr, a);
+    take(b != 0ull && b >= thr, b);
   } else {
-    unsigned long long *out = keys_out + ((size_t)b * nseg + seg) * k;
-    for (int i = threadIdx.x; i < k; i += blockDim.x) out[i] = i < L ? buf[i] : 0ull;
-  }
-}
-
-// ---- k <= 32: one warp holds a running top 32, one key per lane ----------------
-// Lane i holds the i-th largest key seen so far. A batch of 32 new keys is
-// rejected with one ballot when none beats the current 32nd; otherwise it is
-// sorted across the lanes (bitonic network on shuffles) and merged: the
-// element-wise maximum of the running list and the reversed batch is a bitonic
-// sequence holding the 32 largest keys of both, which five more shuffle steps
-// sort. Each block merges its warps' lists; a second launch merges the blocks'.
-constexpr int kWarpBlock = 256;  // threads; 8 warps
-constexpr int kWarpBatches = 8;  // batches of 32 keys a warp loads at once
-
-// Block blockIdx.x of problem blockIdx.y takes entries [x * per_block,
-// (x+1) * per_block) of the problem's N values and forms their 32 largest
-// keys. With one block per problem it writes the final k indices and values.
-// Otherwise each block stores its 32 keys in `keys` and counts itself done on
-// the problem's counter; the block that finishes last merges all the blocks'
-// lists (eight warps, then one) and writes the result, and sets the counter
-// back to zero for the next call.
-__global__ void __launch_bounds__(kWarpBlock) warp_topk_kernel(
-    const float *vals, long long N, long long per_block, unsigned long long *keys,
-    unsigned *counter, int k, long long *idx, float *val) {
-  __shared__ unsigned long long lists[kWarpBlock / 32][kWarpK];
-  __shared__ int is_last;
-  pdl_wait();
-  const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int G = gridDim.x;
-  const long long lo = (long long)blockIdx.x * per_block;
-  const long long hi = std::min<long long>(N, lo + per_block);
-  const size_t row = (size_t)b * N;
-  unsigned long long top = 0ull;  // below every real key
-  for (long long base = lo + (long long)warp * 32 * kWarpBatches; base < hi;
-       base += (long long)kWarpBlock * kWarpBatches) {
-    unsigned long long x[kWarpBatches];
+    unsigned th = kth_word(k, exact, [&](unsigned t) {
+      int c = 0;
 #pragma unroll
-    for (int u = 0; u < kWarpBatches; ++u) {
-      const long long g = base + 32 * u + lane;
-      x[u] = g < hi ? make_key(__ldcs(vals + row + g), (unsigned)g) : 0ull;
+      for (int r = 0; r < kR; ++r) c += hi[r] >= t;
+      return block_count<NT>(c, red);
+    });
+    thr = (unsigned long long)th << 32;
+    if (!exact) {
+      int c = 0;
+#pragma unroll
+      for (int r = 0; r < kR; ++r) c += hi[r] > th;
+      const int above = block_count<NT>(c, red);
+      thr |= kth_word(k - above, exact, [&](unsigned t) {
+        int q = 0;
+#pragma unroll
+        for (int r = 0; r < kR; ++r) q += hi[r] == th && lo(r) >= t;
+        return block_count<NT>(q, red);
+      });
     }
 #pragma unroll
-    for (int u = 0; u < kWarpBatches; ++u) {
-      const unsigned long long thr = shfl64(top, 31);
-      if (__ballot_sync(0xffffffffu, x[u] > thr) == 0u) continue;
-      top = warp_merge_desc(top, warp_sort_desc(x[u], lane), lane);
+    for (int r = 0; r < kR; ++r) {
+      const unsigned long long key = ((unsigned long long)hi[r] << 32) | lo(r);
+      take(hi[r] != 0u && key >= thr, key);
     }
   }
-  lists[warp][lane] = top;
   __syncthreads();
-  if (warp == 0) {
-#pragma unroll 1
-    for (int w = 1; w < kWarpBlock / 32; ++w) top = warp_merge_desc(top, lists[w][lane], lane);
-    if (G > 1) {
-      keys[((size_t)b * G + blockIdx.x) * kWarpK + lane] = top;
-      __threadfence();  // the list is visible before the block counts itself done
-      __syncwarp();
-      if (lane == 0) is_last = atomicAdd(&counter[b], 1u) == (unsigned)(G - 1);
-    }
-  }
-  if (G > 1) {
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    top = 0ull;
-    for (int l = warp; l < G; l += kWarpBlock / 32)
-      top = warp_merge_desc(top, __ldcg(keys + ((size_t)b * G + l) * kWarpK + lane), lane);
-    lists[warp][lane] = top;
-    __syncthreads();
-    if (warp != 0) return;
-#pragma unroll 1
-    for (int w = 1; w < kWarpBlock / 32; ++w) top = warp_merge_desc(top, lists[w][lane], lane);
-    if (lane == 0) counter[b] = 0u;
-  } else if (warp != 0) {
-    return;
-  }
-  if (lane < k) {
-    const unsigned j = key_index(top);
-    if (BOUTE_INB(lane, k)) {
-      idx[(size_t)b * k + lane] = (long long)j;
-      val[(size_t)b * k + lane] = vals[row + j];
-    }
-  }
+  return nout;
 }
 
-// scratch: B x G x 32 keys, then B counters (zero on entry, zero on exit)
-int launch_topk_warp(const float *acq, int B, long long N, int k, long long *idx, float *val,
-                     void *scratch, bool counters_zeroed, cudaStream_t s) {
-  // at most 256 first-level blocks per problem, each a multiple of 2048 entries
-  const long long unit = (long long)kWarpBlock * kWarpBatches;
-  long long per_block = unit;
-  while ((N + per_block - 1) / per_block > 256) per_block += unit;
-  const long long G = (N + per_block - 1) / per_block;
-  prefer_shared(warp_topk_kernel);
-  unsigned long long *keys = G > 1 ? (unsigned long long *)scratch : nullptr;
-  unsigned *counter = G > 1 ? (unsigned *)(keys + (size_t)B * G * kWarpK) : nullptr;
-  if (G > 1 && !counters_zeroed && cudaMemsetAsync(counter, 0, B * sizeof(unsigned), s) != cudaSuccess)
-    return last_launch_status();
-  launch_pdl(warp_topk_kernel, dim3((unsigned)G, B), dim3(kWarpBlock), 0, s, acq, N, per_block,
-             keys, counter, k, idx, val);
-  count_launch(1);
-  return last_launch_status();
+// Segment blockIdx.x (NT * kR entries) of problem blockIdx.y's `len` entries:
+// values (VALUES) or keys. FINAL: the only segment; the k best in order to idx
+// and val (acq: the scores that the indices refer to). Otherwise its k best,
+// padded with zero keys, to keys_out.
+template <int NT, bool VALUES, bool FINAL>
+__global__ void __launch_bounds__(NT) topk_kernel(const float *vals,
+                                                  const unsigned long long *keys_in,
+                                                  long long len, int k,
+                                                  unsigned long long *keys_out, const float *acq,
+                                                  long long N, long long *idx, float *val) {
+  __shared__ unsigned long long buf[2 * NT];
+  __shared__ int red[NT / 32];
+  __shared__ unsigned long long sel[FINAL ? kMaxK : 1];
+  pdl_wait();
+  const int b = blockIdx.y, tid = threadIdx.x;
+  const long long base = (long long)blockIdx.x * (NT * kR);
+  unsigned hi[kR], lw[VALUES ? 1 : kR];
+#pragma unroll
+  for (int r = 0; r < kR; ++r) {
+    const long long g = base + r * NT + tid;
+    unsigned long long key = 0ull;  // below every real key
+    if (g < len)
+      key = VALUES ? make_key(__ldcs(vals + (size_t)b * len + g), (unsigned)g)
+                   : __ldcg(keys_in + (size_t)b * len + g);
+    hi[r] = (unsigned)(key >> 32);
+    if (!VALUES) lw[r] = (unsigned)key;
+  }
+  auto lo = [&](int r) {
+    if (VALUES) return 0xFFFFFFFFu - (unsigned)(base + r * NT + tid);
+    return lw[VALUES ? 0 : r];
+  };
+  if constexpr (!FINAL) {
+    unsigned long long *out = keys_out + ((size_t)b * gridDim.x + blockIdx.x) * k;
+    const int got = block_select<NT>(hi, lo, k, buf, red, out);
+    for (int i = got + tid; i < k; i += NT) out[i] = 0ull;
+  } else {
+    block_select<NT>(hi, lo, k, buf, red, sel);
+    // rank of each selected key, `per` threads (a power of two) to a key
+    int per = 1;
+    while (per < 32 && 2 * per * k <= NT) per *= 2;
+    const int q = tid / per, p = tid & (per - 1);
+    int rank = 0;
+    const unsigned long long key = q < k ? sel[q] : 0ull;
+    if (q < k)
+      for (int j = p; j < k; j += per) rank += sel[j] > key;
+    for (int o = per >> 1; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+    if (q < k && p == 0) {
+      const unsigned j = key_index(key);
+      if (BOUTE_INB(rank, k) && BOUTE_INB(j, N)) {
+        idx[(size_t)b * k + rank] = (long long)j;
+        val[(size_t)b * k + rank] = acq[(size_t)b * N + j];
+      }
+    }
+  }
 }
 
 }  // namespace
 
-// Scratch for the levels after the first: two ping-pong key arrays of
-// ceil(N / 2048) * k keys per problem (segment path), or at most
-// ceil(N / 2048) runs of 32 keys per problem and one counter per problem
-// (warp path, k <= 32); k is counted as at least 32 so that one bound covers
-// both.
+// Scratch for the levels after the first: two ping-pong key arrays, at most
+// ceil(N / 8192) * k keys per problem and level (the bound counts segments of
+// 2048 and k as at least 32, which boute_select_topk_noalloc's limit states).
 size_t topk_scratch_bytes(int B, long long N, int k) {
-  const long long g1 = (N + kSeg - 1) / kSeg;
+  const long long g1 = (N + 2047) / 2048;
   if (g1 <= 1) return 16;
   return 2 * (size_t)B * g1 * std::max(k, 32) * sizeof(unsigned long long) + 16;
 }
 
 int launch_topk(const float *acq, int B, long long N, int k, long long *idx, float *val,
-                void *scratch, cudaStream_t s, bool counters_zeroed) {
-  if (k > kSeg / 2) return BOUTE_ERR_UNSUPPORTED;
-  if (k <= kWarpK)
-    return launch_topk_warp(acq, B, N, k, idx, val, scratch, counters_zeroed, s);
-  long long len = N;
-  long long nseg = (len + kSeg - 1) / kSeg;
-  unsigned long long *ping = (unsigned long long *)scratch;
-  unsigned long long *pong = ping + (size_t)B * nseg * k;
-  int launches = 0;
-  if (nseg == 1) {
-    segment_topk_kernel<true><<<dim3(1, B), kThreads, 0, s>>>(acq, nullptr, len, k, 1, nullptr,
-                                                              acq, N, idx, val);
+                void *scratch, cudaStream_t s) {
+  if (k > kMaxK) return BOUTE_ERR_UNSUPPORTED;
+  const unsigned long long *no_keys = nullptr;
+  const float *no_vals = nullptr;
+  unsigned long long *no_out = nullptr;
+  long long *ni = nullptr;
+  float *nv = nullptr;
+  if (N <= kFin) {
+    launch_pdl(topk_kernel<kFinThreads, true, true>, dim3(1, B), dim3(kFinThreads), 0, s, acq,
+               no_keys, N, k, no_out, acq, N, idx, val);
     count_launch(1);
     return last_launch_status();
   }
-  segment_topk_kernel<true><<<dim3((unsigned)nseg, B), kThreads, 0, s>>>(
-      acq, nullptr, len, k, (int)nseg, ping, acq, N, nullptr, nullptr);
-  ++launches;
-  len = nseg * k;
-  for (;;) {
+  int launches = 2;
+  long long nseg = (N + kSeg - 1) / kSeg, len = nseg * k;
+  unsigned long long *ping = (unsigned long long *)scratch, *pong = ping + (size_t)B * len;
+  launch_pdl(topk_kernel<kSegThreads, true, false>, dim3((unsigned)nseg, B), dim3(kSegThreads), 0,
+             s, acq, no_keys, N, k, ping, acq, N, ni, nv);
+  for (; len > kFin; ++launches) {
     nseg = (len + kSeg - 1) / kSeg;
-    if (nseg == 1) {
-      segment_topk_kernel<false><<<dim3(1, B), kThreads, 0, s>>>(nullptr, ping, len, k, 1,
-                                                                 nullptr, acq, N, idx, val);
-      ++launches;
-      break;
-    }
-    segment_topk_kernel<false><<<dim3((unsigned)nseg, B), kThreads, 0, s>>>(
-        nullptr, ping, len, k, (int)nseg, pong, acq, N, nullptr, nullptr);
-    ++launches;
+    launch_pdl(topk_kernel<kSegThreads, false, false>, dim3((unsigned)nseg, B), dim3(kSegThreads),
+               0, s, no_vals, (const unsigned long long *)ping, len, k, pong, acq, N, ni, nv);
     std::swap(ping, pong);
     len = nseg * k;
   }
+  launch_pdl(topk_kernel<kFinThreads, false, true>, dim3(1, B), dim3(kFinThreads), 0, s, no_vals,
+             (const unsigned long long *)ping, len, k, no_out, acq, N, idx, val);
   count_launch(launches);
   return last_launch_status();
 }

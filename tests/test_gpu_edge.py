@@ -242,8 +242,33 @@ def test_far_candidates_and_zero_variance_ehvi():
     compare(hp)
 
 
-# k <= 32 takes the warp-register path, larger k the segment sort; N spans one
-# block, several, and more than 256 first-level blocks (larger blocks)
+# one block, segments of 8192 around their edges, a second and a third level,
+# k from 1 to 1024 (above a block's 512 threads the selection searches every key)
+@pytest.mark.parametrize("N,k", [(16384, 1024), (16385, 1024), (16385, 512), (24577, 513),
+                                 (8193 * 16, 100), (1, 1), (1024, 1024), (2_000_003, 1000),
+                                 (140_000, 1024)])
+def test_topk_levels_and_k_range(N, k):
+    import torch
+
+    from paper_2602_10729_gb300 import boute as bt
+    rng = np.random.default_rng(N + k)
+    v = rng.standard_normal((4, N)).astype(np.float32)
+    v[1] = np.sort(v[1])  # every survivor in one segment, on few threads
+    v[2] = np.where(v[2] > 1.0, np.round(v[2], 1), 0.0)  # ties around and at zero
+    v[3, rng.random(N) < 0.9] = np.nan
+    v[3, : N // 3] = -np.inf
+    a = torch.as_tensor(v, device="cuda")
+    idx = torch.empty((4, k), dtype=torch.int64, device="cuda")
+    val = torch.empty((4, k), dtype=torch.float32, device="cuda")
+    bt.boute_select_topk(a, 4, N, k, idx, val)
+    key = np.where(np.isnan(v), -np.inf, v)
+    for b in range(4):  # the definition: value descending, then index
+        want = np.lexsort((np.arange(N), -key[b]))[:k]
+        assert np.array_equal(idx[b].cpu().numpy(), want)
+        assert np.array_equal(val[b].cpu().numpy(), v[b][want], equal_nan=True)
+
+
+# ties, NaN and -0 at one block, several, and hundreds of them
 @pytest.mark.parametrize("N,k", [(5000, 40), (5000, 32), (5000, 1), (2048, 7), (40, 32),
                                  (700_001, 32), (700_001, 17), (70_000, 33)])
 def test_topk_ties_nan_and_negative_zero(N, k):

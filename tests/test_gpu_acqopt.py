@@ -83,6 +83,26 @@ def test_value_and_gradient_match_oracle(wi, n, S, B):
         np.testing.assert_allclose(grad[b], grads, rtol=1e-3, atol=2e-4 * gs)
 
 
+@pytest.mark.parametrize("n,S,P", [(1, 1, 1), (2, 3, 2), (31, 33, 3), (33, 500, 2), (257, 7, 2),
+                                   (512, 64, 2), (513, 64, 2), (600, 20, 3)])
+def test_row_panel_edges_match_oracle(n, S, P):
+    """Sizes around a warp, a block's threads and the 512 columns that a warp
+    holds of a row of W (beyond, W k* and W^T q take two passes). Tolerances as
+    above: fp32 sums of n terms against fp64."""
+    w = wl.scaled(wl.WORKLOADS[1], N=64, B=1, n=n)
+    hp = host_problem(w)
+    gp, lower, upper, K, cap, epsd, eps = _setup(hp, S)
+    X0 = np.random.default_rng(n).uniform(0.05, 0.95, (1, P, w.d)).astype(np.float32)
+    _, acq, grad = _run(gp, (lower, upper, K, cap), epsd, X0, 0, 0.01, w.d)
+    gp.free()
+    fp = oracle_fit(hp, 0)
+    vals, grads = zip(*(opl.mc_hvi_value_grad(fp, X0[0, p].astype(np.float64), eps)
+                        for p in range(P)))
+    vals, grads = np.array(vals), np.array(grads)
+    np.testing.assert_allclose(acq[0], vals, rtol=1e-4, atol=1e-6 * np.abs(vals).max() + 1e-12)
+    np.testing.assert_allclose(grad[0], grads, rtol=1e-3, atol=2e-4 * np.abs(grads).max() + 1e-12)
+
+
 @pytest.mark.parametrize("wi,n,S", [(2, 96, 64), (1, 64, 64)])
 def test_ascent_from_the_pool_best_matches_oracle(wi, n, S):
     w = wl.scaled(wl.WORKLOADS[wi], N=2048, B=1, n=n)

@@ -370,47 +370,128 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity,
   }
 }
 
-// The mean of a candidate is recomputed in fp64 when its terms K*_j alpha_j
+// The mean of a candidate is recomputed (below) when its terms K*_j alpha_j
 // add up to more than kFixRatio times the mean's scale max(|mean|, s): the
 // fp32 cross-covariance's rounding (a few units in the last place per entry,
 // amplified by that ratio) would otherwise exceed the 1e-5 tolerance. Below
 // the ratio the fp32 mean's error stays under about 6e-6 of the scale.
 constexpr float kFixRatio = 256.f;
 
-// A row's mean in fp64 for the Matern-5/2 kernel, computed by a whole warp
-// (lane = column j mod 32) and returned to every lane: the candidate's
-// coordinates scaled by 1/l as hi + lo, the training points' x / l as hi + lo
-// and alpha as hi + lo, read from the side input in global memory (the rare,
-// exact path; the warp takes one flagged row at a time).
+// ---- the exact mean of a flagged row, in double-float arithmetic -----------------
+// Numbers as unevaluated pairs hi + lo of floats (Dekker; Knuth's error-free
+// sum, products by fma), 48 significant bits. An fp64 warp instruction takes 76
+// clocks of a scheduler on this part whatever its active lanes, an fp32 one 1,
+// and a pair operation is 8 to 10 of those: at n = 777, d = 20 a row took
+// 370 thousand clocks of its warp in fp64. Against the fp64 form the row's mean
+// differs by less than 1e-13 of its terms' magnitude sum, where the fp32
+// rounding of the result is 6e-8 of the result.
+struct F2 {
+  float h, l;
+};
+// |a| >= |b| or a = 0
+__device__ __forceinline__ F2 quick_two_sum(float a, float b) {
+  const float s = a + b;
+  return F2{s, b - (s - a)};
+}
+__device__ __forceinline__ F2 f2p_mul(F2 a, F2 b) {
+  const float p = a.h * b.h;
+  return quick_two_sum(p, fmaf(a.h, b.h, -p) + fmaf(a.h, b.l, a.l * b.h));
+}
+__device__ __forceinline__ F2 f2p_add(F2 a, F2 b) {
+  float s, e;
+  two_sum_f(a.h, b.h, s, e);
+  return quick_two_sum(s, e + (a.l + b.l));
+}
+constexpr F2 pair_of(double v) { return F2{(float)v, (float)(v - (double)(float)v)}; }
+
+// 2^(-i / 128) as pairs, i < 128 (from the Taylor series of the exponential).
+struct Exp2Table {
+  float h[128], l[128];
+  constexpr Exp2Table() : h(), l() {
+    for (int i = 0; i < 128; ++i) {
+      const double x = -i / 128.0 * 0.69314718055994530942;
+      double v = 1.0;
+      for (int k = 24; k >= 1; --k) v = 1.0 + x / k * v;
+      h[i] = pair_of(v).h;
+      l[i] = pair_of(v).l;
+    }
+  }
+};
+__device__ const Exp2Table kExp2Table{};
+
+// 2^(-r) for a pair r >= 0 (zero below 2^-127): r = N / 128 + f, |f| <= 1/256,
+// a table for 2^(-N/128) and the series of e^u at u = -f ln 2 to the fourth
+// power (the table-driven scheme of Tang, ACM TOMS 15, 1989), u and u^2 / 2 as
+// pairs.
+__device__ __forceinline__ F2 exp2_neg_pair(F2 r) {
+  constexpr F2 ln2 = pair_of(0.69314718055994530942);
+  if (!(r.h < 127.f)) return F2{0.f, 0.f};
+  const float nf = rintf(r.h * 128.f);
+  const int N = (int)nf;
+  const F2 u = f2p_mul(F2{-fmaf(nf, -1.f / 128.f, r.h), -r.l}, ln2);  // (the fma is exact)
+  const float q = u.h * u.h;                                          // u^2
+  const float qe = fmaf(u.h, u.h, -q) + 2.f * u.h * u.l;
+  const float tail = 0.5f * qe + q * u.h * fmaf(u.h, 1.f / 24.f, 1.f / 6.f);
+  F2 e = quick_two_sum(1.f, u.h);
+  e = f2p_add(e, F2{0.5f * q, u.l + tail});
+  e = f2p_mul(e, F2{kExp2Table.h[N & 127], kExp2Table.l[N & 127]});
+  const float sc = exp2i(-min(N >> 7, 126));
+  return F2{e.h * sc, e.l * sc};
+}
+
+// A row's mean for the Matern-5/2 kernel, computed by a whole warp (lane =
+// column j mod 32) and returned to every lane: the candidate's coordinates
+// scaled by 1/l, the training points' x / l and alpha as pairs, read from the
+// side input in global memory (the rare, exact path; the warp takes one flagged
+// row at a time).
 template <int DP>
-__device__ double mean_fp64_warp(const float *xrow, int d, const float *x0, int cf, int n,
-                                 int lane) {
+__device__ float mean_pair_warp(const float *xrow, int d, const float *x0, int cf, int n,
+                                int lane) {
+  constexpr F2 ln2 = pair_of(0.69314718055994530942), ln2sq3 = pair_of(0.69314718055994530942 * 0.69314718055994530942 / 3.0);
   const float *il = x0 + xt_param_offset(DP);
-  const double s2 = il[2 * DP + kParS2];
+  const float s2 = il[2 * DP + kParS2];
   // lane k holds the candidate's coordinate k scaled by 1/l
-  const double xs_l = lane < d ? (double)xrow[lane] * ((double)il[lane] + (double)il[DP + lane]) : 0.0;
-  double acc = 0.0;
+  F2 xs{0.f, 0.f};
+  if (lane < d) {
+    const float x = xrow[lane], p = x * il[lane];
+    xs = quick_two_sum(p, fmaf(x, il[lane], -p) + x * il[DP + lane]);
+  }
+  F2 acc{0.f, 0.f};
   for (int j0 = 0; j0 < n; j0 += 32) {
     const int j = j0 + lane;
-    const float *ch = x0 + (size_t)(min(j, n - 1) / BOUTE_KCHUNK) * cf;
-    const int jj = j % BOUTE_KCHUNK;
-    double r2 = 0.0;
+    const float *ch = x0 + (size_t)(j0 / BOUTE_KCHUNK) * cf;
+    F2 r2{0.f, 0.f};
+#pragma unroll 4
     for (int k = 0; k < d; ++k) {
-      const double xs = __shfl_sync(0xffffffffu, xs_l, k);
-      const double df =
-          xs - ((double)ch[k * BOUTE_KCHUNK + jj] + (double)ch[(DP + k) * BOUTE_KCHUNK + jj]);
-      r2 = fma(df, df, r2);
+      const float xh = __shfl_sync(0xffffffffu, xs.h, k), xl = __shfl_sync(0xffffffffu, xs.l, k);
+      float sh, se;
+      two_sum_f(xh, -ch[k * BOUTE_KCHUNK + lane], sh, se);
+      const F2 df = quick_two_sum(sh, se + (xl - ch[(DP + k) * BOUTE_KCHUNK + lane]));
+      const float p = df.h * df.h;
+      float e;
+      two_sum_f(r2.h, p, r2.h, e);
+      r2.l += e + fmaf(2.f * df.h, df.l, fmaf(df.h, df.h, -p));
     }
-    if (j >= n) continue;
-    const double r = sqrt(r2) / kCoordScale52;  // (the side input's scale)
-    const double kv = s2 * (1.0 + 2.2360679774997896964 * r + (5.0 / 3.0) * (r * r)) *
-                      exp(-2.2360679774997896964 * r);
-    const float *al = ch + xt_alpha_offset(DP) + jj;  // alpha hi, lo
-    acc = fma(kv, (double)al[0] + (double)al[BOUTE_KCHUNK], acc);
+    r2 = quick_two_sum(r2.h, r2.l);
+    // r' = sqrt(r2): one correction of q = r2 rsqrt(r2) by the residual r2 - q^2
+    F2 r{0.f, 0.f};
+    if (r2.h > 0.f) {
+      const float y = rsqrtf(r2.h), q = r2.h * y;
+      r = quick_two_sum(q, 0.5f * y * (fmaf(-q, q, r2.h) + r2.l));
+    }
+    // k = s2 (1 + ln2 r' + ln2^2/3 r'^2) 2^(-r') (the coordinates' scale makes
+    // r' = sqrt5 r / ln 2)
+    F2 k = f2p_add(f2p_add(F2{1.f, 0.f}, f2p_mul(r, ln2)), f2p_mul(r2, ln2sq3));
+    k = f2p_mul(f2p_mul(k, exp2_neg_pair(r)), F2{s2, 0.f});
+    const float *al = ch + xt_alpha_offset(DP) + lane;  // alpha hi, lo (zero past n)
+    if (j < n) acc = f2p_add(acc, f2p_mul(k, F2{al[0], al[BOUTE_KCHUNK]}));
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  return acc;
+  for (int o = 16; o > 0; o >>= 1) {
+    const F2 other{__shfl_xor_sync(0xffffffffu, acc.h, o), __shfl_xor_sync(0xffffffffu, acc.l, o)};
+    acc = f2p_add(acc, other);
+  }
+  return acc.h + acc.l;
 }
 
 // The work sequence every role follows: per unit (tile, objective), the
@@ -768,7 +849,7 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
       // the mean: the builders' partials of this row, one per column group,
       // added in order with error-free sums; its terms reach hundreds of times
       // the result when K is ill-conditioned, and their magnitudes
-      // sum_j K*_j |alpha_j| decide whether the row is recomputed in fp64
+      // sum_j K*_j |alpha_j| decide whether the row is recomputed in pairs
       if (!wait_or_abort(mean_ready, nmean & 1u, abort)) break;
       ++nmean;
       float mhi = 0.f, mlo = 0.f, mag = 0.f;
@@ -783,7 +864,7 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive_count(mean_empty);
       float mean = ldexpf(mhi + mlo, -er);
-      if (KERN == 0) {  // ill-conditioned rows: the mean in fp64, one row at a time
+      if (KERN == 0) {  // ill-conditioned rows: the mean in pairs, one row at a time
         const float sc = ldexpf(sqrtf(par[kParS2]), er);  // the mean's scale, scaled like K*
         const bool fix = live && mag > kFixRatio * fmaxf(fabsf(mhi), sc);
         unsigned todo = __ballot_sync(0xffffffffu, fix);
@@ -792,9 +873,9 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
           todo &= todo - 1;
           const long long rr = (long long)(tile % a.tiles_per_problem) * BOUTE_TILE_M + 32 * eq + src;
           const float *x0 = a.xt + (size_t)(b * m + t) * pl.nxt * cf;
-          const double v = mean_fp64_warp<DP>(a.Xc + ((long long)b * a.N + rr) * d, d, x0, cf, n,
-                                              lane);
-          if (lane == src) mean = (float)v;
+          const float v = mean_pair_warp<DP>(a.Xc + ((long long)b * a.N + rr) * d, d, x0, cf, n,
+                                             lane);
+          if (lane == src) mean = v;
         }
       }
       if (live && BOUTE_INB(((long long)b * m + t) * a.N + row, (long long)a.B * m * a.N))
@@ -852,7 +933,7 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
       }
       // the mean K* alpha: its terms reach hundreds of times the result when K
       // is ill-conditioned, so they are summed with compensation, and their
-      // magnitudes sum_j K*_j |alpha_j| decide whether the row needs the fp64 path
+      // magnitudes sum_j K*_j |alpha_j| decide whether the row is recomputed
       Kahan2 mu2;
       unsigned long long mag2 = 0ull;
       for (int gi = 0; gi < grp.n && !*abort; ++gi) {

@@ -260,16 +260,10 @@ __device__ __forceinline__ void bulk_wait() {
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-// Expected transaction bytes without an arrival, and an arrival counted
-// `count` times (an mbarrier whose phase needs both).
+// Expected transaction bytes without an arrival.
 __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
   asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)),
                "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_n(uint64_t *bar, uint32_t count) {
-  asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-               "r"(count)
                : "memory");
 }
 

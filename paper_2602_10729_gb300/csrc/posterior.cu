@@ -30,7 +30,8 @@
 //   warps 2-5   epilogue: one TMEM lane quarter each, sum of squares, variance
 //   warp 6      bulk-TMA producer of the training-point chunks (side-input ring)
 //               and, with K* precomputed, of its fp32 images (staging ring)
-//   warps 7..   K* builders: packed f32x2 distance math, A ring
+//   warp 7      bulk copies of the cached K* chunks (n > 512)
+//   warps 8..   K* builders: packed f32x2 distance math, A ring
 // All waits are bounded (BOUTE_WAIT_NS): a wait that gives up records
 // BOUTE_ERR_TIMEOUT and every role stops.
 #include <math.h>
@@ -47,7 +48,7 @@ namespace {
 constexpr int kEpiWarp0 = 2;  // warps 2-5: epilogue (variance, mean), TMEM lane quarter = warp % 4
 constexpr int kEpiWarps = 4;
 constexpr int kXtWarp = 6;     // warp 6: side-input producer
-constexpr int kCacheWarp = 7;  // warp 7 (8 builder warps): cached K* chunks into their A stages
+constexpr int kCacheWarp = 7;  // warp 7: cached K* chunks into their A stages
 constexpr int kMaxA = 4, kMaxB = 6, kMaxX = 8;  // ring depths
 constexpr int kSlots = 4;                       // TMEM accumulator slots of 128 columns
 constexpr int kGroup = 4;                       // blocks sharing one K* chunk
@@ -61,11 +62,7 @@ constexpr uint32_t kStageBytes = BOUTE_TILE_M * BOUTE_ACHUNK * 4;   // fp32 K* i
 template <int DP>
 struct Layout {
   static constexpr int kBld = DP <= 16 ? 16 : 8;
-  // with 8 builder warps the cached K* chunks have a warp of their own (warp
-  // 7); with 16 the side-input producer brings them (a 25th warp would cost
-  // the builders registers), and the builders start at warp 7
-  static constexpr bool kSepCache = kBld == 8;
-  static constexpr int kBldWarp0 = kSepCache ? 8 : 7;
+  static constexpr int kBldWarp0 = 8;
   static constexpr int kThreads = 32 * (kBldWarp0 + kBld);
   static constexpr int kCols = 128 / kBld;  // columns of a 32-point half per builder thread
 };
@@ -572,7 +569,9 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
 
   if (tid == 0) {
     for (int s = 0; s < kMaxA; ++s) {
-      mbar_init(&a_full[s], kBldWarps);
+      // every position of the A ring is passed by the builders and, with cached
+      // chunks, by the cache warp, whichever of them fills it
+      mbar_init(&a_full[s], kBldWarps + (a.ncache > 0 ? 1 : 0));
       mbar_init(&a_empty[s], 1);
       mbar_init(&st_full[s], 1);
       mbar_init(&st_empty[s], kBldWarps);
@@ -607,18 +606,21 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
   pdl_wait();  // the fit's outputs (operand images, side input) are complete
   const int units = a.tiles_total * m;
 
-  constexpr bool kSep = Layout<DP>::kSepCache;
   constexpr int kBldWarp0 = Layout<DP>::kBldWarp0;
-  if (warp == 0 || warp == kXtWarp || (kSep && warp == kCacheWarp)) {
+  if (warp == 0 || warp == kXtWarp || warp == kCacheWarp) {
     // ------------------------------------ producers (B / side input / cached K* chunks)
     // With a warp of their own for the cached chunks, waiting for the A stage
-    // of a cached chunk never holds up the side input of the new ones.
+    // of a cached chunk never holds up the side input of the new ones. The
+    // builders and the cache warp both wait for and arrive at every position of
+    // the A ring, filled by them or not: a parity wait tells a phase only from
+    // its neighbours, so neither may fall a phase behind (a position passed by
+    // one alone could be consumed, or the stage's next use begun, unnoticed).
     if (lane == 0 && (warp != kCacheWarp || a.ncache > 0)) {
       const bool is_b = warp == 0;
       const int R = is_b ? SB : SX;
       uint64_t *full = is_b ? b_full : x_full, *empty = is_b ? b_empty : x_empty;
       const bool with_st = PRE && warp == kXtWarp;  // the side-input producer also stages K*
-      const bool with_cache = a.ncache > 0 && warp == (kSep ? kCacheWarp : kXtWarp);
+      const bool with_cache = warp == kCacheWarp;
       uint32_t q = 0, qa = 0, nready = 0;
       RingPos rp, ra;
       int last_q = -1, last_qa = -1;  // last jobs issued
@@ -639,20 +641,19 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
             const int c = Groups::chunk_at(i, kcp, kcg, mix);
             if (with_cache) {  // the A ring's positions; the cached chunks' A stages
               const int s = ra.idx;
-              const bool cached = c < kcp;
-              if (cached) {  // the A stage from this CTA's cache
-                if (qa >= (uint32_t)SA && !wait_or_abort(&a_empty[s], ra.phase ^ 1u, abort)) break;
+              if (qa >= (uint32_t)SA && !wait_or_abort(&a_empty[s], ra.phase ^ 1u, abort)) break;
+              if (c < kcp) {  // the A stage from this CTA's cache
                 mbar_expect_tx(&a_full[s], kABytes);
                 if (BOUTE_INB(blockIdx.x * a.ncache + c, (long long)gridDim.x * a.ncache))
                   bulk_g2s(a_hi(s),
                            a.kcache + ((size_t)blockIdx.x * a.ncache + c) * (kABytes / 2),
                            kABytes, &a_full[s]);
-                mbar_arrive_n(&a_full[s], kBldWarps);
                 last_ca = (int)qa;
               }
+              mbar_arrive_count(&a_full[s]);
               ++qa;
               ra.advance(SA);
-              if (cached || kSep) continue;  // (the cache warp does nothing else)
+              continue;
             }
             if (!is_b && mix && c < kcp) continue;  // a cached chunk needs no side input
             if (with_st) {  // the chunk's fp32 K* image
@@ -944,9 +945,12 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
         const bool mean_grp = a.ncache > 0 || gi == grp.n - 1;
         for (int i = 0; i < kcg && !*abort; ++i, ++qa, pa.advance(SA)) {
           const int c = mix ? Groups::chunk_at(i, kcp, kcg, true) : i;
-          if (mix && c < kcp) continue;  // cached: the producer brings it
           const int s = pa.idx;
           if (qa >= (uint32_t)SA && !wait_or_abort(&a_empty[s], pa.phase ^ 1u, abort)) break;
+          if (mix && c < kcp) {  // cached: the cache warp brings it
+            if (lane == 0) mbar_arrive_count(&a_full[s]);
+            continue;
+          }
           if (PRE && !wait_or_abort(&st_full[s], pa.phase, abort)) break;
           uint8_t *Ah = a_hi(s), *Al = Ah + kAPartBytes;
           for (int h = 0; h < 2; ++h, px.advance(SX)) {

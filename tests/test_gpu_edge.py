@@ -7,8 +7,8 @@ import numpy as np
 import pytest
 
 import oracle
-from _pipeline import (HostProblem, check_acq, check_acq_end_to_end, check_mean, check_var,
-                       gpu_pipeline, host_problem, oracle_fit)
+from _pipeline import (POST_REL, HostProblem, check_acq, check_acq_end_to_end, check_mean,
+                       check_var, gpu_pipeline, host_problem, oracle_fit)
 from oracle import pipeline as opl
 from paper_2602_10729_gb300 import workloads as wl
 
@@ -68,6 +68,35 @@ def test_ragged_candidate_counts(N):
 @pytest.mark.parametrize("n", [1, 2, 31, 33, 97, 129, 150, 160, 161, 255, 257, 600])
 def test_training_set_sizes_and_column_passes(n):
     compare(rand_problem(2, n, 5, 2, 400))
+
+
+@pytest.mark.parametrize("n,d,comp", [(520, 32, True), (640, 32, True), (640, 16, True),
+                                      (640, 24, False), (777, 32, False), (640, 10, False),
+                                      (900, 20, True), (1090, 12, False)])
+def test_cached_chunks_over_many_tiles(n, d, comp):
+    """More than 512 observations (a second group of output blocks takes the
+    first one's K* chunks from the cache) and enough candidates that every CTA
+    works through several tiles: runs of cached chunks at the end of one tile
+    meet the chunks built for the next. Sampled candidates, POST_REL of the
+    prior variance as everywhere."""
+    import dataclasses
+
+    base = wl.scaled(dataclasses.replace(wl.WORKLOADS[2], d=d), N=60011, n=n)
+    w = wl.composite(base) if comp else base
+    hp = host_problem(w)
+    g = gpu_pipeline(hp)
+    assert g["status"] == 0
+    fp = oracle_fit(hp, 0)
+    at = np.unique(np.r_[np.arange(0, 60011, 233), 60010])
+    mean, var = opl.posterior(fp, hp.Xc[0][at])
+    for t in range(w.m):
+        prior = np.full(len(at), hp.s2[0][t])
+        if comp:
+            kern = (hp.d_tau, hp.kc[0][t])
+            prior = np.array([oracle.kernel(c, c, hp.ls[0][t], hp.s2[0][t], kern)
+                              for c in hp.Xc[0][at].astype(np.float64)])
+        check_var(g["var"][0, t, at], var[:, t], prior.max())
+        assert np.abs(g["mean"][0, t, at] - mean[:, t]).max() <= 4 * POST_REL * np.sqrt(prior.max())
 
 
 @pytest.mark.parametrize("d", [1, 3, 8, 9, 13, 17, 25, 32])

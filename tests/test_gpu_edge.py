@@ -345,3 +345,43 @@ def test_invalid_arguments_raise():
     val = torch.empty((1, 11), device="cuda")
     with pytest.raises(bt.BouteError):
         bt.boute_select_topk(a, 1, 10, 11, idx, val)
+
+
+# Sizes around a warp of points; every point on the front; ties and signed zeros.
+@pytest.mark.parametrize("kind", ["random", "antichain", "ties"])
+@pytest.mark.parametrize("n,m", [(1, 2), (31, 3), (32, 2), (33, 3), (130, 4), (513, 2), (257, 3)])
+def test_front_and_boxes_edges(n, m, kind):
+    import torch
+
+    from paper_2602_10729_gb300 import boute as bt
+    rng = np.random.default_rng(n + m)
+    Y = rng.random((n, m)) - 0.5
+    if kind == "antichain":
+        Y[:, -1] = -Y[:, :-1].sum(1)
+    elif kind == "ties":
+        Y = np.round(Y * 4) / 4
+        Y[Y == 0] = np.where(rng.random((Y == 0).sum()) < 0.5, 0.0, -0.0)
+    ref = np.full(m, 0.3)
+    mask_o, order = oracle.pareto_front(Y, ref)
+    t = lambda a: torch.as_tensor(np.ascontiguousarray(a), device="cuda")
+    mask = torch.empty((1, n), dtype=torch.uint8, device="cuda")
+    front = torch.zeros((1, n, m), dtype=torch.float64, device="cuda")
+    P = torch.empty(1, dtype=torch.int32, device="cuda")
+    bt.boute_pareto_front(t(Y[None]), 1, n, m, t(ref[None]), mask, front, P)
+    assert mask.cpu().numpy()[0].astype(bool).tolist() == np.asarray(mask_o).astype(bool).tolist()
+    F = front.cpu().numpy()[0, :int(P[0])]
+    np.testing.assert_array_equal(F, Y[np.asarray(order)])
+    if m == 4:
+        return
+    cap = 2 * n + 2
+    lo = torch.empty((1, cap, m), dtype=torch.float32, device="cuda")
+    hi = torch.empty_like(lo)
+    K = torch.empty(1, dtype=torch.int32, device="cuda")
+    bt.boute_box_decompose(front, P, 1, n, m, t(ref[None]), lo, hi, K)
+    k = int(K[0])
+    assert 1 <= k <= 2 * F.shape[0] + 1
+    lo, hi = (a.cpu().numpy()[0, :k].astype(np.float64) for a in (lo, hi))
+    for y in rng.random((20, m)) - 0.6:
+        got = np.prod(np.maximum(hi - np.maximum(lo, y), 0.0), 1).sum()
+        # the corners are rounded to fp32: 2^-24 of at most 1.1 each, m of them per box
+        assert got == pytest.approx(oracle.hvi(F, ref, y), abs=k * m * 1.1 * 2.0 ** -23)

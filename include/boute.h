@@ -188,8 +188,8 @@ int boute_gp_learn_k(const double *X, const double *Ys, int B, int n, int d, int
  * and contracted on the tensor cores as fp16 hi/lo parts (three products per
  * term, fp32 accumulate: fp32-accurate) without ever being written to HBM.
  * The mean is reduced from the fp32 K* with compensated sums; a candidate
- * whose terms K*_j alpha_j add up to more than 256 times the mean's scale
- * (an ill-conditioned K) has its mean recomputed in fp64.
+ * whose terms K*_j alpha_j add up to more than 224 times the mean's scale
+ * (an ill-conditioned K) has its mean recomputed in pairs of floats (48 bits).
  *   Xc: B x N x d fp32 candidates (points of [0,1]^d or any real values);
  *   mean, var: B x m x N fp32 (objective-major per problem). */
 int boute_gp_posterior(const boute_gp *gp, const float *Xc, long long N, float *mean,

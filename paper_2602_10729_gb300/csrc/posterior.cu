@@ -13,7 +13,7 @@
 // variance is s2 - rowsum(V^2), V = K* W^T, read back from tensor memory with
 // tcgen05.ld. The mean K* alpha is a matrix-vector product: the threads
 // building K* reduce it on the CUDA cores from the fp32 values, with
-// compensated (Kahan) accumulation across chunks, which is more accurate than
+// compensated accumulation across chunks, which is more accurate than
 // the tensor core's fp32 accumulation and takes no operand column. K* never
 // reaches HBM.
 //
@@ -58,7 +58,7 @@ constexpr uint32_t kStageBytes = BOUTE_TILE_M * BOUTE_ACHUNK * 4;   // fp32 K* i
 
 // builder warps: 16 (8 columns of each 32-point half per thread) when the
 // candidate coordinates are short enough to keep in registers, else 8 (16
-// columns of one row, or 8 columns of two rows: kstar_pair)
+// columns of one row, or half of them of two rows: kstar_pair)
 template <int DP>
 struct Layout {
   static constexpr int kBld = DP <= 16 ? 16 : 8;
@@ -116,14 +116,18 @@ __device__ __forceinline__ float ex2_approx(float x) {
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kLn2Sq3 = 0.16015100463940046f;  // (ln 2)^2 / 3
 
-// Compensated (Kahan) accumulation of packed pairs: s + c carries the sum
-// of the terms with the rounding error of every addition.
+// Compensated (Kahan) accumulation of packed pairs of products: s + c carries the sum
+// with the rounding error of every addition, the correction entering with the next
+// product's rounding. The fma is written out: a product and a sum of two pairs may be
+// contracted to one (here they are, .rn or not), and the paths that build and that
+// stage K* have to round alike. (An error-free product and sum, 4 more operations per
+// pair, cost 12 % at n = 512, d = 16 and left the mean's error as it is: K* sets it.)
 struct Kahan2 {
   unsigned long long s = 0ull, c = 0ull;
-  __device__ __forceinline__ void add(unsigned long long x) {
-    const unsigned long long y = f2_sub(x, c);
+  __device__ __forceinline__ void add(unsigned long long x, unsigned long long a) {
+    const unsigned long long y = f2_fma(x, a, c);
     const unsigned long long t = f2_add(s, y);
-    c = f2_sub(f2_sub(t, s), y);
+    c = f2_sub(y, f2_sub(t, s));
     s = t;
   }
 };
@@ -371,8 +375,9 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity,
 // add up to more than kFixRatio times the mean's scale max(|mean|, s): the
 // fp32 cross-covariance's rounding (a few units in the last place per entry,
 // amplified by that ratio) would otherwise exceed the 1e-5 tolerance. Below
-// the ratio the fp32 mean's error stays under about 6e-6 of the scale.
-constexpr float kFixRatio = 256.f;
+// the ratio the fp32 mean's error stays under about 8e-6 of the scale (up to 256
+// it reached 1.1e-5: row 190 of n = 70, lengthscales 0.5 .. 2).
+constexpr float kFixRatio = 224.f;
 
 // ---- the exact mean of a flagged row, in double-float arithmetic -----------------
 // Numbers as unevaluated pairs hi + lo of floats (Dekker; Knuth's error-free
@@ -525,13 +530,18 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
     posterior_kernel(const __grid_constant__ PostArgs a) {
   constexpr int kBldWarps = Layout<DP>::kBld;
   constexpr int COLS = Layout<DP>::kCols;   // columns of a half per builder thread
-  // 8 builder warps building the Matern kernel here: each builder thread
-  // covers two candidate rows (kstar_pair), so that every training coordinate
-  // it loads serves two K* entries (half the shared-memory loads per entry)
-  constexpr bool kPair = !PRE && KERN == 0 && kBldWarps == 8;
+  // The Matern kernel built here: each builder thread covers two candidate rows
+  // (kstar_pair), so that every training coordinate it loads serves two K*
+  // entries (half the shared-memory wavefronts per entry, which beside the tensor
+  // cores' operand reads and with the latency of the loads hold the builders back.
+  // One row and twice the columns with 16 warps: n = 512, d = 16, 2^20 candidates
+  // 2487 against 2210 us; n = 256, d = 10, 2^22 candidates 4092 against 4024 us.
+  // Two rows held singly and duplicated instead of the training coordinate: 2480.)
+  constexpr bool kPair = !PRE && KERN == 0;
   constexpr int RP = kPair ? 2 : 1;  // candidate rows per builder thread
   constexpr int CT = COLS / RP;      // its columns of a 32-point half
-  constexpr int GPT = 32 / CT;       // column groups (partial means per row)
+  constexpr int GPT = 32 / CT;       // column groups
+  constexpr int kParts = 64 / COLS;  // partial means per row
   constexpr int RPT = 32 / GPT;      // builder threads of a warp along the rows
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // 1024-byte alignment (the 128-byte swizzle atom) as an offset from the
@@ -855,7 +865,7 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
       ++nmean;
       float mhi = 0.f, mlo = 0.f, mag = 0.f;
 #pragma unroll
-      for (int q = 0; q < GPT; ++q) {
+      for (int q = 0; q < kParts; ++q) {
         const float *rp = red + ((size_t)q * BOUTE_TILE_M + 32 * eq + lane) * 3;
         float e;
         two_sum_f(mhi, rp[0], mhi, e);
@@ -984,10 +994,10 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
               // mean's terms summed per row; a ragged last half zeroes the
               // columns beyond n
               auto emit2 = [&](auto ragged) {
-                static_assert(CT == 8, "one 16-byte store per row and part");
-                uint32_t hi[2][4], lo[2][4];
+                static_assert(CT == 4 || CT == 8, "one 8- or 16-byte store per row and part");
+                uint32_t hi[2][CT / 2], lo[2][CT / 2];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
+                for (int e = 0; e < CT / 2; ++e) {
                   const int kk = 2 * e;
                   unsigned long long va = kvp[kk], vb = kvp[kk + 1];
                   if (decltype(ragged)::value) {
@@ -996,8 +1006,8 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
                   }
                   if (mean_grp) {  // (each chunk's terms once)
                     const float a0 = alg[kk], a1 = alg[kk + 1];
-                    mu2.add(f2_mul(va, f2_dup(a0)));
-                    mu2.add(f2_mul(vb, f2_dup(a1)));
+                    mu2.add(va, f2_dup(a0));
+                    mu2.add(vb, f2_dup(a1));
                     mag2 = f2_fma(va, f2_dup(fabsf(a0)), mag2);  // (K* >= 0)
                     mag2 = f2_fma(vb, f2_dup(fabsf(a1)), mag2);
                   }
@@ -1010,9 +1020,14 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
                   const int o = sw128_off16(r + q * RPT, col0) * 2;  // bytes
-                  if (BOUTE_INB(o + 15, (long long)kAPartBytes)) {
-                    *(uint4 *)(Ah + o) = make_uint4(hi[q][0], hi[q][1], hi[q][2], hi[q][3]);
-                    *(uint4 *)(Al + o) = make_uint4(lo[q][0], lo[q][1], lo[q][2], lo[q][3]);
+                  if (BOUTE_INB(o + 2 * CT - 1, (long long)kAPartBytes)) {
+                    if constexpr (CT == 8) {
+                      *(uint4 *)(Ah + o) = make_uint4(hi[q][0], hi[q][1], hi[q][2], hi[q][3]);
+                      *(uint4 *)(Al + o) = make_uint4(lo[q][0], lo[q][1], lo[q][2], lo[q][3]);
+                    } else {
+                      *(uint2 *)(Ah + o) = make_uint2(hi[q][0], hi[q][1]);
+                      *(uint2 *)(Al + o) = make_uint2(lo[q][0], lo[q][1]);
+                    }
                   }
                 }
               };
@@ -1036,8 +1051,24 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
               const int jbase = BOUTE_ACHUNK * c + col0;
               const float *alg = alp + COLS * g;
               // kernel values of this thread's COLS columns into the A stage as
-              // fp16 hi/lo; a ragged last half zeroes the columns beyond n
+              // fp16 hi/lo; a ragged last half zeroes the columns beyond n. The mean's
+              // terms in two sums, one per half of the columns, as where a thread holds
+              // half the columns of two rows.
               auto emit = [&](auto ragged) {
+                if (mean_grp) {  // (each chunk's terms once)
+                  constexpr int H = COLS / 2;
+#pragma unroll
+                  for (int e = 0; e < H; ++e) {
+                    float v0 = kv[e], v1 = kv[e + H];
+                    if (decltype(ragged)::value) {
+                      v0 = (jbase + e < n) ? v0 : 0.f;
+                      v1 = (jbase + e + H < n) ? v1 : 0.f;
+                    }
+                    const unsigned long long v2 = f2_pack(v0, v1);
+                    mu2.add(v2, f2_pack(alg[e], alg[e + H]));
+                    mag2 = f2_fma(v2, f2_pack(fabsf(alg[e]), fabsf(alg[e + H])), mag2);
+                  }
+                }
 #pragma unroll
                 for (int u = 0; u < COLS / 8; ++u) {
                   uint32_t hi[4], lo[4];
@@ -1048,12 +1079,6 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
                     if (decltype(ragged)::value) {
                       v0 = (jbase + kk < n) ? v0 : 0.f;
                       v1 = (jbase + kk + 1 < n) ? v1 : 0.f;
-                    }
-                    if (mean_grp) {  // (each chunk's terms once)
-                      const unsigned long long v2 = f2_pack(v0, v1);
-                      const unsigned long long a2 = *(const unsigned long long *)(alg + kk);
-                      mu2.add(f2_mul(v2, a2));
-                      mag2 = f2_fma(v2, a2 & 0x7fffffff7fffffffull, mag2);  // (K* >= 0)
                     }
                     split_f16x2(v0, v1, hi[e], lo[e]);
                   }
@@ -1088,23 +1113,15 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
       f2_split(mag2, me, mo);
       if (nmean > 0 && !wait_or_abort(mean_empty, (nmean - 1) & 1u, abort)) break;
       ++nmean;
-      float *rp = red + ((size_t)g * BOUTE_TILE_M + r) * 3;
-      if constexpr (kPair) {  // the pair's lanes are the two rows, each a Kahan sum s - c
-        float *rq = red + ((size_t)g * BOUTE_TILE_M + r + RPT) * 3;
-        rp[0] = se;
-        rp[1] = -ce;
-        rp[2] = me;
-        rq[0] = so;
-        rq[1] = -co;
-        rq[2] = mo;
-      } else {  // the pair's lanes are two sets of the row's columns
-        float hi, lo;
-        two_sum_f(se, so, hi, lo);
-        lo -= ce + co;
-        rp[0] = hi;
-        rp[1] = lo;
-        rp[2] = me + mo;
-      }
+      // the lanes: two rows' sums, or the row's over the two halves of the columns
+      float *rp = red + ((size_t)(kPair ? g : 2 * g) * BOUTE_TILE_M + r) * 3;
+      float *rq = rp + (kPair ? RPT : BOUTE_TILE_M) * 3;
+      rp[0] = se;
+      rp[1] = ce;
+      rp[2] = me;
+      rq[0] = so;
+      rq[1] = co;
+      rq[2] = mo;
       __syncwarp();
       if (lane == 0) mbar_arrive_count(mean_ready);
     }
@@ -1158,20 +1175,20 @@ int launch_dp(const Gp *gp, const float *Xc, const float *kst, long long N, floa
   for (int q = 0; q < a.plan.nblk; ++q) wmax = std::max(wmax, a.plan.ncol[q]);
   a.b_bytes = (uint32_t)(2 * wmax * 128);
   a.x_bytes = (uint32_t)round_up(xt_chunk_floats(DP) * 4, 16);
-  // alignment slack, barriers, TMEM address, flag; the partial means (twice
-  // the column groups where the builders take rows in pairs)
-  const bool pair = !kst && !gp->kern && Layout<DP>::kBld == 8;
-  const size_t fixed =
-      1024 + 512 + (size_t)(32 / Layout<DP>::kCols) * (pair ? 2 : 1) * BOUTE_TILE_M * 3 * 4;
+  // alignment slack, barriers, TMEM address, flag; the partial means
+  const size_t fixed = 1024 + 512 + (size_t)(64 / Layout<DP>::kCols) * BOUTE_TILE_M * 3 * 4;
   const size_t budget = 227 * 1024 - fixed;
   const size_t st = kst ? kStageBytes : 0;  // staging beside each A stage (PRE)
   // K* stages before B stages: a deeper A ring lets the builders run ahead of
   // the tensor cores through the groups where the MMAs outweigh the building
-  // (measured best: 4 A + 2 B stages with 8 builder warps, 3 + 3 with 16),
+  // (measured best: 4 A + 2 B stages; n = 512, d = 16 with 3 + 3: 2251 against
+  // 2210 us for 2^20 candidates. With in-sample draws, whose dense blocks make more B
+  // stages per A stage, 3 + 3: noisy step at n = 128 471 against 463 us),
   // then the side input's ring as deep as what is left allows
   a.sx = kMaxX;
-  a.sa = Layout<DP>::kBld == 8 ? 4 : 3;
-  a.sb = Layout<DP>::kBld == 8 ? 2 : 3;
+  const bool dense = Layout<DP>::kBld == 16 && a.plan.S_in > 0;
+  a.sa = dense ? 3 : 4;
+  a.sb = dense ? 3 : 2;
   while ((size_t)a.sa * (kABytes + st) + (size_t)a.sb * a.b_bytes + (size_t)a.sx * a.x_bytes >
          budget) {
     if (a.sx > 4) --a.sx;

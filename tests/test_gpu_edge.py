@@ -385,3 +385,19 @@ def test_front_and_boxes_edges(n, m, kind):
         got = np.prod(np.maximum(hi - np.maximum(lo, y), 0.0), 1).sum()
         # the corners are rounded to fp32: 2^-24 of at most 1.1 each, m of them per box
         assert got == pytest.approx(oracle.hvi(F, ref, y), abs=k * m * 1.1 * 2.0 ** -23)
+
+
+# Rows in pairs (four or eight rows apart) and four or eight columns of a half chunk
+# per thread: rows and columns at their edges, every coordinate width.
+@pytest.mark.parametrize("d,n,N", [(3, 1, 1), (3, 35, 4), (9, 4, 5), (9, 61, 129), (16, 5, 8),
+                                   (16, 33, 133), (20, 7, 9), (24, 41, 137), (32, 9, 127)])
+def test_row_pairs_and_column_groups(d, n, N):
+    hp = rand_problem(100 + d + n, n, d, 2, N)
+    hp.ls[0] = 0.2 * np.sqrt(d)
+    g = gpu_pipeline(hp)
+    assert g["status"] == 0
+    fp = oracle_fit(hp, 0)
+    mean, var = opl.posterior(fp, hp.Xc[0])
+    for t in range(2):
+        check_mean(g["mean"][0, t], mean[:, t], fp.s2[t])
+        check_var(g["var"][0, t], var[:, t], fp.s2[t])

@@ -218,11 +218,11 @@ __global__ void __launch_bounds__(kSetupThreads) fit_setup_kernel(
 // even), zero above the diagonal and beyond n. Returns false if a scaled
 // element reaches the fp16 range (W beyond four times its bound 1/sigma_n:
 // the fp32 factor is numerically singular).
-__device__ __forceinline__ bool pack_pair(const float *wrow, int g, int k, const PostPlan &plan,
-                                          float scale, uint16_t *img) {
+__device__ __forceinline__ bool pack_values(float w0, float w1, int g, int k, const PostPlan &plan,
+                                            float scale, uint16_t *img) {
   const int n = plan.n;
-  const float v0 = (k < n && g < n && k <= g) ? wrow[k] * scale : 0.f;
-  const float v1 = (k + 1 < n && g < n && k + 1 <= g) ? wrow[k + 1] * scale : 0.f;
+  const float v0 = (k < n && g < n && k <= g) ? w0 * scale : 0.f;
+  const float v1 = (k + 1 < n && g < n && k + 1 <= g) ? w1 * scale : 0.f;
   uint32_t hi, lo;
   split_f16x2(v0, v1, hi, lo);
   const int q = g / BOUTE_BLKCOLS, c = k / BOUTE_ACHUNK, ncol = plan.ncol[q];
@@ -237,23 +237,11 @@ __device__ __forceinline__ bool pack_pair(const float *wrow, int g, int k, const
   }
   return fabsf(v0) < 32768.f && fabsf(v1) < 32768.f;
 }
-
-// All of W's image elements, pairs [first, total) by stride (rows of the
-// blocks' padded widths, the chunks each block needs).
-__device__ __forceinline__ bool pack_elems(const float *W, int ld, const PostPlan &plan,
-                                           float scale, uint16_t *img, long long first,
-                                           long long stride) {
-  const int nblk = plan.nwblk;
-  const long long rows = (long long)BOUTE_BLKCOLS * (nblk - 1) + plan.ncol[nblk - 1];
-  const int kmax = BOUTE_ACHUNK * plan.kc[nblk - 1];  // pairs per row: kmax / 2
-  const long long total = rows * (kmax / 2);
-  bool ok = true;
-  for (long long e = first; e < total; e += stride) {
-    const int g = (int)(e / (kmax / 2)), k = 2 * (int)(e % (kmax / 2));
-    if (k / BOUTE_ACHUNK >= plan.kc[g / BOUTE_BLKCOLS]) continue;
-    ok &= pack_pair(W + (size_t)(g < plan.npad ? g : 0) * ld, g, k, plan, scale, img);
-  }
-  return ok;
+// The same from row g of W.
+__device__ __forceinline__ bool pack_pair(const float *wrow, int g, int k, const PostPlan &plan,
+                                          float scale, uint16_t *img) {
+  const bool in0 = k < plan.n && k <= g, in1 = k + 1 < plan.n && k + 1 <= g;
+  return pack_values(in0 ? wrow[k] : 0.f, in1 ? wrow[k + 1] : 0.f, g, k, plan, scale, img);
 }
 
 // Error-free product and sum on fp32 pairs (Dekker / Knuth).
@@ -322,18 +310,14 @@ __device__ __forceinline__ void composite_wmax(float *xt, int bt, const PostPlan
 // against the fp64-accurate K = hi + lo with double-float residuals. A pivot
 // at or below 16 * eps32 times its original diagonal entry counts as not
 // positive. Matrix and inverse live in shared memory (row stride NP+1, NP = n
-// rounded up to 32, padded with the identity) when they fit, else in the
-// handle's global workspace.
-// Threads per block of the two variants: the shared-memory variant runs more
-// warps to hide the latency of its short, dependent phases.
-template <bool SMEM>
-constexpr int fit_threads() { return SMEM ? 512 : 256; }
+// rounded up to 32, padded with the identity), n <= 160; fitc_kernel takes the
+// larger problems.
+constexpr int kFitThreads = 512;
 
-template <bool SMEM>
-__global__ void __launch_bounds__(fit_threads<SMEM>(), 1) fit32_kernel(
+__global__ void __launch_bounds__(kFitThreads, 1) fit32_kernel(
     const float *Kh_all, const float *Kl_all, const double *Ys, int standardize, int n, int m,
-    float *Aws, float *Wws, float *xt, int DP, int npad, PostPlan plan, uint16_t *bop,
-    int kl_smem, int early_trigger, int comp, int *status, const int *fbad, float *Wkeep) {
+    float *xt, int DP, int npad, PostPlan plan, uint16_t *bop, int kl_smem, int early_trigger,
+    int comp, int *status, float *Wkeep) {
   extern __shared__ __align__(16) float sm[];
   __shared__ int bad;
   __shared__ uint64_t lbar, lbar_lo;  // K hi; K lo (needed only by the residual)
@@ -345,11 +329,9 @@ __global__ void __launch_bounds__(fit_threads<SMEM>(), 1) fit32_kernel(
             nw = nthr >> 5;
   const int NP = npad, ld = NP + 1;
   const float *Kh = Kh_all + (size_t)bt * n * n, *Kl = Kl_all + (size_t)bt * n * n;
-  float *A = SMEM ? sm : Aws + (size_t)bt * NP * ld;
-  float *W = SMEM ? sm + (size_t)NP * ld : Wws + (size_t)bt * NP * ld;
-  float *vec = SMEM ? sm + 2 * (size_t)NP * ld : sm;  // ylo, dg, y, tv, al, r: 6 x NP
-  float *ylo = vec, *dg = vec + NP, *yv = vec + 2 * NP, *tv = vec + 3 * NP, *al = vec + 4 * NP,
-        *rv = vec + 5 * NP;
+  float *A = sm, *W = sm + (size_t)NP * ld;
+  float *vec = sm + 2 * (size_t)NP * ld;  // ylo, dg, y, al, r: 5 x NP
+  float *ylo = vec, *dg = vec + NP, *yv = vec + 2 * NP, *al = vec + 3 * NP, *rv = vec + 4 * NP;
   const double *y = Ys + (size_t)b * n * m + t;
   if (early_trigger) pdl_trigger();  // every block is resident: the posterior may launch
   // standardize != 0: Ys holds raw outcomes; this column is standardised here
@@ -361,8 +343,8 @@ __global__ void __launch_bounds__(fit_threads<SMEM>(), 1) fit32_kernel(
   // residual), padded with the identity to NP x NP. In shared memory with n
   // even, K hi (and, for n <= 128, K lo) arrive by bulk copy, K hi staged in
   // the W area.
-  float *Kls = kl_smem ? vec + 6 * NP : nullptr;  // K lo, n x n (shared)
-  const bool bulk = SMEM && (n % 2 == 0);
+  float *Kls = kl_smem ? vec + 5 * NP : nullptr;  // K lo, n x n (shared)
+  const bool bulk = n % 2 == 0;
   if (bulk) {
     if (tid == 0) {
       mbar_init(&lbar, 1);
@@ -379,7 +361,7 @@ __global__ void __launch_bounds__(fit_threads<SMEM>(), 1) fit32_kernel(
         bulk_g2s(Kls, Kl, bytes, &lbar_lo);
       }
     }
-  } else if (!fbad) {  // eight independent loads per thread in flight before their stores
+  } else {  // eight independent loads per thread in flight before their stores
     const int nn = n * n;
     for (int base = 0; base < nn; base += 8 * nthr) {
       float v[8], w8[8];
@@ -400,7 +382,7 @@ __global__ void __launch_bounds__(fit_threads<SMEM>(), 1) fit32_kernel(
       }
     }
   }
-  for (int e = tid; e < (NP - n) * NP && !fbad; e += nthr) {
+  for (int e = tid; e < (NP - n) * NP; e += nthr) {
     const int i = n + e / NP, k = e % NP;
     if (k <= i) A[(size_t)i * ld + k] = (k == i) ? 1.f : 0.f;
   }
@@ -427,7 +409,7 @@ __global__ void __launch_bounds__(fit_threads<SMEM>(), 1) fit32_kernel(
     ylo[i] = (float)(ys - (double)yv[i]);
     dg[i] = A[(size_t)i * ld + i];
   }
-  if (tid == 0) bad = fbad ? fbad[bt] : 0;  // (factored by the blocked kernels)
+  if (tid == 0) bad = 0;
   for (int e = tid; e < 32 * 64; e += nthr) (&colL[0][0])[e] = 0.f;
   __syncthreads();
   // Operand images of W for the posterior (n <= 160): rows [g_lo, g_hi) of W,
@@ -459,7 +441,7 @@ __global__ void __launch_bounds__(fit_threads<SMEM>(), 1) fit32_kernel(
   // for T_pJ and W_pJ).
   const int nb = NP / 32;
   const unsigned FULL = 0xffffffffu;
-  for (int p = 0; p < nb && !fbad; ++p) {
+  for (int p = 0; p < nb; ++p) {
     const int p0 = 32 * p;
     if (warp == 0) {
       // Factor. Lane = row of the block. a[] is a window on the lane's row
@@ -533,7 +515,7 @@ __global__ void __launch_bounds__(fit_threads<SMEM>(), 1) fit32_kernel(
       float *Wr = W + (size_t)(p0 + lane) * ld + p0;
 #pragma unroll
       for (int c = 0; c < 32; ++c) Wr[c] = w[c] * myinv;
-    } else if (SMEM && p > 0) {
+    } else if (p > 0) {
       // the other warps pack the previous block row of W meanwhile
       pack_rows(p0 - 32, p0, warp - 2, nw - 2);
     }
@@ -652,11 +634,11 @@ __global__ void __launch_bounds__(fit_threads<SMEM>(), 1) fit32_kernel(
     return;
   }
   // ---- alpha0 = W^T (W y), refined twice against K = hi + lo ---------------------
-  // out = W^T (W rhs). Shared-memory variant: the 32 x 32 blocks (I >= J) of
+  // out = W^T (W rhs): the 32 x 32 blocks (I >= J) of
   // W, one warp per block (the diagonal blocks hold zeros above the diagonal,
   // the padding the identity), with the block partial sums in the space of
   // colL (free after the factorisation), added in a fixed order.
-  auto solve_blocks = [&](const float *rhs, float *out) {
+  auto solve = [&](const float *rhs, float *out) {
     float *pw = &colL[0][0], *pt = pw + nb * NP;  // nb x NP each (nb <= 5, NP <= 160)
     const int nblk = nb * (nb + 1) / 2;
     auto block = [&](int e, int &I, int &J) {
@@ -704,42 +686,6 @@ __global__ void __launch_bounds__(fit_threads<SMEM>(), 1) fit32_kernel(
     }
     __syncthreads();
   };
-  // global variant: a warp per row of W (coalesced loads, lanes combined by
-  // shuffles in a fixed order), then a thread per column (4 accumulators)
-  auto solve = [&](const float *rhs, float *out) {
-    if constexpr (SMEM) {
-      solve_blocks(rhs, out);
-    } else {
-    for (int i = warp; i < NP; i += nw) {
-      const float *wr = W + (size_t)i * ld;
-      float s0 = 0.f, s1 = 0.f;
-      int k = lane;
-      for (; k + 32 <= i; k += 64) {
-        s0 = fmaf(wr[k], rhs[k], s0);
-        s1 = fmaf(wr[k + 32], rhs[k + 32], s1);
-      }
-      if (k <= i) s0 = fmaf(wr[k], rhs[k], s0);
-      float v = s0 + s1;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-      if (lane == 0) tv[i] = v;
-    }
-    __syncthreads();
-    for (int k = tid; k < NP; k += nthr) {
-      float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-      int i = k;
-      for (; i + 3 < NP; i += 4) {
-        s0 = fmaf(W[(size_t)i * ld + k], tv[i], s0);
-        s1 = fmaf(W[(size_t)(i + 1) * ld + k], tv[i + 1], s1);
-        s2 = fmaf(W[(size_t)(i + 2) * ld + k], tv[i + 2], s2);
-        s3 = fmaf(W[(size_t)(i + 3) * ld + k], tv[i + 3], s3);
-      }
-      for (; i < NP; ++i) s0 = fmaf(W[(size_t)i * ld + k], tv[i], s0);
-      out[k] = (s0 + s1) + (s2 + s3);
-    }
-    __syncthreads();
-    }
-  };
   solve(yv, al);
   if (lo_copy && !mbar_wait(&lbar_lo, 0)) {  // the copy never completed: report, drain, leave
     if (tid == 0) set_status(status, BOUTE_ERR_TIMEOUT);
@@ -747,7 +693,7 @@ __global__ void __launch_bounds__(fit_threads<SMEM>(), 1) fit32_kernel(
     return;
   }
   auto residual = [&]() {
-    // residual r = y - K alpha in double-float. Shared-memory variant: one
+    // residual r = y - K alpha in double-float: one
     // warp per 32 x 32 block (I, J) of K, lane = row, two independent chains per
     // lane; K lo through its symmetry (K lo[k][i], conflict-free across the
     // lanes), from shared memory when it fits there; K hi from the upper
@@ -758,107 +704,60 @@ __global__ void __launch_bounds__(fit_threads<SMEM>(), 1) fit32_kernel(
     // alpha is zero there (padding), so those terms add exact zeros. The block
     // partial sums (hi, lo) go to the space of colL and are added per row in a
     // fixed order.
-    if (SMEM) {
-      float *ph = &colL[0][0], *pl = ph + nb * NP;  // nb x NP each
-      const float *Klsm = vec + 6 * NP;  // = Kls when kl_smem (shared-space pointer)
-      for (int e = warp; e < nb * nb; e += nw) {
-        const int I = e / nb, J = e - I * nb, ci = min(32 * I + lane, n - 1);
-        const float *alJ = al + 32 * J;
-        float sh[2] = {0.f, 0.f}, sl[2] = {0.f, 0.f};
-        auto run = [&](auto form, auto lo_smem) {
-          constexpr int F = decltype(form)::value;  // 0: below, 1: above, 2: diagonal block
-          constexpr bool LS = decltype(lo_smem)::value;
-          const float di = dg[ci];
+    float *ph = &colL[0][0], *pl = ph + nb * NP;  // nb x NP each
+    const float *Klsm = vec + 5 * NP;  // = Kls when kl_smem (shared-space pointer)
+    for (int e = warp; e < nb * nb; e += nw) {
+      const int I = e / nb, J = e - I * nb, ci = min(32 * I + lane, n - 1);
+      const float *alJ = al + 32 * J;
+      float sh[2] = {0.f, 0.f}, sl[2] = {0.f, 0.f};
+      auto run = [&](auto form, auto lo_smem) {
+        constexpr int F = decltype(form)::value;  // 0: below, 1: above, 2: diagonal block
+        constexpr bool LS = decltype(lo_smem)::value;
+        const float di = dg[ci];
   #pragma unroll 8
-          for (int kk = 0; kk < 32; ++kk) {
-            const int kc = min(32 * J + kk, n - 1);
-            float h;
-            if (F == 0) {
-              h = A[kc * ld + ci];
-            } else if (F == 1) {
-              h = A[ci * ld + kc];
-            } else {
-              const float x = A[kc * ld + ci], y = A[ci * ld + kc];
-              h = kc < ci ? x : y;
-              h = kc == ci ? di : h;
-            }
-            const float l = LS ? Klsm[kc * n + ci] : Kl[(size_t)kc * n + ci];
-            const float a = alJ[kk];  // zero from n on
-            float pr, er, s_, e2;
-            two_prod(h, a, pr, er);
-            two_sum(sh[kk & 1], pr, s_, e2);
-            sh[kk & 1] = s_;
-            sl[kk & 1] += e2 + fmaf(l, a, er);
+        for (int kk = 0; kk < 32; ++kk) {
+          const int kc = min(32 * J + kk, n - 1);
+          float h;
+          if (F == 0) {
+            h = A[kc * ld + ci];
+          } else if (F == 1) {
+            h = A[ci * ld + kc];
+          } else {
+            const float x = A[kc * ld + ci], y = A[ci * ld + kc];
+            h = kc < ci ? x : y;
+            h = kc == ci ? di : h;
           }
-        };
-        auto pick = [&](auto lo_smem) {
-          if (I > J) run(std::integral_constant<int, 0>{}, lo_smem);
-          else if (I < J) run(std::integral_constant<int, 1>{}, lo_smem);
-          else run(std::integral_constant<int, 2>{}, lo_smem);
-        };
-        if (kl_smem) pick(std::true_type{});
-        else pick(std::false_type{});
+          const float l = LS ? Klsm[kc * n + ci] : Kl[(size_t)kc * n + ci];
+          const float a = alJ[kk];  // zero from n on
+          float pr, er, s_, e2;
+          two_prod(h, a, pr, er);
+          two_sum(sh[kk & 1], pr, s_, e2);
+          sh[kk & 1] = s_;
+          sl[kk & 1] += e2 + fmaf(l, a, er);
+        }
+      };
+      auto pick = [&](auto lo_smem) {
+        if (I > J) run(std::integral_constant<int, 0>{}, lo_smem);
+        else if (I < J) run(std::integral_constant<int, 1>{}, lo_smem);
+        else run(std::integral_constant<int, 2>{}, lo_smem);
+      };
+      if (kl_smem) pick(std::true_type{});
+      else pick(std::false_type{});
+      float s_, e2;
+      two_sum(sh[0], sh[1], s_, e2);
+      ph[J * NP + 32 * I + lane] = s_;
+      pl[J * NP + 32 * I + lane] = (sl[0] + sl[1]) + e2;
+    }
+    __syncthreads();
+    for (int i = tid; i < NP; i += nthr) {
+      float sh = 0.f, sl = 0.f;
+      for (int J = 0; J < nb; ++J) {
         float s_, e2;
-        two_sum(sh[0], sh[1], s_, e2);
-        ph[J * NP + 32 * I + lane] = s_;
-        pl[J * NP + 32 * I + lane] = (sl[0] + sl[1]) + e2;
+        two_sum(sh, ph[J * NP + i], s_, e2);
+        sh = s_;
+        sl += pl[J * NP + i] + e2;
       }
-      __syncthreads();
-      for (int i = tid; i < NP; i += nthr) {
-        float sh = 0.f, sl = 0.f;
-        for (int J = 0; J < nb; ++J) {
-          float s_, e2;
-          two_sum(sh, ph[J * NP + i], s_, e2);
-          sh = s_;
-          sl += pl[J * NP + i] + e2;
-        }
-        if (i < n) rv[i] = (yv[i] - sh) + (ylo[i] - sl);
-      }
-    } else {
-      // global variant: two rows per half warp at a time, all their loads
-      // issued before the arithmetic
-      const int half = lane >> 4, hl = lane & 15;
-      for (int i0 = 2 * warp + half; i0 < NP; i0 += 4 * nw) {
-        const int rows[2] = {i0, i0 + 2 * nw};
-        float sh[2] = {0.f, 0.f}, sl[2] = {0.f, 0.f};
-        for (int k0 = 0; k0 < n; k0 += 128) {
-          float h8[2][8], l8[2][8], a8[8];
-  #pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int k = k0 + hl + 16 * u;
-            a8[u] = k < n ? al[k] : 0.f;
-  #pragma unroll
-            for (int q = 0; q < 2; ++q) {
-              const bool ok = k < n && rows[q] < n;
-              h8[q][u] = ok ? Kh[(size_t)rows[q] * n + k] : 0.f;
-              l8[q][u] = ok ? Kl[(size_t)rows[q] * n + k] : 0.f;
-            }
-          }
-  #pragma unroll
-          for (int q = 0; q < 2; ++q)
-  #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-              float pr, e, s_, e2;
-              two_prod(h8[q][u], a8[u], pr, e);
-              two_sum(sh[q], pr, s_, e2);
-              sh[q] = s_;
-              sl[q] += e2 + fmaf(l8[q][u], a8[u], e);
-            }
-        }
-  #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-  #pragma unroll
-          for (int o = 8; o > 0; o >>= 1) {  // within the half warp
-            const float oh = __shfl_xor_sync(FULL, sh[q], o);
-            const float ol = __shfl_xor_sync(FULL, sl[q], o);
-            float s_, e;
-            two_sum(sh[q], oh, s_, e);
-            sh[q] = s_;
-            sl[q] += ol + e;
-          }
-          if (hl == 0 && rows[q] < n) rv[rows[q]] = (yv[rows[q]] - sh[q]) + (ylo[rows[q]] - sl[q]);
-        }
-      }
+      if (i < n) rv[i] = (yv[i] - sh) + (ylo[i] - sl);
     }
   };
   // two refinement steps: alpha carries the condition number of K, and the
@@ -882,11 +781,9 @@ __global__ void __launch_bounds__(fit_threads<SMEM>(), 1) fit32_kernel(
     }
     __syncthreads();
   }
-  // outputs: the operand images of W (packed here from shared memory; the
-  // global variant leaves W in the workspace for pack_kernel), alpha into the
-  // side input
-  if (SMEM) pack_rows(NP - 32, NP, warp, nw);  // the last block row (the others: above)
-  if (SMEM && Wkeep) {  // W in global memory too (the in-sample preparation, the
+  // outputs: the operand images of W, alpha into the side input
+  pack_rows(NP - 32, NP, warp, nw);  // the last block row (the others: above)
+  if (Wkeep) {  // W in global memory too (the in-sample preparation, the
                         // acquisition's gradient), its lower triangle
     float *dst = Wkeep + (size_t)bt * NP * ld;
     for (int i = warp; i < n; i += nw)
@@ -902,474 +799,556 @@ __global__ void __launch_bounds__(fit_threads<SMEM>(), 1) fit32_kernel(
   if (comp && warp == nw - 1) composite_wmax(xt, bt, plan, DP, n, lane);
 }
 
-// ---- the global-workspace factorisation across many blocks -------------------------
-// For n > 160 the three phases of every 32-column panel of fit32_kernel's loop
-// run as three kernels, each over as many blocks as its tiles fill (a grid of
-// x blocks per problem-objective y), with programmatic dependent launch in
-// between: (a) fitb_diag_kernel factors and inverts the diagonal block, (b)
-// fitb_panel_kernel forms the panel below and the partial sums of T_pJ, (c)
-// fitb_update_kernel applies the trailing update, adds the partials in a fixed
-// order (the result does not depend on the grid), forms W's block row and
-// copies the panel into A. The tiles' arithmetic is the same as in the
-// one-block loop; the fitr_* kernels then form alpha from the factored
-// workspace. A non-positive pivot marks the problem-objective in fbad
-// and its later kernels return at once.
-constexpr int kFitbThreads = 256;
+// ---- factorisation on a thread-block cluster (n > 160) --------------------------
+// One cluster of C = Pr x Pc CTAs per problem-objective runs the whole fit after
+// the set-up in one launch: K's lower triangle as 32 x 32 tiles, tile (I, J) owned
+// by the CTA (I mod Pr, J mod Pc) and kept in its shared memory (in the workspace
+// Aws when it does not fit), updated in place:
+//   before panel J it holds A_IJ (the trailing matrix), afterwards the transpose of
+//   R_IJ = -sum_{J <= K <= p} L_IK W_KJ, and W_IJ^T = (W_II R_IJ)^T from panel I on.
+// Panel p: two warps of the owner factor the diagonal tile and invert it (fc_diagonal)
+// and send W_pp to the CTAs of its block row and column; cluster barrier; these form
+// L_Ip = A_Ip W_pp^T (I > p) and W_pJ = W_pp R_pJ (J < p) and send each to the CTAs
+// whose tiles need it; cluster barrier; every CTA updates its tiles, A_IJ -= L_Ip L_Jp^T
+// (J > p) and R_IJ -= L_Ip W_pJ (J <= p), the owner of the next diagonal tile that one
+// first and factoring it beside the rest, and the owners of block row p write W and its
+// operand images. Then alpha and its two refinement steps from the tiles. Tiles and
+// vectors travel by stores to the other CTAs' shared memory, ordered by the barriers.
+// The arithmetic is fp32 as in fit32_kernel; sums run in an order that does not depend
+// on C. What bounds it is the chain of a panel (two barriers, two tile products, the
+// diagonal tile), for n = 1024 as much the updates' shared-memory reads.
+// Fit with its set-up, against three launches a panel, nine for alpha and one block
+// per problem-objective in large batches: n = 203, m = 3 174 -> 98 us; n = 512, m = 2
+// 385 -> 230 us; n = 777, B = 3, m = 2 1193 -> 754 us; n = 1024, m = 3 1226 -> 943 us;
+// n = 256, B = 16, m = 2 560 -> 250 us.
+constexpr int kFcThreads = 512, kFcGroups = kFcThreads / 64;
+constexpr int kFcTile = 32 * 32;
+constexpr int kFcMaxCluster = 16;
 
-// A = K hi below the diagonal, the identity on the padding; fbad cleared.
-__global__ void __launch_bounds__(kFitbThreads) fitb_load_kernel(const float *Kh_all, int n,
-                                                                 int NP, float *Aws, int *fbad) {
-  pdl_wait();
-  pdl_trigger();
-  const int bt = blockIdx.y, ld = NP + 1;
-  const float *Kh = Kh_all + (size_t)bt * n * n;
-  float *A = Aws + (size_t)bt * NP * ld;
-  const long long tot = (long long)NP * NP;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < tot;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(e / NP), k = (int)(e % NP);
-    if (k > i) continue;
-    A[(size_t)i * ld + k] = i < n ? Kh[(size_t)i * n + k] : (k == i ? 1.f : 0.f);
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) fbad[bt] = 0;
+// Word of element (r, q) of a tile: 16-byte groups permuted by the row's quad, so
+// that a product's operand reads (rows 4 apart) and result accesses are free of conflicts.
+__device__ __forceinline__ int fc_off(int r, int q) {
+  return r * 32 + ((((q >> 2) ^ (r >> 2)) & 7) << 2) + (q & 3);
 }
 
-// (a) one block of two warps per problem-objective: warp 0 factors A_pp in
-// registers (the pivot test against K's own diagonal), warp 1 inverts it one
-// column behind into W_pp, as in fit32_kernel.
-__global__ void __launch_bounds__(64) fitb_diag_kernel(const float *Kh_all, int n, int NP,
-                                                       float *Aws, float *Wws, int p,
-                                                       int *fbad) {
-  __shared__ __align__(16) float colL[32][64];
-  __shared__ float invs[32];
-  pdl_wait();
-  pdl_trigger();
-  const int bt = blockIdx.x, ld = NP + 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (fbad[bt]) return;
-  const float *Kh = Kh_all + (size_t)bt * n * n;
-  float *A = Aws + (size_t)bt * NP * ld, *W = Wws + (size_t)bt * NP * ld;
-  const int p0 = 32 * p;
-  const unsigned FULL = 0xffffffffu;
-  for (int e = threadIdx.x; e < 32 * 64; e += 64) (&colL[0][0])[e] = 0.f;
-  __syncthreads();
-  if (warp == 0) {
-    float a[32];
-    float *Ar = A + (size_t)(p0 + lane) * ld + p0;
-#pragma unroll
-    for (int c = 0; c < 32; ++c) a[c] = (c <= lane) ? Ar[c] : 0.f;
-    const int gi = p0 + lane;
-    const float dgl = gi < n ? Kh[(size_t)gi * n + gi] : 1.f;
-    bool ok = true;
-    float piv = __shfl_sync(FULL, a[0], 0);
-    auto quarter = [&](auto nk, int c0) {
-      constexpr int NK = decltype(nk)::value;
-#pragma unroll 1
-      for (int c = c0; c < c0 + 8; ++c) {
-        if (!(piv > 16.f * 1.1920929e-7f * __shfl_sync(FULL, dgl, c))) ok = false;
-        float inv = rsqrtf(piv);
-        inv = inv * fmaf(-0.5f * piv * inv, inv, 1.5f);  // one Newton step; 1 / L_cc
-        const float l = lane > c ? a[0] * inv : (lane == c ? piv * inv : 0.f);
-        piv = __shfl_sync(FULL, fmaf(-l, l, a[1]), (c + 1) & 31);
-        if (lane >= c) Ar[c] = l;
-        colL[c][lane] = l;
-        if (lane == 0) invs[c] = inv;
-        __syncwarp();
-        named_barrier_sync(1, 64);  // column c is ready for warp 1
-#pragma unroll
-        for (int k = 0; k < NK; ++k) a[k] = fmaf(-l, colL[c][c + 1 + k], a[k + 1]);
-      }
-    };
-    quarter(std::integral_constant<int, 31>{}, 0);
-    quarter(std::integral_constant<int, 23>{}, 8);
-    quarter(std::integral_constant<int, 15>{}, 16);
-    quarter(std::integral_constant<int, 7>{}, 24);
-    if (__any_sync(FULL, !ok) && lane == 0) fbad[bt] = 1;
-  } else {
-    float w[32];
-#pragma unroll
-    for (int c = 0; c < 32; ++c) w[c] = (c == lane) ? 1.f : 0.f;
-    float myinv = 0.f;
-    auto quarter = [&](auto nk, int c0) {
-      constexpr int NK = decltype(nk)::value;
-#pragma unroll 1
-      for (int c = c0; c < c0 + 8; ++c) {
-        named_barrier_sync(1, 64);  // wait for column c
-        const float l = colL[c][lane], inv = invs[c];
-        if (lane == c) myinv = inv;
-        const float lw = lane > c ? l * inv : 0.f;
-#pragma unroll
-        for (int k = 0; k < NK; ++k) w[k] = fmaf(-lw, __shfl_sync(FULL, w[k], c), w[k]);
-      }
-    };
-    quarter(std::integral_constant<int, 8>{}, 0);
-    quarter(std::integral_constant<int, 16>{}, 8);
-    quarter(std::integral_constant<int, 24>{}, 16);
-    quarter(std::integral_constant<int, 32>{}, 24);
-    float *Wr = W + (size_t)(p0 + lane) * ld + p0;
-#pragma unroll
-    for (int c = 0; c < 32; ++c) Wr[c] = w[c] * myinv;
-  }
-}
-
-// The 32 x 32 tiles of (b) and (c): a block of kFitbThreads threads stages
-// its two operand tiles in shared memory (row stride 33) with coalesced loads
-// and forms a 2 x 2 output tile per thread (rows rb, rb + 1, columns cb,
-// cb + 1), each output an fmaf chain over q = 0..31 in order.
-using Tile = float[32][33];
-
-__device__ __forceinline__ void fitb_tile_load(Tile &dst, const float *src, int ld, int tid) {
-#pragma unroll
-  for (int j = 0; j < 1024 / kFitbThreads; ++j) {
-    const int x = tid + kFitbThreads * j, r = x >> 5, c = x & 31;
-    dst[r][c] = src[(size_t)r * ld + c];
-  }
-}
-
-// acc[u][v] += sum_q X[rb + u][q] Y[cb + v][q]  (X Y^T)
-__device__ __forceinline__ void fitb_mma_abt(const Tile &X, const Tile &Y, int rb, int cb,
-                                             float (&acc)[2][2]) {
-#pragma unroll 8
-  for (int q = 0; q < 32; ++q) {
-    const float x0 = X[rb][q], x1 = X[rb + 1][q], y0 = Y[cb][q], y1 = Y[cb + 1][q];
-    acc[0][0] = fmaf(x0, y0, acc[0][0]);
-    acc[0][1] = fmaf(x0, y1, acc[0][1]);
-    acc[1][0] = fmaf(x1, y0, acc[1][0]);
-    acc[1][1] = fmaf(x1, y1, acc[1][1]);
-  }
-}
-
-// acc[u][v] += sum_q X[rb + u][q] Y[q][cb + v]  (X Y)
-__device__ __forceinline__ void fitb_mma_ab(const Tile &X, const Tile &Y, int rb, int cb,
-                                            float (&acc)[2][2]) {
-#pragma unroll 8
-  for (int q = 0; q < 32; ++q) {
-    const float x0 = X[rb][q], x1 = X[rb + 1][q], y0 = Y[q][cb], y1 = Y[q][cb + 1];
-    acc[0][0] = fmaf(x0, y0, acc[0][0]);
-    acc[0][1] = fmaf(x0, y1, acc[0][1]);
-    acc[1][0] = fmaf(x1, y0, acc[1][0]);
-    acc[1][1] = fmaf(x1, y1, acc[1][1]);
-  }
-}
-
-// (b) the panel, L_Rp = A_Rp W_pp^T, in place in A for every block row R > p
-// (one work item each), and the partial sums of T_pJ = sum_{K=J}^{p-1} L_pK
-// W_KJ (J < p) into the workspace tpart: T_pJ's K range is split into chunks
-// of kFitbChunk blocks, one work item each, so that no item runs more than
-// kFitbChunk tile steps and the panel's critical path stays short for every p.
-// tpart holds, per problem-objective, nbw x ncw tiles of 32 x 32 floats (J,
-// chunk), nbw = NP / 32 and ncw = ceil(nbw / kFitbChunk).
-constexpr int kFitbChunk = 4;
-__host__ __device__ __forceinline__ int fitb_t_items(int p) {
+__host__ __device__ inline int fc_rows(int C) { return C >= 8 ? 4 : C >= 2 ? 2 : 1; }
+// tiles of the lower triangle owned by CTA (a, b) of Pr x Pc
+__host__ __device__ inline int fc_slots(int nb, int a, int b, int Pr, int Pc) {
   int t = 0;
-  for (int J = 0; J < p; ++J) t += (p - J + kFitbChunk - 1) / kFitbChunk;
+  for (int I = a; I < nb; I += Pr) t += I >= b ? (I - b) / Pc + 1 : 0;
   return t;
 }
-
-__global__ void __launch_bounds__(kFitbThreads) fitb_panel_kernel(int NP, float *Aws,
-                                                                  const float *Wws, int p,
-                                                                  const int *fbad, float *tpart) {
-  __shared__ Tile Xs, Ys;
-  pdl_wait();
-  pdl_trigger();
-  const int bt = blockIdx.y, ld = NP + 1, tid = threadIdx.x;
-  if (fbad[bt]) return;
-  float *A = Aws + (size_t)bt * NP * ld;
-  const float *W = Wws + (size_t)bt * NP * ld;
-  const int nbw = NP / 32, ncw = (nbw + kFitbChunk - 1) / kFitbChunk, p0 = 32 * p;
-  const int nr = nbw - 1 - p, items = nr + fitb_t_items(p);
-  const int rb = 2 * (tid >> 4), cb = 2 * (tid & 15);
-  bool wpp = false;  // W_pp staged in Ys
-  for (int item = blockIdx.x; item < items; item += gridDim.x) {
-    float acc[2][2] = {};
-    if (item < nr) {  // L_Rp = A_Rp W_pp^T
-      float *ar = A + (size_t)(p0 + 32 + 32 * item) * ld + p0;
-      __syncthreads();  // the previous item's tiles are consumed
-      fitb_tile_load(Xs, ar, ld, tid);
-      if (!wpp) fitb_tile_load(Ys, W + (size_t)p0 * ld + p0, ld, tid);
-      wpp = true;
-      __syncthreads();
-      fitb_mma_abt(Xs, Ys, rb, cb, acc);
-#pragma unroll
-      for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int v = 0; v < 2; ++v) ar[(size_t)(rb + u) * ld + cb + v] = acc[u][v];
-      continue;
+// the largest number of tiles of any CTA, and the operand tiles of a panel
+__host__ __device__ inline int fc_max_slots(int nb, int C) {
+  const int Pr = fc_rows(C), Pc = C / Pr;
+  int t = 0;
+  for (int a = 0; a < Pr; ++a)
+    for (int b = 0; b < Pc; ++b) {
+      const int q = fc_slots(nb, a, b, Pr, Pc);
+      t = q > t ? q : t;
     }
-    // the item's (J, c): K in [J + c kFitbChunk, min(J + (c + 1) kFitbChunk, p))
-    int J = 0, rest = item - nr;
-    while (rest >= (p - J + kFitbChunk - 1) / kFitbChunk) {
-      rest -= (p - J + kFitbChunk - 1) / kFitbChunk;
-      ++J;
-    }
-    const int c = rest, Kb = J + c * kFitbChunk, Ke = min(Kb + kFitbChunk, p);
-    wpp = false;
-    for (int K = Kb; K < Ke; ++K) {
-      __syncthreads();
-      fitb_tile_load(Xs, A + (size_t)p0 * ld + 32 * K, ld, tid);
-      fitb_tile_load(Ys, W + (size_t)(32 * K) * ld + 32 * J, ld, tid);
-      __syncthreads();
-      fitb_mma_ab(Xs, Ys, rb, cb, acc);
-    }
-    const size_t tile = ((size_t)bt * nbw + J) * ncw + c;
-    if (!BOUTE_INB(tile, (size_t)gridDim.y * nbw * ncw)) continue;
-    float *tp = tpart + tile * 1024;
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-#pragma unroll
-      for (int v = 0; v < 2; ++v) tp[(rb + u) * 32 + cb + v] = acc[u][v];
-  }
+  return t;
 }
-
-// (c) W_pJ = -W_pp T_pJ for J < p (one work item each; T_pJ the partials
-// added in chunk order, so the result does not depend on the grid), then the
-// trailing update A_IJ -= L_Ip L_Jp^T for p < J <= I (one item per 32 x 32
-// tile; the lower triangle of the diagonal tiles).
-__global__ void __launch_bounds__(kFitbThreads) fitb_update_kernel(int NP, float *Aws,
-                                                                   float *Wws, int p,
-                                                                   const int *fbad,
-                                                                   const float *tpart) {
-  __shared__ Tile Xs, Ys;
-  pdl_wait();
-  pdl_trigger();
-  const int bt = blockIdx.y, ld = NP + 1, tid = threadIdx.x;
-  if (fbad[bt]) return;
-  float *A = Aws + (size_t)bt * NP * ld;
-  float *W = Wws + (size_t)bt * NP * ld;
-  const int nbw = NP / 32, ncw = (nbw + kFitbChunk - 1) / kFitbChunk, p0 = 32 * p;
-  const int T = nbw - 1 - p, items = p + T * (T + 1) / 2;
-  const int rb = 2 * (tid >> 4), cb = 2 * (tid & 15);
-  bool wpp = false;  // W_pp staged in Xs
-  for (int item = blockIdx.x; item < items; item += gridDim.x) {
-    float acc[2][2] = {};
-    if (item < p) {  // W_pJ, J = item
-      const int J = item, nc = (p - J + kFitbChunk - 1) / kFitbChunk;
-      const float *tp = tpart + ((size_t)bt * nbw + J) * ncw * 1024;
-      __syncthreads();
-      if (!wpp) fitb_tile_load(Xs, W + (size_t)p0 * ld + p0, ld, tid);
-      wpp = true;
+__host__ __device__ inline int fc_ops(int nb, int C) {
+  const int Pr = fc_rows(C), Pc = C / Pr;
+  return (nb + Pr - 1) / Pr + (nb + Pc - 1) / Pc;
+}
+// acc[u][v] = sum_q X(4 ty + u, q) Y(4 tx + v, q) by 64 threads (t = 8 ty + tx), each
+// an fmaf chain over q = 0 .. 31 in order.
+__device__ __forceinline__ void fc_product(const float *X, const float *Y, int t,
+                                           float (&acc)[4][4]) {
+  const int tx = t & 7, ty = t >> 3;
 #pragma unroll
-      for (int j = 0; j < 1024 / kFitbThreads; ++j) {
-        const int x = tid + kFitbThreads * j;
-        float t = 0.f;
-        for (int c = 0; c < nc; ++c) t += tp[(size_t)c * 1024 + x];
-        Ys[x >> 5][x & 31] = t;
+  for (int u = 0; u < 4; ++u)
+#pragma unroll
+    for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
+  const float4 *X4 = (const float4 *)X + 4 * ty * 8, *Y4 = (const float4 *)Y + 4 * tx * 8;
+#pragma unroll 2
+  for (int g = 0; g < 8; ++g) {
+    float4 x[4], y[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = X4[u * 8 + (g ^ ty)];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) y[v] = Y4[v * 8 + (g ^ tx)];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        acc[u][v] = fmaf(x[u].x, y[v].x, acc[u][v]);
+        acc[u][v] = fmaf(x[u].y, y[v].y, acc[u][v]);
+        acc[u][v] = fmaf(x[u].z, y[v].z, acc[u][v]);
+        acc[u][v] = fmaf(x[u].w, y[v].w, acc[u][v]);
       }
-      __syncthreads();
-      fitb_mma_ab(Xs, Ys, rb, cb, acc);
-      float *wr = W + (size_t)p0 * ld + 32 * J;
-#pragma unroll
-      for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int v = 0; v < 2; ++v) wr[(size_t)(rb + u) * ld + cb + v] = -acc[u][v];
-      continue;
-    }
-    const int e = item - p;
-    int ti = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);
-    while (ti * (ti + 1) / 2 > e) --ti;
-    while ((ti + 1) * (ti + 2) / 2 <= e) ++ti;
-    const int tj = e - ti * (ti + 1) / 2, I = p + 1 + ti, J = p + 1 + tj;
-    wpp = false;
-    __syncthreads();
-    fitb_tile_load(Xs, A + (size_t)(32 * I) * ld + p0, ld, tid);
-    fitb_tile_load(Ys, A + (size_t)(32 * J) * ld + p0, ld, tid);
-    __syncthreads();
-    fitb_mma_abt(Xs, Ys, rb, cb, acc);
-    float *ar = A + (size_t)(32 * I) * ld + 32 * J;
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-#pragma unroll
-      for (int v = 0; v < 2; ++v)
-        if (I != J || cb + v <= rb + u) ar[(size_t)(rb + u) * ld + cb + v] -= acc[u][v];
   }
 }
 
-// ---- alpha on the blocked path, across many blocks -----------------------------
-// After the blocked factorisation, fit32_kernel's alpha (alpha0 = W^T (W y),
-// then two refinement steps against K = hi + lo with double-float residuals,
-// the second correction kept as alpha's lo part) runs as a chain of kernels,
-// each spread over many blocks per problem-objective (a grid of x blocks per
-// problem-objective y): fitr_init_kernel (the standardised y, the output
-// padding), then per solve fitr_wx_kernel (t = W rhs, a warp per row) and
-// fitr_wtx_kernel (W^T t, 32 columns per block, the rows split over its warps
-// and added in a fixed order), and fitr_resid_kernel (r = y - K alpha, a half
-// warp per row) between the solves. The vectors live in the workspace fvec,
-// kFitrVecs x NP floats per problem-objective.
-enum { kVy = 0, kVylo = 1, kVal = 2, kVlo = 3, kVt = 4, kVr = 5, kFitrVecs = 6 };
+// The diagonal tile by warps 0 and 1: tile = L L^T factored by warp 0 (lane = row) and
+// W_pp = L^-1 formed by warp 1 (lane = column of W_pp), eight columns of L behind. W_pp
+// goes to wpp (row, column) and, transposed, to wtpp and into the tile. dg: the tile's
+// diagonal of K. Each warp holds a window of its row (column) that moves four columns
+// per iteration, so that register indices are static and the code stays small (unrolled
+// over the 32 columns it ran three times longer, waiting for instructions); column c
+// of L reaches the row updates as broadcast 16-byte loads, and only the entry that the
+// next pivot waits for as a shuffle.
+struct FcDiag {
+  float colL[34 * 32];  // columns of L_pp (rows from the diagonal on); the windows' reads
+                        // run up to 28 words past a column
+  float invs[32];       // 1 / L_cc
+};
+__device__ __forceinline__ void fc_diagonal(float *tile, const float *dg, FcDiag &sh, float *wpp,
+                                            float *wtpp, int *fbad) {
+  const int lane = threadIdx.x & 31;
+  const unsigned FULL = 0xffffffffu;
+  if (threadIdx.x < 32) {
+    float a[36];  // columns c0 .. c0 + 31 of the lane's row (those beyond 31: never used)
+#pragma unroll
+    for (int g = 0; g < 8; ++g) {
+      const float4 v = ((const float4 *)tile)[lane * 8 + ((g ^ (lane >> 2)) & 7)];
+      a[4 * g] = v.x;
+      a[4 * g + 1] = v.y;
+      a[4 * g + 2] = v.z;
+      a[4 * g + 3] = v.w;
+    }
+    a[32] = a[33] = a[34] = a[35] = 0.f;
+    bool ok = true;
+    float piv = __shfl_sync(FULL, a[0], 0);
+#pragma unroll 1
+    for (int c0 = 0; c0 < 32; c0 += 4) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int c = c0 + j;
+        if (!(piv > 16.f * 1.1920929e-7f * dg[c])) ok = false;
+        float inv = rsqrtf(piv);
+        inv = inv * fmaf(-0.5f * piv * inv, inv, 1.5f);  // one Newton step; 1 / L_cc
+        const float l = lane == c ? piv * inv : a[j] * inv;  // (rows above c: never used)
+        float *col = sh.colL + c * 32;
+        col[lane] = l;
+        if (lane == 0) sh.invs[c] = inv;
+        // the next pivot: lane c + 1's entry, which needs that lane's l alone
+        piv = __shfl_sync(FULL, fmaf(-l, l, a[j + 1]), (c + 1) & 31);
+        a[j + 1] = fmaf(-l, __shfl_sync(FULL, l, (c + 1) & 31), a[j + 1]);
+        __syncwarp();
+#pragma unroll
+        for (int g = (j + 2) / 4; g < 8; ++g) {  // the window's columns j + 2 ..
+          const float4 v = *(const float4 *)(col + c0 + 4 * g);
+          if (4 * g > j + 1) a[4 * g] = fmaf(-l, v.x, a[4 * g]);
+          if (4 * g + 1 > j + 1) a[4 * g + 1] = fmaf(-l, v.y, a[4 * g + 1]);
+          if (4 * g + 2 > j + 1) a[4 * g + 2] = fmaf(-l, v.z, a[4 * g + 2]);
+          if (4 * g + 3 > j + 1) a[4 * g + 3] = fmaf(-l, v.w, a[4 * g + 3]);
+        }
+      }
+      if (c0 & 4) named_barrier_arrive(9 + (c0 >> 3), 64);  // eight columns for warp 1
+#pragma unroll
+      for (int k = 0; k < 32; ++k) a[k] = a[k + 4];
+    }
+    if (!ok && lane == 0) __stcg(fbad, 1);
+  } else {
+    float r[36];  // rows c0 .. c0 + 31 of column `lane`: the remainders
+#pragma unroll
+    for (int c = 0; c < 36; ++c) r[c] = (c == lane) ? 1.f : 0.f;
+#pragma unroll 1
+    for (int c0 = 0; c0 < 32; c0 += 4) {
+      if (!(c0 & 4)) named_barrier_sync(9 + (c0 >> 3), 64);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int c = c0 + j;
+        const float *col = sh.colL + c * 32;
+        r[j] *= sh.invs[c];  // W_c,lane
+#pragma unroll
+        for (int g = (j + 1) / 4; g < 8; ++g) {  // r_i -= L_ic W_c,lane, rows below c
+          const float4 v = *(const float4 *)(col + c0 + 4 * g);
+          if (4 * g > j) r[4 * g] = fmaf(-v.x, r[j], r[4 * g]);
+          if (4 * g + 1 > j) r[4 * g + 1] = fmaf(-v.y, r[j], r[4 * g + 1]);
+          if (4 * g + 2 > j) r[4 * g + 2] = fmaf(-v.z, r[j], r[4 * g + 2]);
+          if (4 * g + 3 > j) r[4 * g + 3] = fmaf(-v.w, r[j], r[4 * g + 3]);
+        }
+        wpp[fc_off(c, lane)] = r[j];
+      }
+      const float4 v = make_float4(r[0], r[1], r[2], r[3]);
+      const int o = lane * 8 + (((c0 >> 2) ^ (lane >> 2)) & 7);
+      ((float4 *)wtpp)[o] = v;
+      ((float4 *)tile)[o] = v;
+#pragma unroll
+      for (int k = 0; k < 32; ++k) r[k] = r[k + 4];
+    }
+  }
+  __syncwarp();
+}
 
-__global__ void __launch_bounds__(256) fitr_init_kernel(const double *Ys, int standardize, int n,
-                                                        int m, int NP, float *fvec, float *xt,
-                                                        int DP, PostPlan plan, int comp,
-                                                        int *status, const int *fbad) {
+// Shared memory of CTA `rank` of the cluster at this CTA's address p, and stores there.
+__device__ __forceinline__ uint32_t fc_remote(const float *p, int rank) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void fc_store4(uint32_t a, const float4 &v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y),
+               "f"(v.z), "f"(v.w)
+               : "memory");
+}
+__device__ __forceinline__ void fc_store1(uint32_t a, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+
+// TS: the tiles in shared memory.
+template <bool TS>
+__global__ void __launch_bounds__(kFcThreads, 1) fitc_kernel(
+    const float *Kh_all, const float *Kl_all, const double *Ys, int standardize, int n, int m,
+    int NP, int C, int max_slots, float *Aws, float *Wws, float *xt, int DP, PostPlan plan,
+    uint16_t *bop, int comp, int *status, int *fbad_all) {
+  extern __shared__ __align__(16) float sm[];
+  __shared__ __align__(16) FcDiag dsh;
   __shared__ double ymu, yisd;
-  pdl_wait();
-  pdl_trigger();
-  const int bt = blockIdx.x, b = bt / m, t = bt % m, tid = threadIdx.x, lane = tid & 31;
-  if (fbad[bt]) {
-    if (tid == 0) set_status(status, BOUTE_ERR_NOT_PD);
-    return;
+  __shared__ int row_first[BOUTE_MAX_N / 32 + 1];  // the first slot of each block row of this CTA
+  __shared__ int next_item, item[kFcGroups];       // the updates' queue beside a diagonal tile
+  const int bt = blockIdx.x / C, rank = blockIdx.x % C, b = bt / m, t = bt % m;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = kFcThreads / 32;
+  const int grp = tid >> 6, gt = tid & 63;
+  const int nb = NP / 32, Pr = fc_rows(C), Pc = C / Pr, ra = rank % Pr, rb = rank / Pr;
+  const int sr = 31 - __clz(Pr), sc = 31 - __clz(Pc);  // (powers of two)
+  const int nR = (nb + Pr - 1) / Pr, nC = (nb + Pc - 1) / Pc;
+  // operand tiles of a panel (rows: L_Ip; columns: L_Jp or W_pJ^T), W_pp, W_pp^T of
+  // two panels, K's diagonal at this CTA's block rows, the slots' block coordinates
+  float *rop = sm, *cop = rop + (size_t)nR * kFcTile, *wpp = cop + (size_t)nC * kFcTile;
+  float *wt = wpp + kFcTile, *dg = wt + 2 * kFcTile;
+  unsigned short *slotI = (unsigned short *)(dg + 32 * nR), *slotJ = slotI + max_slots;
+  float *tiles = TS ? dg + 32 * nR + ((max_slots + 3) & ~3) : Aws + (size_t)bt * NP * (NP + 1);
+  if (!TS)  // this CTA's share: the owners' tiles one after another
+    for (int r = 0; r < rank; ++r) tiles += (size_t)fc_slots(nb, r % Pr, r / Pr, Pr, Pc) * kFcTile;
+  int *fbad = fbad_all + bt;
+  auto sync = [&]() {
+    __syncwarp();
+    if (C > 1)
+      asm volatile(
+          "barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
+              : "memory");
+    else
+      __syncthreads();
+  };
+  // this CTA's block rows I = ra + Pr i, each with the columns J = rb + Pc j <= I
+  const int lrows = ra < nb ? ((nb - 1 - ra) >> sr) + 1 : 0;
+  auto row_count = [&](int I) { return I >= rb ? ((I - rb) >> sc) + 1 : 0; };
+  for (int i = tid; i <= lrows; i += kFcThreads) {
+    int q = 0;
+    for (int e = 0; e < i; ++e) q += row_count(ra + (e << sr));
+    row_first[i] = q;
   }
+  __syncthreads();
+  const int nslots = row_first[lrows];
+  for (int i = warp; i < lrows; i += nw)
+    for (int j = lane; j < row_count(ra + (i << sr)); j += 32) {
+      slotI[row_first[i] + j] = (unsigned short)(ra + (i << sr));
+      slotJ[row_first[i] + j] = (unsigned short)(rb + (j << sc));
+    }
   const double *y = Ys + (size_t)b * n * m + t;
-  if (tid < 32) standardize_stats(y, n, m, standardize, lane, ymu, yisd);
-  __syncthreads();
-  float *v = fvec + (size_t)bt * kFitrVecs * NP;
-  for (int i = tid; i < NP; i += blockDim.x) {  // standardised y as an fp32 pair
-    const double ys = i < n ? (y[(size_t)i * m] - ymu) * yisd : 0.0;
-    const float hi = (float)ys;
-    v[kVy * NP + i] = hi;
-    v[kVylo * NP + i] = (float)(ys - (double)hi);
-  }
-  const int cf = xt_chunk_floats(DP);
-  float *xa = xt + (size_t)bt * plan.nxt * cf + xt_alpha_offset(DP);
-  for (int k = n + tid; k < BOUTE_KCHUNK * plan.nxt; k += blockDim.x) {  // alpha's padding
-    float *q = xa + (size_t)(k / BOUTE_KCHUNK) * cf + k % BOUTE_KCHUNK;
-    q[0] = 0.f;
-    q[BOUTE_KCHUNK] = 0.f;
-  }
-  if (comp && tid < 32) composite_wmax(xt, bt, plan, DP, n, lane);
-}
-
-// t = W rhs (W lower triangular): a warp per row, two accumulators per lane,
-// the lanes combined by shuffles in a fixed order.
-__global__ void __launch_bounds__(256) fitr_wx_kernel(int NP, const float *Wws, float *fvec,
-                                                      int src, const int *fbad) {
+  if (warp == nw - 1) standardize_stats(y, n, m, standardize, lane, ymu, yisd);
+  // everything below reads what the set-up kernel wrote
   pdl_wait();
-  pdl_trigger();
-  const int bt = blockIdx.y, ld = NP + 1, lane = threadIdx.x & 31;
-  if (fbad[bt]) return;
-  const float *W = Wws + (size_t)bt * NP * ld;
-  float *v = fvec + (size_t)bt * kFitrVecs * NP;
-  const float *rhs = v + src * NP;
-  const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (i >= NP) return;
-  const float *wr = W + (size_t)i * ld;
-  float s0 = 0.f, s1 = 0.f;
-  int k = lane;
-  for (; k + 32 <= i; k += 64) {
-    s0 = fmaf(wr[k], rhs[k], s0);
-    s1 = fmaf(wr[k + 32], rhs[k + 32], s1);
-  }
-  if (k <= i) s0 = fmaf(wr[k], rhs[k], s0);
-  float r = s0 + s1;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-  if (lane == 0 && BOUTE_INB(i, NP)) v[kVt * NP + i] = r;
-}
-
-// W^T t for columns [32 x, 32 x + 32): lane = column, warp w takes the rows
-// i = k0 + w, k0 + w + 8, ... (those at or below the column's diagonal), the
-// eight partial sums added in a fixed order. mode 0: alpha = the result;
-// mode 1: alpha += the result; mode 2: alpha + the result kept exactly as a
-// pair (hi, lo), written with alpha's padding into the side input.
-__global__ void __launch_bounds__(256) fitr_wtx_kernel(int NP, int n, const float *Wws,
-                                                       float *fvec, int mode, float *xt, int DP,
-                                                       PostPlan plan, const int *fbad) {
-  __shared__ float part[8][33];
-  pdl_wait();
-  pdl_trigger();
-  const int bt = blockIdx.y, ld = NP + 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (fbad[bt]) return;
-  const float *W = Wws + (size_t)bt * NP * ld;
-  float *v = fvec + (size_t)bt * kFitrVecs * NP;
-  const float *tv = v + kVt * NP;
-  const int k0 = 32 * blockIdx.x, k = k0 + lane;
-  float s0 = 0.f, s1 = 0.f;  // entries above the diagonal are never loaded
-  int i = k0 + warp;
-  for (; i + 8 < NP; i += 16) {
-    const float w0 = i >= k ? W[(size_t)i * ld + k] : 0.f;
-    const float w1 = i + 8 >= k ? W[(size_t)(i + 8) * ld + k] : 0.f;
-    s0 = fmaf(w0, tv[i], s0);
-    s1 = fmaf(w1, tv[i + 8], s1);
-  }
-  if (i < NP && i >= k) s0 = fmaf(W[(size_t)i * ld + k], tv[i], s0);
-  part[warp][lane] = s0 + s1;
-  __syncthreads();
-  if (warp == 0 && BOUTE_INB(k, NP)) {
-    const float out = ((part[0][lane] + part[1][lane]) + (part[2][lane] + part[3][lane])) +
-                      ((part[4][lane] + part[5][lane]) + (part[6][lane] + part[7][lane]));
-    float *al = v + kVal * NP;
-    if (mode == 0) {
-      al[k] = out;
-    } else if (mode == 1) {
-      al[k] += out;
-    } else {
-      float hi, lo;
-      two_sum(al[k], out, hi, lo);
-      al[k] = hi;
-      v[kVlo * NP + k] = lo;
-      if (k < n) {
-        const int cf = xt_chunk_floats(DP);
-        float *q = xt + (size_t)bt * plan.nxt * cf + xt_alpha_offset(DP) +
-                   (size_t)(k / BOUTE_KCHUNK) * cf + k % BOUTE_KCHUNK;
-        q[0] = hi;
-        q[BOUTE_KCHUNK] = lo;
-      }
-    }
-  }
-}
-
-// r = y - K alpha in double-float (K = hi + lo, alpha zero from n on): a half
-// warp per row, eight loads of each of K hi and K lo per lane in flight, the
-// lanes combined by shuffles in a fixed order; zero from n on.
-__global__ void __launch_bounds__(256) fitr_resid_kernel(const float *Kh_all, const float *Kl_all,
-                                                         int n, int NP, float *fvec,
-                                                         const int *fbad) {
-  pdl_wait();
-  pdl_trigger();
-  const int bt = blockIdx.y, lane = threadIdx.x & 31, hl = lane & 15;
-  if (fbad[bt]) return;
   const float *Kh = Kh_all + (size_t)bt * n * n, *Kl = Kl_all + (size_t)bt * n * n;
-  float *v = fvec + (size_t)bt * kFitrVecs * NP;
-  const float *al = v + kVal * NP;
-  const int i = blockIdx.x * 16 + (threadIdx.x >> 4);
-  if (i >= NP) return;  // a whole half warp
-  float sh = 0.f, sl = 0.f;
-  if (i < n) {
-    for (int k0 = 0; k0 < n; k0 += 128) {
-      float h8[8], l8[8], a8[8];
+  if (rank == 0 && tid == 0) __stcg(fbad, 0);
+  for (int e = tid; e < 32 * lrows; e += kFcThreads) {
+    const int i = 32 * (ra + ((e >> 5) << sr)) + (e & 31);
+    dg[e] = i < n ? Kh[(size_t)i * n + i] : 1.f;
+  }
+  __syncthreads();
+  for (int e = warp; e < 4 * nslots; e += nw) {  // eight rows of a tile per warp
+    const int s = e >> 2, r0 = 8 * (e & 3), i0 = 32 * slotI[s] + r0, k = 32 * slotJ[s] + lane;
+    float v[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int k = k0 + hl + 16 * u;
-        const bool ok = k < n;
-        a8[u] = ok ? al[k] : 0.f;
-        h8[u] = ok ? Kh[(size_t)i * n + k] : 0.f;
-        l8[u] = ok ? Kl[(size_t)i * n + k] : 0.f;
-      }
+    for (int u = 0; u < 8; ++u) {
+      const int i = i0 + u;
+      v[u] = (i < n && k < n) ? Kh[(size_t)i * n + k] : (i == k ? 1.f : 0.f);
+    }
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        float pr, e, s_, e2;
-        two_prod(h8[u], a8[u], pr, e);
-        two_sum(sh, pr, s_, e2);
-        sh = s_;
-        sl += e2 + fmaf(l8[u], a8[u], e);
+    for (int u = 0; u < 8; ++u) tiles[(size_t)s * kFcTile + fc_off(r0 + u, lane)] = v[u];
+  }
+  __syncthreads();
+  auto at = [&](const float *q, int r) { return fc_remote(q, r); };
+  // W_pp and W_pp^T, from this CTA's wpp and wt, to the CTAs of block row and column p
+  auto send_diagonal = [&](int p) {
+    const int a = p & (Pr - 1), c = p & (Pc - 1), par = p & 1;
+    float4 v[4], w[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      v[u] = ((const float4 *)wpp)[gt + 64 * u];
+      w[u] = ((const float4 *)(wt + par * kFcTile))[gt + 64 * u];
+    }
+    for (int q = 0; q < Pr + Pc; ++q) {
+      const int r = q < Pr ? q + Pr * c : a + Pr * (q - Pr);
+      if (r == rank) continue;
+      const uint32_t dst = at(wpp, r) + 16 * gt, dwt = at(wt + par * kFcTile, r) + 16 * gt;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        fc_store4(dst + 1024 * u, v[u]);
+        if (q < Pr) fc_store4(dwt + 1024 * u, w[u]);
       }
     }
+  };
+  sync();  // every CTA of the cluster runs: its shared memory may be written
+  if (rank == 0 && grp == 0) {
+    fc_diagonal(tiles, dg, dsh, wpp, wt, fbad);
+    named_barrier_sync(1, 64);
+    send_diagonal(0);
   }
-  const unsigned half = 0xffffu << (lane & 16);
+  float acc[4][4];
+  const int tx = gt & 7, ty = gt >> 3;
+  // block row p of W (final after panel p's products): W itself and its operand images
+  const int cf = xt_chunk_floats(DP);
+  float *x0 = xt + (size_t)bt * plan.nxt * cf;
+  const float wscale = exp2i((int)x0[xt_param_offset(DP) + 2 * DP + kParEW]);
+  const int gmax = BOUTE_BLKCOLS * (plan.nwblk - 1) + plan.ncol[plan.nwblk - 1];
+  uint16_t *img = bop + (size_t)bt * plan.image_halves;
+  float *W = Wws + (size_t)bt * NP * (NP + 1);
+  bool fits = true;
+  auto output_row = [&](int p) {
+    const int f = row_first[(p - ra) >> sr], cnt = 4 * row_count(p);
+#pragma unroll 1
+    for (int e = warp; e < cnt; e += nw) {  // eight rows of a tile per warp
+      const int s = f + (e >> 2), r0 = 8 * (e & 3), J = slotJ[s];
+      const float *T = tiles + (size_t)s * kFcTile;
 #pragma unroll
-  for (int o = 8; o > 0; o >>= 1) {  // within the half warp
-    const float oh = __shfl_xor_sync(half, sh, o);
-    const float ol = __shfl_xor_sync(half, sl, o);
-    float s_, e;
-    two_sum(sh, oh, s_, e);
-    sh = s_;
-    sl += ol + e;
+      for (int u = 0; u < 8; ++u) {
+        const int i = 32 * p + r0 + u, k = 32 * J + lane;
+        if (i < n && k <= i) W[(size_t)i * (NP + 1) + k] = T[fc_off(lane, r0 + u)];
+      }
+      const int kk = 2 * (lane & 15);
+#pragma unroll 1
+      for (int u = 0; u < 8; u += 2) {
+        const int r = r0 + u + (lane >> 4), g = 32 * p + r;
+        if (g >= gmax) continue;
+        fits &= pack_values(T[fc_off(kk, r)], T[fc_off(kk + 1, r)], g, 32 * J + kk, plan, wscale, img);
+        if (p == J)  // zeros right of the diagonal tile, as far as the block's chunks reach
+#pragma unroll 1
+          for (int k = 32 * (J + 1) + kk; k < BOUTE_ACHUNK * plan.kc[g / BOUTE_BLKCOLS]; k += 32)
+            pack_values(0.f, 0.f, g, k, plan, wscale, img);
+      }
+    }
+    __syncwarp();
+  };
+  for (int p = 0; p < nb; ++p) {
+    sync();  // W_pp has arrived; the previous panel's operands are consumed
+    // L_Ip = A_Ip W_pp^T and W_pJ^T = R_pJ^T W_pp^T
+    const int i1 = p < ra ? 0 : ((p - ra) >> sr) + 1;  // first block row of this CTA below p
+    const int f1 = row_first[i1], a = p & (Pr - 1), c = p & (Pc - 1);
+    const int nl = rb == c ? lrows - i1 : 0;
+    const int nwt = ra == a ? row_count(p) - (rb == c ? 1 : 0) : 0;
+    if (tid == 0) next_item = f1;
+    for (int e = grp; e < nl + nwt; e += kFcGroups) {
+      int s, X;
+      if (e < nl) {
+        X = ra + ((i1 + e) << sr);
+        s = row_first[i1 + e] + ((p - rb) >> sc);
+      } else {
+        s = row_first[(p - ra) >> sr] + (e - nl);
+        X = rb + ((e - nl) << sc);
+      }
+      float *T = tiles + (size_t)s * kFcTile;
+      fc_product(T, wpp, gt, acc);
+      // to the column operands of CTAs (., X mod Pc) and, L_Ip, the row operands of
+      // CTAs (X mod Pr, .)
+      const int o = ((4 * ty) * 8 + (tx ^ ty)) * 16;
+      if (p < nb - 1)
+        for (int q = 0; q < (e < nl ? Pr + Pc : Pr); ++q) {
+          const uint32_t dst =
+              o + (q < Pr ? at(cop + (size_t)(X >> sc) * kFcTile, q + Pr * (X & (Pc - 1)))
+                          : at(rop + (size_t)(X >> sr) * kFcTile, (X & (Pr - 1)) + Pr * (q - Pr)));
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            fc_store4(dst + 128 * u, make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]));
+        }
+      if (e >= nl) {
+        named_barrier_sync(1 + grp, 64);  // the tile is read
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          ((float4 *)T)[(4 * ty + u) * 8 + (tx ^ ty)] =
+              make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
+      }
+    }
+    if (p == nb - 1) break;
+    sync();  // L_Ip and W_pJ have arrived
+    // update: the slots from block row i1 on; the next diagonal tile first, by group 0
+    auto update = [&](int s) {
+      const int I = slotI[s], J = slotJ[s];
+      const float *L = rop + (size_t)(I >> sr) * kFcTile;
+      const float *Q = J == p ? wt + (p & 1) * kFcTile : cop + (size_t)(J >> sc) * kFcTile;
+      float *T = tiles + (size_t)s * kFcTile;
+      fc_product(J > p ? L : Q, J > p ? Q : L, gt, acc);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        float4 *q = (float4 *)T + (4 * ty + u) * 8 + (tx ^ ty);
+        float4 v = J == p ? make_float4(0.f, 0.f, 0.f, 0.f) : *q;
+        v.x -= acc[u][0];
+        v.y -= acc[u][1];
+        v.z -= acc[u][2];
+        v.w -= acc[u][3];
+        *q = v;
+      }
+    };
+    const bool own = ((p + 1) & (Pr - 1)) == ra && ((p + 1) & (Pc - 1)) == rb;
+    if (own) {
+      // Beside the diagonal tile's two warps only the groups of the other two
+      // schedulers work (odd groups); the rest join them afterwards.
+      const int sd = row_first[i1] + ((p + 1) >> sc);  // the diagonal tile's slot
+      if (grp == 0) {
+        update(sd);
+        named_barrier_sync(1, 64);
+        fc_diagonal(tiles + (size_t)sd * kFcTile, dg + 32 * i1, dsh, wpp, wt + ((p + 1) & 1) * kFcTile,
+                    fbad);
+        named_barrier_sync(1, 64);
+        send_diagonal(p + 1);
+      }
+      if (!(grp & 1)) named_barrier_sync(13, 32 * nw / 2);
+      for (;;) {
+        if (gt == 0) item[grp] = atomicAdd(&next_item, 1);
+        __syncwarp();
+        named_barrier_sync(1 + grp, 64);
+        const int s = item[grp];
+        if (s >= nslots) break;
+        if (s != sd) update(s);
+        named_barrier_sync(1 + grp, 64);  // (item is read)
+      }
+    } else {
+      for (int s = f1 + grp; s < nslots; s += kFcGroups) update(s);
+    }
+    if (ra == a) output_row(p);
   }
-  if (hl == 0 && BOUTE_INB(i, NP))
-    v[kVr * NP + i] = i < n ? (v[kVy * NP + i] - sh) + (v[kVylo * NP + i] - sl) : 0.f;
-}
-
-// ---- operand images of L^-1 as fp16 hi/lo, swizzled (global-workspace fit) ----
-__global__ void pack_kernel(const float *Wws, PostPlan plan, uint16_t *bop, const float *xt,
-                            int DP, int *status) {
-  if (*status == BOUTE_ERR_NOT_PD) return;
-  const size_t bt = blockIdx.y;
-  const int ld = plan.npad + 1;
-  const float *xpar = xt + bt * plan.nxt * xt_chunk_floats(DP) + xt_param_offset(DP) + 2 * DP;
-  if (!pack_elems(Wws + bt * plan.npad * ld, ld, plan, exp2i((int)xpar[kParEW]),
-                  bop + bt * plan.image_halves,
-                  (long long)blockIdx.x * blockDim.x + threadIdx.x,
-                  (long long)gridDim.x * blockDim.x))
-    set_status(status, BOUTE_ERR_NOT_PD);
+  pdl_trigger();
+  __syncthreads();
+  if (ra == ((nb - 1) & (Pr - 1))) output_row(nb - 1);
+  // ---- alpha0 = W^T (W y), refined twice against K = hi + lo ----------------------
+  // (vectors in the operands' space: x, alpha, y hi, y lo, the partial sums of the CTA's
+  // block rows and of every column, four classes of tiles each)
+  float *x = sm, *al = x + NP, *yv = al + NP, *ylo = yv + NP, *pt = ylo + NP, *pw = pt + 4 * NP;
+  {
+    const double mu = ymu, isd = yisd;
+    for (int i = tid; i < NP; i += kFcThreads) {  // standardised y as an fp32 pair
+      const double ys = i < n ? (y[(size_t)i * m] - mu) * isd : 0.0;
+      yv[i] = x[i] = (float)ys;
+      ylo[i] = (float)(ys - (double)yv[i]);
+    }
+  }
+  __syncthreads();
+  // out(k, (W^T (W x))_k) for every k, in every CTA. W x: a warp per block row and class
+  // J mod 4, lane = row; W^T: a warp per block column and class I mod 4, lane = column;
+  // tiles in ascending order, then the classes.
+  const int kr = 4 / Pr, kcl = 4 / Pc;  // classes of block rows and columns in this CTA
+  const int lcols = rb < nb ? ((nb - 1 - rb) >> sc) + 1 : 0;
+  auto solve = [&](auto out) {
+#pragma unroll 1
+    for (int e = warp; e < lrows * kcl; e += nw) {
+      const int i = e / kcl, q = rb + Pc * (e % kcl), I = ra + (i << sr);
+      float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll 1
+      for (int J = q; J <= I; J += 4) {
+        const float *T = tiles + (size_t)(row_first[i] + (J >> sc)) * kFcTile, *xj = x + 32 * J;
+#pragma unroll
+        for (int k = 0; k < 32; k += 4) {
+          s0 = fmaf(T[fc_off(k, lane)], xj[k], s0);
+          s1 = fmaf(T[fc_off(k + 1, lane)], xj[k + 1], s1);
+          s2 = fmaf(T[fc_off(k + 2, lane)], xj[k + 2], s2);
+          s3 = fmaf(T[fc_off(k + 3, lane)], xj[k + 3], s3);
+        }
+      }
+      const float v = (s0 + s1) + (s2 + s3);
+      for (int r = 0; r < Pc; ++r) fc_store1(at(pw + q * 32 * nR + 32 * i + lane, ra + Pr * r), v);
+    }
+    sync();
+    for (int e = tid; e < 32 * lrows; e += kFcThreads) {  // (class 0's words take the sum)
+      const int w = 32 * nR;
+      pw[e] = (pw[e] + pw[e + w]) + (pw[e + 2 * w] + pw[e + 3 * w]);
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int e = warp; e < lcols * kr; e += nw) {
+      const int j = e / kr, q = ra + Pr * (e % kr), J = rb + (j << sc);
+      float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll 1
+      for (int I = q; I < nb; I += 4) {
+        if (I < J) continue;
+        const int i = (I - ra) >> sr;
+        const float4 *T4 = (const float4 *)(tiles + (size_t)(row_first[i] + j) * kFcTile) + lane * 8;
+        const float4 *v4 = (const float4 *)(pw + 32 * i);
+#pragma unroll
+        for (int g = 0; g < 8; ++g) {
+          const float4 w = T4[(g ^ (lane >> 2)) & 7], v = v4[g];
+          s0 = fmaf(w.x, v.x, s0);
+          s1 = fmaf(w.y, v.y, s1);
+          s2 = fmaf(w.z, v.z, s2);
+          s3 = fmaf(w.w, v.w, s3);
+        }
+      }
+      const float v = (s0 + s1) + (s2 + s3);
+      for (int r = 0; r < C; ++r) fc_store1(at(pt + q * NP + 32 * J + lane, r), v);
+    }
+    sync();
+    for (int k = tid; k < NP; k += kFcThreads)
+      out(k, (pt[k] + pt[k + NP]) + (pt[k + 2 * NP] + pt[k + 3 * NP]));
+    __syncthreads();
+  };
+  solve([&](int k, float v) { al[k] = v; });
+#pragma unroll 1
+  for (int step = 0; step < 2; ++step) {
+    // r = y - K alpha in double-float, a half warp per row, eight loads of each of K
+    // hi and K lo per lane in flight; to every CTA's x
+    const int hl = lane & 15;
+#pragma unroll 1
+    for (int i = rank * (kFcThreads / 16) + (tid >> 4); i < NP; i += C * (kFcThreads / 16)) {
+      float sh = 0.f, sl = 0.f;
+      if (i < n) {
+#pragma unroll 1
+        for (int k0 = 0; k0 < n; k0 += 128) {
+          float h8[8], l8[8], a8[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const int k = k0 + hl + 16 * u;
+            const bool in = k < n;
+            a8[u] = in ? al[k] : 0.f;
+            h8[u] = in ? Kh[(size_t)i * n + k] : 0.f;
+            l8[u] = in ? Kl[(size_t)i * n + k] : 0.f;
+          }
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            float pr, e, s_, e2;
+            two_prod(h8[u], a8[u], pr, e);
+            two_sum(sh, pr, s_, e2);
+            sh = s_;
+            sl += e2 + fmaf(l8[u], a8[u], e);
+          }
+        }
+      }
+      const unsigned half = 0xffffu << (lane & 16);
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) {  // within the half warp
+        const float oh = __shfl_xor_sync(half, sh, o);
+        const float ol = __shfl_xor_sync(half, sl, o);
+        float s_, e;
+        two_sum(sh, oh, s_, e);
+        sh = s_;
+        sl += ol + e;
+      }
+      const float r = i < n ? (yv[i] - sh) + (ylo[i] - sl) : 0.f;
+      if (hl < C) fc_store1(at(x + i, hl), r);
+    }
+    sync();
+    // the second correction is kept exactly: alpha = hi + lo, hi = fl(alpha + delta)
+    solve([&](int k, float v) {
+      float s_, e;
+      two_sum(al[k], v, s_, e);
+      al[k] = s_;
+      if (step == 1) x[k] = e;  // (before that other CTAs may be sending the next residual)
+    });
+  }
+  // (cluster barriers lie between the last pivot and here)
+  const bool bad = __ldcg(fbad) != 0;
+  if (bad || !fits) set_status(status, BOUTE_ERR_NOT_PD);
+  if (bad) return;
+  float *xa = x0 + xt_alpha_offset(DP);
+  for (int k = rank * kFcThreads + tid; k < BOUTE_KCHUNK * plan.nxt; k += C * kFcThreads) {
+    float *q = xa + (size_t)(k / BOUTE_KCHUNK) * cf + k % BOUTE_KCHUNK;
+    q[0] = k < n ? al[k] : 0.f;
+    q[BOUTE_KCHUNK] = k < n ? x[k] : 0.f;
+  }
+  if (comp && rank == 0 && warp == nw - 1) composite_wmax(xt, bt, plan, DP, n, lane);
 }
 
 }  // namespace
@@ -1400,22 +1379,68 @@ int launch_standardize(const double *Y, int B, int n, int m, int codes, double *
 // The shared-memory variant holds n up to 160 (n rounded up to 32).
 bool fit_uses_smem(int npad) { return npad <= 160; }
 
-size_t fit_tpart_floats(int npad, int BM) {
-  if (fit_uses_smem(npad) || 4 * BM > num_sms()) return 0;  // no blocked factorisation
-  const int nbw = npad / 32, ncw = (nbw + kFitbChunk - 1) / kFitbChunk;
-  return (size_t)BM * nbw * ncw * 1024;
-}
-
-size_t fit_fvec_floats(int npad, int BM) {
-  return fit_tpart_floats(npad, BM) ? (size_t)BM * kFitrVecs * npad : 0;
-}
-
-// Dynamic shared memory of the shared-memory fit: A and W (np x (np+1)), six
+// Dynamic shared memory of the shared-memory fit: A and W (np x (np+1)), five
 // vectors, and K lo (n x n) when n <= 128.
 static bool fit_kl_in_smem(int n) { return n <= 128; }
 size_t fit_smem_bytes(int np, int n) {
-  return (2 * (size_t)np * (np + 1) + 6 * (size_t)np + (fit_kl_in_smem(n) ? (size_t)n * n : 0)) *
+  return (2 * (size_t)np * (np + 1) + 5 * (size_t)np + (fit_kl_in_smem(n) ? (size_t)n * n : 0)) *
          sizeof(float);
+}
+
+// Dynamic shared memory of fitc_kernel with clusters of C (tiles: its tiles too).
+static size_t fitc_smem(int npad, int C, bool tiles) {
+  const int nb = npad / 32, ms = fc_max_slots(nb, C);
+  return ((size_t)(fc_ops(nb, C) + 3 + (tiles ? ms : 0)) * kFcTile +
+          32 * ((nb + fc_rows(C) - 1) / fc_rows(C)) + ((ms + 3) & ~3)) *
+         sizeof(float);
+}
+constexpr size_t kFcMaxSmem = 227 * 1024 - 5 * 1024;  // (its static part: 4.9 KB)
+
+// n > 160: clusters of the largest size with which every problem-objective runs at
+// once, and large enough that the operands, and if any size allows it the tiles, fit
+// shared memory (n = 256 on single CTAs, n = 1024 on 16; above that the tiles stay in
+// the workspace).
+static int launch_fitc(Gp *gp, const double *Ys, int standardize, cudaStream_t s) {
+  const int n = gp->n, m = gp->m, npad = gp->plan.npad, nb = npad / 32;
+  const long long BM = (long long)gp->B * m, sms = num_sms();
+  int C = 1;
+  while (C < kFcMaxCluster && (fitc_smem(npad, C, true) > kFcMaxSmem || 2 * C * BM <= sms)) C *= 2;
+  auto go = [&](auto kern, bool tiles) {
+    prefer_shared(kern);
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFcMaxSmem);
+    if (C > 8) cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)(BM * C));
+    cfg.blockDim = dim3(kFcThreads);
+    cfg.dynamicSmemBytes = fitc_smem(npad, C, tiles);
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int fit = 0;
+    if (C > 1 && (cudaOccupancyMaxActiveClusters(&fit, kern, &cfg) != cudaSuccess || fit == 0)) {
+      cudaGetLastError();
+      return false;
+    }
+    cfg.numAttrs = 2;
+    cudaLaunchKernelEx(&cfg, kern, (const float *)gp->Kh, (const float *)gp->Kl, Ys, standardize, n,
+                       m, npad, C, fc_max_slots(nb, C), gp->Aws, gp->Wws, gp->xt, gp->DP, gp->plan,
+                       gp->bop, gp->kern, gp->status, gp->fbad);
+    return true;
+  };
+  // (a partitioned device may not place the larger clusters)
+  for (;; C /= 2) {
+    const bool tiles = fitc_smem(npad, C, true) <= kFcMaxSmem;
+    if (tiles ? go(fitc_kernel<true>, true) : go(fitc_kernel<false>, false)) break;
+    if (C == 1 || fitc_smem(npad, C / 2, false) > kFcMaxSmem) return BOUTE_ERR_CUDA;
+  }
+  count_launch(2);
+  return last_launch_status();
 }
 
 // Ys: standardised outcomes, or raw outcomes when standardize != 0.
@@ -1444,87 +1469,17 @@ static int launch_fit_impl(Gp *gp, const double *X, const double *Ys, int standa
   if (gp->kern) setup(fit_setup_kernel<true>);
   else setup(fit_setup_kernel<false>);
   if (setup_done && cudaEventRecord(setup_done, s) != cudaSuccess) return last_launch_status();
-  // the one-block fits already fill the GPU when there are many problem-
-  // objectives; with few, the blocked factorisation spreads each over blocks
-  const bool blocked = !fit_uses_smem(npad) && 4 * BM <= sms && gp->tpart && gp->fvec;
-  if (fit_uses_smem(npad) || !blocked) {
-    const bool sm_fit = fit_uses_smem(npad);
-    if (sm_fit) {
-      const size_t smem = fit_smem_bytes(npad, n);
-      prefer_shared(fit32_kernel<true>);
-      cudaFuncSetAttribute(fit32_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem);
-      launch_pdl(fit32_kernel<true>, dim3(BM), dim3(fit_threads<true>()), smem, s, gp->Kh,
-                 gp->Kl, Ys, standardize, n, m, gp->Aws, gp->Wws, gp->xt, gp->DP, npad, gp->plan,
-                 gp->bop, fit_kl_in_smem(n) ? 1 : 0, fit_early, gp->kern, gp->status,
-                 (const int *)nullptr, gp->Wws);  // W kept in global memory as well
-      count_launch(2);
-    } else {  // one block per problem-objective on the global workspace
-      launch_pdl(fit32_kernel<false>, dim3(BM), dim3(fit_threads<false>()),
-                 6 * npad * sizeof(float), s, gp->Kh, gp->Kl, Ys, standardize, n, m, gp->Aws,
-                 gp->Wws, gp->xt, gp->DP, npad, gp->plan, gp->bop, 0, 0, gp->kern, gp->status,
-                 (const int *)nullptr, (float *)nullptr);
-      const long long tot = (long long)gp->plan.nwblk * BOUTE_BLKCOLS * gp->plan.nchunk * 32;
-      pack_kernel<<<dim3((unsigned)std::min<long long>((tot + 255) / 256, 4096), BM), 256, 0,
-                    s>>>(gp->Wws, gp->plan, gp->bop, gp->xt, gp->DP, gp->status);
-      count_launch(3);
-    }
-  } else {
-    // the factorisation across many blocks, panel by panel, then alpha across
-    // many blocks and the operand images
-    const int cap = std::max(1, 2 * sms / BM);
-    auto ctas = [&](long long tiles) {
-      return (unsigned)std::max(1LL, std::min<long long>(cap, (tiles + kFitbThreads - 1) / kFitbThreads));
-    };
-    auto grid = [&](long long items) {  // one block per item up to 4 blocks per SM
-      return (unsigned)std::max(1LL, std::min<long long>(std::max(1, 4 * sms / BM), items));
-    };
-    int nl = 0;
-    launch_pdl(fitb_load_kernel, dim3(ctas((long long)npad * npad / 2), BM), dim3(kFitbThreads), 0, s,
-               (const float *)gp->Kh, n, npad, gp->Aws, gp->fbad);
-    ++nl;
-    const int nbw = npad / 32;
-    for (int p = 0; p < nbw; ++p) {
-      const int T = nbw - 1 - p;
-      launch_pdl(fitb_diag_kernel, dim3(BM), dim3(64), 0, s, (const float *)gp->Kh, n, npad,
-                 gp->Aws, gp->Wws, p, gp->fbad);
-      ++nl;
-      // items: the panel's block rows below p, then one per (J, chunk) of T_pJ
-      const long long items = (long long)T + fitb_t_items(p);
-      if (items > 0) {
-        launch_pdl(fitb_panel_kernel, dim3(grid(items), BM), dim3(kFitbThreads), 0, s, npad,
-                   gp->Aws, (const float *)gp->Wws, p, (const int *)gp->fbad, gp->tpart);
-        ++nl;
-      }
-      // items: W_pJ for J < p, then the trailing tiles
-      const long long uitems = (long long)p + (long long)T * (T + 1) / 2;
-      if (uitems > 0) {
-        launch_pdl(fitb_update_kernel, dim3(grid(uitems), BM), dim3(kFitbThreads), 0, s, npad,
-                   gp->Aws, gp->Wws, p, (const int *)gp->fbad, (const float *)gp->tpart);
-        ++nl;
-      }
-    }
-    // alpha: W^T (W y) and two refinement steps, each matvec over many blocks
-    const int *fb = gp->fbad;
-    launch_pdl(fitr_init_kernel, dim3(BM), dim3(256), 0, s, Ys, standardize, n, m, npad,
-               gp->fvec, gp->xt, gp->DP, gp->plan, gp->kern, gp->status, fb);
-    for (int step = 0; step < 3; ++step) {
-      if (step > 0)
-        launch_pdl(fitr_resid_kernel, dim3((npad + 15) / 16, BM), dim3(256), 0, s,
-                   (const float *)gp->Kh, (const float *)gp->Kl, n, npad, gp->fvec, fb);
-      launch_pdl(fitr_wx_kernel, dim3((npad + 7) / 8, BM), dim3(256), 0, s, npad,
-                 (const float *)gp->Wws, gp->fvec, step == 0 ? (int)kVy : (int)kVr, fb);
-      launch_pdl(fitr_wtx_kernel, dim3(npad / 32, BM), dim3(256), 0, s, npad, n,
-                 (const float *)gp->Wws, gp->fvec, step, gp->xt, gp->DP, gp->plan, fb);
-      nl += step > 0 ? 3 : 2;
-    }
-    count_launch(nl + 1);
-    const long long tot = (long long)gp->plan.nwblk * BOUTE_BLKCOLS * gp->plan.nchunk * 32;
-    pack_kernel<<<dim3((unsigned)std::min<long long>((tot + 255) / 256, 4096), BM), 256, 0, s>>>(
-        gp->Wws, gp->plan, gp->bop, gp->xt, gp->DP, gp->status);
-    count_launch(1);
+  if (fit_uses_smem(npad)) {
+    const size_t smem = fit_smem_bytes(npad, n);
+    prefer_shared(fit32_kernel);
+    cudaFuncSetAttribute(fit32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    launch_pdl(fit32_kernel, dim3(BM), dim3(kFitThreads), smem, s, gp->Kh, gp->Kl, Ys, standardize,
+               n, m, gp->xt, gp->DP, npad, gp->plan, gp->bop, fit_kl_in_smem(n) ? 1 : 0, fit_early,
+               gp->kern, gp->status, gp->Wws);  // W kept in global memory as well
+    count_launch(2);
+    return last_launch_status();
   }
-  return last_launch_status();
+  return launch_fitc(gp, Ys, standardize, s);
 }
 
 int launch_fit(Gp *gp, const double *X, const double *Ys, const double *ls, const double *s2,

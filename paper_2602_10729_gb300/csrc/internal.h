@@ -15,7 +15,8 @@ struct Gp {
   int B, n, d, m, DP;  // DP = d rounded up to a multiple of 4 (register tile)
   PostPlan plan;
   float *Kh, *Kl;  // B*m x n x n: kernel matrix (lower) as an fp32 pair hi + lo
-  float *Aws;      // B*m x np x (np+1): factorisation workspace (large n; np = npad)
+  float *Aws;      // B*m x np x (np+1): the factorisation's tiles when they do not fit shared memory
+                   // (n > 1024; np = npad)
   float *Wws;      // B*m x np x (np+1): L^-1 (lower, row stride np+1)
   uint16_t *bop;  // B*m x plan.image_halves: L^-1 as fp16 hi/lo operand images
   // the posterior's cache of K* chunks that later groups of output blocks
@@ -28,9 +29,7 @@ struct Gp {
   float *xt;      // B*m x nxt x xt_chunk_floats(DP): X/lengthscale hi/lo, alpha
   float *s2f;     // B*m: outputscale
   int *status;    // device status word (first error wins)
-  int *fbad;      // B*m: a non-positive pivot in the blocked factorisation (n > 160)
-  float *tpart;   // the blocked factorisation's partial sums of T_pJ (fit_tpart_floats)
-  float *fvec;    // the blocked path's alpha vectors (fit_fvec_floats)
+  int *fbad;      // B*m: a non-positive pivot in the cluster factorisation (n > 160)
   // the FP64 tier (prec = BOUTE_PREC_FP64): W = L^-1 (B*m x n x n), alpha
   // (B*m x n), X / lengthscale (B*m x n x d), lengthscales (B*m x d) and
   // outputscales (B*m) of the last fit, all fp64
@@ -89,12 +88,6 @@ inline int num_sms() {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   return sms;
 }
-
-// floats of the blocked factorisation's partial-sum workspace for B*m = BM
-// problem-objectives at padded size npad (0 when that size never takes it)
-size_t fit_tpart_floats(int npad, int BM);
-// floats of the blocked path's alpha vectors (0 likewise)
-size_t fit_fvec_floats(int npad, int BM);
 
 void count_launch(int k = 1);
 unsigned long long launch_count();

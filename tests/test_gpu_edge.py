@@ -401,3 +401,20 @@ def test_row_pairs_and_column_groups(d, n, N):
     for t in range(2):
         check_mean(g["mean"][0, t], mean[:, t], fp.s2[t])
         check_var(g["var"][0, t], var[:, t], fp.s2[t])
+
+
+# Tiles of 32, from six block rows on: sizes at their edges, batches that take
+# clusters of 16, 8, 4, 2 and 1 CTAs, and tiles that stay in the workspace.
+@pytest.mark.parametrize("n,B", [(161, 1), (192, 2), (193, 1), (224, 40), (256, 40), (288, 20),
+                                 (321, 12), (511, 6), (1024, 1), (1025, 1)])
+def test_cluster_fit_edges(n, B):
+    w = wl.scaled(wl.WORKLOADS[4], N=130, B=B, n=n)
+    hp = host_problem(w)
+    g = gpu_pipeline(hp)
+    assert g["status"] == 0
+    for b in sorted({0, B // 2, B - 1}):
+        fp = oracle_fit(hp, b)
+        mean, var = opl.posterior(fp, hp.Xc[b])
+        for t in range(w.m):
+            check_mean(g["mean"][b, t], mean[:, t], fp.s2[t])
+            check_var(g["var"][b, t], var[:, t], fp.s2[t])

@@ -72,6 +72,7 @@ __global__ void __launch_bounds__(256) ehvi2d_kernel(const float *mean, const fl
                                                      const double *cons, float *acq) {
   extern __shared__ float cells[];  // bnd[n+1] (b_i), up[n+1] (u_i)
   pdl_wait();
+  pdl_trigger();
   const int b = blockIdx.y;
   const int Pb = P[b];
   float *bnd = cells, *up = cells + (n + 1);
@@ -231,6 +232,7 @@ __global__ void __launch_bounds__(512) mchvi_kernel(const float *mean, const flo
   extern __shared__ float boxes[];  // per problem in this block: lo[K][M], hi[K][M]
   __shared__ float4 stage[16][64];  // per warp: 32 boxes' constants (mc_hvi_regs)
   pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
   const int b = blockIdx.y;
   const int K = BOUTE_INB(Kc[b], box_cap + 1) ? Kc[b] : 0;
@@ -351,6 +353,7 @@ __global__ void __launch_bounds__(512, 2) mchvi2_kernel(const float *mean, const
   // 1 + a multiple of 4 (they add exactly nothing), box_cap + 4 in all
   extern __shared__ float4 strips4[];
   pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
   const int b = blockIdx.y;
   const int K = mc2_load_strips(strips4, lower, upper, Kc, b, box_cap, threadIdx.x, blockDim.x);

@@ -284,6 +284,7 @@ __global__ void __launch_bounds__(kInsThreads, 1)
   __syncthreads();
   for (int e = tid; e < n * n; e += kInsThreads)
     wsb[(size_t)n * n + e] = Kb[(size_t)(e / n) * ldk + e % n];
+  pdl_trigger();
   // H^T's operand images (output rows of the H blocks) and scale
   const int eh = scale_exp(__uint_as_float(mxh));
   if (tid == 0) x0[xt_param_offset(DP) + 2 * DP + kParEH] = (float)eh;
@@ -311,6 +312,7 @@ __global__ void __launch_bounds__(kDrawThreads)
   float *F = sm, *Ht = F + (size_t)n * ld, *zs = Ht + (size_t)n * ld, *mu = zs + kInsDraws * kInsMaxN;
   float *wsb = ws + (size_t)bt * ins_ws_floats(n);
   pdl_wait();
+  pdl_trigger();
   if (*status == BOUTE_ERR_NOT_PD) return;
   for (int i = warp; i < n; i += kInsDraws) {  // a warp per row, eight loads in flight
     float f[kInsMaxN / 32], h[kInsMaxN / 32];
@@ -374,6 +376,7 @@ __global__ void __launch_bounds__(256)
                          int nxt, uint16_t *bop, PostPlan plan, const int *status) {
   const int bt = blockIdx.y;
   pdl_wait();
+  pdl_trigger();
   if (*status == BOUTE_ERR_NOT_PD) return;
   const float *wsb = ws + (size_t)bt * ins_ws_floats(n);
   const int eg = scale_exp(wsb[2 * (size_t)n * n + n]);
@@ -445,6 +448,7 @@ __global__ void __launch_bounds__(32 * kFrontWarps)
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int bs = blockIdx.x * kFrontWarps + w;  // (problem, draw)
   pdl_wait();
+  pdl_trigger();
   if (bs >= B * S) return;
   const int b = bs / S, s = bs % S;
   const float r1 = (float)ref[(size_t)b * 2], r2 = (float)ref[(size_t)b * 2 + 1];
@@ -543,6 +547,7 @@ __global__ void __launch_bounds__(kAcqThreads)
   const int b = blockIdx.y;
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   pdl_wait();
+  pdl_trigger();
   const float4 *stb = strips + (size_t)b * S * (n + 1);
   const int *cnt = counts + (size_t)b * S;
   // exclusive scan of the counts (S <= 1024): loaded by all, scanned by warp 0

@@ -160,6 +160,7 @@ __global__ void __launch_bounds__(NT) topk_kernel(const float *vals,
   __shared__ int red[NT / 32];
   __shared__ unsigned long long sel[FINAL ? kMaxK : 1];
   pdl_wait();
+  if (!FINAL) pdl_trigger();
   const int b = blockIdx.y, tid = threadIdx.x;
   const long long base = (long long)blockIdx.x * (NT * kR);
   unsigned hi[kR], lw[VALUES ? 1 : kR];

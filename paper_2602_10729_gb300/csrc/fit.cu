@@ -237,13 +237,6 @@ __device__ __forceinline__ bool pack_values(float w0, float w1, int g, int k, co
   }
   return fabsf(v0) < 32768.f && fabsf(v1) < 32768.f;
 }
-// The same from row g of W.
-__device__ __forceinline__ bool pack_pair(const float *wrow, int g, int k, const PostPlan &plan,
-                                          float scale, uint16_t *img) {
-  const bool in0 = k < plan.n && k <= g, in1 = k + 1 < plan.n && k + 1 <= g;
-  return pack_values(in0 ? wrow[k] : 0.f, in1 ? wrow[k + 1] : 0.f, g, k, plan, scale, img);
-}
-
 // Error-free product and sum on fp32 pairs (Dekker / Knuth).
 __device__ __forceinline__ void two_prod(float a, float b, float &p, float &e) {
   p = a * b;
@@ -299,507 +292,12 @@ __device__ __forceinline__ void composite_wmax(float *xt, int bt, const PostPlan
   if (lane == 0) x0[xt_param_offset(DP) + 2 * DP + kParWmax] = wm;
 }
 
-// ---- factorisation: one block per (problem, objective) -------------------------
-// Blocked right-looking Cholesky of K (its fp32 rounding) in 32-column panels,
-// with W = L^-1 formed block row by block row inside the same loop: one warp
-// factors and inverts each diagonal block in registers, the panel below is the
-// product with that inverse, W_pJ = -W_pp sum_{K=J}^{p-1} L_pK W_KJ, and the
-// trailing update uses 4 x 4 register tiles. fp32 arithmetic on the FP32
-// pipes: the fp32 factor is as accurate as the posterior needs, while alpha,
-// which carries the condition number, gets two steps of iterative refinement
-// against the fp64-accurate K = hi + lo with double-float residuals. A pivot
-// at or below 16 * eps32 times its original diagonal entry counts as not
-// positive. Matrix and inverse live in shared memory (row stride NP+1, NP = n
-// rounded up to 32, padded with the identity), n <= 160; fitc_kernel takes the
-// larger problems.
-constexpr int kFitThreads = 512;
-
-__global__ void __launch_bounds__(kFitThreads, 1) fit32_kernel(
-    const float *Kh_all, const float *Kl_all, const double *Ys, int standardize, int n, int m,
-    float *xt, int DP, int npad, PostPlan plan, uint16_t *bop, int kl_smem, int early_trigger,
-    int comp, int *status, float *Wkeep) {
-  extern __shared__ __align__(16) float sm[];
-  __shared__ int bad;
-  __shared__ uint64_t lbar, lbar_lo;  // K hi; K lo (needed only by the residual)
-  __shared__ double ymu, yisd;
-  __shared__ __align__(16) float colL[32][64];  // columns of L_pp, zero-padded
-  __shared__ float invs[32];                    // 1 / L_cc
-  const int bt = blockIdx.x, b = bt / m, t = bt % m;
-  const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5,
-            nw = nthr >> 5;
-  const int NP = npad, ld = NP + 1;
-  const float *Kh = Kh_all + (size_t)bt * n * n, *Kl = Kl_all + (size_t)bt * n * n;
-  float *A = sm, *W = sm + (size_t)NP * ld;
-  float *vec = sm + 2 * (size_t)NP * ld;  // ylo, dg, y, al, r: 5 x NP
-  float *ylo = vec, *dg = vec + NP, *yv = vec + 2 * NP, *al = vec + 3 * NP, *rv = vec + 4 * NP;
-  const double *y = Ys + (size_t)b * n * m + t;
-  if (early_trigger) pdl_trigger();  // every block is resident: the posterior may launch
-  // standardize != 0: Ys holds raw outcomes; this column is standardised here
-  // (zero mean, unit sample standard deviation, as standardize_kernel does)
-  if (warp == 0) standardize_stats(y, n, m, standardize, lane, ymu, yisd);  // few fp64 ops
-  // everything below reads what the set-up kernel wrote
-  pdl_wait();
-  // A = K (hi; the lower triangle becomes L, the upper triangle keeps K for the
-  // residual), padded with the identity to NP x NP. In shared memory with n
-  // even, K hi (and, for n <= 128, K lo) arrive by bulk copy, K hi staged in
-  // the W area.
-  float *Kls = kl_smem ? vec + 5 * NP : nullptr;  // K lo, n x n (shared)
-  const bool bulk = n % 2 == 0;
-  if (bulk) {
-    if (tid == 0) {
-      mbar_init(&lbar, 1);
-      mbar_init(&lbar_lo, 1);
-      fence_mbar_init();
-    }
-    __syncthreads();
-    if (tid == 0) {
-      const uint32_t bytes = (uint32_t)n * n * sizeof(float);
-      mbar_arrive_expect_tx(&lbar, bytes);
-      bulk_g2s(W, Kh, bytes, &lbar);
-      if (kl_smem) {  // lands while the factorisation runs
-        mbar_arrive_expect_tx(&lbar_lo, bytes);
-        bulk_g2s(Kls, Kl, bytes, &lbar_lo);
-      }
-    }
-  } else {  // eight independent loads per thread in flight before their stores
-    const int nn = n * n;
-    for (int base = 0; base < nn; base += 8 * nthr) {
-      float v[8], w8[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int e = base + j * nthr + tid;
-        v[j] = e < nn ? Kh[e] : 0.f;
-        w8[j] = (e < nn && kl_smem) ? Kl[e] : 0.f;
-      }
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int e = base + j * nthr + tid;
-        if (e < nn) {
-          const int i = e / n, k = e - i * n;
-          A[(size_t)i * ld + k] = v[j];
-          if (kl_smem) Kls[e] = w8[j];
-        }
-      }
-    }
-  }
-  for (int e = tid; e < (NP - n) * NP; e += nthr) {
-    const int i = n + e / NP, k = e % NP;
-    if (k <= i) A[(size_t)i * ld + k] = (k == i) ? 1.f : 0.f;
-  }
-  __syncthreads();
-  const double mu_y = ymu, isd_y = yisd;
-  if (bulk) {
-    if (!mbar_wait(&lbar, 0)) {  // the copy never completed: report, drain, leave
-      if (tid == 0) set_status(status, BOUTE_ERR_TIMEOUT);
-      mbar_wait(&lbar, 0);
-      if (kl_smem) mbar_wait(&lbar_lo, 0);
-      return;
-    }
-    for (int i = warp; i < n; i += nw) {  // a warp per row: no division per entry
-      const float *src = W + (size_t)i * n;
-      float *dst = A + (size_t)i * ld;
-#pragma unroll 4
-      for (int k = lane; k < n; k += 32) dst[k] = src[k];
-    }
-    __syncthreads();
-  }
-  for (int i = tid; i < NP; i += nthr) {  // standardised y as an fp32 pair
-    const double ys = i < n ? (y[(size_t)i * m] - mu_y) * isd_y : 0.0;
-    yv[i] = (float)ys;
-    ylo[i] = (float)(ys - (double)yv[i]);
-    dg[i] = A[(size_t)i * ld + i];
-  }
-  if (tid == 0) bad = 0;
-  for (int e = tid; e < 32 * 64; e += nthr) (&colL[0][0])[e] = 0.f;
-  __syncthreads();
-  // Operand images of W for the posterior (n <= 160): rows [g_lo, g_hi) of W,
-  // warps w0, w0 + nws, ... one row each, lane = pair of columns 2 lane of
-  // each 64-wide chunk, scaled by 2^e_W. A block row of W is final once its
-  // panel's trailing update is done.
-  const float *xpar = xt + (size_t)bt * plan.nxt * xt_chunk_floats(DP) + xt_param_offset(DP) +
-                      2 * DP;
-  const float wscale = exp2i((int)xpar[kParEW]);
-  const int gmax = BOUTE_BLKCOLS * (plan.nwblk - 1) + plan.ncol[plan.nwblk - 1];
-  auto pack_rows = [&](int g_lo, int g_hi, int w0, int nws) {
-    uint16_t *img = bop + (size_t)bt * plan.image_halves;
-    for (int g = g_lo + w0; g < g_hi && g < gmax; g += nws) {
-      const float *wr = W + (size_t)g * ld;
-      const int kc = plan.kc[g / BOUTE_BLKCOLS];
-      for (int c = 0; c < kc; ++c)
-        if (!pack_pair(wr, g, BOUTE_ACHUNK * c + 2 * lane, plan, wscale, img))
-          set_status(status, BOUTE_ERR_NOT_PD);
-    }
-  };
-  // ---- blocked Cholesky and W = L^-1, 32-column panels -------------------------
-  // Iteration p: (a) warp 0 factors the diagonal block, A_pp = L_pp L_pp^T,
-  // and warp 1 inverts it one column behind, W_pp = L_pp^-1, both
-  // register-resident (lane = row of the block); (b) the panel below, L_rp = A_rp W_pp^T, goes to the still-unused
-  // block column p of W, and T_pJ = sum_{K=J}^{p-1} L_pK W_KJ (J < p) is
-  // parked, transposed, in the unused upper triangle of W; (c) the trailing
-  // update A_ij -= sum_q L_iq L_jq (rows and columns below the panel), the
-  // copy of the panel into A, and W_pJ = -W_pp T_pJ. 4 x 4 register tiles (4 x 2
-  // for T_pJ and W_pJ).
-  const int nb = NP / 32;
-  const unsigned FULL = 0xffffffffu;
-  for (int p = 0; p < nb; ++p) {
-    const int p0 = 32 * p;
-    if (warp == 0) {
-      // Factor. Lane = row of the block. a[] is a window on the lane's row
-      // that moves one column right every step (a[0] is always column c), so
-      // the step loop runs with static register indices and stays small.
-      // Each column of L_pp and 1 / L_cc go to warp 1 through shared memory,
-      // one named-barrier handshake per step.
-      float a[32];
-      float *Ar = A + (size_t)(p0 + lane) * ld + p0;
-#pragma unroll
-      for (int c = 0; c < 32; ++c) a[c] = (c <= lane) ? Ar[c] : 0.f;
-      const float dgl = dg[p0 + lane];
-      bool ok = true;
-      // steps c0 .. c0 + 7; after step c only a[0 .. 30 - c] still lie in the
-      // block, so each quarter of the panel shifts and updates NK entries
-      // (the rest are right of the block: never stored, left as they are)
-      // The pivot of step c + 1 is lane c + 1's entry after step c, which
-      // needs only that lane's own l: it is formed and broadcast before the
-      // stores and the row update, whose issue then hides its latency.
-      float piv = __shfl_sync(FULL, a[0], 0);
-      auto quarter = [&](auto nk, int c0) {
-        constexpr int NK = decltype(nk)::value;
-#pragma unroll 1
-        for (int c = c0; c < c0 + 8; ++c) {
-          if (!(piv > 16.f * 1.1920929e-7f * __shfl_sync(FULL, dgl, c))) ok = false;
-          float inv = rsqrtf(piv);
-          inv = inv * fmaf(-0.5f * piv * inv, inv, 1.5f);  // one Newton step; 1 / L_cc
-          const float l = lane > c ? a[0] * inv : (lane == c ? piv * inv : 0.f);
-          piv = __shfl_sync(FULL, fmaf(-l, l, a[1]), (c + 1) & 31);  // (unused after c = 31)
-          if (lane >= c) Ar[c] = l;
-          colL[c][lane] = l;  // colL[c][32..63] stay zero
-          if (lane == 0) invs[c] = inv;
-          __syncwarp();
-          named_barrier_sync(1, 64);  // column c is ready for warp 1
-          // trailing update of the lane's row, shifted one column: entries
-          // above the lane's diagonal collect values never stored
-#pragma unroll
-          for (int k = 0; k < NK; ++k) a[k] = fmaf(-l, colL[c][c + 1 + k], a[k + 1]);
-        }
-      };
-      quarter(std::integral_constant<int, 31>{}, 0);
-      quarter(std::integral_constant<int, 23>{}, 8);
-      quarter(std::integral_constant<int, 15>{}, 16);
-      quarter(std::integral_constant<int, 7>{}, 24);
-      if (!ok && lane == 0) bad = 1;
-    } else if (warp == 1) {
-      // Inverse, one column behind the factor. w[] is the lane's row of
-      // R = e_lane - sum_{j<c} L_lane,j W_j, which becomes W_pp's row after
-      // the division by L_lane,lane. R_c has no entries right of c, so the
-      // update at step c touches w[0 .. c] only (NK per quarter of the panel).
-      float w[32];
-#pragma unroll
-      for (int c = 0; c < 32; ++c) w[c] = (c == lane) ? 1.f : 0.f;
-      float myinv = 0.f;
-      auto quarter = [&](auto nk, int c0) {
-        constexpr int NK = decltype(nk)::value;
-#pragma unroll 1
-        for (int c = c0; c < c0 + 8; ++c) {
-          named_barrier_sync(1, 64);  // wait for column c
-          const float l = colL[c][lane], inv = invs[c];
-          if (lane == c) myinv = inv;
-          const float lw = lane > c ? l * inv : 0.f;  // R_i -= (L_ic / L_cc) R_c, rows below c
-#pragma unroll
-          for (int k = 0; k < NK; ++k) w[k] = fmaf(-lw, __shfl_sync(FULL, w[k], c), w[k]);
-        }
-      };
-      quarter(std::integral_constant<int, 8>{}, 0);
-      quarter(std::integral_constant<int, 16>{}, 8);
-      quarter(std::integral_constant<int, 24>{}, 16);
-      quarter(std::integral_constant<int, 32>{}, 24);
-      float *Wr = W + (size_t)(p0 + lane) * ld + p0;
-#pragma unroll
-      for (int c = 0; c < 32; ++c) Wr[c] = w[c] * myinv;
-    } else if (p > 0) {
-      // the other warps pack the previous block row of W meanwhile
-      pack_rows(p0 - 32, p0, warp - 2, nw - 2);
-    }
-    __syncthreads();
-    if (bad) break;
-    const int r0 = p0 + 32, rows = NP - r0;
-    // (b)
-    {
-      const int ntr = (rows / 4) * 8, ntt = p * 128;
-      for (int tix = tid; tix < ntr + ntt; tix += nthr) {
-        float acc[4][4] = {};
-        if (tix < ntr) {  // L_rp tile: rows i0.., columns c0.. of the panel
-          const int i0 = r0 + 4 * (tix >> 3), c0 = 4 * (tix & 7);
-#pragma unroll 4
-          for (int q = 0; q < 32; ++q) {
-            float x[4], y4[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              x[u] = A[(size_t)(i0 + u) * ld + p0 + q];
-              y4[u] = W[(size_t)(p0 + c0 + u) * ld + p0 + q];
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-              for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(x[u], y4[v], acc[u][v]);
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) W[(size_t)(i0 + u) * ld + p0 + c0 + v] = acc[u][v];
-        } else {
-          // T_pJ tile of 4 rows x 2 columns (8 x 16 tiles per 32 x 32 block):
-          // the sums run over 32 (p - J) terms, so the long ones get twice
-          // the threads that 4 x 4 tiles would give them
-          const int e = tix - ntr, J = e >> 7, rb = 4 * ((e >> 4) & 7), cb = 2 * (e & 15);
-#pragma unroll 4
-          for (int q = 32 * J; q < p0; ++q) {
-            float x[4], y2[2];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) x[u] = A[(size_t)(p0 + rb + u) * ld + q];
-#pragma unroll
-            for (int v = 0; v < 2; ++v) y2[v] = W[(size_t)q * ld + 32 * J + cb + v];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-              for (int v = 0; v < 2; ++v) acc[u][v] = fmaf(x[u], y2[v], acc[u][v]);
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 2; ++v) W[(size_t)(32 * J + cb + v) * ld + p0 + rb + u] = acc[u][v];
-        }
-      }
-    }
-    __syncthreads();
-    // (c)
-    {
-      const int th = rows / 4, ntile = th * (th + 1) / 2, nwt = p * 128;
-      for (int tix = tid; tix < ntile + nwt; tix += nthr) {
-        float acc[4][4] = {};
-        if (tix < ntile) {  // trailing tile (i, j) of the lower triangle
-          int ti = (int)((sqrtf(8.f * tix + 1.f) - 1.f) * 0.5f);
-          while (ti * (ti + 1) / 2 > tix) --ti;
-          while ((ti + 1) * (ti + 2) / 2 <= tix) ++ti;
-          const int tj = tix - ti * (ti + 1) / 2;
-          const int i0 = r0 + 4 * ti, j0 = r0 + 4 * tj;
-#pragma unroll 4
-          for (int q = 0; q < 32; ++q) {
-            float x[4], y4[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              x[u] = W[(size_t)(i0 + u) * ld + p0 + q];
-              y4[u] = W[(size_t)(j0 + u) * ld + p0 + q];
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-              for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(x[u], y4[v], acc[u][v]);
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v)
-              if (ti != tj || v <= u) A[(size_t)(i0 + u) * ld + j0 + v] -= acc[u][v];
-        } else {  // W_pJ tile = -W_pp T_pJ (W_pp lower, zeros above), 4 rows x 2 columns
-          const int e = tix - ntile, J = e >> 7, rb = 4 * ((e >> 4) & 7), cb = 2 * (e & 15);
-#pragma unroll 4
-          for (int q = 0; q < 32; ++q) {
-            float x[4], y2[2];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) x[u] = W[(size_t)(p0 + rb + u) * ld + p0 + q];
-#pragma unroll
-            for (int v = 0; v < 2; ++v) y2[v] = W[(size_t)(32 * J + cb + v) * ld + p0 + q];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-              for (int v = 0; v < 2; ++v) acc[u][v] = fmaf(x[u], y2[v], acc[u][v]);
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 2; ++v) W[(size_t)(p0 + rb + u) * ld + 32 * J + cb + v] = -acc[u][v];
-        }
-      }
-      for (int e = tid; e < rows * 32; e += nthr) {  // the panel into A
-        const size_t o = (size_t)(r0 + (e >> 5)) * ld + p0 + (e & 31);
-        A[o] = W[o];
-      }
-    }
-    __syncthreads();
-  }
-  const bool lo_copy = bulk && kl_smem;  // K lo is on its way by bulk copy
-  if (bad) {
-    if (tid == 0) set_status(status, BOUTE_ERR_NOT_PD);
-    if (lo_copy) mbar_wait(&lbar_lo, 0);  // let it land before the block exits
-    return;
-  }
-  // ---- alpha0 = W^T (W y), refined twice against K = hi + lo ---------------------
-  // out = W^T (W rhs): the 32 x 32 blocks (I >= J) of
-  // W, one warp per block (the diagonal blocks hold zeros above the diagonal,
-  // the padding the identity), with the block partial sums in the space of
-  // colL (free after the factorisation), added in a fixed order.
-  auto solve = [&](const float *rhs, float *out) {
-    float *pw = &colL[0][0], *pt = pw + nb * NP;  // nb x NP each (nb <= 5, NP <= 160)
-    const int nblk = nb * (nb + 1) / 2;
-    auto block = [&](int e, int &I, int &J) {
-      I = 0;
-      while ((I + 1) * (I + 2) / 2 <= e) ++I;
-      J = e - I * (I + 1) / 2;
-    };
-    for (int e = warp; e < nblk; e += nw) {  // (W rhs) restricted to block (I, J): lane = row
-      int I, J;
-      block(e, I, J);
-      const float *wr = W + (size_t)(32 * I + lane) * ld + 32 * J;
-      const float *x = rhs + 32 * J;
-      float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll
-      for (int k = 0; k < 32; k += 4) {
-        s0 = fmaf(wr[k], x[k], s0);
-        s1 = fmaf(wr[k + 1], x[k + 1], s1);
-        s2 = fmaf(wr[k + 2], x[k + 2], s2);
-        s3 = fmaf(wr[k + 3], x[k + 3], s3);
-      }
-      pw[J * NP + 32 * I + lane] = (s0 + s1) + (s2 + s3);
-    }
-    __syncthreads();
-    for (int e = warp; e < nblk; e += nw) {  // W^T (W rhs) restricted to block (I, J): lane = column
-      int I, J;
-      block(e, I, J);
-      float v = 0.f;  // (W rhs) of row 32 I + lane
-      for (int q = 0; q <= I; ++q) v += pw[q * NP + 32 * I + lane];
-      const float *wc = W + (size_t)(32 * I) * ld + 32 * J + lane;
-      float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll
-      for (int r = 0; r < 32; r += 4) {
-        s0 = fmaf(wc[(size_t)r * ld], __shfl_sync(FULL, v, r), s0);
-        s1 = fmaf(wc[(size_t)(r + 1) * ld], __shfl_sync(FULL, v, r + 1), s1);
-        s2 = fmaf(wc[(size_t)(r + 2) * ld], __shfl_sync(FULL, v, r + 2), s2);
-        s3 = fmaf(wc[(size_t)(r + 3) * ld], __shfl_sync(FULL, v, r + 3), s3);
-      }
-      pt[I * NP + 32 * J + lane] = (s0 + s1) + (s2 + s3);
-    }
-    __syncthreads();
-    for (int k = tid; k < NP; k += nthr) {
-      float v = 0.f;
-      for (int q = k >> 5; q < nb; ++q) v += pt[q * NP + k];
-      out[k] = v;
-    }
-    __syncthreads();
-  };
-  solve(yv, al);
-  if (lo_copy && !mbar_wait(&lbar_lo, 0)) {  // the copy never completed: report, drain, leave
-    if (tid == 0) set_status(status, BOUTE_ERR_TIMEOUT);
-    mbar_wait(&lbar_lo, 0);
-    return;
-  }
-  auto residual = [&]() {
-    // residual r = y - K alpha in double-float: one
-    // warp per 32 x 32 block (I, J) of K, lane = row, two independent chains per
-    // lane; K lo through its symmetry (K lo[k][i], conflict-free across the
-    // lanes), from shared memory when it fits there; K hi from the upper
-    // triangle of A: at (k, i) below the diagonal blocks, at (i, k) above them,
-    // each with one fixed load form (a per-entry choice of address costs more
-    // than the arithmetic), and in the diagonal blocks both loaded and the
-    // value selected, the diagonal from dg. Indices past n are clamped and
-    // alpha is zero there (padding), so those terms add exact zeros. The block
-    // partial sums (hi, lo) go to the space of colL and are added per row in a
-    // fixed order.
-    float *ph = &colL[0][0], *pl = ph + nb * NP;  // nb x NP each
-    const float *Klsm = vec + 5 * NP;  // = Kls when kl_smem (shared-space pointer)
-    for (int e = warp; e < nb * nb; e += nw) {
-      const int I = e / nb, J = e - I * nb, ci = min(32 * I + lane, n - 1);
-      const float *alJ = al + 32 * J;
-      float sh[2] = {0.f, 0.f}, sl[2] = {0.f, 0.f};
-      auto run = [&](auto form, auto lo_smem) {
-        constexpr int F = decltype(form)::value;  // 0: below, 1: above, 2: diagonal block
-        constexpr bool LS = decltype(lo_smem)::value;
-        const float di = dg[ci];
-  #pragma unroll 8
-        for (int kk = 0; kk < 32; ++kk) {
-          const int kc = min(32 * J + kk, n - 1);
-          float h;
-          if (F == 0) {
-            h = A[kc * ld + ci];
-          } else if (F == 1) {
-            h = A[ci * ld + kc];
-          } else {
-            const float x = A[kc * ld + ci], y = A[ci * ld + kc];
-            h = kc < ci ? x : y;
-            h = kc == ci ? di : h;
-          }
-          const float l = LS ? Klsm[kc * n + ci] : Kl[(size_t)kc * n + ci];
-          const float a = alJ[kk];  // zero from n on
-          float pr, er, s_, e2;
-          two_prod(h, a, pr, er);
-          two_sum(sh[kk & 1], pr, s_, e2);
-          sh[kk & 1] = s_;
-          sl[kk & 1] += e2 + fmaf(l, a, er);
-        }
-      };
-      auto pick = [&](auto lo_smem) {
-        if (I > J) run(std::integral_constant<int, 0>{}, lo_smem);
-        else if (I < J) run(std::integral_constant<int, 1>{}, lo_smem);
-        else run(std::integral_constant<int, 2>{}, lo_smem);
-      };
-      if (kl_smem) pick(std::true_type{});
-      else pick(std::false_type{});
-      float s_, e2;
-      two_sum(sh[0], sh[1], s_, e2);
-      ph[J * NP + 32 * I + lane] = s_;
-      pl[J * NP + 32 * I + lane] = (sl[0] + sl[1]) + e2;
-    }
-    __syncthreads();
-    for (int i = tid; i < NP; i += nthr) {
-      float sh = 0.f, sl = 0.f;
-      for (int J = 0; J < nb; ++J) {
-        float s_, e2;
-        two_sum(sh, ph[J * NP + i], s_, e2);
-        sh = s_;
-        sl += pl[J * NP + i] + e2;
-      }
-      if (i < n) rv[i] = (yv[i] - sh) + (ylo[i] - sl);
-    }
-  };
-  // two refinement steps: alpha carries the condition number of K, and the
-  // posterior mean amplifies its error by sum_j |K*_j alpha_j| / |mean|
-  // The second correction is kept exactly: alpha = hi + lo, hi = fl(alpha +
-  // delta), lo its rounding error (in rv), for the posterior's fp64 path.
-  for (int step = 0; step < 2; ++step) {
-    residual();
-    for (int i = n + tid; i < NP; i += nthr) rv[i] = 0.f;
-    __syncthreads();
-    solve(rv, rv);
-    for (int k = tid; k < NP; k += nthr) {
-      if (step == 0) {
-        al[k] += rv[k];
-      } else {
-        float s_, e;
-        two_sum(al[k], rv[k], s_, e);
-        al[k] = s_;
-        rv[k] = e;
-      }
-    }
-    __syncthreads();
-  }
-  // outputs: the operand images of W, alpha into the side input
-  pack_rows(NP - 32, NP, warp, nw);  // the last block row (the others: above)
-  if (Wkeep) {  // W in global memory too (the in-sample preparation, the
-                        // acquisition's gradient), its lower triangle
-    float *dst = Wkeep + (size_t)bt * NP * ld;
-    for (int i = warp; i < n; i += nw)
-      for (int k = lane; k <= i; k += 32) dst[(size_t)i * ld + k] = W[(size_t)i * ld + k];
-  }
-  const int cf = xt_chunk_floats(DP);
-  float *xa = xt + (size_t)bt * plan.nxt * cf + xt_alpha_offset(DP);
-  for (int k = tid; k < BOUTE_KCHUNK * plan.nxt; k += nthr) {
-    float *q = xa + (size_t)(k / BOUTE_KCHUNK) * cf + k % BOUTE_KCHUNK;
-    q[0] = k < n ? al[k] : 0.f;
-    q[BOUTE_KCHUNK] = k < n ? rv[k] : 0.f;
-  }
-  if (comp && warp == nw - 1) composite_wmax(xt, bt, plan, DP, n, lane);
-}
-
-// ---- factorisation on a thread-block cluster (n > 160) --------------------------
+// ---- factorisation on a thread-block cluster ---------------------------------------
+// The Cholesky factor of K (its fp32 rounding), W = L^-1 and alpha. fp32 arithmetic on
+// the FP32 pipes: the fp32 factor is as accurate as the posterior needs, while alpha,
+// which carries the condition number, gets two steps of iterative refinement against
+// the fp64-accurate K = hi + lo with double-float residuals. A pivot at or below 16 *
+// eps32 times its original diagonal entry counts as not positive.
 // One cluster of C = Pr x Pc CTAs per problem-objective runs the whole fit after
 // the set-up in one launch: K's lower triangle as 32 x 32 tiles, tile (I, J) owned
 // by the CTA (I mod Pr, J mod Pc) and kept in its shared memory (in the workspace
@@ -814,13 +312,14 @@ __global__ void __launch_bounds__(kFitThreads, 1) fit32_kernel(
 // first and factoring it beside the rest, and the owners of block row p write W and its
 // operand images. Then alpha and its two refinement steps from the tiles. Tiles and
 // vectors travel by stores to the other CTAs' shared memory, ordered by the barriers.
-// The arithmetic is fp32 as in fit32_kernel; sums run in an order that does not depend
-// on C. What bounds it is the chain of a panel (two barriers, two tile products, the
+// Sums run in an order that does not depend on C. What bounds it is the chain of a panel (two barriers, two tile products, the
 // diagonal tile), for n = 1024 as much the updates' shared-memory reads.
 // Fit with its set-up, against three launches a panel, nine for alpha and one block
 // per problem-objective in large batches: n = 203, m = 3 174 -> 98 us; n = 512, m = 2
 // 385 -> 230 us; n = 777, B = 3, m = 2 1193 -> 754 us; n = 1024, m = 3 1226 -> 943 us;
-// n = 256, B = 16, m = 2 560 -> 250 us.
+// n = 256, B = 16, m = 2 560 -> 250 us. Against one block per problem-objective with K
+// and W as matrices in shared memory (n <= 160, m = 2): n = 32 32 -> 28 us, n = 128
+// 69 -> 50 us, n = 160 100 -> 65 us.
 constexpr int kFcThreads = 512, kFcGroups = kFcThreads / 64;
 constexpr int kFcTile = 32 * 32;
 constexpr int kFcMaxCluster = 16;
@@ -911,30 +410,37 @@ __device__ __forceinline__ void fc_diagonal(float *tile, const float *dg, FcDiag
     }
     a[32] = a[33] = a[34] = a[35] = 0.f;
     bool ok = true;
-    float piv = __shfl_sync(FULL, a[0], 0);
+    auto recip_root = [](float piv) {  // 1 / L_cc: one Newton step
+      const float inv = rsqrtf(piv);
+      return inv * fmaf(-0.5f * piv * inv, inv, 1.5f);
+    };
+    float piv = __shfl_sync(FULL, a[0], 0), inv = recip_root(piv);
 #pragma unroll 1
     for (int c0 = 0; c0 < 32; c0 += 4) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int c = c0 + j;
-        if (!(piv > 16.f * 1.1920929e-7f * dg[c])) ok = false;
-        float inv = rsqrtf(piv);
-        inv = inv * fmaf(-0.5f * piv * inv, inv, 1.5f);  // one Newton step; 1 / L_cc
         const float l = lane == c ? piv * inv : a[j] * inv;  // (rows above c: never used)
         float *col = sh.colL + c * 32;
         col[lane] = l;
         if (lane == 0) sh.invs[c] = inv;
-        // the next pivot: lane c + 1's entry, which needs that lane's l alone
-        piv = __shfl_sync(FULL, fmaf(-l, l, a[j + 1]), (c + 1) & 31);
+        // the next pivot: lane c + 1's entry, which needs that lane's l alone; its
+        // reciprocal root is formed while the row's update waits for its operands
+        const float next = __shfl_sync(FULL, fmaf(-l, l, a[j + 1]), (c + 1) & 31);
         a[j + 1] = fmaf(-l, __shfl_sync(FULL, l, (c + 1) & 31), a[j + 1]);
         __syncwarp();
+        float4 v[8];
+#pragma unroll
+        for (int g = (j + 2) / 4; g < 8; ++g) v[g] = *(const float4 *)(col + c0 + 4 * g);
+        if (!(piv > 16.f * 1.1920929e-7f * dg[c])) ok = false;
+        piv = next;
+        inv = recip_root(piv);  // (unused after c = 31)
 #pragma unroll
         for (int g = (j + 2) / 4; g < 8; ++g) {  // the window's columns j + 2 ..
-          const float4 v = *(const float4 *)(col + c0 + 4 * g);
-          if (4 * g > j + 1) a[4 * g] = fmaf(-l, v.x, a[4 * g]);
-          if (4 * g + 1 > j + 1) a[4 * g + 1] = fmaf(-l, v.y, a[4 * g + 1]);
-          if (4 * g + 2 > j + 1) a[4 * g + 2] = fmaf(-l, v.z, a[4 * g + 2]);
-          if (4 * g + 3 > j + 1) a[4 * g + 3] = fmaf(-l, v.w, a[4 * g + 3]);
+          if (4 * g > j + 1) a[4 * g] = fmaf(-l, v[g].x, a[4 * g]);
+          if (4 * g + 1 > j + 1) a[4 * g + 1] = fmaf(-l, v[g].y, a[4 * g + 1]);
+          if (4 * g + 2 > j + 1) a[4 * g + 2] = fmaf(-l, v[g].z, a[4 * g + 2]);
+          if (4 * g + 3 > j + 1) a[4 * g + 3] = fmaf(-l, v[g].w, a[4 * g + 3]);
         }
       }
       if (c0 & 4) named_barrier_arrive(9 + (c0 >> 3), 64);  // eight columns for warp 1
@@ -1376,17 +882,6 @@ int launch_standardize(const double *Y, int B, int n, int m, int codes, double *
   return last_launch_status();
 }
 
-// The shared-memory variant holds n up to 160 (n rounded up to 32).
-bool fit_uses_smem(int npad) { return npad <= 160; }
-
-// Dynamic shared memory of the shared-memory fit: A and W (np x (np+1)), five
-// vectors, and K lo (n x n) when n <= 128.
-static bool fit_kl_in_smem(int n) { return n <= 128; }
-size_t fit_smem_bytes(int np, int n) {
-  return (2 * (size_t)np * (np + 1) + 5 * (size_t)np + (fit_kl_in_smem(n) ? (size_t)n * n : 0)) *
-         sizeof(float);
-}
-
 // Dynamic shared memory of fitc_kernel with clusters of C (tiles: its tiles too).
 static size_t fitc_smem(int npad, int C, bool tiles) {
   const int nb = npad / 32, ms = fc_max_slots(nb, C);
@@ -1396,15 +891,18 @@ static size_t fitc_smem(int npad, int C, bool tiles) {
 }
 constexpr size_t kFcMaxSmem = 227 * 1024 - 5 * 1024;  // (its static part: 4.9 KB)
 
-// n > 160: clusters of the largest size with which every problem-objective runs at
-// once, and large enough that the operands, and if any size allows it the tiles, fit
-// shared memory (n = 256 on single CTAs, n = 1024 on 16; above that the tiles stay in
-// the workspace).
+// Clusters of the largest size with which every problem-objective runs at once, no
+// more CTAs than block rows (n = 32 on one CTA 28 us, on two 30; n = 128 on four 50, on
+// eight 53; n = 203 on four 101, on eight 98), and enough that the operands, and if any
+// size allows it the tiles, fit shared memory (n = 256 on single CTAs, n = 1024 on 16;
+// above that the tiles stay in the workspace).
 static int launch_fitc(Gp *gp, const double *Ys, int standardize, cudaStream_t s) {
   const int n = gp->n, m = gp->m, npad = gp->plan.npad, nb = npad / 32;
   const long long BM = (long long)gp->B * m, sms = num_sms();
   int C = 1;
-  while (C < kFcMaxCluster && (fitc_smem(npad, C, true) > kFcMaxSmem || 2 * C * BM <= sms)) C *= 2;
+  while (C < kFcMaxCluster &&
+         (fitc_smem(npad, C, true) > kFcMaxSmem || (2 * C * BM <= sms && C < nb)))
+    C *= 2;
   auto go = [&](auto kern, bool tiles) {
     prefer_shared(kern);
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFcMaxSmem);
@@ -1448,7 +946,7 @@ static int launch_fit_impl(Gp *gp, const double *X, const double *Ys, int standa
                            const double *ls, const double *s2, const double *noise,
                            cudaStream_t s, cudaEvent_t setup_done = nullptr) {
   const int n = gp->n, d = gp->d, m = gp->m, BM = gp->B * gp->m;
-  const int npad = gp->plan.npad, xpad = BOUTE_KCHUNK * gp->plan.nxt;
+  const int xpad = BOUTE_KCHUNK * gp->plan.nxt;
   const int nkt = kmat_units(n);
   const int sms = num_sms();
   // side-input blocks: as many as leave one block per SM (K blocks first), 2 .. 16
@@ -1458,7 +956,6 @@ static int launch_fit_impl(Gp *gp, const double *X, const double *Ys, int standa
   // that waiting successors can never hold resources a later block needs
   const long long setup_blocks = (long long)(nkt + nprep) * BM;
   const int setup_early = setup_blocks <= 8LL * (sms - BM) ? 1 : 0;
-  const int fit_early = 2 * BM <= sms ? 1 : 0;
   auto setup = [&](auto kern) {
     prefer_shared(kern);
     kern<<<dim3(nkt + nprep, BM), kSetupThreads, 0, s>>>(X, n, d, m, gp->DP, xpad, ls, s2, noise,
@@ -1469,16 +966,6 @@ static int launch_fit_impl(Gp *gp, const double *X, const double *Ys, int standa
   if (gp->kern) setup(fit_setup_kernel<true>);
   else setup(fit_setup_kernel<false>);
   if (setup_done && cudaEventRecord(setup_done, s) != cudaSuccess) return last_launch_status();
-  if (fit_uses_smem(npad)) {
-    const size_t smem = fit_smem_bytes(npad, n);
-    prefer_shared(fit32_kernel);
-    cudaFuncSetAttribute(fit32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_pdl(fit32_kernel, dim3(BM), dim3(kFitThreads), smem, s, gp->Kh, gp->Kl, Ys, standardize,
-               n, m, gp->xt, gp->DP, npad, gp->plan, gp->bop, fit_kl_in_smem(n) ? 1 : 0, fit_early,
-               gp->kern, gp->status, gp->Wws);  // W kept in global memory as well
-    count_launch(2);
-    return last_launch_status();
-  }
   return launch_fitc(gp, Ys, standardize, s);
 }
 

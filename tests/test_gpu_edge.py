@@ -403,9 +403,9 @@ def test_row_pairs_and_column_groups(d, n, N):
         check_var(g["var"][0, t], var[:, t], fp.s2[t])
 
 
-# Tiles of 32, from six block rows on: sizes at their edges, batches that take
-# clusters of 16, 8, 4, 2 and 1 CTAs, and tiles that stay in the workspace.
-@pytest.mark.parametrize("n,B", [(161, 1), (192, 2), (193, 1), (224, 40), (256, 40), (288, 20),
+# Tiles of 32: sizes at their edges, batches that take clusters of 16, 8, 4, 2 and 1
+# CTAs, and tiles that stay in the workspace.
+@pytest.mark.parametrize("n,B", [(1, 1), (32, 3), (33, 1), (65, 40), (97, 2), (160, 1), (161, 1), (192, 2), (193, 1), (224, 40), (256, 40), (288, 20),
                                  (321, 12), (511, 6), (1024, 1), (1025, 1)])
 def test_cluster_fit_edges(n, B):
     w = wl.scaled(wl.WORKLOADS[4], N=130, B=B, n=n)

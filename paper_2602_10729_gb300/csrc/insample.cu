@@ -26,6 +26,7 @@
 #include <algorithm>
 
 #include "internal.h"
+#include "tile32.cuh"
 
 namespace boute {
 
@@ -36,8 +37,6 @@ constexpr int kInsThreads = 512;
 // Row stride of the shared-memory matrices: odd, so that a warp reading one
 // column (32 consecutive rows) touches 32 different banks.
 __host__ __device__ __forceinline__ int ins_ld(int n) { return n | 1; }
-__host__ __device__ __forceinline__ int ins_lda(int n) { return round_up(n, 32) + 4; }
-__host__ __device__ __forceinline__ int ins_ldk(int n) { return round_up(n, 32) + 8; }
 
 __device__ __forceinline__ void atomic_max_pos(unsigned *a, float v) {
   atomicMax(a, __float_as_uint(v));  // non-negative floats order as their bits
@@ -53,9 +52,9 @@ __host__ __device__ __forceinline__ size_t ins_ws_floats(int n) {
 
 // The operand image of one output row of a dense block: K positions k, k + 1
 // of row `row` of block q, scaled, as fp16 hi/lo pairs (zero beyond n).
-__device__ __forceinline__ void pack_dense_pair(const float *src, int n, int k, float scl, int q,
+__device__ __forceinline__ void pack_dense_pair(float w0, float w1, int n, int k, float scl, int q,
                                                 int row, const PostPlan &plan, uint16_t *img) {
-  const float v0 = k < n ? src[k] * scl : 0.f, v1 = k + 1 < n ? src[k + 1] * scl : 0.f;
+  const float v0 = k < n ? w0 * scl : 0.f, v1 = k + 1 < n ? w1 * scl : 0.f;
   uint32_t hi, lo;
   split_f16x2(v0, v1, hi, lo);
   const int ncol = plan.ncol[q], cidx = k / BOUTE_ACHUNK;
@@ -73,7 +72,12 @@ __device__ __forceinline__ void pack_dense_pair(const float *src, int n, int k, 
 // (1) one CTA per problem-objective: the sequential part. K^-1 = W^T W, the
 // jittered in-sample covariance and its Cholesky factor F, H^T = sigma^2
 // F^-1 K^-1 by forward substitution; F, H^T and mu_n go to the workspace,
-// H^T's operand images and scale exponent to the handle.
+// H^T's operand images and scale exponent to the handle. Everything is 32 x 32 tiles
+// in shared memory, products by eight groups of 64 threads: W and H as transposes
+// (tile (K, I) of WT holds W_KI^T), the right-hand sides H updated with the factor's
+// trailing matrix in one right-looking loop, so that what bounds it is four diagonal
+// tiles' chains and about 100 tile products (n = 128: 149 -> 46 us; scalar loops
+// over rows and columns, with serial substitutions, before).
 __global__ void __launch_bounds__(kInsThreads, 1)
     insample_factor_kernel(const float *Wws, int npad, float *xt, int DP, int nxt,
                            const double *Ys, const double *s2, const double *noise, int n, int m,
@@ -83,11 +87,14 @@ __global__ void __launch_bounds__(kInsThreads, 1)
   __shared__ unsigned mxh;
   const int bt = blockIdx.x;
   const int tid = threadIdx.x;
-  // row strides: A (L, read along rows by four lanes per row) = 4 mod 32,
-  // Kb (K^-1 then H^T, read down columns by eight columns x four k phases)
-  // = 8 mod 32, so that neither pattern repeats a bank within a warp
-  const int ld = ins_lda(n), ldk = ins_ldk(n);
-  float *A = sm, *Kb = A + (size_t)n * ld, *part = Kb + (size_t)n * ldk, *mu = part + 4 * 128;
+  const int nb = (n + 31) / 32, nt = nb * (nb + 1) / 2;
+  // W^T (then F) and the covariance: lower tiles; H^T transposed: nb x nb tiles, column
+  // tile c of block row q at (q nb + c); the diagonal tile's inverse, both ways
+  float *WT = sm, *A = WT + nt * kFcTile, *HT = A + nt * kFcTile;
+  float *vpp = HT + nb * nb * kFcTile, *vtt = vpp + kFcTile, *mu = vtt + kFcTile;
+  __shared__ __align__(16) FcDiag dsh;
+  __shared__ float zero[32];
+  auto tri = [](int I, int J) { return (I * (I + 1) / 2 + J) * kFcTile; };
   const double s2d = s2[bt];
   const double nzd = noise[bt] > 1e-12 * s2d ? noise[bt] : 1e-12 * s2d;  // the fit's floor
   const float sig2 = (float)nzd, jit = (float)(kInsJitter * s2d);
@@ -103,17 +110,20 @@ __global__ void __launch_bounds__(kInsThreads, 1)
   // W (lower triangle) and mu_n = y - sigma^2 alpha (alpha = hi + lo)
   const float *W = Wws + (size_t)bt * npad * (npad + 1);
   const int warp = tid >> 5, lane = tid & 31;
-  for (int i = warp; i < n; i += kInsThreads / 32) {  // a warp per row, four loads in flight
-    float v[kInsMaxN / 32];
+  for (int e = warp; e < 4 * nt; e += kInsThreads / 32) {  // eight rows of a tile per warp
+    int I = 0;
+    while ((I + 1) * (I + 2) / 2 <= (e >> 2)) ++I;
+    const int J = (e >> 2) - I * (I + 1) / 2, r0 = 8 * (e & 3), k = 32 * J + lane;
+    float v[8];
 #pragma unroll
-    for (int r = 0; r < kInsMaxN / 32; ++r) {
-      const int k = lane + 32 * r;
-      v[r] = k <= i ? W[(size_t)i * (npad + 1) + k] : 0.f;
+    for (int u = 0; u < 8; ++u) {
+      const int i = 32 * I + r0 + u;
+      v[u] = (i < n && k <= i) ? W[(size_t)i * (npad + 1) + k] : 0.f;
     }
 #pragma unroll
-    for (int r = 0; r < kInsMaxN / 32; ++r)
-      if (lane + 32 * r < n) A[(size_t)i * ld + lane + 32 * r] = v[r];
+    for (int u = 0; u < 8; ++u) WT[tri(I, J) + fc_off(lane, r0 + u)] = v[u];
   }
+  if (tid < 32) zero[tid] = 0.f;
   const int b = bt / m, t = bt % m;
   for (int i = tid; i < n; i += kInsThreads) {
     const float *ca = x0 + (size_t)(i / BOUTE_KCHUNK) * cf + xt_alpha_offset(DP) + i % BOUTE_KCHUNK;
@@ -123,167 +133,123 @@ __global__ void __launch_bounds__(kInsThreads, 1)
   }
   __syncthreads();
   if (bad) return;
-  // K^-1 = W^T W: (i, j), j <= i, sum over k >= i of W_ki W_kj (two chains)
-  const int npairs = n * (n + 1) / 2;
-  for (int e = tid; e < npairs; e += kInsThreads) {
-    int i = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);
-    while (i * (i + 1) / 2 > e) --i;
-    while ((i + 1) * (i + 2) / 2 <= e) ++i;
-    const int j = e - i * (i + 1) / 2;
-    float a0 = 0.f, a1 = 0.f;
-    int k = i;
-    for (; k + 1 < n; k += 2) {
-      a0 = fmaf(A[(size_t)k * ld + i], A[(size_t)k * ld + j], a0);
-      a1 = fmaf(A[(size_t)(k + 1) * ld + i], A[(size_t)(k + 1) * ld + j], a1);
+  const int grp = tid >> 6, gt = tid & 63, tx = gt & 7, ty = gt >> 3;
+  constexpr int kGroups = kInsThreads / 64;
+  float acc[4][4];
+  auto store = [&](float *T) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      ((float4 *)T)[(4 * ty + u) * 8 + (tx ^ ty)] =
+          make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
+  };
+  // K^-1 = W^T W by lower tiles, sum over K >= I of W_KI^T W_KJ; from it sigma^2 K^-1
+  // (H's right-hand sides, both triangles) and the covariance Sigma + jitter s2 I =
+  // sigma^2 (I - sigma^2 K^-1) + jitter s2 I (the longest sums first)
+  for (int e = grp; e < nt; e += kGroups) {
+    int I = 0;
+    while ((I + 1) * (I + 2) / 2 <= e) ++I;
+    const int J = e - I * (I + 1) / 2;
+    float sum[4][4] = {};
+    for (int K = I; K < nb; ++K) {
+      fc_product(WT + tri(K, I), WT + tri(K, J), gt, acc);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) sum[u][v] += acc[u][v];
     }
-    if (k < n) a0 = fmaf(A[(size_t)k * ld + i], A[(size_t)k * ld + j], a0);
-    const float acc = a0 + a1;
-    Kb[(size_t)i * ldk + j] = acc;
-    Kb[(size_t)j * ldk + i] = acc;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const int r = 4 * ty + u, c = 4 * tx + v;
+        const float kv = sig2 * sum[u][v];  // sigma^2 K^-1
+        HT[(J * nb + I) * kFcTile + fc_off(r, c)] = kv;  // (row tile J, column tile I)^T
+        if (I != J) HT[(I * nb + J) * kFcTile + fc_off(c, r)] = kv;
+        const bool dia = I == J && r == c;
+        const float a = sig2 * ((dia ? 1.f : 0.f) - kv);
+        acc[u][v] = dia ? a + jit : a;
+      }
+    store(A + tri(I, J));
   }
-  __syncthreads();
-  // Sigma + jitter s2 I = sigma^2 (I - sigma^2 K^-1) + jitter s2 I (lower)
-  for (int e = tid; e < n * n; e += kInsThreads) {
-    const int i = e / n, j = e % n;
-    if (j <= i) {
-      const float v = sig2 * ((i == j ? 1.f : 0.f) - sig2 * Kb[(size_t)i * ldk + j]);
-      A[(size_t)i * ld + j] = i == j ? v + jit : v;
-    }
-  }
-  __syncthreads();
-  // Cholesky in 32-column panels: (a) the panel's columns c, rows i >= p0,
-  // take the earlier panels' products, A_ic -= sum_{k<p0} L_ik L_ck (a thread
-  // holds one row and eight columns c = cg + 4u); (b) warp 0 factors the
-  // 32 x 32 diagonal block in registers (lane = row; rows past n are the
-  // identity); (c) the rows below solve L_i,panel = A_i,panel L_dd^-T, a
-  // thread per row in registers.
-  const unsigned FULL = 0xffffffffu;
-  const int nb = (n + 31) / 32;
   __shared__ int badp;
   if (tid == 0) badp = 0;
+  __syncthreads();
+  // Panel p: the diagonal tile's factor and inverse V = F_pp^-1 (any positive pivot is
+  // accepted); F_Ip = A_Ip V^T into F's tiles (the space of W^T) and H_p^T = V (its
+  // right-hand sides); then A_IJ -= F_Ip F_Jp^T and H_I^T -= F_Ip H_p^T.
+  float *F = WT;
+  float hmax = 0.f;
   for (int p = 0; p < nb; ++p) {
-    const int p0 = 32 * p, R = n - p0;
-    if (p0 > 0) {
-      const int ii = tid >> 2, cg = tid & 3;
-      if (ii < R) {
-        const float *Li = A + (size_t)(p0 + ii) * ld;
-        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int k = 0; k < p0; ++k) {
-          const float l = Li[k];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) acc[u] = fmaf(l, A[(size_t)(p0 + cg + 4 * u) * ld + k], acc[u]);
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-          if (cg + 4 * u <= ii) A[(size_t)(p0 + ii) * ld + p0 + cg + 4 * u] -= acc[u];
-      }
-      __syncthreads();
-    }
-    if (warp == 0) {
-      // a[k] holds column p0 + c + k of this lane's row: a window that moves
-      // one column right every step, so that the step loop keeps static
-      // register indices
-      const int row = p0 + lane;
-      const bool live = row < n;
-      float a[32];
-#pragma unroll
-      for (int k = 0; k < 32; ++k)
-        a[k] = (live && k <= lane) ? A[(size_t)row * ld + p0 + k] : (k == lane ? 1.f : 0.f);
-      bool okp = true;
-      for (int c = 0; c < 32; ++c) {
-        const float piv = __shfl_sync(FULL, a[0], c);
-        okp = okp && piv > 0.f;
-        const float d = sqrtf(fmaxf(piv, 1e-30f));
-        const float l = lane == c ? d : (lane > c ? a[0] / d : 0.f);  // L_{lane,c}
-#pragma unroll
-        for (int k = 1; k < 32; ++k) {
-          const float lk = __shfl_sync(FULL, l, (c + k) & 31);  // L_{c+k,c}
-          if (c + k < 32 && lane >= c + k) a[k] = fmaf(-l, lk, a[k]);
-        }
-        if (live && lane >= c) A[(size_t)row * ld + p0 + c] = l;
-#pragma unroll
-        for (int k = 0; k < 31; ++k) a[k] = a[k + 1];
-        a[31] = 0.f;
-      }
-      if (lane == 0 && !okp) badp = 1;
+    if (grp == 0) {
+      fc_diagonal(A + tri(p, p), zero, dsh, vpp, vtt, &badp);
     }
     __syncthreads();
     if (badp) {  // (uniform)
       if (tid == 0) set_status(status, BOUTE_ERR_NOT_PD);
       return;
     }
-    if (tid < R - 32) {
-      const int i = p0 + 32 + tid;
-      const float *Ld = A + (size_t)p0 * ld + p0;  // L_dd, read as broadcasts
-      float bv[32];
-#pragma unroll
-      for (int c = 0; c < 32; ++c) bv[c] = A[(size_t)i * ld + p0 + c];
-#pragma unroll
-      for (int c = 0; c < 32; ++c) {
-        float sv = bv[c];
-#pragma unroll
-        for (int k = 0; k < c; ++k) sv = fmaf(-bv[k], Ld[(size_t)c * ld + k], sv);
-        bv[c] = sv / Ld[(size_t)c * ld + c];
-      }
-#pragma unroll
-      for (int c = 0; c < 32; ++c) A[(size_t)i * ld + p0 + c] = bv[c];
+    for (int e = tid; e < kFcTile; e += kInsThreads) {  // F_pp, zero above the diagonal
+      const int r = e & 31, c = e >> 5;
+      F[tri(p, p) + fc_off(r, c)] = c <= r ? dsh.colL[c * 32 + r] : 0.f;
     }
-    __syncthreads();
-  }
-  for (int e = tid; e < n * n; e += kInsThreads) {  // F, zero above the diagonal
-    const int i = e / n, k = e % n;
-    wsb[e] = k <= i ? A[(size_t)i * ld + k] : 0.f;
-  }
-  // H^T = sigma^2 F^-1 K^-1 by forward substitution (in place of K^-1) in
-  // blocks of 32 rows: (a) the block's right-hand sides sigma^2 K^-1_rc -
-  // sum_{k<r0} F_rk H^T_kc (a thread holds one column and eight rows), then
-  // (b) a thread per column solves the block's triangle in registers.
-  float hmax = 0.f;
-  for (int q = 0; q < nb; ++q) {
-    const int r0 = 32 * q;
-    {
-      const int c = tid & 127, rg = tid >> 7;
-      if (c < n) {
-        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int k = 0; k < r0; ++k) {
-          const float hk = Kb[(size_t)k * ldk + c];
+    const int T = nb - 1 - p;
+    for (int e = grp; e < T + nb; e += kGroups) {
+      if (e < T) {
+        const int I = p + 1 + e;
+        fc_product(A + tri(I, p), vpp, gt, acc);
+        store(F + tri(I, p));
+      } else {
+        float *H = HT + (p * nb + e - T) * kFcTile;
+        fc_product(H, vpp, gt, acc);
+        named_barrier_sync(1 + grp, 64);  // the tile is read
+        store(H);
 #pragma unroll
-          for (int u = 0; u < 8; ++u) acc[u] = fmaf(A[(size_t)(r0 + 8 * rg + u) * ld + k], hk, acc[u]);
-        }
+        for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int r = r0 + 8 * rg + u;
-          if (r < n) Kb[(size_t)r * ldk + c] = fmaf(sig2, Kb[(size_t)r * ldk + c], -acc[u]);
-        }
+          for (int v = 0; v < 4; ++v) hmax = fmaxf(hmax, fabsf(acc[u][v]));
       }
     }
     __syncthreads();
-    if (tid < n) {
-      const int c = tid;
-      float hv[32];
-#pragma unroll
-      for (int rr = 0; rr < 32; ++rr) hv[rr] = r0 + rr < n ? Kb[(size_t)(r0 + rr) * ldk + c] : 0.f;
-#pragma unroll
-      for (int rr = 0; rr < 32; ++rr) {
-        if (r0 + rr < n) {
-          const float *Fr = A + (size_t)(r0 + rr) * ld + r0;
-          float sv = hv[rr];
-#pragma unroll
-          for (int k = 0; k < rr; ++k) sv = fmaf(-Fr[k], hv[k], sv);
-          hv[rr] = sv / Fr[rr];
-          hmax = fmaxf(hmax, fabsf(hv[rr]));
-        }
+    const int na = T * (T + 1) / 2;
+    for (int e = grp; e < na + T * nb; e += kGroups) {
+      float *D;
+      if (e < na) {
+        int i = 0;
+        while ((i + 1) * (i + 2) / 2 <= e) ++i;
+        const int I = p + 1 + i, J = p + 1 + e - i * (i + 1) / 2;
+        fc_product(F + tri(I, p), F + tri(J, p), gt, acc);
+        D = A + tri(I, J);
+      } else {
+        const int I = p + 1 + (e - na) / nb, c = (e - na) % nb;
+        fc_product(HT + (p * nb + c) * kFcTile, F + tri(I, p), gt, acc);
+        D = HT + (I * nb + c) * kFcTile;
       }
 #pragma unroll
-      for (int rr = 0; rr < 32; ++rr)
-        if (r0 + rr < n) Kb[(size_t)(r0 + rr) * ldk + c] = hv[rr];
+      for (int u = 0; u < 4; ++u) {
+        float4 *q = (float4 *)D + (4 * ty + u) * 8 + (tx ^ ty);
+        float4 v = *q;
+        v.x -= acc[u][0];
+        v.y -= acc[u][1];
+        v.z -= acc[u][2];
+        v.w -= acc[u][3];
+        *q = v;
+      }
     }
     __syncthreads();
   }
-  if (tid < n) atomic_max_pos(&mxh, hmax);
+  for (int i = warp; i < n; i += kInsThreads / 32)  // F, zero above the diagonal
+    for (int k = lane; k < n; k += 32)
+      wsb[(size_t)i * n + k] =
+          k <= i ? F[tri(i >> 5, k >> 5) + fc_off(i & 31, k & 31)] : 0.f;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) hmax = fmaxf(hmax, __shfl_xor_sync(0xffffffffu, hmax, o));
+  if (lane == 0) atomic_max_pos(&mxh, hmax);
   __syncthreads();
-  for (int e = tid; e < n * n; e += kInsThreads)
-    wsb[(size_t)n * n + e] = Kb[(size_t)(e / n) * ldk + e % n];
+  auto hval = [&](int r, int c) {  // H^T
+    return HT[((r >> 5) * nb + (c >> 5)) * kFcTile + fc_off(c & 31, r & 31)];
+  };
+  for (int i = warp; i < n; i += kInsThreads / 32)
+    for (int k = lane; k < n; k += 32) wsb[(size_t)n * n + (size_t)i * n + k] = hval(i, k);
   pdl_trigger();
   // H^T's operand images (output rows of the H blocks) and scale
   const int eh = scale_exp(__uint_as_float(mxh));
@@ -291,11 +257,12 @@ __global__ void __launch_bounds__(kInsThreads, 1)
   const float sh = exp2i(eh);
   const int kpairs = plan.nchunk * (BOUTE_ACHUNK / 2);
   uint16_t *img = bop + (size_t)bt * plan.image_halves;
-  for (int e = tid; e < n * kpairs; e += kInsThreads) {
-    const int row = e / kpairs, k = 2 * (e % kpairs);
-    pack_dense_pair(Kb + (size_t)row * ldk, n, k, sh, plan.nwblk + row / BOUTE_BLKCOLS, row, plan,
-                    img);
-  }
+  for (int row = warp; row < n; row += kInsThreads / 32)
+    for (int e = lane; e < kpairs; e += 32) {
+      const int k = 2 * e;
+      pack_dense_pair(k < n ? hval(row, k) : 0.f, k + 1 < n ? hval(row, k + 1) : 0.f, n, k, sh,
+                      plan.nwblk + row / BOUTE_BLKCOLS, row, plan, img);
+    }
 }
 
 // (2) the draws, kInsDraws per CTA (grid: draw groups x problem-objectives),
@@ -388,15 +355,17 @@ __global__ void __launch_bounds__(256)
   const float *gb = gws + (size_t)bt * S * n;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < S * kpairs; e += gridDim.x * blockDim.x) {
     const int row = e / kpairs, k = 2 * (e % kpairs);
-    pack_dense_pair(gb + (size_t)row * n, n, k, sg, plan.nwblk + plan.nhblk + row / BOUTE_BLKCOLS,
-                    row, plan, img);
+    const float *g = gb + (size_t)row * n;
+    pack_dense_pair(k < n ? g[k] : 0.f, k + 1 < n ? g[k + 1] : 0.f, n, k, sg,
+                    plan.nwblk + plan.nhblk + row / BOUTE_BLKCOLS, row, plan, img);
   }
 }
 
 }  // namespace
 
 size_t insample_smem_bytes(int n) {
-  return ((size_t)n * (ins_lda(n) + ins_ldk(n)) + 4 * 128 + 128) * sizeof(float);
+  const int nb = (n + 31) / 32;
+  return ((size_t)(nb * (nb + 1) + nb * nb + 2) * kFcTile + 32 * nb) * sizeof(float);
 }
 
 size_t insample_ws_floats(int n) { return ins_ws_floats(n); }

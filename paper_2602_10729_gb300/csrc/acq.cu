@@ -222,6 +222,77 @@ __device__ __forceinline__ float mc_hvi_regs(const float *e, int S, const float 
   return s0 + s1;
 }
 
+// Any other S: passes of 128 samples, four per lane in registers (sample 32 j + lane of
+// the pass), so that a box's bounds are read from shared memory once per four samples
+// and a box that lies below every sample of the pass adds nothing and is passed over.
+// Each sample adds prod_t (u_t - max(l_t, y_t))_+ as written. (A lane that took the
+// samples one by one read six bounds per sample and box: S = 100, 20 000 candidates
+// 155 -> 52 us.)
+template <int M, bool CONS>
+__device__ __forceinline__ float mc_hvi_any(const float *e, int S, const float (&mu)[M],
+                                            const float (&sg)[M], const float (&kc)[M],
+                                            const float *lo, const float *hi, int K, int lane,
+                                            float4 *stage) {
+  static_assert(M <= 3, "a box's bounds fit two float4");
+  constexpr int NS = 4;
+  float sum = 0.f;
+  for (int s0 = 0; s0 < S; s0 += 32 * NS) {
+    float y[NS][M], ymin[M];
+#pragma unroll
+    for (int t = 0; t < M; ++t) ymin[t] = INFINITY;
+#pragma unroll
+    for (int j = 0; j < NS; ++j) {
+      const int s = s0 + 32 * j + lane;
+      const bool in = s < S;
+      bool ok = in;
+#pragma unroll
+      for (int t = 0; t < M; ++t) {
+        y[j][t] = fmaf(sg[t], in ? __ldcs(e + (size_t)t * S + s) : 0.f, mu[t]);
+        if (in) ymin[t] = y[j][t] == y[j][t] ? fminf(ymin[t], y[j][t]) : -INFINITY;
+        if (CONS) ok = ok && y[j][t] <= kc[t];
+      }
+      if (!ok) y[j][0] = kInfeasible;
+    }
+#pragma unroll
+    for (int t = 0; t < M; ++t)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+        ymin[t] = fminf(ymin[t], __shfl_xor_sync(0xffffffffu, ymin[t], o));
+    for (int k0 = 0; k0 < K; k0 += 32) {
+      const int kb = k0 + lane;
+      float l[3] = {0.f, 0.f, 0.f}, h[3] = {0.f, 0.f, 0.f};
+      bool lv = kb < K;
+      if (kb < K) {
+#pragma unroll
+        for (int t = 0; t < M; ++t) {
+          l[t] = lo[kb * M + t];
+          h[t] = hi[kb * M + t];
+          lv = lv && !(h[t] <= ymin[t]);
+        }
+      }
+      __syncwarp();  // the previous group's bounds are read
+      stage[lane] = make_float4(l[0], l[1], l[2], 0.f);
+      stage[32 + lane] = make_float4(h[0], h[1], h[2], 0.f);
+      __syncwarp();
+      unsigned todo = __ballot_sync(0xffffffffu, lv);
+      while (todo) {
+        const int jb = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const float4 l4 = stage[jb], h4 = stage[32 + jb];
+        const float lb[3] = {l4.x, l4.y, l4.z}, hb[3] = {h4.x, h4.y, h4.z};
+#pragma unroll
+        for (int j = 0; j < NS; ++j) {
+          float v = fmaxf(hb[0] - fmaxf(lb[0], y[j][0]), 0.f);
+#pragma unroll
+          for (int t = 1; t < M; ++t) v *= fmaxf(hb[t] - fmaxf(lb[t], y[j][t]), 0.f);
+          sum += v;
+        }
+      }
+    }
+  }
+  return sum;
+}
+
 template <int M, bool CONS>
 __global__ void __launch_bounds__(512) mchvi_kernel(const float *mean, const float *var, int B,
                                                     long long N, const float *lower,
@@ -265,62 +336,8 @@ __global__ void __launch_bounds__(512) mchvi_kernel(const float *mean, const flo
       sum = mc_hvi_regs<M, CONS, 2>(e, S, mu, sg, kc, lo, hi, K, lane, stage[warp]);
     } else if (vec && S == 128) {
       sum = mc_hvi_regs<M, CONS, 1>(e, S, mu, sg, kc, lo, hi, K, lane, stage[warp]);
-    } else if (vec) {
-      for (int s0 = 4 * lane; s0 < S; s0 += 128) {
-        float4 z[M];
-#pragma unroll
-        for (int t = 0; t < M; ++t) z[t] = __ldcs((const float4 *)(e + (size_t)t * S + s0));
-        float y[4][M];
-#pragma unroll
-        for (int t = 0; t < M; ++t) {
-          y[0][t] = fmaf(sg[t], z[t].x, mu[t]);
-          y[1][t] = fmaf(sg[t], z[t].y, mu[t]);
-          y[2][t] = fmaf(sg[t], z[t].z, mu[t]);
-          y[3][t] = fmaf(sg[t], z[t].w, mu[t]);
-        }
-        if (CONS) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            bool ok = true;
-#pragma unroll
-            for (int t = 0; t < M; ++t) ok = ok && y[j][t] <= kc[t];
-            if (!ok) y[j][0] = kInfeasible;
-          }
-        }
-        for (int k = 0; k < K; ++k) {
-          float l[M], h[M];
-#pragma unroll
-          for (int t = 0; t < M; ++t) {
-            l[t] = lo[k * M + t];
-            h[t] = hi[k * M + t];
-          }
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            float v = fmaxf(h[0] - fmaxf(l[0], y[j][0]), 0.f);
-#pragma unroll
-            for (int t = 1; t < M; ++t) v *= fmaxf(h[t] - fmaxf(l[t], y[j][t]), 0.f);
-            sum += v;
-          }
-        }
-      }
     } else {
-      for (int s = lane; s < S; s += 32) {
-        float y[M];
-#pragma unroll
-        for (int t = 0; t < M; ++t) y[t] = fmaf(sg[t], e[(size_t)t * S + s], mu[t]);
-        if (CONS) {
-          bool ok = true;
-#pragma unroll
-          for (int t = 0; t < M; ++t) ok = ok && y[t] <= kc[t];
-          if (!ok) y[0] = kInfeasible;
-        }
-        for (int k = 0; k < K; ++k) {
-          float v = fmaxf(hi[k * M] - fmaxf(lo[k * M], y[0]), 0.f);
-#pragma unroll
-          for (int t = 1; t < M; ++t) v *= fmaxf(hi[k * M + t] - fmaxf(lo[k * M + t], y[t]), 0.f);
-          sum += v;
-        }
-      }
+      sum = mc_hvi_any<M, CONS>(e, S, mu, sg, kc, lo, hi, K, lane, stage[warp]);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);

@@ -418,3 +418,17 @@ def test_cluster_fit_edges(n, B):
         for t in range(w.m):
             check_mean(g["mean"][b, t], mean[:, t], fp.s2[t])
             check_var(g["var"][b, t], var[:, t], fp.s2[t])
+
+
+# Three objectives: passes of 128 samples with a ragged last one, one sample, and a
+# count the register path takes (with and without thresholds).
+@pytest.mark.parametrize("S", [1, 31, 100, 127, 129, 200, 256, 300])
+def test_three_objective_sample_counts(S):
+    hp = rand_problem(S, 25, 4, 3, 77, mode="mc", S=S)
+    compare(hp)
+    cons = np.full((1, 3), 0.4)
+    g = gpu_pipeline(hp, cons=cons)
+    fp = oracle_fit(hp, 0)
+    want = opl.acquisition(fp, g["mean"][0].T.astype(np.float64), g["var"][0].T.astype(np.float64),
+                           "mc", hp.eps[0], cons=cons[0])
+    check_acq(g["acq"][0], want)

@@ -156,15 +156,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// The composite kernel's per-candidate inputs (Sec. 5.2 "Additive kernels"
-// and S5, as Sec. 6 assembles them): the routing features are dimensions
-// [0, dtau), the candidate's preference weight w* = exp(beta <s, c*>), the
-// outputscales of the weighted deployment term and of the interaction term.
-struct CompIn {
-  int dtau;
-  float ws, s2c, s2x;
-};
-
 // The side input's composite-kernel entries within a chunk (the block after
 // the scaled coordinates): row 0 the chunk's training-point preference weights
 // w_j, row 1 beta * s_k per dimension (zero for routing features); the
@@ -174,10 +165,6 @@ __device__ __forceinline__ const float *chunk_weights(const float *chunk, int DP
 }
 __device__ __forceinline__ const float *chunk_pref(const float *chunk, int DP) {
   return chunk + BOUTE_KCHUNK * DP + BOUTE_KCHUNK;
-}
-__device__ __forceinline__ CompIn chunk_comp(const float *chunk, int DP) {
-  const float *pb = chunk + xt_param_offset(DP) + 2 * DP;
-  return CompIn{(int)pb[3], 0.f, pb[1], pb[2]};
 }
 
 // A candidate's preference weight from its raw coordinates.
@@ -189,113 +176,67 @@ __device__ __forceinline__ float cand_weight(const float (&xr)[DP], const float 
   return expf(e);
 }
 
-// The K* values of one builder thread's COLS columns of a 32-point chunk:
-// squared scaled distances in packed pairs (candidate x*_k / l_k as a
-// duplicated pair, minus the chunk's training coordinates x_k / l_k, both
-// times the side input's coordinate scale), then
-// k = s2 (1 + sqrt5 r + 5/3 r^2) exp(-sqrt5 r) = s2 (1 + ln2 r' + ln2^2/3 r'^2) 2^(-r').
-// KERN = 1, the composite kernel: the distances over the routing features
-// (r_t) and the deployment features (r_c) are accumulated apart, and
-//   k = k52(r_t) (s2 + s2_x k32(r_c)) + s2_c w_j w* k32(r_c),
-//   k52(r) = (1 + sqrt5 r + 5/3 r^2) e^(-sqrt5 r), k32(r) = (1 + sqrt3 r) e^(-sqrt3 r),
-// each in its own scaled distance (the deployment features carry sqrt3 / ln 2).
-// Both the fused builders and the stand-alone K* kernel use this, so their
-// values are identical.
-template <int DP, int COLS, int KERN = 0>
-__device__ __forceinline__ void kstar_cols(const unsigned long long (&xs2)[DP], const float *xth,
-                                           int g, float s2, float (&kv)[COLS],
-                                           const CompIn &ci = CompIn{}) {
-  unsigned long long acc2[COLS / 2], accc[COLS / 2];
-#pragma unroll
-  for (int e = 0; e < COLS / 2; ++e) {
-    acc2[e] = 0ull;
-    accc[e] = 0ull;
-  }
-#pragma unroll
-  for (int k = 0; k < DP; ++k) {
-    // 16-byte loads: two training points' coordinate pairs each
-    const ulonglong2 *h4 = (const ulonglong2 *)(xth + k * BOUTE_KCHUNK + COLS * g);
-    unsigned long long h2[COLS / 2];
-#pragma unroll
-    for (int e = 0; e < COLS / 4; ++e) {
-      const ulonglong2 v = h4[e];
-      h2[2 * e] = v.x;
-      h2[2 * e + 1] = v.y;
-    }
-    if (KERN == 1 && k >= ci.dtau) {  // a deployment feature (uniform branch)
-#pragma unroll
-      for (int e = 0; e < COLS / 2; ++e) {
-        const unsigned long long df = f2_sub(xs2[k], h2[e]);
-        accc[e] = f2_fma(df, df, accc[e]);
-      }
-    } else {
-#pragma unroll
-      for (int e = 0; e < COLS / 2; ++e) {
-        const unsigned long long df = f2_sub(xs2[k], h2[e]);
-        acc2[e] = f2_fma(df, df, acc2[e]);
-      }
-    }
-  }
-  if (KERN == 1) {
-    const float *wj = chunk_weights(xth, DP) + COLS * g;
-#pragma unroll
-    for (int e = 0; e < COLS / 2; ++e) {
-      float r2[2], c2[2];
-      f2_split(acc2[e], r2[0], r2[1]);
-      f2_split(accc[e], c2[0], c2[1]);
-#pragma unroll
-      for (int z = 0; z < 2; ++z) {
-        const float rr = sqrt_approx(r2[z]);
-        const float k52 = fmaf(kLn2Sq3, r2[z], fmaf(kLn2, rr, 1.0f)) * ex2_approx(-rr);
-        const float rc = sqrt_approx(c2[z]);
-        const float k32 = fmaf(kLn2, rc, 1.0f) * ex2_approx(-rc);
-        kv[2 * e + z] = fmaf(k52, fmaf(ci.s2x, k32, s2), ci.s2c * (wj[2 * e + z] * ci.ws) * k32);
-      }
-    }
-    return;
-  }
-  // packed pairs: k = (s2 + s2 ln2 r' + s2 ln2^2/3 r'^2) 2^(-r'); the exponent
-  // is the scaled distance itself, so the exponential is as accurate as ex2
-  const unsigned long long c0 = f2_dup(s2), c1 = f2_dup(s2 * kLn2), c2 = f2_dup(s2 * kLn2Sq3);
-#pragma unroll
-  for (int e = 0; e < COLS / 2; ++e) {
-    float ra, rb;
-    f2_split(acc2[e], ra, rb);
-    const float r0 = sqrt_approx(ra), r1 = sqrt_approx(rb);
-    const unsigned long long ex = f2_pack(ex2_approx(-r0), ex2_approx(-r1));
-    const unsigned long long t = f2_fma(acc2[e], c2, f2_fma(f2_pack(r0, r1), c1, c0));
-    f2_split(f2_mul(t, ex), kv[2 * e], kv[2 * e + 1]);
-  }
+// The exponent e_r of a candidate row's K* scale (kstar_scale_exp of the
+// row's bound on K*): the outputscale for the Matern-5/2 kernel; for the
+// composite kernel s2 + s2_x + s2_c w* max_j w_j (each factor k52, k32 <= 1).
+// Builders, the epilogue and the K* kernel all derive it here.
+__device__ __forceinline__ int row_exp(int kern, const float *par, float ws) {
+  float bound = par[kParS2];
+  if (kern) bound = fmaf(par[kParS2c] * ws, par[kParWmax], par[kParS2] + par[kParS2x]);
+  if (!(bound > 0.f) || !(bound < 3.0e38f)) bound = 1.f;
+  return kstar_scale_exp(bound);
 }
 
-// A candidate's scaled coordinates as duplicated pairs, x*_k (1/l_k hi + lo),
-// from the objective's parameters (1/l hi [DP], 1/l lo [DP], s2) of a chunk.
+// A pair of candidate rows as (row 0, row 1) pairs: the scaled coordinates
+// x*_k (1/l_k hi + lo), and the kernel's outputscales times 2^e_r, s2 and, composite
+// kernel, s2_x and s2_c w* (w* = exp(beta <s, c*>), the row's preference weight).
 template <int DP>
-__device__ __forceinline__ void scaled_candidate(const float (&xr)[DP], const float *il,
-                                                 unsigned long long (&xs2)[DP]) {
-#pragma unroll
-  for (int k = 0; k < DP; ++k) xs2[k] = f2_dup(fmaf(xr[k], il[k], xr[k] * il[DP + k]));
-}
-
-// Two candidates' scaled coordinates as (row 0, row 1) pairs.
-template <int DP>
-__device__ __forceinline__ void scaled_pair(const float (&x0)[DP], const float (&x1)[DP],
-                                            const float *il, unsigned long long (&xs2)[DP]) {
+struct PairIn {
+  unsigned long long x[DP], s2, s2x, s2cw;
+  int dtau;
+};
+// x0, x1: the rows' raw coordinates; chunk: the objective's first side-input chunk;
+// par: its scalars.
+template <int DP, int KERN>
+__device__ __forceinline__ void pair_rows(const float (&x0)[DP], const float (&x1)[DP],
+                                          const float *chunk, const float *par, PairIn<DP> &in) {
+  const float *il = chunk + xt_param_offset(DP);
+  if (KERN == 0) {
+    in.s2 = f2_dup(ldexpf(par[kParS2], row_exp(0, par, 0.f)));
+  } else {
+    const float w0 = cand_weight<DP>(x0, chunk_pref(chunk, DP));
+    const float w1 = cand_weight<DP>(x1, chunk_pref(chunk, DP));
+    const int e0 = row_exp(1, par, w0), e1 = row_exp(1, par, w1);
+    in.dtau = (int)par[kParDtau];
+    in.s2 = f2_pack(ldexpf(par[kParS2], e0), ldexpf(par[kParS2], e1));
+    in.s2x = f2_pack(ldexpf(par[kParS2x], e0), ldexpf(par[kParS2x], e1));
+    in.s2cw = f2_pack(ldexpf(par[kParS2c], e0) * w0, ldexpf(par[kParS2c], e1) * w1);
+  }
 #pragma unroll
   for (int k = 0; k < DP; ++k)
-    xs2[k] = f2_pack(fmaf(x0[k], il[k], x0[k] * il[DP + k]), fmaf(x1[k], il[k], x1[k] * il[DP + k]));
+    in.x[k] = f2_pack(fmaf(x0[k], il[k], x0[k] * il[DP + k]), fmaf(x1[k], il[k], x1[k] * il[DP + k]));
 }
 
-// kstar_cols for a pair of candidate rows (Matern-5/2): C columns of a 32-point
-// chunk, each value a (row 0, row 1) pair; every training coordinate is loaded
-// once for the two rows and duplicated in registers. Per entry the same
-// operations in the same order as kstar_cols, so the values are identical.
-template <int DP, int C>
-__device__ __forceinline__ void kstar_pair(const unsigned long long (&xs2)[DP], const float *xth,
-                                           int g, float s2, unsigned long long (&kv)[C]) {
-  unsigned long long acc[C];
+// The K* values of C columns of a 32-point chunk for a pair of candidate rows, each
+// value a (row 0, row 1) pair: squared scaled distances in packed pairs (candidate
+// minus the chunk's training coordinates x_k / l_k, both times the side input's
+// coordinate scale; every training coordinate is loaded once for the two rows), then
+//   k = s2 (1 + sqrt5 r + 5/3 r^2) exp(-sqrt5 r) = s2 (1 + ln2 r' + ln2^2/3 r'^2) 2^(-r'),
+// whose exponent is the scaled distance itself, so the exponential is as accurate as ex2.
+// KERN = 1, the composite kernel (Sec. 5.2 "Additive kernels" and S5, as Sec. 6
+// assembles them): the distances over the routing features [0, dtau) (r_t) and the
+// deployment features (r_c) are accumulated apart, and
+//   k = k52(r_t) (s2 + s2_x k32(r_c)) + s2_c w_j w* k32(r_c),
+//   k52(r) = (1 + sqrt5 r + 5/3 r^2) e^(-sqrt5 r), k32(r) = (1 + sqrt3 r) e^(-sqrt3 r),
+// each in its own scaled distance (the deployment features carry sqrt3 / ln 2). Both
+// the fused builders and the stand-alone K* kernel use this, so their values are
+// identical.
+template <int DP, int C, int KERN>
+__device__ __forceinline__ void kstar_pair(const PairIn<DP> &in, const float *xth, int g,
+                                           unsigned long long (&kv)[C]) {
+  unsigned long long acc[C], accd[C];
 #pragma unroll
-  for (int e = 0; e < C; ++e) acc[e] = 0ull;
+  for (int e = 0; e < C; ++e) acc[e] = accd[e] = 0ull;
 #pragma unroll
   for (int k = 0; k < DP; ++k) {
     const float4 *h4 = (const float4 *)(xth + k * BOUTE_KCHUNK + C * g);
@@ -308,34 +249,51 @@ __device__ __forceinline__ void kstar_pair(const unsigned long long (&xs2)[DP], 
       h[4 * e + 2] = v.z;
       h[4 * e + 3] = v.w;
     }
+    if (KERN == 1 && k >= in.dtau) {  // a deployment feature (uniform branch)
 #pragma unroll
-    for (int e = 0; e < C; ++e) {
-      const unsigned long long df = f2_sub(xs2[k], f2_dup(h[e]));
-      acc[e] = f2_fma(df, df, acc[e]);
+      for (int e = 0; e < C; ++e) {
+        const unsigned long long df = f2_sub(in.x[k], f2_dup(h[e]));
+        accd[e] = f2_fma(df, df, accd[e]);
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < C; ++e) {
+        const unsigned long long df = f2_sub(in.x[k], f2_dup(h[e]));
+        acc[e] = f2_fma(df, df, acc[e]);
+      }
     }
   }
-  const unsigned long long c0 = f2_dup(s2), c1 = f2_dup(s2 * kLn2), c2 = f2_dup(s2 * kLn2Sq3);
-#pragma unroll
-  for (int e = 0; e < C; ++e) {
+  auto root_exp = [](unsigned long long a, unsigned long long &r, unsigned long long &ex) {
     float ra, rb;
-    f2_split(acc[e], ra, rb);
+    f2_split(a, ra, rb);
     const float r0 = sqrt_approx(ra), r1 = sqrt_approx(rb);
-    const unsigned long long ex = f2_pack(ex2_approx(-r0), ex2_approx(-r1));
-    const unsigned long long t = f2_fma(acc[e], c2, f2_fma(f2_pack(r0, r1), c1, c0));
-    kv[e] = f2_mul(t, ex);
+    r = f2_pack(r0, r1);
+    ex = f2_pack(ex2_approx(-r0), ex2_approx(-r1));
+  };
+  if (KERN == 0) {
+    float s2, s2_;
+    f2_split(in.s2, s2, s2_);  // (the rows' are equal)
+    const unsigned long long c1 = f2_dup(s2 * kLn2), c2 = f2_dup(s2 * kLn2Sq3);
+#pragma unroll
+    for (int e = 0; e < C; ++e) {
+      unsigned long long r, ex;
+      root_exp(acc[e], r, ex);
+      kv[e] = f2_mul(f2_fma(acc[e], c2, f2_fma(r, c1, in.s2)), ex);
+    }
+  } else {
+    const unsigned long long one = f2_dup(1.f), l1 = f2_dup(kLn2), l2 = f2_dup(kLn2Sq3);
+    const float *wj = chunk_weights(xth, DP) + C * g;
+#pragma unroll
+    for (int e = 0; e < C; ++e) {
+      unsigned long long r, ex, rd, exd;
+      root_exp(acc[e], r, ex);
+      root_exp(accd[e], rd, exd);
+      const unsigned long long k52 = f2_mul(f2_fma(acc[e], l2, f2_fma(r, l1, one)), ex);
+      const unsigned long long k32 = f2_mul(f2_fma(rd, l1, one), exd);
+      kv[e] = f2_fma(k52, f2_fma(in.s2x, k32, in.s2),
+                     f2_mul(f2_mul(in.s2cw, f2_dup(wj[e])), k32));
+    }
   }
-}
-
-
-// The exponent e_r of a candidate row's K* scale (kstar_scale_exp of the
-// row's bound on K*): the outputscale for the Matern-5/2 kernel; for the
-// composite kernel s2 + s2_x + s2_c w* max_j w_j (each factor k52, k32 <= 1).
-// Builders, the epilogue and the K* kernel all derive it here.
-__device__ __forceinline__ int row_exp(int kern, const float *par, float ws) {
-  float bound = par[kParS2];
-  if (kern) bound = fmaf(par[kParS2c] * ws, par[kParWmax], par[kParS2] + par[kParS2x]);
-  if (!(bound > 0.f) || !(bound < 3.0e38f)) bound = 1.f;
-  return kstar_scale_exp(bound);
 }
 
 // Position in a ring of R stages: the stage index and the parity of the
@@ -530,14 +488,13 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
     posterior_kernel(const __grid_constant__ PostArgs a) {
   constexpr int kBldWarps = Layout<DP>::kBld;
   constexpr int COLS = Layout<DP>::kCols;   // columns of a half per builder thread
-  // The Matern kernel built here: each builder thread covers two candidate rows
-  // (kstar_pair), so that every training coordinate it loads serves two K*
+  // K* built here: each builder thread covers two candidate rows (kstar_pair), so that every training coordinate it loads serves two K*
   // entries (half the shared-memory wavefronts per entry, which beside the tensor
   // cores' operand reads and with the latency of the loads hold the builders back.
   // One row and twice the columns with 16 warps: n = 512, d = 16, 2^20 candidates
   // 2487 against 2210 us; n = 256, d = 10, 2^22 candidates 4092 against 4024 us.
   // Two rows held singly and duplicated instead of the training coordinate: 2480.)
-  constexpr bool kPair = !PRE && KERN == 0;
+  constexpr bool kPair = !PRE;
   constexpr int RP = kPair ? 2 : 1;  // candidate rows per builder thread
   constexpr int CT = COLS / RP;      // its columns of a 32-point half
   constexpr int GPT = 32 / CT;       // column groups
@@ -915,18 +872,12 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
       const int tile = unit / m;
       const int b = tile / a.tiles_per_problem;
       const long long row = (long long)(tile % a.tiles_per_problem) * BOUTE_TILE_M + r;
-      float xr[DP];  // (unused with rows in pairs)
-      unsigned long long xs2[DP];
-      float s2 = 0.f;
-      CompIn ci{};
-      int er = 0;
+      PairIn<DP> in;
       if constexpr (kPair) {
         // both rows' scaled coordinates now, with the objective's scales read
         // from the side input in global memory, so that the raw coordinates
         // die here instead of living through the chunk loop
-        const float *il = a.xt + (size_t)(b * m + unit % m) * pl.nxt * cf + xt_param_offset(DP);
-        er = row_exp(0, il + 2 * DP, 0.f);
-        s2 = ldexpf(il[2 * DP + kParS2], er);
+        const float *x00 = a.xt + (size_t)(b * m + unit % m) * pl.nxt * cf;
         float x0[DP], x1[DP];
         const long long row1 = row + RPT;
         const float *xrow = a.Xc + ((long long)b * a.N + row) * d;
@@ -936,11 +887,7 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
           x0[k] = (k < d && row < a.N) ? xrow[k] : 0.f;
           x1[k] = (k < d && row1 < a.N) ? xrow1[k] : 0.f;
         }
-        scaled_pair<DP>(x0, x1, il, xs2);
-      } else if (!PRE || KERN == 1) {
-        const float *xrow = a.Xc + ((long long)b * a.N + row) * d;
-#pragma unroll
-        for (int k = 0; k < DP; ++k) xr[k] = (k < d && row < a.N) ? xrow[k] : 0.f;
+        pair_rows<DP, KERN>(x0, x1, x00, x00 + xt_param_offset(DP) + 2 * DP, in);
       }
       // the mean K* alpha: its terms reach hundreds of times the result when K
       // is ill-conditioned, so they are summed with compensation, and their
@@ -968,26 +915,10 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
             if (!wait_or_abort(&x_full[j], px.phase, abort)) break;
             const float *xth = xt_reg(j);
             const float *alp = xth + xt_alpha_offset(DP);
-            if (!kPair && gi == 0 && c == 0 && h == 0) {  // new objective: its parameters came with the chunk
-              const float *il = xth + xt_param_offset(DP);
-              const float *par = il + 2 * DP;
-              if (KERN == 1) ci = chunk_comp(xth, DP);
-              const float ws = KERN == 1 ? cand_weight<DP>(xr, chunk_pref(xth, DP)) : 0.f;
-              er = row_exp(KERN, par, ws);
-              if (!PRE) {
-                scaled_candidate<DP>(xr, il, xs2);
-                s2 = ldexpf(par[kParS2], er);
-                if (KERN == 1) {
-                  ci.ws = ws;
-                  ci.s2c = ldexpf(ci.s2c, er);
-                  ci.s2x = ldexpf(ci.s2x, er);
-                }
-              }
-            }
             if constexpr (kPair) {
               const int col0 = BOUTE_KCHUNK * h + CT * g;  // first column within the chunk
               unsigned long long kvp[CT];  // (row r, row r + RPT) per column
-              kstar_pair<DP, CT>(xs2, xth, g, s2, kvp);
+              kstar_pair<DP, CT, KERN>(in, xth, g, kvp);
               const int jbase = BOUTE_ACHUNK * c + col0;
               const float *alg = alp + CT * g;
               // both rows' CT = 8 columns into the A stage as fp16 hi/lo, the
@@ -1036,17 +967,13 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
             } else {
               float kv[COLS];
               const int col0 = BOUTE_KCHUNK * h + COLS * g;  // first column within the chunk
-              if (PRE) {  // this thread's COLS values, from the staged fp32 image
 #pragma unroll
-                for (int e = 0; e < COLS / 4; ++e) {
-                  const float4 v = *(const float4 *)(stage(s) + st_off32(r, col0 + 4 * e));
-                  kv[4 * e] = v.x;
-                  kv[4 * e + 1] = v.y;
-                  kv[4 * e + 2] = v.z;
-                  kv[4 * e + 3] = v.w;
-                }
-              } else {
-                kstar_cols<DP, COLS, KERN>(xs2, xth, g, s2, kv, ci);
+              for (int e = 0; e < COLS / 4; ++e) {  // its values, from the staged fp32 image
+                const float4 v = *(const float4 *)(stage(s) + st_off32(r, col0 + 4 * e));
+                kv[4 * e] = v.x;
+                kv[4 * e + 1] = v.y;
+                kv[4 * e + 2] = v.z;
+                kv[4 * e + 3] = v.w;
               }
               const int jbase = BOUTE_ACHUNK * c + col0;
               const float *alg = alp + COLS * g;
@@ -1229,20 +1156,24 @@ template <int DP, int KERN>
 __global__ void __launch_bounds__(Layout<DP>::kBld * 32) kstar_kernel(
     const float *Xc, const float *xt, long long N, int d, int m, int n, int tiles_per_problem,
     int nxt, float *kst) {
-  constexpr int COLS = Layout<DP>::kCols, GPR = 32 / COLS, RPW = 32 / GPR;
+  // rows in pairs, RPT apart, C columns of each half per thread, as the fused builders
+  constexpr int C = Layout<DP>::kCols / 2, RPT = C;
   extern __shared__ __align__(16) float xs[];  // nxt side-input chunks
   __shared__ float wmax_s;
   const int unit = blockIdx.x, tile = unit / m, t = unit % m, b = tile / tiles_per_problem;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r = warp * RPW + lane % RPW, g = lane / RPW;
+  const int r = warp * 2 * RPT + lane % RPT, g = lane / RPT;
   const long long row = (long long)(tile % tiles_per_problem) * BOUTE_TILE_M + r;
   const int cf = xt_chunk_floats(DP);  // a multiple of 4
   const float4 *x4 = (const float4 *)(xt + (size_t)(b * m + t) * nxt * cf);
   for (int e = threadIdx.x; e < nxt * cf / 4; e += blockDim.x) ((float4 *)xs)[e] = x4[e];
-  const float *xrow = Xc + ((long long)b * N + row) * d;
-  float xr[DP];
+  const float *xrow = Xc + ((long long)b * N + row) * d, *xrow1 = xrow + (long long)RPT * d;
+  float x0[DP], x1[DP];
 #pragma unroll
-  for (int k = 0; k < DP; ++k) xr[k] = (k < d && row < N) ? xrow[k] : 0.f;
+  for (int k = 0; k < DP; ++k) {
+    x0[k] = (k < d && row < N) ? xrow[k] : 0.f;
+    x1[k] = (k < d && row + RPT < N) ? xrow1[k] : 0.f;
+  }
   __syncthreads();
   const float *il = xs + xt_param_offset(DP);
   float par[8];
@@ -1260,33 +1191,26 @@ __global__ void __launch_bounds__(Layout<DP>::kBld * 32) kstar_kernel(
     __syncthreads();
     par[kParWmax] = wmax_s;
   }
-  unsigned long long xs2[DP];
-  scaled_candidate<DP>(xr, il, xs2);
-  CompIn ci{};
-  float ws = 0.f;
-  if (KERN == 1) {
-    ci = chunk_comp(xs, DP);
-    ws = cand_weight<DP>(xr, chunk_pref(xs, DP));
-  }
-  const int er = row_exp(KERN, par, ws);
-  const float s2 = ldexpf(par[kParS2], er);
-  if (KERN == 1) {
-    ci.ws = ws;
-    ci.s2c = ldexpf(ci.s2c, er);
-    ci.s2x = ldexpf(ci.s2x, er);
-  }
+  PairIn<DP> in;
+  pair_rows<DP, KERN>(x0, x1, xs, par, in);
   for (int c = 0; c < nxt; ++c) {  // 32-point halves
-    float kv[COLS];
-    kstar_cols<DP, COLS, KERN>(xs2, xs + (size_t)c * cf, g, s2, kv, ci);
-    const int jbase = c * BOUTE_KCHUNK + COLS * g;
-#pragma unroll
-    for (int kk = 0; kk < COLS; ++kk) kv[kk] = (jbase + kk < n) ? kv[kk] : 0.f;
+    unsigned long long kvp[C];
+    kstar_pair<DP, C, KERN>(in, xs + (size_t)c * cf, g, kvp);
+    const int jbase = c * BOUTE_KCHUNK + C * g;
     float *img = kst + ((size_t)unit * (nxt / 2) + c / 2) * (kStageBytes / 4);
-    const int col0 = BOUTE_KCHUNK * (c & 1) + COLS * g;
+    const int col0 = BOUTE_KCHUNK * (c & 1) + C * g;
+    float kv[2][C];
 #pragma unroll
-    for (int g4 = 0; g4 < COLS / 4; ++g4)
-      *(float4 *)(img + st_off32(r, col0 + 4 * g4)) =
-          make_float4(kv[4 * g4], kv[4 * g4 + 1], kv[4 * g4 + 2], kv[4 * g4 + 3]);
+    for (int kk = 0; kk < C; ++kk) {
+      f2_split(kvp[kk], kv[0][kk], kv[1][kk]);
+      if (jbase + kk >= n) kv[0][kk] = kv[1][kk] = 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int g4 = 0; g4 < C / 4; ++g4)
+        *(float4 *)(img + st_off32(r + q * RPT, col0 + 4 * g4)) =
+            make_float4(kv[q][4 * g4], kv[q][4 * g4 + 1], kv[q][4 * g4 + 2], kv[q][4 * g4 + 3]);
   }
 }
 

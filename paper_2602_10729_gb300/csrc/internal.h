@@ -12,7 +12,7 @@ namespace boute {
 
 // The boute_gp handle: fp64 factors plus the prepacked tensor-core operands.
 struct Gp {
-  int B, n, d, m, DP;  // DP = d rounded up to a multiple of 4 (register tile)
+  int B, n, d, m, DP;  // DP = d rounded up to one of BOUTE_PADDED_DIMS (register tile)
   PostPlan plan;
   float *Kh, *Kl;  // B*m x n x n: kernel matrix (lower) as an fp32 pair hi + lo
   float *Aws;      // B*m x np x (np+1): the factorisation's tiles when they do not fit shared memory
@@ -44,6 +44,9 @@ struct Gp {
   // the preparation's workspace (F, H^T, mu_n, max |G|: insample_ws_floats)
   float *gws, *iws;
 };
+
+// X(DP) for every padded dimension count the posterior's kernels are built for.
+#define BOUTE_PADDED_DIMS(X) X(6) X(8) X(10) X(12) X(14) X(16) X(20) X(24) X(28) X(32)
 
 // An NVTX range over one call of the C-ABI (visible in a profiler's timeline;
 // a few nanoseconds when no tool is attached).

@@ -1243,11 +1243,10 @@ int launch_posterior_joint(const Gp *gp, const float *Xc, long long N, float *me
                            float *shift, cudaStream_t s, const float *kst) {
   if (N <= 0) return BOUTE_OK;
   switch (gp->DP) {
-    case 8: return launch_dp<8>(gp, Xc, kst, N, mean, cvar, s, shift);
-    case 12: return launch_dp<12>(gp, Xc, kst, N, mean, cvar, s, shift);
-    case 16: return launch_dp<16>(gp, Xc, kst, N, mean, cvar, s, shift);
-    case 24: return launch_dp<24>(gp, Xc, kst, N, mean, cvar, s, shift);
-    case 32: return launch_dp<32>(gp, Xc, kst, N, mean, cvar, s, shift);
+#define BOUTE_CASE(DP) \
+  case DP: return launch_dp<DP>(gp, Xc, kst, N, mean, cvar, s, shift);
+    BOUTE_PADDED_DIMS(BOUTE_CASE)
+#undef BOUTE_CASE
   }
   return BOUTE_ERR_UNSUPPORTED;
 }
@@ -1272,11 +1271,10 @@ size_t kstar_floats(const Gp *gp, long long N) {
 int launch_kstar(const Gp *gp, const float *Xc, long long N, float *kst, cudaStream_t s) {
   if (N <= 0) return BOUTE_OK;
   switch (gp->DP) {
-    case 8: return launch_kstar_dp<8>(gp, Xc, N, kst, s);
-    case 12: return launch_kstar_dp<12>(gp, Xc, N, kst, s);
-    case 16: return launch_kstar_dp<16>(gp, Xc, N, kst, s);
-    case 24: return launch_kstar_dp<24>(gp, Xc, N, kst, s);
-    case 32: return launch_kstar_dp<32>(gp, Xc, N, kst, s);
+#define BOUTE_CASE(DP) \
+  case DP: return launch_kstar_dp<DP>(gp, Xc, N, kst, s);
+    BOUTE_PADDED_DIMS(BOUTE_CASE)
+#undef BOUTE_CASE
   }
   return BOUTE_ERR_UNSUPPORTED;
 }

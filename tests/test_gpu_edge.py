@@ -390,7 +390,9 @@ def test_front_and_boxes_edges(n, m, kind):
 # Rows in pairs (four or eight rows apart) and four or eight columns of a half chunk
 # per thread: rows and columns at their edges, every coordinate width.
 @pytest.mark.parametrize("d,n,N", [(3, 1, 1), (3, 35, 4), (9, 4, 5), (9, 61, 129), (16, 5, 8),
-                                   (16, 33, 133), (20, 7, 9), (24, 41, 137), (32, 9, 127)])
+                                   (16, 33, 133), (20, 7, 9), (24, 41, 137), (32, 9, 127),
+                                   (7, 34, 70), (11, 66, 130), (13, 40, 131), (14, 3, 200),
+                                   (17, 37, 65), (21, 70, 66), (25, 36, 90), (29, 35, 129)])
 def test_row_pairs_and_column_groups(d, n, N):
     hp = rand_problem(100 + d + n, n, d, 2, N)
     hp.ls[0] = 0.2 * np.sqrt(d)

@@ -434,3 +434,23 @@ def test_three_objective_sample_counts(S):
     want = opl.acquisition(fp, g["mean"][0].T.astype(np.float64), g["var"][0].T.astype(np.float64),
                            "mc", hp.eps[0], cons=cons[0])
     check_acq(g["acq"][0], want)
+
+
+def test_ehvi_over_the_normal_tail():
+    """One front point: EHVI's standardised distances from 0 to 12 on both sides,
+    relative. The tail factor is good to 3e-7, phi's exponent t^2 / 2 to an ulp of its
+    product (t <= 12: 5e-6), sums and products of a few such terms: 2e-5."""
+    import torch
+
+    from paper_2602_10729_gb300 import boute as bt
+    z = np.linspace(-12, 12, 2001)
+    N = z.size
+    mean = np.stack([z, 0.3 * z], 0)[None].astype(np.float32)
+    var = np.ones((1, 2, N), np.float32)
+    F, ref = np.array([[0.0, 0.0]]), np.array([1.1, 1.1])
+    t = lambda a: torch.as_tensor(np.ascontiguousarray(a), device="cuda")
+    acq = torch.empty((1, N), dtype=torch.float32, device="cuda")
+    bt.boute_acq_ehvi(t(mean), t(var), 1, N, t(F[None]), torch.ones(1, dtype=torch.int32, device="cuda"),
+                      1, t(ref[None]), acq)
+    want = oracle.ehvi2d(mean[0].T.astype(np.float64), var[0].T.astype(np.float64), F, ref)
+    np.testing.assert_allclose(acq.cpu().numpy()[0], want, rtol=2e-5, atol=1e-36)

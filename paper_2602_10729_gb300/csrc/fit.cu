@@ -313,8 +313,9 @@ __device__ __forceinline__ void composite_wmax(float *xt, int bt, const PostPlan
 // first and factoring it beside the rest, and the owners of block row p write W and its
 // operand images. Then alpha and its two refinement steps from the tiles. Tiles and
 // vectors travel by stores to the other CTAs' shared memory, ordered by the barriers.
-// Sums run in an order that does not depend on C. What bounds it is the chain of a panel (two barriers, two tile products, the
-// diagonal tile), for n = 1024 as much the updates' shared-memory reads.
+// Sums run in an order that does not depend on C. What bounds it is the chain of a
+// panel (two barriers, two tile products, the diagonal tile: about 15 thousand clocks at
+// n = 512), for n = 1024 as much the updates' shared-memory reads.
 // Fit with its set-up, against three launches a panel, nine for alpha and one block
 // per problem-objective in large batches: n = 203, m = 3 174 -> 98 us; n = 512, m = 2
 // 385 -> 230 us; n = 777, B = 3, m = 2 1193 -> 754 us; n = 1024, m = 3 1226 -> 943 us;

@@ -14,9 +14,9 @@
 // cvar = k(x,x) - |W k*|^2 - |H^T k*|^2. H^T and G^T therefore become dense
 // output blocks of the posterior's tensor-core contraction beside W.
 //
-//   insample_kernel        one CTA per problem-objective after the fit: K^-1,
-//                          F, the in-sample draws, H, G and their operand
-//                          images (fp32 arithmetic in shared memory, n <= 128)
+//   insample_factor_kernel one CTA per problem-objective after the fit: K^-1, F and H
+//                          (fp32 tiles in shared memory, n <= 128); then
+//   insample_draws_kernel, insample_pack_kernel: the draws, G, and its operand images
 //   insample_front_kernel  one warp per (problem, draw): the Pareto front of
 //                          the feasible in-sample draws as vertical strips
 //   nehvi2_kernel          one thread per candidate: the draws' hypervolume

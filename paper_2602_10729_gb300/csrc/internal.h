@@ -29,7 +29,7 @@ struct Gp {
   float *xt;      // B*m x nxt x xt_chunk_floats(DP): X/lengthscale hi/lo, alpha
   float *s2f;     // B*m: outputscale
   int *status;    // device status word (first error wins)
-  int *fbad;      // B*m: a non-positive pivot in the cluster factorisation (n > 160)
+  int *fbad;      // B*m: a non-positive pivot in the factorisation
   // the FP64 tier (prec = BOUTE_PREC_FP64): W = L^-1 (B*m x n x n), alpha
   // (B*m x n), X / lengthscale (B*m x n x d), lengthscales (B*m x d) and
   // outputscales (B*m) of the last fit, all fp64

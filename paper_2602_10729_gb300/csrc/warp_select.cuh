@@ -63,14 +63,6 @@ __device__ __forceinline__ unsigned long long warp_merge_desc(unsigned long long
   return u;
 }
 
-// Insert one key (the same in every lane) into a sorted warp list.
-__device__ __forceinline__ unsigned long long warp_insert_desc(unsigned long long top,
-                                                               unsigned long long key, int lane) {
-  const int pos = __popc(__ballot_sync(0xffffffffu, top > key));  // keys above the new one
-  const unsigned long long up = __shfl_up_sync(0xffffffffu, top, 1);
-  return lane < pos ? top : (lane == pos ? key : up);
-}
-
 // A warp's running top-32 fed one key at a time (the same key in every lane):
 // keys wait in a lane each (lane i holds the i-th since the last merge) and
 // are sorted and merged into the list 32 at a time, so that adding a key

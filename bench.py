@@ -184,14 +184,14 @@ def stage_roofline(w: wl.Workload, stage: str, ms: float, hbm, tens, sm_mhz):
         byts = float(B) * N * 4
         return dict(bound="hbm", achieved=byts / (ms * 1e-3) / 1e9, peak=hbm, unit="GB/s",
                     per_launch=byts,
-                    kernel="warp_topk_kernel" if w.k <= 32 else "segment_topk_kernel")
+                    kernel="topk_kernel")
     # the fit: Cholesky n^3/3 + triangular inverse n^3/3 flops per (problem,
     # objective) in fp32 on the CUDA cores, against the whole GPU's FP32 FMA
     # peak at the clock measured during the run
     flops = float(B) * m * 2 * n ** 3 / 3
     peak = NUM_SMS * FMA_LANES_PER_SM * 2 * (sm_mhz or 2070.0) * 1e6 / 1e12
     return dict(bound="alu", achieved=flops / (ms * 1e-3) / 1e12, peak=peak, unit="TFLOP/s",
-                per_launch=flops, kernel="fit32_kernel")
+                per_launch=flops, kernel="fitc_kernel")
 
 
 def pass_roofline(w: wl.Workload, ms_pass: float, hbm, tens, tens_tf32):

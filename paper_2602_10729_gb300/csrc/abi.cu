@@ -571,8 +571,12 @@ void boute_engine_free(boute_engine *e) {
 }
 
 // Largest K* buffer an engine keeps (it lets the posterior's K* be computed
-// beside the fit); larger workloads build K* inside the posterior.
-constexpr size_t kKstarMaxBytes = size_t(512) << 20;
+// beside the fit); larger workloads build K* inside the posterior. The line is the
+// L2's size: beyond it K* goes to HBM and back, which takes longer than the fit it
+// hides behind (271 MB at n = 49, d = 15, m = 3: step 659 us, built inside 638; 307 MB
+// at n = 203, d = 7: 325 either way; 67 MB at n = 128, d = 12: posterior 26 us
+// against 54 built inside).
+constexpr size_t kKstarMaxBytes = size_t(128) << 20;
 
 // The selection runs inside the acquisition kernel for 2-objective
 // Monte-Carlo steps with k <= 32 (not in stage-timing mode, which times the

@@ -1110,10 +1110,11 @@ int launch_dp(const Gp *gp, const float *Xc, const float *kst, long long N, floa
   // the tensor cores through the groups where the MMAs outweigh the building
   // (measured best: 4 A + 2 B stages; n = 512, d = 16 with 3 + 3: 2251 against
   // 2210 us for 2^20 candidates. With in-sample draws, whose dense blocks make more B
-  // stages per A stage, 3 + 3: noisy step at n = 128 471 against 463 us),
+  // stages per A stage, and with staged K*, 3 + 3: noisy step at n = 128 471 against
+  // 463 us),
   // then the side input's ring as deep as what is left allows
   a.sx = kMaxX;
-  const bool dense = Layout<DP>::kBld == 16 && a.plan.S_in > 0;
+  const bool dense = Layout<DP>::kBld == 16 && (a.plan.S_in > 0 || kst);
   a.sa = dense ? 3 : 4;
   a.sb = dense ? 3 : 2;
   while ((size_t)a.sa * (kABytes + st) + (size_t)a.sb * a.b_bytes + (size_t)a.sx * a.x_bytes >
@@ -1166,7 +1167,6 @@ __global__ void __launch_bounds__(Layout<DP>::kBld * 32) kstar_kernel(
   const long long row = (long long)(tile % tiles_per_problem) * BOUTE_TILE_M + r;
   const int cf = xt_chunk_floats(DP);  // a multiple of 4
   const float4 *x4 = (const float4 *)(xt + (size_t)(b * m + t) * nxt * cf);
-  for (int e = threadIdx.x; e < nxt * cf / 4; e += blockDim.x) ((float4 *)xs)[e] = x4[e];
   const float *xrow = Xc + ((long long)b * N + row) * d, *xrow1 = xrow + (long long)RPT * d;
   float x0[DP], x1[DP];
 #pragma unroll
@@ -1174,6 +1174,7 @@ __global__ void __launch_bounds__(Layout<DP>::kBld * 32) kstar_kernel(
     x0[k] = (k < d && row < N) ? xrow[k] : 0.f;
     x1[k] = (k < d && row + RPT < N) ? xrow1[k] : 0.f;
   }
+  for (int e = threadIdx.x; e < nxt * cf / 4; e += blockDim.x) ((float4 *)xs)[e] = x4[e];
   __syncthreads();
   const float *il = xs + xt_param_offset(DP);
   float par[8];

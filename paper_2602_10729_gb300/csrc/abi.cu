@@ -95,7 +95,8 @@ struct boute_engine {
   bool fuse_sel;
   // K* of the candidates, computed on a second side stream while the fit
   // runs (it needs the fit's set-up, not its results); the posterior then
-  // only contracts it. Null when it would take more than kKstarMaxBytes.
+  // only contracts it. Null when it would take more than kKstarMaxBytes; unused while
+  // n is too large for the K* kernel (kstar_fits).
   float *kst;
   cudaStream_t side2;
   cudaEvent_t ev_setup, join2;
@@ -722,8 +723,9 @@ static int engine_run(boute_engine *e, const double *X, const double *Y, const d
     if ((r = launch_outcome_transform(Y, (long long)B * n * m, m, e->tcodes, e->Yt, s))) return r;
     Y = e->Yt;
   }
-  // K* beside the fit (not in serialised timing, where the posterior builds it)
-  const float *kst = serial ? nullptr : e->kst;
+  // K* beside the fit (not in serialised timing, where the posterior builds it, nor
+  // while the K* kernel cannot hold the side input of the engine's present n)
+  const float *kst = serial || !kstar_fits(&e->gp->g) ? nullptr : e->kst;
   // The graph has one root, the fit's set-up: the front stage (which needs
   // the raw outcomes only) and K* (which needs the set-up's side input) fork
   // after it and run beside the fit (one root launches sooner than two).

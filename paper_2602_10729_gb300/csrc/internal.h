@@ -154,6 +154,9 @@ constexpr size_t kKstarChunkHalves = 2 * BOUTE_TILE_M * BOUTE_ACHUNK;
 // row's 2^e_r): kstar_floats(gp, N) 4-byte words. Reads the fit set-up's side
 // input (not the fit's results) and the candidates.
 size_t kstar_floats(const Gp *gp, long long N);
+// Whether the K* kernel can run: the side input of all n observations fits a block's
+// shared memory (with n it grows past it at n = 833 for d > 28, n = 1601 for d = 16).
+bool kstar_fits(const Gp *gp);
 int launch_kstar(const Gp *gp, const float *Xc, long long N, float *kst, cudaStream_t s);
 int launch_pareto(const double *Ys, int B, int n, int m, const double *ref, unsigned char *mask,
                   double *front, int *P, cudaStream_t s);

@@ -1215,11 +1215,16 @@ __global__ void __launch_bounds__(Layout<DP>::kBld * 32) kstar_kernel(
   }
 }
 
+// The side input that a block of kstar_kernel stages.
+size_t kstar_smem(const Gp *gp) {
+  return (size_t)gp->plan.nxt * xt_chunk_floats(gp->DP) * sizeof(float);
+}
+
 template <int DP>
 int launch_kstar_dp(const Gp *gp, const float *Xc, long long N, float *kst, cudaStream_t s) {
   const int tpp = (int)((N + BOUTE_TILE_M - 1) / BOUTE_TILE_M);
   const int units = tpp * gp->B * gp->m;
-  const size_t smem = (size_t)gp->plan.nxt * xt_chunk_floats(DP) * sizeof(float);
+  const size_t smem = kstar_smem(gp);
   auto go = [&](auto kern) {
     prefer_shared(kern);
     // (set on every launch: the kernel's static array counts against the same
@@ -1268,6 +1273,9 @@ size_t kstar_floats(const Gp *gp, long long N) {
   const size_t tpp = (size_t)((N + BOUTE_TILE_M - 1) / BOUTE_TILE_M);
   return tpp * gp->B * gp->m * gp->plan.nchunk * (kStageBytes / 4);
 }
+
+// (beside the kernel's static word and its alignment)
+bool kstar_fits(const Gp *gp) { return kstar_smem(gp) <= 227 * 1024 - 16; }
 
 int launch_kstar(const Gp *gp, const float *Xc, long long N, float *kst, cudaStream_t s) {
   if (N <= 0) return BOUTE_OK;

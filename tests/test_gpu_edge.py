@@ -70,6 +70,29 @@ def test_training_set_sizes_and_column_passes(n):
     compare(rand_problem(2, n, 5, 2, 400))
 
 
+def check_posterior_at(hp, at, mean_g, var_g):
+    """Problem 0's means and variances (m x N) at the candidates `at`: POST_REL of the
+    prior's scale. The composite kernel's means are never recomputed, so they get in
+    addition what rounding K* (a few units in the last place of each value, 16 allowed
+    for its exponents) leaves of the terms K*_j alpha_j."""
+    fp = oracle_fit(hp, 0)
+    mean, var = opl.posterior(fp, hp.Xc[0][at])
+    for t in range(hp.w.m):
+        g = mean_g[t, at].astype(np.float64)
+        if hp.kc is None:
+            check_mean(g, mean[:, t], fp.s2[t])
+            check_var(var_g[t, at], var[:, t], fp.s2[t])
+            continue
+        kern, x = (hp.d_tau, hp.kc[0][t]), hp.Xc[0][at].astype(np.float64)
+        args = (hp.ls[0][t], hp.s2[0][t], kern)
+        prior = max(oracle.kernel(c, c, *args) for c in x)
+        terms = [sum(oracle.kernel(c, r, *args) * abs(a) for r, a in zip(hp.X[0], fp.alpha[t]))
+                 for c in x]
+        bound = 16 * 2.0 ** -23 * np.array(terms) + POST_REL * np.sqrt(prior)
+        assert np.all(np.isfinite(g)) and np.all(np.abs(g - mean[:, t]) <= bound)
+        check_var(var_g[t, at], var[:, t], prior)
+
+
 @pytest.mark.parametrize("n,d,comp", [(520, 32, True), (640, 32, True), (640, 16, True),
                                       (640, 24, False), (777, 32, False), (640, 10, False),
                                       (900, 20, True), (1090, 12, False)])
@@ -148,6 +171,44 @@ def test_kstar_side_input_near_48kb(n):
     for tt in range(w.m):
         check_mean(mean[0, tt].cpu().numpy(), mo[:, tt], fp.s2[tt])
         check_var(var[0, tt].cpu().numpy(), vo[:, tt], fp.s2[tt])
+
+
+# The K* kernel stages the whole side input, which passes a block's shared memory from
+# n = 833 at 29 .. 32 dimensions, 961 at 25 .. 28, 1089 at 21 .. 24 and 1601 at 15 or 16
+# on: an engine then builds K* inside the posterior, also with so few candidates that
+# its buffer is small. Both sides of the lines; then fewer observations in the same engine.
+@pytest.mark.parametrize("n,d,comp", [(832, 32, False), (833, 32, False), (1000, 28, False),
+                                      (960, 25, True), (961, 25, True), (1024, 32, True),
+                                      (1088, 24, False), (1089, 24, False), (1601, 16, False)])
+def test_engine_where_the_side_input_passes_shared_memory(n, d, comp):
+    import dataclasses
+
+    import torch
+
+    from paper_2602_10729_gb300 import boute as bt
+    base = wl.scaled(dataclasses.replace(wl.WORKLOADS[2], d=d), N=300, n=n)
+    w = wl.composite(base) if comp else base
+    hp = host_problem(w)
+    t = lambda a, dt=torch.float64: torch.as_tensor(np.ascontiguousarray(a), dtype=dt, device="cuda")
+    e = bt.Engine(1, n, d, w.m, w.N, bt.BOUTE_ACQ_EHVI2D, 0, w.k)
+    if comp:
+        bt.boute_engine_set_kernel(e, hp.d_tau, hp.kc)
+        bt.boute_engine_set_outcome_transforms(e, list(hp.transforms))
+    idx = torch.empty((1, w.k), dtype=torch.int64, device="cuda")
+    val = torch.empty((1, w.k), dtype=torch.float32, device="cuda")
+    mean = torch.empty((1, w.m, w.N), dtype=torch.float32, device="cuda")
+    var = torch.empty_like(mean)
+    at = np.arange(0, 300, 7)
+    for rows in (n, 65):
+        if rows < n:
+            bt.boute_engine_set_n(e, rows)
+            hp.X, hp.Y = hp.X[:, :rows], hp.Y[:, :rows]
+        bt.boute_engine_step(e, t(hp.X), t(hp.Y), t(hp.ls), t(hp.s2), t(hp.noise), t(hp.ref),
+                             t(hp.Xc, torch.float32), None, idx, val)
+        bt.boute_engine_scores(e, None, mean, var)
+        torch.cuda.synchronize()
+        check_posterior_at(hp, at, mean[0].cpu().numpy(), var[0].cpu().numpy())
+    e.free()
 
 
 def test_ill_conditioned_problem_meets_fp32_error_bound():

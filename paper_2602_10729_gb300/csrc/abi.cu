@@ -55,6 +55,13 @@ static int dalloc(T **p, size_t count) {
   return BOUTE_OK;
 }
 
+// Waits for what a call queued on the legacy default stream (clears, copies from pageable
+// memory, which may still be on their way when the copy returns): the caller's next call
+// may be on a non-blocking stream, which nothing orders against that one.
+static int default_stream_done() {
+  return cudaStreamSynchronize(nullptr) == cudaSuccess ? BOUTE_OK : last_launch_status();
+}
+
 // The builders' distances run over the padded dimensions: even up to 16, multiples of 4
 // above (BOUTE_PADDED_DIMS; a copied chunk of the side input is a multiple of 16 bytes for
 // every even count). d = 10 padded to 12, 64 problems of n = 256 and 2^18 candidates each:
@@ -243,6 +250,10 @@ int boute_gp_create(int B, int n, int d, int m, boute_gp **out) {
   // padding never holds stale bits
   cudaMemset(g.bop, 0, BM * (size_t)g.plan.image_halves * sizeof(uint16_t));
   cudaMemset(g.xt, 0, BM * (size_t)g.plan.nxt * xt_chunk_floats(g.DP) * sizeof(float));
+  if ((r = default_stream_done()) != BOUTE_OK) {
+    boute_gp_free(h);
+    return r;
+  }
   *out = h;
   return BOUTE_OK;
 }
@@ -321,7 +332,8 @@ int boute_gp_set_insample(boute_gp *gp, int S) {
     cudaFree(iws);
     return BOUTE_ERR_OOM;
   }
-  if (cudaMemset(bop, 0, BM * (size_t)cap.image_halves * sizeof(uint16_t)) != cudaSuccess) {
+  if (cudaMemset(bop, 0, BM * (size_t)cap.image_halves * sizeof(uint16_t)) != cudaSuccess ||
+      default_stream_done() != BOUTE_OK) {
     cudaGetLastError();
     cudaFree(bop);
     cudaFree(gws);
@@ -392,11 +404,16 @@ int boute_acq_nehvi2d(const float *mean, const float *cvar, const float *shift, 
 int boute_gp_status(boute_gp *gp, void *stream) {
   BOUTE_TRACE();
   if (!gp) return BOUTE_ERR_INVALID_ARG;
-  if (cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) return last_launch_status();
+  // on the caller's stream alone: on the default stream the copy would wait for all other
+  // work there, and the clear would not be ordered against the next call
+  const cudaStream_t s = (cudaStream_t)stream;
   int st = 0;
-  if (cudaMemcpy(&st, gp->g.status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+  if (cudaMemcpyAsync(&st, gp->g.status, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
     return last_launch_status();
-  cudaMemset(gp->g.status, 0, sizeof(int));
+  if (st && (cudaMemsetAsync(gp->g.status, 0, sizeof(int), s) != cudaSuccess ||
+             cudaStreamSynchronize(s) != cudaSuccess))
+    return last_launch_status();
   return st;
 }
 
@@ -464,6 +481,7 @@ int boute_gp_set_kernel(boute_gp *gp, int d_tau, const double *params) {
   if (cudaMemcpy(g.kpar, h.data(), h.size() * sizeof(double), cudaMemcpyHostToDevice) !=
       cudaSuccess)
     return last_launch_status();
+  if (int r = default_stream_done()) return r;
   g.kern = 1;
   g.dtau = d_tau;
   return BOUTE_OK;
@@ -673,6 +691,7 @@ int boute_engine_create(int B, int n, int d, int m, long long N, int mode, int S
       cudaGetLastError();
       r = BOUTE_ERR_CUDA;
     }
+  if (r == BOUTE_OK) r = default_stream_done();  // (the in-sample normals, the clears)
   if (r != BOUTE_OK) {
     boute_engine_free(e);
     return BOUTE_ERR_OOM;
@@ -875,6 +894,7 @@ static void engine_reset_counters(boute_engine *e) {
   cudaDeviceSynchronize();
   cudaGetLastError();
   if (e->sel) cudaMemset(e->sel, 0, e->sel_bytes);
+  default_stream_done();
   cudaGetLastError();
 }
 
@@ -1067,7 +1087,7 @@ static int gp_set_n(Gp &g, int n) {
     cudaGetLastError();
     return BOUTE_ERR_CUDA;
   }
-  return BOUTE_OK;
+  return default_stream_done();
 }
 
 int boute_engine_optimize(boute_engine *e, const float *eps, int S, const float *X0, int P,
@@ -1106,7 +1126,7 @@ int boute_engine_set_n(boute_engine *e, int n) {
         return BOUTE_ERR_OOM;
       }
       e->sel_bytes = bytes;
-      if (cudaMemset(e->sel, 0, bytes) != cudaSuccess) {
+      if (cudaMemset(e->sel, 0, bytes) != cudaSuccess || default_stream_done() != BOUTE_OK) {
         cudaGetLastError();
         return BOUTE_ERR_CUDA;
       }
@@ -1228,6 +1248,7 @@ int boute_engine_set_constraints(boute_engine *e, const double *cons) {
     if (!e->cons && dalloc(&e->cons, count) != BOUTE_OK) return BOUTE_ERR_OOM;
     if (cudaMemcpy(e->cons, cons, count * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
       return last_launch_status();
+    if (int r = default_stream_done()) return r;
   }
   const int on = cons != nullptr;
   if (on != e->has_cons) {  // the step's acquisition kernel changes: recapture

@@ -515,3 +515,51 @@ def test_ehvi_over_the_normal_tail():
                       1, t(ref[None]), acq)
     want = oracle.ehvi2d(mean[0].T.astype(np.float64), var[0].T.astype(np.float64), F, ref)
     np.testing.assert_allclose(acq.cpu().numpy()[0], want, rtol=2e-5, atol=1e-36)
+
+
+def test_status_and_new_handles_beside_a_busy_default_stream():
+    """Steps on a stream of their own while something else holds the default stream: a
+    status is read and cleared without waiting for it, and a new handle's buffers are
+    cleared before they are used, not when the default stream comes to it."""
+    import time
+
+    import torch
+
+    from paper_2602_10729_gb300 import boute as bt
+    hp = rand_problem(21, 70, 5, 2, 300)
+    t = lambda a, dt=torch.float64: torch.as_tensor(np.ascontiguousarray(a), dtype=dt, device="cuda")
+    X, ls, s2, nz, Xc = t(hp.X), t(hp.ls), t(hp.s2), t(hp.noise), t(hp.Xc, torch.float32)
+    Ys = torch.empty_like(t(hp.Y))
+    bt.boute_standardize(t(hp.Y), Ys)
+    flat = torch.zeros_like(X)  # equal points, no noise: not positive definite
+    mean = torch.empty((1, 2, 300), dtype=torch.float32, device="cuda")
+    var = torch.empty_like(mean)
+    s = torch.cuda.Stream()
+    torch.cuda._sleep(1000)
+    torch.cuda.synchronize()
+    busy = int(1.2e9)  # clocks: half a second or more
+    torch.cuda._sleep(busy)
+    gp = bt.boute_gp_create(1, 70, 5, 2)
+    with torch.cuda.stream(s):
+        bt.boute_gp_fit(gp, X, Ys, ls, s2, nz)
+    torch.cuda.synchronize()
+    bt.boute_gp_posterior(gp, Xc, 300, mean, var)
+    torch.cuda.synchronize()
+    fp = oracle_fit(hp, 0)
+    mo, vo = opl.posterior(fp, hp.Xc[0])
+    for k in range(2):
+        check_mean(mean[0, k].cpu().numpy(), mo[:, k], fp.s2[k])
+        check_var(var[0, k].cpu().numpy(), vo[:, k], fp.s2[k])
+    torch.cuda._sleep(busy)
+    t0 = time.monotonic()
+    with torch.cuda.stream(s):
+        bt.boute_gp_fit(gp, flat, Ys, ls, s2, torch.zeros_like(nz))
+        assert bt.boute_gp_status(gp) == bt.BOUTE_ERR_NOT_PD
+        assert bt.boute_gp_status(gp) == bt.BOUTE_OK
+        bt.boute_gp_fit(gp, flat, Ys, ls, s2, torch.zeros_like(nz))
+        s.synchronize()
+        assert bt.boute_gp_status(gp) == bt.BOUTE_ERR_NOT_PD
+    waited = time.monotonic() - t0
+    torch.cuda.synchronize()
+    assert waited < 0.25
+    gp.free()

@@ -757,19 +757,24 @@ static size_t fitc_smem(int npad, int C, bool tiles) {
 }
 constexpr size_t kFcMaxSmem = 227 * 1024 - 5 * 1024;  // (its static part: 4.9 KB)
 
-// Clusters of the largest size with which every problem-objective runs at once, no
-// more CTAs than block rows (n = 32 on one CTA 28 us, on two 30; n = 128 on four 50, on
+// Clusters of the largest size of which the device holds one per problem-objective at
+// once (a cluster lies within a GPC, so of 152 SMs clusters of 16 reach 112, of 8 120 and
+// of 4 144: the held clusters are asked for, not the SMs divided. n = 512, 16
+// problem-objectives: 535 us on clusters of 4, 655 in two waves of 8; n = 256: 154
+// against 215; n = 128, 38 of them: 93 on clusters of 2, 122 in two waves of 4), no more
+// CTAs than block rows (n = 32 on one CTA 28 us, on two 30; n = 128 on four 50, on
 // eight 53; n = 203 on four 101, on eight 98), and enough that the operands, and if any
 // size allows it the tiles, fit shared memory (n = 256 on single CTAs, n = 1024 on 16;
 // above that the tiles stay in the workspace).
 static int launch_fitc(Gp *gp, const double *Ys, int standardize, cudaStream_t s) {
   const int n = gp->n, m = gp->m, npad = gp->plan.npad, nb = npad / 32;
   const long long BM = (long long)gp->B * m, sms = num_sms();
-  int C = 1;
-  while (C < kFcMaxCluster &&
-         (fitc_smem(npad, C, true) > kFcMaxSmem || (2 * C * BM <= sms && C < nb)))
-    C *= 2;
-  auto go = [&](auto kern, bool tiles) {
+  int least = 1;
+  while (least < kFcMaxCluster && fitc_smem(npad, least, true) > kFcMaxSmem) least *= 2;
+  int C = least;
+  while (C < kFcMaxCluster && C < nb && 2 * C * BM <= sms) C *= 2;
+  // launches unless the device cannot hold `want` clusters of C
+  auto go = [&](auto kern, bool tiles, long long want) {
     prefer_shared(kern);
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFcMaxSmem);
     if (C > 8) cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -786,8 +791,8 @@ static int launch_fitc(Gp *gp, const double *Ys, int standardize, cudaStream_t s
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    int fit = 0;
-    if (C > 1 && (cudaOccupancyMaxActiveClusters(&fit, kern, &cfg) != cudaSuccess || fit == 0)) {
+    int held = 0;
+    if (C > 1 && (cudaOccupancyMaxActiveClusters(&held, kern, &cfg) != cudaSuccess || held < want)) {
       cudaGetLastError();
       return false;
     }
@@ -797,10 +802,11 @@ static int launch_fitc(Gp *gp, const double *Ys, int standardize, cudaStream_t s
                        gp->bop, gp->kern, gp->status, gp->fbad);
     return true;
   };
-  // (a partitioned device may not place the larger clusters)
+  // (below `least`: a partitioned device may not place the larger clusters)
   for (;; C /= 2) {
     const bool tiles = fitc_smem(npad, C, true) <= kFcMaxSmem;
-    if (tiles ? go(fitc_kernel<true>, true) : go(fitc_kernel<false>, false)) break;
+    const long long want = C > least ? BM : 1;
+    if (tiles ? go(fitc_kernel<true>, true, want) : go(fitc_kernel<false>, false, want)) break;
     if (C == 1 || fitc_smem(npad, C / 2, false) > kFcMaxSmem) return BOUTE_ERR_CUDA;
   }
   count_launch(2);

@@ -563,3 +563,39 @@ def test_status_and_new_handles_beside_a_busy_default_stream():
     torch.cuda.synchronize()
     assert waited < 0.25
     gp.free()
+
+
+def _median_us(f, reps=15):
+    import torch
+    for _ in range(3):
+        f()
+    out = []
+    for _ in range(reps):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        f()
+        b.record()
+        torch.cuda.synchronize()
+        out.append(a.elapsed_time(b) * 1e3)
+    return float(np.median(out))
+
+
+@pytest.mark.parametrize("n", [256, 512])
+def test_fit_of_problem_objectives_beyond_the_held_clusters(n):
+    """15 clusters of 8 fit the device, though 16 of them have no more CTAs than it has
+    SMs: 16 problem-objectives take smaller clusters at once, not a second wave (which
+    costs half as much again or more; the smaller clusters a quarter)."""
+    import torch
+
+    from paper_2602_10729_gb300 import boute as bt
+    us = []
+    for B in (7, 8):
+        hp = host_problem(wl.scaled(wl.WORKLOADS[4], N=1, B=B, n=n))
+        t = lambda a: torch.as_tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")
+        args = [t(a) for a in (hp.X, hp.Y, hp.ls, hp.s2, hp.noise)]
+        bt.boute_standardize(args[1], args[1])
+        gp = bt.boute_gp_create(B, n, hp.w.d, 2)
+        us.append(_median_us(lambda: bt.boute_gp_fit(gp, *args)))
+        assert bt.boute_gp_status(gp) == 0
+        gp.free()
+    assert us[1] < 1.35 * us[0], us

@@ -488,36 +488,41 @@ int launch_learn(const double *X, const double *Ys, int B, int n, int d, int m,
     cudaGetLastError();
     return BOUTE_ERR_OOM;
   }
-  // the largest cluster with which every restart still runs at once, and no
-  // more CTAs than the triangle has tiles
+  // the largest cluster of which the device holds one per restart at once, an SM to each
+  // CTA (clusters lie within a GPC, so fewer fit than SMs / C: 7 of 16 CTAs; 8 restarts
+  // at n = 128 took 3.39 ms for 10 Adam steps on clusters of 16, 2.23 on clusters of 8), and
+  // no more CTAs than the power of two that covers the triangle's tiles (n = 20, 3 tiles,
+  // 20 steps: 1.06 ms on four CTAs, 1.36 on two; n = 48, 6 tiles: 1.37 on eight, 1.71 on four)
   const int nb = learn_tiles(n), nt = nb * (nb + 1) / 2;
   const long long sms = num_sms();
   int C = kMaxCluster;
-  while (C > 1 && (C * (long long)blocks > sms || C > nt)) C /= 2;
+  while (C > 1 && (C * (long long)blocks > sms || C / 2 >= nt)) C /= 2;
   const size_t smem = (size_t)(d + 5) * kLearnWork * sizeof(double);
   int st = BOUTE_OK;
   auto go = [&](auto kern) {
     prefer_shared(kern);
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr size_t kAlone = 120 * 1024;  // more than half an SM's shared memory
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAlone);
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.blockDim = dim3(kLearnThreads);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = kAlone;
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (C > 8)
       cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    for (;; C /= 2) {  // (a partitioned device may not place the larger clusters)
+    for (;; C /= 2) {
       attr[0].val.clusterDim.x = C;
       cfg.gridDim = dim3((unsigned)(blocks * C));
-      int fit = 0;
-      if (C == 1 || (cudaOccupancyMaxActiveClusters(&fit, kern, &cfg) == cudaSuccess && fit > 0))
+      int held = 0;
+      if (C == 1 || (cudaOccupancyMaxActiveClusters(&held, kern, &cfg) == cudaSuccess && held >= blocks))
         break;
       cudaGetLastError();
     }
+    cfg.dynamicSmemBytes = smem;
     cudaLaunchKernelEx(&cfg, kern, X, Ys, n, d, m, R, C, theta0, iters, lr, theta, mll, grad, ws,
                        dtau, pref);
   };

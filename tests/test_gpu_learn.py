@@ -158,3 +158,35 @@ def test_composite_likelihood_gradient_and_trajectory_match_oracle(wi, n, R):
                                       kernel=(dtau, pref[0, t]))
         np.testing.assert_allclose(theta[0, t], th_o, rtol=0, atol=1e-7)
         np.testing.assert_allclose(mll[0, t], mll_o, rtol=1e-9, atol=1e-8)
+
+
+def _median_ms(n, R, iters):
+    import torch
+
+    from paper_2602_10729_gb300 import boute as bt
+    _, X, Ys, theta0 = _problem(1, 1, n, R)
+    t = lambda a: torch.as_tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")
+    X, Ys, th0 = t(X), t(Ys), t(theta0)
+    theta, grad = torch.empty_like(th0), torch.empty_like(th0)
+    mll = torch.empty(theta0.shape[:3], dtype=torch.float64, device="cuda")
+    out = []
+    for _ in range(9):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        bt.boute_gp_learn(X, Ys, th0, iters, 0.05, theta, mll, grad)
+        b.record()
+        torch.cuda.synchronize()
+        out.append(a.elapsed_time(b))
+    return float(np.median(out[2:]))
+
+
+def test_restarts_beyond_the_held_clusters_run_at_once():
+    """Seven clusters of 16 CTAs fit the device with an SM to each CTA: eight restarts
+    take smaller clusters, not a second wave or a shared SM (twice the time)."""
+    assert _median_ms(128, 4, 5) < 1.5 * _median_ms(128, 3, 5)
+
+
+def test_a_few_tiles_get_a_cta_each():
+    """n = 20 has three tiles of 16 where n = 16 has one: with a CTA each (a cluster of
+    four) a step takes 1.4 times as long, on two CTAs 1.8."""
+    assert _median_ms(20, 1, 20) < 1.6 * _median_ms(16, 1, 20)

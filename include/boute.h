@@ -148,9 +148,10 @@ int boute_gp_set_kernel(boute_gp *gp, int d_tau, const double *params);
  *   optional, same layout as theta): the gradient at the final theta.
  *   All device pointers; iters >= 0 (0: evaluate at theta0); R >= 1.
  * A restart whose K is not positive definite stops there: its theta is kept
- * and its mll (and grad) are NaN. One cluster of up to 16 blocks per (b, t, r);
- * its workspace (about 16 n^2 bytes) is stream-ordered pool memory.
- * Asynchronous on `stream`. */
+ * and its mll (and grad) are NaN. One cluster of up to 16 blocks per (b, t, r),
+ * each with a workspace (about 16 n^2 bytes) of stream-ordered pool memory, of
+ * which 1 GiB or one for every SM are taken at most: more restarts than that
+ * run in further launches. Asynchronous on `stream`. */
 #define BOUTE_LOG_LS_MIN (-6.907755278982137)    /* log 1e-3 */
 #define BOUTE_LOG_LS_MAX (6.907755278982137)     /* log 1e3 */
 #define BOUTE_LOG_S2_MIN (-6.907755278982137)    /* log 1e-3 */

@@ -188,8 +188,8 @@ int launch_mchvi(const float *mean, const float *var, int B, long long N, int m,
                  const float *lower, const float *upper, const int *K, int box_cap,
                  const float *eps, int S, long long eps_stride, const double *cons, float *acq,
                  cudaStream_t s);
-// hyperparameter learning (learn.cu): B*m*R blocks, fp64; workspace from the
-// stream-ordered pool when a block's does not fit in shared memory
+// hyperparameter learning (learn.cu), fp64: a cluster per restart, with a bounded number of
+// workspaces from the stream-ordered pool
 // dtau, pref: the composite kernel's routing features and preference entries
 // (B x m x (d - dtau)); pref null: the Matern-5/2 kernel
 int launch_learn(const double *X, const double *Ys, int B, int n, int d, int m,

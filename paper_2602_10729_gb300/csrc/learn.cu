@@ -28,6 +28,8 @@
 // matrix in shared memory and a barrier per column took 26.3 ms).
 #include <math.h>
 
+#include <algorithm>
+
 #include "internal.h"
 
 namespace boute {
@@ -40,6 +42,7 @@ constexpr int kLearnWork = kTE;       // worker threads
 constexpr int kLearnThreads = kTE + 32;  // and one warp for the pivots' reciprocals
 constexpr int kTS = kT + 1;           // row stride of a tile in shared memory
 constexpr int kMaxCluster = 16;
+constexpr size_t kLearnWsBytes = size_t(1) << 30;  // of workspaces (see launch_learn)
 constexpr double kSqrt5d = 2.23606797749978969641;
 constexpr double kSqrt3d = 1.73205080756887729353;
 constexpr double kLog2Pi = 1.83787706640934548356;
@@ -121,9 +124,9 @@ __device__ __forceinline__ void reduce_rows(const double *part, int P, double *o
 
 template <bool COMP>
 __global__ void __launch_bounds__(kLearnThreads, 1) learn_kernel(
-    const double *X, const double *Ys, int n, int d, int m, int R, int C, const double *theta0,
-    int iters, double lr, double *theta_out, double *mll_out, double *grad_out, double *ws,
-    int dtau, const double *pref) {
+    const double *X, const double *Ys, int n, int d, int m, int R, int blk0, int C,
+    const double *theta0, int iters, double lr, double *theta_out, double *mll_out,
+    double *grad_out, double *ws, int dtau, const double *pref) {
   extern __shared__ __align__(16) double part[];  // P x kLearnWork gradient terms
   __shared__ double th[kMaxP], m1[kMaxP], m2[kMaxP], gr[kMaxP];
   __shared__ double il[kMaxP];  // 1 / l_q, then the scales
@@ -133,11 +136,11 @@ __global__ void __launch_bounds__(kLearnThreads, 1) learn_kernel(
   __shared__ double inv_s;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rank = C > 1 ? cluster_rank() : 0;
-  const int blk = blockIdx.x / C, bt = blk / R, b = bt / m, t = bt % m;
+  const int slot = blockIdx.x / C, blk = blk0 + slot, bt = blk / R, b = bt / m, t = bt % m;
   const int P = d + (COMP ? 5 : 2), dc = d - dtau, nb = learn_tiles(n), nt = nb * (nb + 1) / 2;
   const bool work = tid < kLearnWork;
   const int r = tid / kT & (kT - 1), c = tid % kT;  // this thread's entry of a tile
-  double *KT = ws + (size_t)blk * learn_ws_doubles(n), *WT = KT + (size_t)nt * kTE;
+  double *KT = ws + (size_t)slot * learn_ws_doubles(n), *WT = KT + (size_t)nt * kTE;
   double *E1 = WT + (size_t)nt * kTE, *E2 = E1 + (size_t)nt * kTE, *av = E2 + (size_t)nt * kTE;
   double *piv = av + (size_t)nb * kT, *gpart = piv + (size_t)nb * kT;
   volatile int *bad = (volatile int *)(gpart + (size_t)kMaxCluster * (BOUTE_MAX_D + 5));
@@ -481,13 +484,7 @@ __global__ void __launch_bounds__(kLearnThreads, 1) learn_kernel(
 int launch_learn(const double *X, const double *Ys, int B, int n, int d, int m,
                  const double *theta0, int R, int iters, double lr, double *theta, double *mll,
                  double *grad, int dtau, const double *pref, cudaStream_t s) {
-  const size_t per = learn_ws_doubles(n) * sizeof(double);
   const int blocks = B * m * R;
-  double *ws = nullptr;
-  if (cudaMallocAsync((void **)&ws, per * blocks, s) != cudaSuccess) {
-    cudaGetLastError();
-    return BOUTE_ERR_OOM;
-  }
   // the largest cluster of which the device holds one per restart at once, an SM to each
   // CTA (clusters lie within a GPC, so fewer fit than SMs / C: 7 of 16 CTAs; 8 restarts
   // at n = 128 took 3.39 ms for 10 Adam steps on clusters of 16, 2.23 on clusters of 8), and
@@ -498,6 +495,7 @@ int launch_learn(const double *X, const double *Ys, int B, int n, int d, int m,
   int C = kMaxCluster;
   while (C > 1 && (C * (long long)blocks > sms || C / 2 >= nt)) C /= 2;
   const size_t smem = (size_t)(d + 5) * kLearnWork * sizeof(double);
+  double *ws = nullptr;
   int st = BOUTE_OK;
   auto go = [&](auto kern) {
     prefer_shared(kern);
@@ -518,17 +516,34 @@ int launch_learn(const double *X, const double *Ys, int B, int n, int d, int m,
       attr[0].val.clusterDim.x = C;
       cfg.gridDim = dim3((unsigned)(blocks * C));
       int held = 0;
-      if (C == 1 || (cudaOccupancyMaxActiveClusters(&held, kern, &cfg) == cudaSuccess && held >= blocks))
+      if (C == 1 || (cudaOccupancyMaxActiveClusters(&held, kern, &cfg) == cudaSuccess &&
+                     held >= blocks))
         break;
       cudaGetLastError();
     }
     cfg.dynamicSmemBytes = smem;
-    cudaLaunchKernelEx(&cfg, kern, X, Ys, n, d, m, R, C, theta0, iters, lr, theta, mll, grad, ws,
-                       dtau, pref);
+    // Workspaces for what runs at once (a CTA's registers take an SM), or for as many rounds
+    // of that as kLearnWsBytes hold; further restarts follow in launches of their own that
+    // use the same ones, so that the memory does not grow with the restarts. (One launch
+    // whose clusters loop over their restarts cost 1 to 2 % at every size.)
+    const size_t per = learn_ws_doubles(n) * sizeof(double);
+    const long long rounds = std::max<long long>(1, (long long)(kLearnWsBytes / per) / sms);
+    const int wave = C > 1 ? blocks : (int)std::min<long long>(blocks, rounds * sms);
+    if (cudaMallocAsync((void **)&ws, per * wave, s) != cudaSuccess) {
+      cudaGetLastError();
+      st = BOUTE_ERR_OOM;
+      return;
+    }
+    for (int blk0 = 0; blk0 < blocks; blk0 += wave) {
+      cfg.gridDim = dim3((unsigned)(std::min(wave, blocks - blk0) * C));
+      cudaLaunchKernelEx(&cfg, kern, X, Ys, n, d, m, R, blk0, C, theta0, iters, lr, theta, mll,
+                         grad, ws, dtau, pref);
+      count_launch();
+    }
   };
   if (pref) go(learn_kernel<true>);
   else go(learn_kernel<false>);
-  count_launch();
+  if (st) return st;
   st = last_launch_status();
   cudaFreeAsync(ws, s);
   return st;

@@ -190,3 +190,32 @@ def test_a_few_tiles_get_a_cta_each():
     """n = 20 has three tiles of 16 where n = 16 has one: with a CTA each (a cluster of
     four) a step takes 1.4 times as long, on two CTAs 1.8."""
     assert _median_ms(20, 1, 20) < 1.6 * _median_ms(16, 1, 20)
+
+
+def test_many_restarts_take_bounded_memory():
+    """20 000 restarts: workspaces for 1 GiB, used in turn, not one per restart (1.2 GB);
+    the restarts of every launch give what they give alone, also after one that fails."""
+    import ctypes
+
+    import torch
+
+    n, R = 32, 20000
+    _, X, Ys, theta0 = _problem(0, 1, n, 4)
+    theta0 = np.tile(theta0, (1, 1, R // 4, 1))
+    theta0[0, 0, 8888] = theta0[0, 1, 7777] = np.nan  # never positive definite
+    torch.zeros(1, device="cuda")
+    cu, pool, used = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(), ctypes.c_uint64(0)
+    USED_MEM_HIGH = 8
+    assert cu.cuDeviceGetDefaultMemPool(ctypes.byref(pool), torch.cuda.current_device()) == 0
+    assert cu.cuMemPoolSetAttribute(pool, USED_MEM_HIGH, ctypes.byref(used)) == 0
+    theta, mll, grad = _gpu(X, Ys, theta0, 2, 0.05)
+    assert cu.cuMemPoolGetAttribute(pool, USED_MEM_HIGH, ctypes.byref(used)) == 0
+    assert 0 < used.value <= 1 << 30
+    one = _gpu(X, Ys, theta0[:, :, :4], 2, 0.05)
+    assert np.isnan(mll[0, 0, 8888]) and np.isnan(mll[0, 1, 7777]) and np.isnan(mll).sum() == 2
+    for got, want in zip((theta, mll, grad), one):
+        got = got.reshape(2, R // 4, 4, -1)
+        got[0, 2222, 0], got[1, 1944, 1] = got[0, 0, 0], got[1, 0, 1]
+        # (clusters of four CTAs there, one CTA here: the gradient's sums in another order)
+        np.testing.assert_allclose(got, np.broadcast_to(want.reshape(2, 1, 4, -1), got.shape),
+                                   rtol=1e-9, atol=1e-9 * np.abs(want).max())

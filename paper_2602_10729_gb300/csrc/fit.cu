@@ -301,8 +301,8 @@ __device__ __forceinline__ void composite_wmax(float *xt, int bt, const PostPlan
 // eps32 times its original diagonal entry counts as not positive.
 // One cluster of C = Pr x Pc CTAs per problem-objective runs the whole fit after
 // the set-up in one launch: K's lower triangle as 32 x 32 tiles, tile (I, J) owned
-// by the CTA (I mod Pr, J mod Pc) and kept in its shared memory (in the workspace
-// Aws when it does not fit), updated in place:
+// by the CTA (I mod Pr, J mod Pc) and kept in its shared memory (n > 1024: below),
+// updated in place:
 //   before panel J it holds A_IJ (the trailing matrix), afterwards the transpose of
 //   R_IJ = -sum_{J <= K <= p} L_IK W_KJ, and W_IJ^T = (W_II R_IJ)^T from panel I on.
 // Panel p: two warps of the owner factor the diagonal tile and invert it (fc_diagonal)
@@ -362,7 +362,45 @@ __device__ __forceinline__ void fc_store1(uint32_t a, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
 }
 
-// TS: the tiles in shared memory.
+// Word offset of tile (I, J) among the lower triangle's, row by row, and the coordinates
+// of the e-th.
+__device__ __forceinline__ size_t tri_tile(int I, int J) {
+  return (size_t)(I * (I + 1) / 2 + J) * kFcTile;
+}
+__device__ __forceinline__ void tri_coords(int e, int &I, int &J) {
+  I = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);
+  while (I * (I + 1) / 2 > e) --I;
+  while ((I + 1) * (I + 2) / 2 <= e) ++I;
+  J = e - I * (I + 1) / 2;
+}
+
+// Rows r0 .. r0 + 7 of W_IJ, from the final tile T = W_IJ^T, by one warp: W itself and its
+// operand images (false if an element does not fit them).
+__device__ __forceinline__ bool fc_output(const float *T, int I, int J, int r0, int lane, int NP,
+                                          const PostPlan &plan, float wscale, float *W,
+                                          uint16_t *img) {
+  const int n = plan.n, gmax = BOUTE_BLKCOLS * (plan.nwblk - 1) + plan.ncol[plan.nwblk - 1];
+  bool fits = true;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int i = 32 * I + r0 + u, k = 32 * J + lane;
+    if (i < n && k <= i) W[(size_t)i * (NP + 1) + k] = T[fc_off(lane, r0 + u)];
+  }
+  const int kk = 2 * (lane & 15);
+#pragma unroll 1
+  for (int u = 0; u < 8; u += 2) {
+    const int r = r0 + u + (lane >> 4), g = 32 * I + r;
+    if (g >= gmax) continue;
+    fits &= pack_values(T[fc_off(kk, r)], T[fc_off(kk + 1, r)], g, 32 * J + kk, plan, wscale, img);
+    if (I == J)  // zeros right of the diagonal tile, as far as the block's chunks reach
+#pragma unroll 1
+      for (int k = 32 * (J + 1) + kk; k < BOUTE_ACHUNK * plan.kc[g / BOUTE_BLKCOLS]; k += 32)
+        pack_values(0.f, 0.f, g, k, plan, wscale, img);
+  }
+  return fits;
+}
+
+// TS: the tiles in shared memory; otherwise factored tiles in the workspace, alpha alone.
 template <bool TS>
 __global__ void __launch_bounds__(kFcThreads, 1) fitc_kernel(
     const float *Kh_all, const float *Kl_all, const double *Ys, int standardize, int n, int m,
@@ -385,8 +423,6 @@ __global__ void __launch_bounds__(kFcThreads, 1) fitc_kernel(
   float *wt = wpp + kFcTile, *dg = wt + 2 * kFcTile;
   unsigned short *slotI = (unsigned short *)(dg + 32 * nR), *slotJ = slotI + max_slots;
   float *tiles = TS ? dg + 32 * nR + ((max_slots + 3) & ~3) : Aws + (size_t)bt * NP * (NP + 1);
-  if (!TS)  // this CTA's share: the owners' tiles one after another
-    for (int r = 0; r < rank; ++r) tiles += (size_t)fc_slots(nb, r % Pr, r / Pr, Pr, Pc) * kFcTile;
   int *fbad = fbad_all + bt;
   auto sync = [&]() {
     __syncwarp();
@@ -400,193 +436,183 @@ __global__ void __launch_bounds__(kFcThreads, 1) fitc_kernel(
   // this CTA's block rows I = ra + Pr i, each with the columns J = rb + Pc j <= I
   const int lrows = ra < nb ? ((nb - 1 - ra) >> sr) + 1 : 0;
   auto row_count = [&](int I) { return I >= rb ? ((I - rb) >> sc) + 1 : 0; };
-  for (int i = tid; i <= lrows; i += kFcThreads) {
-    int q = 0;
-    for (int e = 0; e < i; ++e) q += row_count(ra + (e << sr));
-    row_first[i] = q;
-  }
-  __syncthreads();
-  const int nslots = row_first[lrows];
-  for (int i = warp; i < lrows; i += nw)
-    for (int j = lane; j < row_count(ra + (i << sr)); j += 32) {
-      slotI[row_first[i] + j] = (unsigned short)(ra + (i << sr));
-      slotJ[row_first[i] + j] = (unsigned short)(rb + (j << sc));
-    }
   const double *y = Ys + (size_t)b * n * m + t;
   if (warp == nw - 1) standardize_stats(y, n, m, standardize, lane, ymu, yisd);
   // everything below reads what the set-up kernel wrote
   pdl_wait();
   const float *Kh = Kh_all + (size_t)bt * n * n, *Kl = Kl_all + (size_t)bt * n * n;
-  if (rank == 0 && tid == 0) __stcg(fbad, 0);
-  for (int e = tid; e < 32 * lrows; e += kFcThreads) {
-    const int i = 32 * (ra + ((e >> 5) << sr)) + (e & 31);
-    dg[e] = i < n ? Kh[(size_t)i * n + i] : 1.f;
-  }
-  __syncthreads();
-  for (int e = warp; e < 4 * nslots; e += nw) {  // eight rows of a tile per warp
-    const int s = e >> 2, r0 = 8 * (e & 3), i0 = 32 * slotI[s] + r0, k = 32 * slotJ[s] + lane;
-    float v[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int i = i0 + u;
-      v[u] = (i < n && k < n) ? Kh[(size_t)i * n + k] : (i == k ? 1.f : 0.f);
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) tiles[(size_t)s * kFcTile + fc_off(r0 + u, lane)] = v[u];
-  }
-  __syncthreads();
-  auto at = [&](const float *q, int r) { return fc_remote(q, r); };
-  // W_pp and W_pp^T, from this CTA's wpp and wt, to the CTAs of block row and column p
-  auto send_diagonal = [&](int p) {
-    const int a = p & (Pr - 1), c = p & (Pc - 1), par = p & 1;
-    float4 v[4], w[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      v[u] = ((const float4 *)wpp)[gt + 64 * u];
-      w[u] = ((const float4 *)(wt + par * kFcTile))[gt + 64 * u];
-    }
-    for (int q = 0; q < Pr + Pc; ++q) {
-      const int r = q < Pr ? q + Pr * c : a + Pr * (q - Pr);
-      if (r == rank) continue;
-      const uint32_t dst = at(wpp, r) + 16 * gt, dwt = at(wt + par * kFcTile, r) + 16 * gt;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        fc_store4(dst + 1024 * u, v[u]);
-        if (q < Pr) fc_store4(dwt + 1024 * u, w[u]);
-      }
-    }
-  };
-  sync();  // every CTA of the cluster runs: its shared memory may be written
-  if (rank == 0 && grp == 0) {
-    fc_diagonal(tiles, dg, dsh, wpp, wt, fbad);
-    named_barrier_sync(1, 64);
-    send_diagonal(0);
-  }
-  float acc[4][4];
-  const int tx = gt & 7, ty = gt >> 3;
-  // block row p of W (final after panel p's products): W itself and its operand images
   const int cf = xt_chunk_floats(DP);
   float *x0 = xt + (size_t)bt * plan.nxt * cf;
-  const float wscale = exp2i((int)x0[xt_param_offset(DP) + 2 * DP + kParEW]);
-  const int gmax = BOUTE_BLKCOLS * (plan.nwblk - 1) + plan.ncol[plan.nwblk - 1];
-  uint16_t *img = bop + (size_t)bt * plan.image_halves;
-  float *W = Wws + (size_t)bt * NP * (NP + 1);
   bool fits = true;
-  auto output_row = [&](int p) {
-    const int f = row_first[(p - ra) >> sr], cnt = 4 * row_count(p);
-#pragma unroll 1
-    for (int e = warp; e < cnt; e += nw) {  // eight rows of a tile per warp
-      const int s = f + (e >> 2), r0 = 8 * (e & 3), J = slotJ[s];
-      const float *T = tiles + (size_t)s * kFcTile;
+  auto at = [&](const float *q, int r) { return fc_remote(q, r); };
+  if constexpr (TS) {
+    for (int i = tid; i <= lrows; i += kFcThreads) {
+      int q = 0;
+      for (int e = 0; e < i; ++e) q += row_count(ra + (e << sr));
+      row_first[i] = q;
+    }
+    __syncthreads();
+    const int nslots = row_first[lrows];
+    for (int i = warp; i < lrows; i += nw)
+      for (int j = lane; j < row_count(ra + (i << sr)); j += 32) {
+        slotI[row_first[i] + j] = (unsigned short)(ra + (i << sr));
+        slotJ[row_first[i] + j] = (unsigned short)(rb + (j << sc));
+      }
+    if (rank == 0 && tid == 0) __stcg(fbad, 0);
+    for (int e = tid; e < 32 * lrows; e += kFcThreads) {
+      const int i = 32 * (ra + ((e >> 5) << sr)) + (e & 31);
+      dg[e] = i < n ? Kh[(size_t)i * n + i] : 1.f;
+    }
+    __syncthreads();
+    for (int e = warp; e < 4 * nslots; e += nw) {  // eight rows of a tile per warp
+      const int s = e >> 2, r0 = 8 * (e & 3), i0 = 32 * slotI[s] + r0, k = 32 * slotJ[s] + lane;
+      float v[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        const int i = 32 * p + r0 + u, k = 32 * J + lane;
-        if (i < n && k <= i) W[(size_t)i * (NP + 1) + k] = T[fc_off(lane, r0 + u)];
+        const int i = i0 + u;
+        v[u] = (i < n && k < n) ? Kh[(size_t)i * n + k] : (i == k ? 1.f : 0.f);
       }
-      const int kk = 2 * (lane & 15);
-#pragma unroll 1
-      for (int u = 0; u < 8; u += 2) {
-        const int r = r0 + u + (lane >> 4), g = 32 * p + r;
-        if (g >= gmax) continue;
-        fits &= pack_values(T[fc_off(kk, r)], T[fc_off(kk + 1, r)], g, 32 * J + kk, plan, wscale, img);
-        if (p == J)  // zeros right of the diagonal tile, as far as the block's chunks reach
-#pragma unroll 1
-          for (int k = 32 * (J + 1) + kk; k < BOUTE_ACHUNK * plan.kc[g / BOUTE_BLKCOLS]; k += 32)
-            pack_values(0.f, 0.f, g, k, plan, wscale, img);
-      }
-    }
-    __syncwarp();
-  };
-  for (int p = 0; p < nb; ++p) {
-    sync();  // W_pp has arrived; the previous panel's operands are consumed
-    // L_Ip = A_Ip W_pp^T and W_pJ^T = R_pJ^T W_pp^T
-    const int i1 = p < ra ? 0 : ((p - ra) >> sr) + 1;  // first block row of this CTA below p
-    const int f1 = row_first[i1], a = p & (Pr - 1), c = p & (Pc - 1);
-    const int nl = rb == c ? lrows - i1 : 0;
-    const int nwt = ra == a ? row_count(p) - (rb == c ? 1 : 0) : 0;
-    if (tid == 0) next_item = f1;
-    for (int e = grp; e < nl + nwt; e += kFcGroups) {
-      int s, X;
-      if (e < nl) {
-        X = ra + ((i1 + e) << sr);
-        s = row_first[i1 + e] + ((p - rb) >> sc);
-      } else {
-        s = row_first[(p - ra) >> sr] + (e - nl);
-        X = rb + ((e - nl) << sc);
-      }
-      float *T = tiles + (size_t)s * kFcTile;
-      fc_product(T, wpp, gt, acc);
-      // to the column operands of CTAs (., X mod Pc) and, L_Ip, the row operands of
-      // CTAs (X mod Pr, .)
-      const int o = ((4 * ty) * 8 + (tx ^ ty)) * 16;
-      if (p < nb - 1)
-        for (int q = 0; q < (e < nl ? Pr + Pc : Pr); ++q) {
-          const uint32_t dst =
-              o + (q < Pr ? at(cop + (size_t)(X >> sc) * kFcTile, q + Pr * (X & (Pc - 1)))
-                          : at(rop + (size_t)(X >> sr) * kFcTile, (X & (Pr - 1)) + Pr * (q - Pr)));
 #pragma unroll
-          for (int u = 0; u < 4; ++u)
-            fc_store4(dst + 128 * u, make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]));
-        }
-      if (e >= nl) {
-        named_barrier_sync(1 + grp, 64);  // the tile is read
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          ((float4 *)T)[(4 * ty + u) * 8 + (tx ^ ty)] =
-              make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
-      }
+      for (int u = 0; u < 8; ++u) tiles[(size_t)s * kFcTile + fc_off(r0 + u, lane)] = v[u];
     }
-    if (p == nb - 1) break;
-    sync();  // L_Ip and W_pJ have arrived
-    // update: the slots from block row i1 on; the next diagonal tile first, by group 0
-    auto update = [&](int s) {
-      const int I = slotI[s], J = slotJ[s];
-      const float *L = rop + (size_t)(I >> sr) * kFcTile;
-      const float *Q = J == p ? wt + (p & 1) * kFcTile : cop + (size_t)(J >> sc) * kFcTile;
-      float *T = tiles + (size_t)s * kFcTile;
-      fc_product(J > p ? L : Q, J > p ? Q : L, gt, acc);
+    __syncthreads();
+    // W_pp and W_pp^T, from this CTA's wpp and wt, to the CTAs of block row and column p
+    auto send_diagonal = [&](int p) {
+      const int a = p & (Pr - 1), c = p & (Pc - 1), par = p & 1;
+      float4 v[4], w[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        float4 *q = (float4 *)T + (4 * ty + u) * 8 + (tx ^ ty);
-        float4 v = J == p ? make_float4(0.f, 0.f, 0.f, 0.f) : *q;
-        v.x -= acc[u][0];
-        v.y -= acc[u][1];
-        v.z -= acc[u][2];
-        v.w -= acc[u][3];
-        *q = v;
+        v[u] = ((const float4 *)wpp)[gt + 64 * u];
+        w[u] = ((const float4 *)(wt + par * kFcTile))[gt + 64 * u];
+      }
+      for (int q = 0; q < Pr + Pc; ++q) {
+        const int r = q < Pr ? q + Pr * c : a + Pr * (q - Pr);
+        if (r == rank) continue;
+        const uint32_t dst = at(wpp, r) + 16 * gt, dwt = at(wt + par * kFcTile, r) + 16 * gt;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          fc_store4(dst + 1024 * u, v[u]);
+          if (q < Pr) fc_store4(dwt + 1024 * u, w[u]);
+        }
       }
     };
-    const bool own = ((p + 1) & (Pr - 1)) == ra && ((p + 1) & (Pc - 1)) == rb;
-    if (own) {
-      // Beside the diagonal tile's two warps only the groups of the other two
-      // schedulers work (odd groups); the rest join them afterwards.
-      const int sd = row_first[i1] + ((p + 1) >> sc);  // the diagonal tile's slot
-      if (grp == 0) {
-        update(sd);
-        named_barrier_sync(1, 64);
-        fc_diagonal(tiles + (size_t)sd * kFcTile, dg + 32 * i1, dsh, wpp, wt + ((p + 1) & 1) * kFcTile,
-                    fbad);
-        named_barrier_sync(1, 64);
-        send_diagonal(p + 1);
-      }
-      if (!(grp & 1)) named_barrier_sync(13, 32 * nw / 2);
-      for (;;) {
-        if (gt == 0) item[grp] = atomicAdd(&next_item, 1);
-        __syncwarp();
-        named_barrier_sync(1 + grp, 64);
-        const int s = item[grp];
-        if (s >= nslots) break;
-        if (s != sd) update(s);
-        named_barrier_sync(1 + grp, 64);  // (item is read)
-      }
-    } else {
-      for (int s = f1 + grp; s < nslots; s += kFcGroups) update(s);
+    sync();  // every CTA of the cluster runs: its shared memory may be written
+    if (rank == 0 && grp == 0) {
+      fc_diagonal(tiles, dg, dsh, wpp, wt, fbad);
+      named_barrier_sync(1, 64);
+      send_diagonal(0);
     }
-    if (ra == a) output_row(p);
+    float acc[4][4];
+    const int tx = gt & 7, ty = gt >> 3;
+    // block row p of W (final after panel p's products): W itself and its operand images
+    const float wscale = exp2i((int)x0[xt_param_offset(DP) + 2 * DP + kParEW]);
+    uint16_t *img = bop + (size_t)bt * plan.image_halves;
+    float *W = Wws + (size_t)bt * NP * (NP + 1);
+    auto output_row = [&](int p) {
+      const int f = row_first[(p - ra) >> sr], cnt = 4 * row_count(p);
+#pragma unroll 1
+      for (int e = warp; e < cnt; e += nw) {  // eight rows of a tile per warp
+        const int s = f + (e >> 2);
+        fits &= fc_output(tiles + (size_t)s * kFcTile, p, slotJ[s], 8 * (e & 3), lane, NP, plan,
+                          wscale, W, img);
+      }
+      __syncwarp();
+    };
+    for (int p = 0; p < nb; ++p) {
+      sync();  // W_pp has arrived; the previous panel's operands are consumed
+      // L_Ip = A_Ip W_pp^T and W_pJ^T = R_pJ^T W_pp^T
+      const int i1 = p < ra ? 0 : ((p - ra) >> sr) + 1;  // first block row of this CTA below p
+      const int f1 = row_first[i1], a = p & (Pr - 1), c = p & (Pc - 1);
+      const int nl = rb == c ? lrows - i1 : 0;
+      const int nwt = ra == a ? row_count(p) - (rb == c ? 1 : 0) : 0;
+      if (tid == 0) next_item = f1;
+      for (int e = grp; e < nl + nwt; e += kFcGroups) {
+        int s, X;
+        if (e < nl) {
+          X = ra + ((i1 + e) << sr);
+          s = row_first[i1 + e] + ((p - rb) >> sc);
+        } else {
+          s = row_first[(p - ra) >> sr] + (e - nl);
+          X = rb + ((e - nl) << sc);
+        }
+        float *T = tiles + (size_t)s * kFcTile;
+        fc_product(T, wpp, gt, acc);
+        // to the column operands of CTAs (., X mod Pc) and, L_Ip, the row operands of
+        // CTAs (X mod Pr, .)
+        const int o = ((4 * ty) * 8 + (tx ^ ty)) * 16;
+        if (p < nb - 1)
+          for (int q = 0; q < (e < nl ? Pr + Pc : Pr); ++q) {
+            const uint32_t dst =
+                o + (q < Pr ? at(cop + (size_t)(X >> sc) * kFcTile, q + Pr * (X & (Pc - 1)))
+                            : at(rop + (size_t)(X >> sr) * kFcTile,
+                                 (X & (Pr - 1)) + Pr * (q - Pr)));
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              fc_store4(dst + 128 * u, make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]));
+          }
+        if (e >= nl) {
+          named_barrier_sync(1 + grp, 64);  // the tile is read
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            ((float4 *)T)[(4 * ty + u) * 8 + (tx ^ ty)] =
+                make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
+        }
+      }
+      if (p == nb - 1) break;
+      sync();  // L_Ip and W_pJ have arrived
+      // update: the slots from block row i1 on; the next diagonal tile first, by group 0
+      auto update = [&](int s) {
+        const int I = slotI[s], J = slotJ[s];
+        const float *L = rop + (size_t)(I >> sr) * kFcTile;
+        const float *Q = J == p ? wt + (p & 1) * kFcTile : cop + (size_t)(J >> sc) * kFcTile;
+        float *T = tiles + (size_t)s * kFcTile;
+        fc_product(J > p ? L : Q, J > p ? Q : L, gt, acc);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          float4 *q = (float4 *)T + (4 * ty + u) * 8 + (tx ^ ty);
+          float4 v = J == p ? make_float4(0.f, 0.f, 0.f, 0.f) : *q;
+          v.x -= acc[u][0];
+          v.y -= acc[u][1];
+          v.z -= acc[u][2];
+          v.w -= acc[u][3];
+          *q = v;
+        }
+      };
+      const bool own = ((p + 1) & (Pr - 1)) == ra && ((p + 1) & (Pc - 1)) == rb;
+      if (own) {
+        // Beside the diagonal tile's two warps only the groups of the other two
+        // schedulers work (odd groups); the rest join them afterwards.
+        const int sd = row_first[i1] + ((p + 1) >> sc);  // the diagonal tile's slot
+        if (grp == 0) {
+          update(sd);
+          named_barrier_sync(1, 64);
+          fc_diagonal(tiles + (size_t)sd * kFcTile, dg + 32 * i1, dsh, wpp,
+                      wt + ((p + 1) & 1) * kFcTile, fbad);
+          named_barrier_sync(1, 64);
+          send_diagonal(p + 1);
+        }
+        if (!(grp & 1)) named_barrier_sync(13, 32 * nw / 2);
+        for (;;) {
+          if (gt == 0) item[grp] = atomicAdd(&next_item, 1);
+          __syncwarp();
+          named_barrier_sync(1 + grp, 64);
+          const int s = item[grp];
+          if (s >= nslots) break;
+          if (s != sd) update(s);
+          named_barrier_sync(1 + grp, 64);  // (item is read)
+        }
+      } else {
+        for (int s = f1 + grp; s < nslots; s += kFcGroups) update(s);
+      }
+      if (ra == a) output_row(p);
+    }
+    pdl_trigger();
+    __syncthreads();
+    if (ra == ((nb - 1) & (Pr - 1))) output_row(nb - 1);
+  } else {  // (factored by the fitg_* kernels)
+    pdl_trigger();
+    sync();  // every CTA of the cluster runs: its shared memory may be written
   }
-  pdl_trigger();
-  __syncthreads();
-  if (ra == ((nb - 1) & (Pr - 1))) output_row(nb - 1);
   // ---- alpha0 = W^T (W y), refined twice against K = hi + lo ----------------------
   // (vectors in the operands' space: x, alpha, y hi, y lo, the partial sums of the CTA's
   // block rows and of every column, four classes of tiles each)
@@ -605,6 +631,11 @@ __global__ void __launch_bounds__(kFcThreads, 1) fitc_kernel(
   // tiles in ascending order, then the classes.
   const int kr = 4 / Pr, kcl = 4 / Pc;  // classes of block rows and columns in this CTA
   const int lcols = rb < nb ? ((nb - 1 - rb) >> sc) + 1 : 0;
+  // tile (row i, column j) of this CTA's; in the workspace the triangle's tiles in order
+  auto tile_at = [&](int i, int j) {
+    if (TS) return tiles + (size_t)(row_first[i] + j) * kFcTile;
+    return tiles + tri_tile(ra + (i << sr), rb + (j << sc));
+  };
   auto solve = [&](auto out) {
 #pragma unroll 1
     for (int e = warp; e < lrows * kcl; e += nw) {
@@ -612,7 +643,7 @@ __global__ void __launch_bounds__(kFcThreads, 1) fitc_kernel(
       float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
 #pragma unroll 1
       for (int J = q; J <= I; J += 4) {
-        const float *T = tiles + (size_t)(row_first[i] + (J >> sc)) * kFcTile, *xj = x + 32 * J;
+        const float *T = tile_at(i, J >> sc), *xj = x + 32 * J;
 #pragma unroll
         for (int k = 0; k < 32; k += 4) {
           s0 = fmaf(T[fc_off(k, lane)], xj[k], s0);
@@ -638,7 +669,7 @@ __global__ void __launch_bounds__(kFcThreads, 1) fitc_kernel(
       for (int I = q; I < nb; I += 4) {
         if (I < J) continue;
         const int i = (I - ra) >> sr;
-        const float4 *T4 = (const float4 *)(tiles + (size_t)(row_first[i] + j) * kFcTile) + lane * 8;
+        const float4 *T4 = (const float4 *)tile_at(i, j) + lane * 8;
         const float4 *v4 = (const float4 *)(pw + 32 * i);
 #pragma unroll
         for (int g = 0; g < 8; ++g) {
@@ -723,6 +754,129 @@ __global__ void __launch_bounds__(kFcThreads, 1) fitc_kernel(
   if (comp && rank == 0 && warp == nw - 1) composite_wmax(xt, bt, plan, DP, n, lane);
 }
 
+// ---- factorisation over the whole GPU -------------------------------------------------
+// More tiles than a cluster's shared memory holds (n > 1024): the same tiles, sums and
+// orders as above, the tiles in the workspace (the triangle's row by row, then L_Ip of the
+// present panel, then W_pp), 64 threads a tile product, two launches a panel over as many
+// blocks as there are products. What bounds it is the products' operands from L2 (16 KB
+// each), for small n the launches (about 6 us a panel). Fit with its set-up, against one
+// cluster per problem-objective, whose 16 SMs do all the products: n = 1025, m = 1 776 ->
+// 451 us; n = 1025, B = 8, m = 2 3178 -> 2311 us; n = 1536, m = 2 1854 -> 964 us; n = 2048,
+// m = 1 3211 -> 1079 us, m = 3 3800 -> 2231 us.
+
+// K's tiles; block 0 factors the first diagonal tile and clears fbad.
+__global__ void __launch_bounds__(64)
+    fitg_load_kernel(const float *Kh_all, int n, int NP, float *Aws, int *fbad_all) {
+  __shared__ __align__(16) float ts[kFcTile];
+  __shared__ __align__(16) FcDiag dsh;
+  __shared__ float dg[32];
+  pdl_wait();
+  pdl_trigger();
+  const int bt = blockIdx.y, tid = threadIdx.x, lane = tid & 31, nb = NP / 32;
+  const float *Kh = Kh_all + (size_t)bt * n * n;
+  float *tiles = Aws + (size_t)bt * NP * (NP + 1), *T = tiles + (size_t)blockIdx.x * kFcTile;
+  float *dst = blockIdx.x == 0 ? ts : T;
+  int I, J;
+  tri_coords(blockIdx.x, I, J);
+#pragma unroll 8
+  for (int r = tid >> 5; r < 32; r += 2) {
+    const int i = 32 * I + r, k = 32 * J + lane;
+    dst[fc_off(r, lane)] = (i < n && k < n) ? Kh[(size_t)i * n + k] : (i == k ? 1.f : 0.f);
+  }
+  if (blockIdx.x) return;
+  if (tid < 32) dg[tid] = tid < n ? Kh[(size_t)tid * n + tid] : 1.f;
+  if (tid == 0) fbad_all[bt] = 0;
+  __syncthreads();
+  fc_diagonal(ts, dg, dsh, tiles + tri_tile(nb + 1, 0) - kFcTile, T, fbad_all + bt);
+}
+
+__device__ __forceinline__ void fitg_copy(float *dst, const float *src, int tid) {
+#pragma unroll
+  for (int u = 0; u < 4; ++u) ((float4 *)dst)[tid + 64 * u] = ((const float4 *)src)[tid + 64 * u];
+}
+
+// Panel p: W_pJ^T (J < p) in place, L_Ip (I > p) beside the tiles.
+__global__ void __launch_bounds__(64) fitg_panel_kernel(int NP, float *Aws, int p) {
+  __shared__ __align__(16) float ts[kFcTile], ws[kFcTile];
+  pdl_wait();
+  pdl_trigger();
+  const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3, nb = NP / 32;
+  float *tiles = Aws + (size_t)blockIdx.y * NP * (NP + 1), *L = tiles + tri_tile(nb, 0);
+  const int X = (int)blockIdx.x < p ? blockIdx.x : blockIdx.x + 1;
+  float *T = tiles + (X > p ? tri_tile(X, p) : tri_tile(p, X));
+  fitg_copy(ts, T, tid);
+  fitg_copy(ws, L + (size_t)nb * kFcTile, tid);
+  __syncthreads();
+  float acc[4][4];
+  fc_product(ts, ws, tid, acc);
+  if (X > p) T = L + (size_t)X * kFcTile;
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+    ((float4 *)T)[(4 * ty + u) * 8 + (tx ^ ty)] =
+        make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
+}
+
+// The tiles of the block rows below panel p; block 0 the next diagonal tile, which it factors.
+__global__ void __launch_bounds__(64)
+    fitg_update_kernel(const float *Kh_all, int n, int NP, float *Aws, int p, int *fbad_all) {
+  __shared__ __align__(16) float ls[kFcTile], qs[kFcTile];
+  __shared__ __align__(16) FcDiag dsh;
+  __shared__ float dg[32];
+  pdl_wait();
+  pdl_trigger();
+  const int bt = blockIdx.y, tid = threadIdx.x, tx = tid & 7, ty = tid >> 3, nb = NP / 32;
+  float *tiles = Aws + (size_t)bt * NP * (NP + 1), *L = tiles + tri_tile(nb, 0);
+  int I = p + 1, J = p + 1;
+  if (blockIdx.x) {  // (the diagonal tile is number p + 1 of its row)
+    const int e = (int)blockIdx.x - 1;
+    tri_coords((p + 1) * (p + 2) / 2 + e + (e > p ? 1 : 0), I, J);
+  }
+  float *T = tiles + tri_tile(I, J);
+  float4 old[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+    old[u] = J == p ? make_float4(0.f, 0.f, 0.f, 0.f)
+                    : ((const float4 *)T)[(4 * ty + u) * 8 + (tx ^ ty)];
+  fitg_copy(ls, L + (size_t)I * kFcTile, tid);
+  fitg_copy(qs, J > p ? L + (size_t)J * kFcTile : tiles + tri_tile(p, J), tid);
+  __syncthreads();
+  float acc[4][4];
+  fc_product(J > p ? ls : qs, J > p ? qs : ls, tid, acc);
+  if (blockIdx.x == 0) __syncthreads();  // (ls is read)
+  float *D = blockIdx.x == 0 ? ls : T;
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+    ((float4 *)D)[(4 * ty + u) * 8 + (tx ^ ty)] =
+        make_float4(old[u].x - acc[u][0], old[u].y - acc[u][1], old[u].z - acc[u][2],
+                    old[u].w - acc[u][3]);
+  if (blockIdx.x) return;
+  const float *Kh = Kh_all + (size_t)bt * n * n;
+  const int i = 32 * I + tid;
+  if (tid < 32) dg[tid] = i < n ? Kh[(size_t)i * n + i] : 1.f;
+  __syncthreads();
+  fc_diagonal(ls, dg, dsh, L + (size_t)nb * kFcTile, T, fbad_all + bt);
+}
+
+// W and its operand images, a tile per block.
+__global__ void __launch_bounds__(64)
+    fitg_output_kernel(int NP, const float *Aws, float *Wws, const float *xt, int DP, PostPlan plan,
+                       uint16_t *bop, int *status, const int *fbad_all) {
+  pdl_wait();
+  pdl_trigger();
+  const int bt = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (fbad_all[bt]) return;  // (fitc_kernel reports it)
+  const float *x0 = xt + (size_t)bt * plan.nxt * xt_chunk_floats(DP);
+  const float *T = Aws + (size_t)bt * NP * (NP + 1) + (size_t)blockIdx.x * kFcTile;
+  const float wscale = exp2i((int)x0[xt_param_offset(DP) + 2 * DP + kParEW]);
+  int I, J;
+  tri_coords(blockIdx.x, I, J);
+  bool fits = true;
+  for (int r0 = 8 * warp; r0 < 32; r0 += 16)
+    fits &= fc_output(T, I, J, r0, lane, NP, plan, wscale, Wws + (size_t)bt * NP * (NP + 1),
+                      bop + (size_t)bt * plan.image_halves);
+  if (!fits) set_status(status, BOUTE_ERR_NOT_PD);
+}
+
 }  // namespace
 
 // Outcome transforms alone (codes != 0), elementwise: Yt = t(Y), count
@@ -748,12 +902,12 @@ int launch_standardize(const double *Y, int B, int n, int m, int codes, double *
   return last_launch_status();
 }
 
-// Dynamic shared memory of fitc_kernel with clusters of C (tiles: its tiles too).
+// Dynamic shared memory of fitc_kernel with clusters of C: operands and tiles, or alpha's
+// vectors alone.
 static size_t fitc_smem(int npad, int C, bool tiles) {
-  const int nb = npad / 32, ms = fc_max_slots(nb, C);
-  return ((size_t)(fc_ops(nb, C) + 3 + (tiles ? ms : 0)) * kFcTile +
-          32 * ((nb + fc_rows(C) - 1) / fc_rows(C)) + ((ms + 3) & ~3)) *
-         sizeof(float);
+  const int nb = npad / 32, ms = fc_max_slots(nb, C), nR = (nb + fc_rows(C) - 1) / fc_rows(C);
+  if (!tiles) return ((size_t)8 * npad + 4 * 32 * nR) * sizeof(float);
+  return ((size_t)(fc_ops(nb, C) + 3 + ms) * kFcTile + 32 * nR + ((ms + 3) & ~3)) * sizeof(float);
 }
 constexpr size_t kFcMaxSmem = 227 * 1024 - 5 * 1024;  // (its static part: 4.9 KB)
 
@@ -763,18 +917,20 @@ constexpr size_t kFcMaxSmem = 227 * 1024 - 5 * 1024;  // (its static part: 4.9 K
 // problem-objectives: 535 us on clusters of 4, 655 in two waves of 8; n = 256: 154
 // against 215; n = 128, 38 of them: 93 on clusters of 2, 122 in two waves of 4), no more
 // CTAs than block rows (n = 32 on one CTA 28 us, on two 30; n = 128 on four 50, on
-// eight 53; n = 203 on four 101, on eight 98), and enough that the operands, and if any
-// size allows it the tiles, fit shared memory (n = 256 on single CTAs, n = 1024 on 16;
-// above that the tiles stay in the workspace).
+// eight 53; n = 203 on four 101, on eight 98), and enough that operands and tiles fit
+// shared memory (n = 256 on single CTAs, n = 1024 on 16; above that the whole GPU factors
+// the tiles and the clusters solve for alpha alone).
 static int launch_fitc(Gp *gp, const double *Ys, int standardize, cudaStream_t s) {
   const int n = gp->n, m = gp->m, npad = gp->plan.npad, nb = npad / 32;
   const long long BM = (long long)gp->B * m, sms = num_sms();
   int least = 1;
   while (least < kFcMaxCluster && fitc_smem(npad, least, true) > kFcMaxSmem) least *= 2;
+  bool tiles = fitc_smem(npad, least, true) <= kFcMaxSmem;
+  if (!tiles) least = 1;
   int C = least;
   while (C < kFcMaxCluster && C < nb && 2 * C * BM <= sms) C *= 2;
   // launches unless the device cannot hold `want` clusters of C
-  auto go = [&](auto kern, bool tiles, long long want) {
+  auto go = [&](auto kern, long long want) {
     prefer_shared(kern);
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFcMaxSmem);
     if (C > 8) cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -792,7 +948,8 @@ static int launch_fitc(Gp *gp, const double *Ys, int standardize, cudaStream_t s
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int held = 0;
-    if (C > 1 && (cudaOccupancyMaxActiveClusters(&held, kern, &cfg) != cudaSuccess || held < want)) {
+    if (C > 1 &&
+        (cudaOccupancyMaxActiveClusters(&held, kern, &cfg) != cudaSuccess || held < want)) {
       cudaGetLastError();
       return false;
     }
@@ -802,13 +959,34 @@ static int launch_fitc(Gp *gp, const double *Ys, int standardize, cudaStream_t s
                        gp->bop, gp->kern, gp->status, gp->fbad);
     return true;
   };
-  // (below `least`: a partitioned device may not place the larger clusters)
-  for (;; C /= 2) {
-    const bool tiles = fitc_smem(npad, C, true) <= kFcMaxSmem;
-    const long long want = C > least ? BM : 1;
-    if (tiles ? go(fitc_kernel<true>, true, want) : go(fitc_kernel<false>, false, want)) break;
-    if (C == 1 || fitc_smem(npad, C / 2, false) > kFcMaxSmem) return BOUTE_ERR_CUDA;
+  auto factor = [&]() {  // (every lower tile a product for each panel above it)
+    const unsigned nt = nb * (nb + 1) / 2, y = (unsigned)BM;
+    launch_pdl(fitg_load_kernel, dim3(nt, y), dim3(64), 0, s, (const float *)gp->Kh, n, npad,
+               gp->Aws, gp->fbad);
+    for (int p = 0; p < nb; ++p) {
+      if (nb > 1) launch_pdl(fitg_panel_kernel, dim3(nb - 1, y), dim3(64), 0, s, npad, gp->Aws, p);
+      if (p + 1 < nb)
+        launch_pdl(fitg_update_kernel, dim3(nt - (p + 1) * (p + 2) / 2, y), dim3(64), 0, s,
+                   (const float *)gp->Kh, n, npad, gp->Aws, p, gp->fbad);
+    }
+    launch_pdl(fitg_output_kernel, dim3(nt, y), dim3(64), 0, s, npad, (const float *)gp->Aws,
+               gp->Wws, (const float *)gp->xt, gp->DP, gp->plan, gp->bop, gp->status,
+               (const int *)gp->fbad);
+    count_launch(2 * nb + 1);
+  };
+  if (tiles) {
+    while (C > least && !go(fitc_kernel<true>, BM)) C /= 2;
+    // (a partitioned device may not place clusters of `least`)
+    if (C > least || go(fitc_kernel<true>, 1)) {
+      count_launch(2);
+      return last_launch_status();
+    }
+    tiles = false;
+    C = 1;
   }
+  factor();
+  while (C > 1 && !go(fitc_kernel<false>, BM)) C /= 2;
+  if (C == 1) go(fitc_kernel<false>, 1);
   count_launch(2);
   return last_launch_status();
 }

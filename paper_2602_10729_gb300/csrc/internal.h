@@ -15,8 +15,8 @@ struct Gp {
   int B, n, d, m, DP;  // DP = d rounded up to one of BOUTE_PADDED_DIMS (register tile)
   PostPlan plan;
   float *Kh, *Kl;  // B*m x n x n: kernel matrix (lower) as an fp32 pair hi + lo
-  float *Aws;      // B*m x np x (np+1): the factorisation's tiles when they do not fit shared memory
-                   // (n > 1024; np = npad)
+  float *Aws;      // B*m x np x (np+1): the factorisation's tiles, and a panel's, when they do
+                   // not fit a cluster's shared memory (n > 1024; np = npad)
   float *Wws;      // B*m x np x (np+1): L^-1 (lower, row stride np+1)
   uint16_t *bop;  // B*m x plan.image_halves: L^-1 as fp16 hi/lo operand images
   // the posterior's cache of K* chunks that later groups of output blocks

@@ -199,13 +199,17 @@ def test_engine_where_the_side_input_passes_shared_memory(n, d, comp):
     mean = torch.empty((1, w.m, w.N), dtype=torch.float32, device="cuda")
     var = torch.empty_like(mean)
     at = np.arange(0, 300, 7)
+    stream = torch.cuda.Stream()  # (steps are captured as graphs)
     for rows in (n, 65):
         if rows < n:
             bt.boute_engine_set_n(e, rows)
             hp.X, hp.Y = hp.X[:, :rows], hp.Y[:, :rows]
-        bt.boute_engine_step(e, t(hp.X), t(hp.Y), t(hp.ls), t(hp.s2), t(hp.noise), t(hp.ref),
-                             t(hp.Xc, torch.float32), None, idx, val)
-        bt.boute_engine_scores(e, None, mean, var)
+        args = [t(hp.X), t(hp.Y), t(hp.ls), t(hp.s2), t(hp.noise), t(hp.ref),
+                t(hp.Xc, torch.float32)]
+        torch.cuda.synchronize()
+        with torch.cuda.stream(stream):
+            bt.boute_engine_step(e, *args, None, idx, val)
+            bt.boute_engine_scores(e, None, mean, var)
         torch.cuda.synchronize()
         check_posterior_at(hp, at, mean[0].cpu().numpy(), var[0].cpu().numpy())
     e.free()
@@ -467,9 +471,10 @@ def test_row_pairs_and_column_groups(d, n, N):
 
 
 # Tiles of 32: sizes at their edges, batches that take clusters of 16, 8, 4, 2 and 1
-# CTAs, and tiles that stay in the workspace.
+# CTAs, and (n > 1024) the factorisation over the whole GPU.
 @pytest.mark.parametrize("n,B", [(1, 1), (32, 3), (33, 1), (65, 40), (97, 2), (160, 1), (161, 1), (192, 2), (193, 1), (224, 40), (256, 40), (288, 20),
-                                 (321, 12), (511, 6), (1024, 1), (1025, 1)])
+                                 (321, 12), (511, 6), (1024, 1), (1025, 1),
+                                 (1057, 5), (1300, 1), (2048, 1)])
 def test_cluster_fit_edges(n, B):
     w = wl.scaled(wl.WORKLOADS[4], N=130, B=B, n=n)
     hp = host_problem(w)
@@ -599,3 +604,22 @@ def test_fit_of_problem_objectives_beyond_the_held_clusters(n):
         assert bt.boute_gp_status(gp) == 0
         gp.free()
     assert us[1] < 1.35 * us[0], us
+
+
+def test_fit_of_many_observations_uses_the_whole_gpu():
+    """n = 2048 has eight times the products of n = 1024: over all SMs a fit of one
+    objective takes less than twice as long, on the 16 SMs of one cluster four times."""
+    import torch
+
+    from paper_2602_10729_gb300 import boute as bt
+    us = []
+    for n in (1024, 2048):
+        hp = host_problem(wl.scaled(wl.WORKLOADS[4], N=1, B=1, n=n))
+        t = lambda a: torch.as_tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")
+        args = [t(hp.X), t(hp.Y[:, :, :1]), t(hp.ls[:, :1]), t(hp.s2[:, :1]), t(hp.noise[:, :1])]
+        bt.boute_standardize(args[1], args[1])
+        gp = bt.boute_gp_create(1, n, hp.w.d, 1)
+        us.append(_median_us(lambda: bt.boute_gp_fit(gp, *args)))
+        assert bt.boute_gp_status(gp) == 0
+        gp.free()
+    assert us[1] < 2.5 * us[0], us

@@ -102,8 +102,8 @@ struct boute_engine {
   bool fuse_sel;
   // K* of the candidates, computed on a second side stream while the fit
   // runs (it needs the fit's set-up, not its results); the posterior then
-  // only contracts it. Null when it would take more than kKstarMaxBytes; unused while
-  // n is too large for the K* kernel (kstar_fits).
+  // only contracts it. Null when that takes longer (kstar_worth); unused while n is too
+  // large for the K* kernel (kstar_fits).
   float *kst;
   cudaStream_t side2;
   cudaEvent_t ev_setup, join2;
@@ -589,13 +589,23 @@ void boute_engine_free(boute_engine *e) {
   delete e;
 }
 
-// Largest K* buffer an engine keeps (it lets the posterior's K* be computed
-// beside the fit); larger workloads build K* inside the posterior. The line is the
-// L2's size: beyond it K* goes to HBM and back, which takes longer than the fit it
-// hides behind (271 MB at n = 49, d = 15, m = 3: step 659 us, built inside 638; 307 MB
-// at n = 203, d = 7: 325 either way; 67 MB at n = 128, d = 12: posterior 26 us
-// against 54 built inside).
-constexpr size_t kKstarMaxBytes = size_t(128) << 20;
+// Largest K* buffer with which an engine computes K* beside the fit; larger workloads build
+// K* inside the posterior. Building it inside costs more the more dimensions there are
+// (from 17 on with half the builder warps), writing and reading it costs the same, and
+// from L2's size on that is HBM's time. Steps with two objectives, beside against inside:
+//   d = 24, any n: n = 32 188 : 190 us at 140 MiB, 570 : 621 at 500; n = 128 166 : 188 and
+//     459 : 495; n = 512 353 : 383 and 637 : 657
+//   d = 16: n = 128 146 : 162 at 140 MiB, 229 : 242 at 260, 404 : 400 at 500; n = 160 199 :
+//     202 at 190, 250 : 243 at 260; n = 384 267 : 288 at 190
+//   d = 12: n = 128 163 : 175 at 190 MiB, 289 : 286 at 380; n = 160 182 : 184 at 190, 228 :
+//     220 at 260; n = 384 262 : 269 at 190; n = 512 339 : 336 at 190
+//   d = 6: n = 160 143 : 141 at 140 MiB, 199 : 192 at 260; n = 384 226 : 219 at 140
+//   up to 64 observations the fit is too short to hide it: d = 12, n = 64 206 : 197 at 190
+//     MiB, 266 : 247 at 260
+static bool kstar_worth(const Gp &g, long long N) {
+  const size_t line = g.DP > 16 ? 512 : g.n > 64 && g.n <= 448 && g.DP > 8 ? 256 : 128;
+  return kstar_floats(&g, N) * sizeof(float) <= line << 20;
+}
 
 // The selection runs inside the acquisition kernel for 2-objective
 // Monte-Carlo steps with k <= 32 (not in stage-timing mode, which times the
@@ -666,7 +676,7 @@ int boute_engine_create(int B, int n, int d, int m, long long N, int mode, int S
       r = BOUTE_ERR_CUDA;
     }
   }
-  if (r == BOUTE_OK && kstar_floats(&e->gp->g, N) * sizeof(float) <= kKstarMaxBytes)
+  if (r == BOUTE_OK && kstar_worth(e->gp->g, N))
     r |= dalloc(&e->kst, kstar_floats(&e->gp->g, N));
   if (r == BOUTE_OK &&
       (cudaStreamCreateWithFlags(&e->side, cudaStreamNonBlocking) != cudaSuccess ||
@@ -744,7 +754,8 @@ static int engine_run(boute_engine *e, const double *X, const double *Y, const d
   }
   // K* beside the fit (not in serialised timing, where the posterior builds it, nor
   // while the K* kernel cannot hold the side input of the engine's present n)
-  const float *kst = serial || !kstar_fits(&e->gp->g) ? nullptr : e->kst;
+  const float *kst =
+      serial || !kstar_fits(&e->gp->g) || !kstar_worth(e->gp->g, e->N) ? nullptr : e->kst;
   // The graph has one root, the fit's set-up: the front stage (which needs
   // the raw outcomes only) and K* (which needs the set-up's side input) fork
   // after it and run beside the fit (one root launches sooner than two).

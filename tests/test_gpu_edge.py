@@ -215,6 +215,34 @@ def test_engine_where_the_side_input_passes_shared_memory(n, d, comp):
     e.free()
 
 
+@pytest.mark.parametrize("n,d,N,beside", [(128, 24, 143323, True), (32, 20, 389083, True),
+                                          (64, 17, 532443, True), (128, 16, 194523, True),
+                                          (128, 16, 532443, False), (64, 16, 389083, False),
+                                          (160, 7, 129627, False), (128, 24, 600000, False),
+                                          (512, 12, 48603, False)])
+def test_kstar_beside_the_fit_where_it_is_faster(n, d, N, beside):
+    """A step with K* beside the fit launches one kernel more (its own), as one with few
+    candidates does: up to 512 MiB of K* from 17 dimensions on, 256 with 9 to 16 and 65 to
+    448 observations, else 128."""
+    import torch
+
+    from paper_2602_10729_gb300 import boute as bt
+    hp = rand_problem(31, n, d, 2, 1, ls=0.2 * np.sqrt(d))
+    t = lambda a: torch.as_tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")
+    count = []
+    for cands in (20000, N):
+        e = bt.Engine(1, n, d, 2, cands, bt.BOUTE_ACQ_EHVI2D, 0, 4)
+        Xc = torch.rand((1, cands, d), device="cuda")
+        idx = torch.empty((1, 4), dtype=torch.int64, device="cuda")
+        val = torch.empty((1, 4), dtype=torch.float32, device="cuda")
+        l0 = bt.boute_launch_count()
+        bt.boute_engine_step(e, t(hp.X), t(hp.Y), t(hp.ls), t(hp.s2), t(hp.noise), t(hp.ref), Xc,
+                             None, idx, val)
+        count.append(bt.boute_launch_count() - l0)
+        e.free()
+    assert count[0] - count[1] == (0 if beside else 1)
+
+
 def test_ill_conditioned_problem_meets_fp32_error_bound():
     """40 points on a line with lengthscale 0.3: cond(K) ~ 2e5, |alpha| ~ 1e3.
     The mean meets 1e-5 (its ill-conditioned rows take the fp64 path); the

@@ -390,6 +390,64 @@ def test_topk_levels_and_k_range(N, k):
         assert np.array_equal(val[b].cpu().numpy(), v[b][want], equal_nan=True)
 
 
+# blocks of 128 to 1024 threads at their edges, one level and two, scores mostly equal:
+# fewer others than k, as many, more, none
+@pytest.mark.parametrize("N,k", [(2048, 128), (2048, 129), (2049, 100), (4096, 256), (4097, 32),
+                                 (8192, 512), (8193, 512), (8192, 513), (16384, 7), (20_000, 40),
+                                 (300_000, 64), (300_000, 700), (60, 60)])
+def test_topk_mostly_equal_scores(N, k):
+    import torch
+
+    from paper_2602_10729_gb300 import boute as bt
+    rng = np.random.default_rng(N + k)
+    v = np.zeros((6, N), np.float32)
+    for b, others in enumerate((k // 2, k, 2 * k, 0)):
+        v[b, rng.permutation(N)[:others]] = rng.random(min(others, N)) + 0.5
+    v[4] = np.where(rng.random(N) < 0.5, -1.0, -2.0)  # ties at and below the k-th value
+    v[5, rng.permutation(N)[: N - N // 8]] = -np.inf
+    a = torch.as_tensor(v, device="cuda")
+    idx = torch.empty((6, k), dtype=torch.int64, device="cuda")
+    val = torch.empty((6, k), dtype=torch.float32, device="cuda")
+    bt.boute_select_topk(a, 6, N, k, idx, val)
+    for b in range(6):
+        want = np.lexsort((np.arange(N), -v[b]))[:k]
+        assert np.array_equal(idx[b].cpu().numpy(), want)
+        assert np.array_equal(val[b].cpu().numpy(), v[b][want])
+
+
+def _graph_us(f, calls=20):
+    """Device time of a call, from a graph of several."""
+    import torch
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        f()
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            for _ in range(calls):
+                f()
+        return _median_us(g.replay, 9) / calls
+
+
+def test_topk_of_mostly_zero_scores_and_of_many_small_problems():
+    """Scores that are mostly zero, or a thousand problems of a thousand scores, take a
+    few times what one problem with distinct scores takes (they took eight times that)."""
+    import torch
+
+    from paper_2602_10729_gb300 import boute as bt
+
+    def us(a, k):
+        idx = torch.empty((len(a), k), dtype=torch.int64, device="cuda")
+        val = torch.empty((len(a), k), dtype=torch.float32, device="cuda")
+        return _graph_us(lambda: bt.boute_select_topk(a, len(a), a.shape[1], k, idx, val))
+
+    a = torch.randn((1, 4096), device="cuda")
+    one = us(a, 8)
+    assert us(torch.where(a > 3.5, a, torch.zeros_like(a)), 8) < 4 * one
+    assert us(torch.randn((1000, 1024), device="cuda"), 32) < 4 * one
+
+
 # ties, NaN and -0 at one block, several, and hundreds of them
 @pytest.mark.parametrize("N,k", [(5000, 40), (5000, 32), (5000, 1), (2048, 7), (40, 32),
                                  (700_001, 32), (700_001, 17), (70_000, 33)])

@@ -14,7 +14,8 @@
 // -sum_k (b_k - max(a_k, y1))+ [y2 < u_k].
 //
 // One CTA per (problem, starting point) runs all its steps; each step is a chain
-// of short phases, so what bounds it is latency. Half of the 16 warps take each
+// of short phases, so what bounds it is latency. Half of its (16, with many starts of few
+// observations 8 or 4) warps take each
 // objective: the threads build k* and its gradient factors over the training
 // points (the fit's side input: scaled coordinates hi + lo, alpha as a pair);
 // a warp takes a row of the fit's W into registers, forms q_i = W_i k* and adds
@@ -27,6 +28,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.h"
 
@@ -34,9 +36,6 @@ namespace boute {
 
 namespace {
 
-constexpr int kOptThreads = 512, kOptWarps = kOptThreads / 32;
-constexpr int kObjWarps = kOptWarps / 2, kObjThreads = kOptThreads / 2;  // per objective
-constexpr int kRowRegs = 16, kPanel = 32 * kRowRegs;  // a row of W in a warp's registers
 constexpr float kLn2f = 0.6931471805599453f;
 constexpr float kLn2Sq3f = 0.16015100463940046f;  // (ln 2)^2 / 3
 // 1 / (the side input's coordinate scale)^2
@@ -63,6 +62,7 @@ __device__ __forceinline__ float warp_sum_f(float v) {
 }
 
 // acc[u] += q w[u] and back: a row's entries j0 + lane + 32 u up to column i
+template <int kRowRegs>
 __device__ __forceinline__ void load_row(const float *wr, int i, int j0, int lane,
                                          float (&w)[kRowRegs]) {
 #pragma unroll
@@ -72,7 +72,11 @@ __device__ __forceinline__ void load_row(const float *wr, int i, int j0, int lan
   }
 }
 
+// kRowRegs: columns of a row of W per lane (n <= 32 kRowRegs, or panels of as many).
+template <int kOptThreads, int kRowRegs>
 __global__ void __launch_bounds__(kOptThreads) acqopt_kernel(const __grid_constant__ OptArgs a) {
+  constexpr int kOptWarps = kOptThreads / 32, kPanel = 32 * kRowRegs;
+  constexpr int kObjWarps = kOptWarps / 2, kObjThreads = kOptThreads / 2;  // per objective
   extern __shared__ __align__(16) float sm[];
   __shared__ float xs[BOUTE_MAX_D], xsc[2][BOUTE_MAX_D];  // x, x / l (scaled)
   __shared__ float dmu_s[2][BOUTE_MAX_D], dvar_s[2][BOUTE_MAX_D];
@@ -334,11 +338,28 @@ int launch_acq_optimize(const Gp *gp, const float *lower, const float *upper, co
   const size_t n = gp->n;
   // (the limit on n and d that the call has always had)
   if ((4 * n + n * gp->d) * sizeof(float) > 200 * 1024) return BOUTE_ERR_UNSUPPORTED;
-  const size_t smem = (6 * n + 2 * (size_t)kObjWarps * std::min<size_t>(n, kPanel) + 3 * (n + 1) +
-                       (n > kPanel ? 2 * n : 0)) * sizeof(float);
-  // (no shared-memory preference: what it leaves of the SM's memory caches W)
-  cudaFuncSetAttribute(acqopt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  launch_pdl(acqopt_kernel, dim3(P, gp->B), dim3(kOptThreads), smem, s, a);
+  auto go = [&](auto threads, auto regs) {
+    constexpr int T = decltype(threads)::value, R = decltype(regs)::value;
+    const size_t panel = 32 * R;
+    const size_t smem = (6 * n + (size_t)(T / 32) * std::min(n, panel) + 3 * (n + 1) +
+                         (n > panel ? 2 * n : 0)) * sizeof(float);
+    // (no shared-memory preference: what it leaves of the SM's memory caches W)
+    cudaFuncSetAttribute(acqopt_kernel<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem);
+    launch_pdl(acqopt_kernel<T, R>, dim3(P, gp->B), dim3(T), smem, s, a);
+  };
+  // With at most 128 columns a row of W takes four registers of a lane, and starts beyond one
+  // per SM share SMs in smaller blocks: n = 32, d = 6, S = 64, 5 steps: 256 starts 27 us
+  // with 256 threads (42 with 512), 1024 starts 49 with 128 (74 with 256, 137 with 512, 171
+  // with 16 registers); n = 100, S = 128, 3 steps, 4096 starts: 274 (749 with 512 and 16).
+  // More columns keep 16 registers and the block of 512: n = 700, 1024 starts, 2 steps 2.0
+  // ms against 2.2 with 128.
+  using std::integral_constant;
+  const long long blocks = (long long)P * gp->B, sms = num_sms();
+  if (n > 128) go(integral_constant<int, 512>{}, integral_constant<int, 16>{});
+  else if (blocks <= sms) go(integral_constant<int, 512>{}, integral_constant<int, 4>{});
+  else if (blocks <= 2 * sms) go(integral_constant<int, 256>{}, integral_constant<int, 4>{});
+  else go(integral_constant<int, 128>{}, integral_constant<int, 4>{});
   count_launch();
   return last_launch_status();
 }

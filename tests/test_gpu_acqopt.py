@@ -103,6 +103,52 @@ def test_row_panel_edges_match_oracle(n, S, P):
     np.testing.assert_allclose(grad[0], grads, rtol=1e-3, atol=2e-4 * np.abs(grads).max() + 1e-12)
 
 
+@pytest.mark.parametrize("n", [1, 33, 100, 128, 129])
+@pytest.mark.parametrize("P", [160, 320])
+def test_many_starts_in_smaller_blocks_match_oracle(n, P):
+    """More starts than SMs, and than twice as many: blocks of 256 and 128 threads, up to
+    128 observations with four registers a lane for a row of W. Tolerances as above."""
+    w = wl.scaled(wl.WORKLOADS[1], N=64, B=1, n=n)
+    hp = host_problem(w)
+    gp, lower, upper, K, cap, epsd, eps = _setup(hp, 33)
+    X0 = np.random.default_rng(n).uniform(0.05, 0.95, (1, 4, w.d)).astype(np.float32)
+    _, acq, grad = _run(gp, (lower, upper, K, cap), epsd, np.tile(X0, (1, P // 4, 1)), 0, 0.01, w.d)
+    gp.free()
+    fp = oracle_fit(hp, 0)
+    vals, grads = zip(*(opl.mc_hvi_value_grad(fp, X0[0, p].astype(np.float64), eps)
+                        for p in range(4)))
+    vals, grads = np.tile(vals, P // 4), np.tile(grads, (P // 4, 1))
+    np.testing.assert_allclose(acq[0], vals, rtol=1e-4, atol=1e-6 * np.abs(vals).max() + 1e-12)
+    np.testing.assert_allclose(grad[0], grads, rtol=1e-3, atol=2e-4 * np.abs(grads).max() + 1e-12)
+
+
+def test_many_starts_share_the_sms():
+    """4096 starts at n = 32 take five times as long as 152: several blocks run on an SM at
+    once (one that fills it at a time: 17 times)."""
+    import torch
+
+    from paper_2602_10729_gb300 import boute as bt
+    w = wl.scaled(wl.WORKLOADS[0], N=64, B=1, n=32)
+    gp, lower, upper, K, cap, epsd, _ = _setup(host_problem(w), 64)
+    lo = torch.zeros(w.d, dtype=torch.float32, device="cuda")
+    ms = []
+    for P in (152, 4096):
+        x0 = torch.rand((1, P, w.d), device="cuda")
+        X, acq = torch.empty_like(x0), torch.empty((1, P), device="cuda")
+        out = []
+        for _ in range(9):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            bt.boute_acq_optimize(gp, lower, upper, K, cap, epsd, 64, x0, P, lo, lo + 1, 20, 0.01,
+                                  X, acq)
+            b.record()
+            torch.cuda.synchronize()
+            out.append(a.elapsed_time(b))
+        ms.append(float(np.median(out[2:])))
+    gp.free()
+    assert ms[1] < 9 * ms[0], ms
+
+
 @pytest.mark.parametrize("wi,n,S", [(2, 96, 64), (1, 64, 64)])
 def test_ascent_from_the_pool_best_matches_oracle(wi, n, S):
     w = wl.scaled(wl.WORKLOADS[wi], N=2048, B=1, n=n)

@@ -109,12 +109,13 @@ __device__ __forceinline__ int block_select(const unsigned (&hi)[kR], Lo lo, int
   unsigned m = 0u;
 #pragma unroll
   for (int r = 0; r < kR; ++r) m = max(m, hi[r]);
-  bool exact;
+  bool exact = true;
   unsigned t0 = 0u;
   if (k <= NT)
     t0 = kth_word(k, 0u, 32, exact, [&](unsigned t) { return __syncthreads_count(m >= t); });
   else __syncthreads();
   t0 = max(t0, 1u);  // (absent keys never survive)
+  const bool value = !exact;  // t0 has all its bits: it may be the k-th value
   // survivors into buf, while they fit
 #pragma unroll
   for (int r = 0; r < kR; ++r) {
@@ -142,7 +143,7 @@ __device__ __forceinline__ int block_select(const unsigned (&hi)[kR], Lo lo, int
         return two ? c + __syncthreads_count(bh > t) : c;
       };
       unsigned th = t0;  // (the k-th value unless k keys lie above it)
-      int above = count_above(t0);
+      int above = value ? count_above(t0) : k;
       exact = false;
       if (above >= k) {
         th = kth_word(k, 0u, 32, exact, [&](unsigned t) {
@@ -177,7 +178,7 @@ __device__ __forceinline__ int block_select(const unsigned (&hi)[kR], Lo lo, int
       return sum[0];
     };
     unsigned th = t0;
-    int above = count_above(t0);
+    int above = value ? count_above(t0) : k;
     exact = false;
     if (above >= k) {
       th = kth_word_all<NT>(k, 0u, 32, red, exact, at_least);

@@ -574,9 +574,9 @@ def test_cluster_fit_edges(n, B):
             check_var(g["var"][b, t], var[:, t], fp.s2[t])
 
 
-# Three objectives: passes of 128 samples with a ragged last one, one sample, and a
-# count the register path takes (with and without thresholds).
-@pytest.mark.parametrize("S", [1, 31, 100, 127, 129, 200, 256, 300])
+# Three objectives: passes of 32, 64 and 128 samples with a ragged last one, one sample, and
+# a count the register path takes (with and without thresholds).
+@pytest.mark.parametrize("S", [1, 31, 32, 33, 64, 65, 100, 127, 129, 200, 256, 300])
 def test_three_objective_sample_counts(S):
     hp = rand_problem(S, 25, 4, 3, 77, mode="mc", S=S)
     compare(hp)
@@ -586,6 +586,28 @@ def test_three_objective_sample_counts(S):
     want = opl.acquisition(fp, g["mean"][0].T.astype(np.float64), g["var"][0].T.astype(np.float64),
                            "mc", hp.eps[0], cons=cons[0])
     check_acq(g["acq"][0], want)
+
+
+def test_few_samples_of_three_objectives_cost_less_than_many():
+    """Sixteen samples in passes of 32, not padded to the 128 of a full pass (with which
+    they took longer than 128 samples do on their own path)."""
+    import torch
+
+    from paper_2602_10729_gb300 import boute as bt
+    rng = np.random.default_rng(5)
+    N, K = 20000, 21
+    t = lambda a: torch.as_tensor(np.ascontiguousarray(a, np.float32), device="cuda")
+    lo = rng.uniform(-2, 0, (1, K, 3))
+    hi = lo + rng.uniform(0.1, 1, (1, K, 3))
+    mean, var = t(rng.standard_normal((1, 3, N))), t(rng.uniform(0.05, 1, (1, 3, N)))
+    lo, hi, Kd = t(lo), t(hi), torch.tensor([K], dtype=torch.int32, device="cuda")
+    acq = torch.empty((1, N), device="cuda")
+
+    def us(S):
+        eps = torch.randn((1, N, 3, S), device="cuda")
+        return _graph_us(lambda: bt.boute_acq_mc_hvi(mean, var, 1, N, 3, lo, hi, Kd, K, eps, S,
+                                                     3 * S, acq))
+    assert us(16) < 0.95 * us(128)
 
 
 def test_ehvi_over_the_normal_tail():

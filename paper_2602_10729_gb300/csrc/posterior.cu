@@ -336,6 +336,14 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity,
 // the ratio the fp32 mean's error stays under about 8e-6 of the scale (up to 256
 // it reached 1.1e-5: row 190 of n = 70, lengthscales 0.5 .. 2).
 constexpr float kFixRatio = 224.f;
+// What the epilogue writes for such a row until the CTA, its last unit done, recomputes it
+// with all its warps: a NaN that no computation gives. (The CTA that marks a mean writes it;
+// nobody reads it before the grid is complete.) Recomputed by the epilogue's own warps, a row
+// at a time, a row held up its CTA for 100 to 200 thousand clocks. 2^18 candidates, n = 1024:
+// d = 24, 476 rows marked 2426 -> 1810 us, d = 16, 24 441 rows 8339 -> 2784; n = 777, d = 20,
+// three problems of 30 011 2673 -> 1124; n = 512, d = 6, 2^15 candidates, 23 769 rows 1705 ->
+// 417; no rows marked: within 1 %, n <= 32 1.5 % slower.
+constexpr uint32_t kFixMark = 0x7fc0a51fu;
 
 // ---- the exact mean of a flagged row, in double-float arithmetic -----------------
 // Numbers as unevaluated pairs hi + lo of floats (Dekker; Knuth's error-free
@@ -399,15 +407,18 @@ __device__ __forceinline__ F2 exp2_neg_pair(F2 r) {
   return F2{e.h * sc, e.l * sc};
 }
 
-// A row's mean for the Matern-5/2 kernel, computed by a whole warp (lane =
-// column j mod 32) and returned to every lane: the candidate's coordinates
-// scaled by 1/l, the training points' x / l and alpha as pairs, read from the
-// side input in global memory (the rare, exact path; the warp takes one flagged
-// row at a time).
+// A row's mean for the Matern-5/2 kernel, computed by a whole warp and returned to every
+// lane: the candidate's coordinates scaled by 1/l, the training points' x / l and alpha as
+// pairs, read from the side input in global memory. Eight lanes to a chunk of 32 points and
+// four points to a lane, so that the loads, 16 bytes each, and the chains of dependent
+// operations overlap four times; with a point per lane the row waited for L2 at every four
+// dimensions.
 template <int DP>
 __device__ float mean_pair_warp(const float *xrow, int d, const float *x0, int cf, int n,
                                 int lane) {
-  constexpr F2 ln2 = pair_of(0.69314718055994530942), ln2sq3 = pair_of(0.69314718055994530942 * 0.69314718055994530942 / 3.0);
+  constexpr F2 ln2 = pair_of(0.69314718055994530942);
+  constexpr F2 ln2sq3 = pair_of(0.69314718055994530942 * 0.69314718055994530942 / 3.0);
+  constexpr int E = 4;
   const float *il = x0 + xt_param_offset(DP);
   const float s2 = il[2 * DP + kParS2];
   // lane k holds the candidate's coordinate k scaled by 1/l
@@ -417,34 +428,48 @@ __device__ float mean_pair_warp(const float *xrow, int d, const float *x0, int c
     xs = quick_two_sum(p, fmaf(x, il[lane], -p) + x * il[DP + lane]);
   }
   F2 acc{0.f, 0.f};
-  for (int j0 = 0; j0 < n; j0 += 32) {
-    const int j = j0 + lane;
-    const float *ch = x0 + (size_t)(j0 / BOUTE_KCHUNK) * cf;
-    F2 r2{0.f, 0.f};
-#pragma unroll 4
+  const int nch = (n + BOUTE_KCHUNK - 1) / BOUTE_KCHUNK;
+  for (int c0 = 0; c0 < nch; c0 += 32 * E / BOUTE_KCHUNK) {
+    const int c = c0 + lane / (BOUTE_KCHUNK / E), jj = E * (lane % (BOUTE_KCHUNK / E));
+    const float *ch = x0 + (size_t)min(c, nch - 1) * cf + jj;
+    F2 r2[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) r2[e] = F2{0.f, 0.f};
+#pragma unroll 2
     for (int k = 0; k < d; ++k) {
       const float xh = __shfl_sync(0xffffffffu, xs.h, k), xl = __shfl_sync(0xffffffffu, xs.l, k);
-      float sh, se;
-      two_sum_f(xh, -ch[k * BOUTE_KCHUNK + lane], sh, se);
-      const F2 df = quick_two_sum(sh, se + (xl - ch[(DP + k) * BOUTE_KCHUNK + lane]));
-      const float p = df.h * df.h;
-      float e;
-      two_sum_f(r2.h, p, r2.h, e);
-      r2.l += e + fmaf(2.f * df.h, df.l, fmaf(df.h, df.h, -p));
+      const float4 h4 = *(const float4 *)(ch + k * BOUTE_KCHUNK);
+      const float4 l4 = *(const float4 *)(ch + (DP + k) * BOUTE_KCHUNK);
+      const float th[E] = {h4.x, h4.y, h4.z, h4.w}, tl[E] = {l4.x, l4.y, l4.z, l4.w};
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        float sh, se;
+        two_sum_f(xh, -th[e], sh, se);
+        const F2 df = quick_two_sum(sh, se + (xl - tl[e]));
+        const float p = df.h * df.h;
+        float er;
+        two_sum_f(r2[e].h, p, r2[e].h, er);
+        r2[e].l += er + fmaf(2.f * df.h, df.l, fmaf(df.h, df.h, -p));
+      }
     }
-    r2 = quick_two_sum(r2.h, r2.l);
-    // r' = sqrt(r2): one correction of q = r2 rsqrt(r2) by the residual r2 - q^2
-    F2 r{0.f, 0.f};
-    if (r2.h > 0.f) {
-      const float y = rsqrtf(r2.h), q = r2.h * y;
-      r = quick_two_sum(q, 0.5f * y * (fmaf(-q, q, r2.h) + r2.l));
+    const float4 a4 = *(const float4 *)(ch + xt_alpha_offset(DP));  // alpha hi, lo
+    const float4 b4 = *(const float4 *)(ch + xt_alpha_offset(DP) + BOUTE_KCHUNK);
+    const float ah[E] = {a4.x, a4.y, a4.z, a4.w}, al[E] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const F2 q2 = quick_two_sum(r2[e].h, r2[e].l);
+      // r' = sqrt(r2): one correction of q = r2 rsqrt(r2) by the residual r2 - q^2
+      F2 r{0.f, 0.f};
+      if (q2.h > 0.f) {
+        const float y = rsqrtf(q2.h), q = q2.h * y;
+        r = quick_two_sum(q, 0.5f * y * (fmaf(-q, q, q2.h) + q2.l));
+      }
+      // k = s2 (1 + ln2 r' + ln2^2/3 r'^2) 2^(-r') (the coordinates' scale makes
+      // r' = sqrt5 r / ln 2)
+      F2 k = f2p_add(f2p_add(F2{1.f, 0.f}, f2p_mul(r, ln2)), f2p_mul(q2, ln2sq3));
+      k = f2p_mul(f2p_mul(k, exp2_neg_pair(r)), F2{s2, 0.f});
+      if (BOUTE_KCHUNK * c + jj + e < n) acc = f2p_add(acc, f2p_mul(k, F2{ah[e], al[e]}));
     }
-    // k = s2 (1 + ln2 r' + ln2^2/3 r'^2) 2^(-r') (the coordinates' scale makes
-    // r' = sqrt5 r / ln 2)
-    F2 k = f2p_add(f2p_add(F2{1.f, 0.f}, f2p_mul(r, ln2)), f2p_mul(r2, ln2sq3));
-    k = f2p_mul(f2p_mul(k, exp2_neg_pair(r)), F2{s2, 0.f});
-    const float *al = ch + xt_alpha_offset(DP) + lane;  // alpha hi, lo (zero past n)
-    if (j < n) acc = f2p_add(acc, f2p_mul(k, F2{al[0], al[BOUTE_KCHUNK]}));
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -525,6 +550,7 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
   uint64_t *mean_ready = cache_ready + 1, *mean_empty = mean_ready + 1;
   uint32_t *tmem_holder = (uint32_t *)(mean_empty + 1);
   volatile int *abort = (volatile int *)(tmem_holder + 1);
+  volatile int *redo = abort + 1;  // means are marked (kFixMark)
   // after the 512-byte barrier area: per column group and row of the tile,
   // a builder thread's partial mean (hi, lo) and magnitude sum
   float *red = (float *)(bars + 64);
@@ -559,7 +585,7 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
     mbar_init(cache_ready, 1);
     mbar_init(mean_ready, kBldWarps);
     mbar_init(mean_empty, kEpiWarps);
-    *abort = 0;
+    *abort = *redo = 0;
     fence_mbar_init();
   }
   if (warp == 1) {
@@ -772,6 +798,9 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
       // the row's K* scale 2^e_r; the in-sample shifts (G blocks) leave with
       // 2^-(e_r + e_G) applied
       const int er = row_exp(a.kern, par, ws);
+      // (loaded here: after the waits below nothing would hide it)
+      const float fix_scale = kFixRatio * sqrtf(par[kParS2]);
+      const int ew = (int)par[kParEW];
       const float gscale = pl.S_in > 0 ? exp2i(-(er + (int)par[kParEG])) : 0.f;
       float* shrow = pl.S_in > 0 ? a.shift + (size_t)(b * m + t) * pl.S_in * a.N + row : nullptr;
       float ss = 0.f, ssh = 0.f;  // W's and H^T's sums of squares
@@ -832,25 +861,16 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive_count(mean_empty);
       float mean = ldexpf(mhi + mlo, -er);
-      if (KERN == 0) {  // ill-conditioned rows: the mean in pairs, one row at a time
-        const float sc = ldexpf(sqrtf(par[kParS2]), er);  // the mean's scale, scaled like K*
-        const bool fix = live && mag > kFixRatio * fmaxf(fabsf(mhi), sc);
-        unsigned todo = __ballot_sync(0xffffffffu, fix);
-        while (todo) {
-          const int src = __ffs(todo) - 1;
-          todo &= todo - 1;
-          const long long rr = (long long)(tile % a.tiles_per_problem) * BOUTE_TILE_M + 32 * eq + src;
-          const float *x0 = a.xt + (size_t)(b * m + t) * pl.nxt * cf;
-          const float v = mean_pair_warp<DP>(a.Xc + ((long long)b * a.N + rr) * d, d, x0, cf, n,
-                                             lane);
-          if (lane == src) mean = v;
-        }
+      // ill-conditioned rows (scales as K*'s): marked, and recomputed after the last unit
+      if (KERN == 0 && live && mag > fmaxf(kFixRatio * fabsf(mhi), ldexpf(fix_scale, er))) {
+        mean = __uint_as_float(kFixMark);
+        *redo = 1;
       }
       if (live && BOUTE_INB(((long long)b * m + t) * a.N + row, (long long)a.B * m * a.N))
         a.mean[((size_t)b * m + t) * a.N + row] = mean;
       if (live) {
         // V carries the scales 2^e_r (K*) and 2^e_W (W); H^T k* 2^e_r and 2^e_H
-        float vv = prior - ldexpf(ss, -2 * (er + (int)par[kParEW]));
+        float vv = prior - ldexpf(ss, -2 * (er + ew));
         if (pl.nhblk > 0) vv -= ldexpf(ssh, -2 * (er + (int)par[kParEH]));
         if (BOUTE_INB(((long long)b * m + t) * a.N + row, (long long)a.B * m * a.N))
           a.var[((size_t)b * m + t) * a.N + row] = vv > 0.f ? vv : 0.f;
@@ -1063,6 +1083,24 @@ __global__ void __launch_bounds__(Layout<DP>::kThreads, 1)
   if (warp == 1) {
     __syncwarp();
     tmem_dealloc(tmem, 512);
+  }
+  if (KERN == 0 && *redo && !*abort) {
+    // this CTA's marked rows, a warp per 32 rows of a unit
+    for (int i = warp;; i += Layout<DP>::kThreads / 32) {
+      const int unit = blockIdx.x + (i >> 2) * gridDim.x;
+      if (unit >= units) break;
+      const int tile = unit / m, t = unit % m, b = tile / a.tiles_per_problem;
+      const long long row0 =
+          (long long)(tile % a.tiles_per_problem) * BOUTE_TILE_M + 32 * (i & 3);
+      float *mu = a.mean + ((size_t)b * m + t) * a.N + row0 + lane;
+      const bool marked = row0 + lane < a.N && __float_as_uint(*mu) == kFixMark;
+      for (unsigned todo = __ballot_sync(0xffffffffu, marked); todo; todo &= todo - 1) {
+        const int src = __ffs(todo) - 1;
+        const float v = mean_pair_warp<DP>(a.Xc + ((long long)b * a.N + row0 + src) * d, d,
+                                           a.xt + (size_t)(b * m + t) * pl.nxt * cf, cf, n, lane);
+        if (lane == src) *mu = v;
+      }
+    }
   }
 }
 

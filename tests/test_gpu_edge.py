@@ -245,7 +245,7 @@ def test_kstar_beside_the_fit_where_it_is_faster(n, d, N, beside):
 
 def test_ill_conditioned_problem_meets_fp32_error_bound():
     """40 points on a line with lengthscale 0.3: cond(K) ~ 2e5, |alpha| ~ 1e3.
-    The mean meets 1e-5 (its ill-conditioned rows take the fp64 path); the
+    The mean meets 1e-5 (its ill-conditioned rows are recomputed in pairs of floats); the
     variance s2 - ||L^-1 k*||^2 must stay within the error bound of an
     fp32-accurate contraction, eps32 * s2 times cond-scaled terms."""
     hp = rand_problem(12, 40, 1, 2, 300)
@@ -262,6 +262,70 @@ def test_ill_conditioned_problem_meets_fp32_error_bound():
         v = Ks @ W.T
         bound_v = 64 * eps32 * 2 * (np.abs(v) * (np.abs(Ks) @ np.abs(W.T))).sum(1) + 1e-5
         assert np.all(np.abs(g["var"][0, t] - var[:, t]) <= bound_v)
+
+
+@pytest.mark.parametrize("n,d,N,B", [(60, 5, 20_000, 2), (33, 9, 130, 1), (129, 20, 999, 3)])
+def test_ill_conditioned_rows_of_many_tiles(n, d, N, B):
+    """Long lengthscales, so that most rows are recomputed, over several tiles per CTA, a
+    ragged last tile, problems and objectives; by the handle (K* built inside the posterior)
+    and by an engine step (K* staged)."""
+    import dataclasses
+
+    import torch
+
+    from paper_2602_10729_gb300 import boute as bt
+    w = wl.scaled(dataclasses.replace(wl.WORKLOADS[4], d=d, k=4), N=N, B=B, n=n)
+    hp = host_problem(w)
+    hp.ls *= 4.0
+    g = gpu_pipeline(hp)
+    t = lambda a, dt=torch.float64: torch.as_tensor(np.ascontiguousarray(a), dtype=dt, device="cuda")
+    e = bt.Engine(B, n, d, 2, N, bt.BOUTE_ACQ_EHVI2D, 0, 4)
+    idx = torch.empty((B, 4), dtype=torch.int64, device="cuda")
+    val = torch.empty((B, 4), dtype=torch.float32, device="cuda")
+    mean = torch.empty((B, 2, N), dtype=torch.float32, device="cuda")
+    bt.boute_engine_step(e, t(hp.X), t(hp.Y), t(hp.ls), t(hp.s2), t(hp.noise), t(hp.ref),
+                         t(hp.Xc, torch.float32), None, idx, val)
+    bt.boute_engine_scores(e, None, mean, None)
+    torch.cuda.synchronize()
+    e.free()
+    at = np.unique(np.r_[np.arange(0, N, 37), N - 1])
+    marked = 0
+    for b in range(B):
+        fp = oracle_fit(hp, b)
+        mo, _ = opl.posterior(fp, hp.Xc[b][at])
+        for k in range(2):
+            check_mean(g["mean"][b, k, at], mo[:, k], fp.s2[k])
+            check_mean(mean[b, k].cpu().numpy()[at], mo[:, k], fp.s2[k])
+            ks = np.array([[oracle.matern52(c, x, hp.ls[b][k], hp.s2[b][k]) for x in hp.X[b]]
+                           for c in hp.Xc[b][at[:20]].astype(np.float64)])
+            terms = ks @ np.abs(fp.alpha[k])
+            marked += int((terms > 224 * np.maximum(np.abs(mo[:20, k]), np.sqrt(fp.s2[k]))).sum())
+    assert marked > 5 * B
+
+
+def test_recomputed_means_do_not_hold_up_the_posterior():
+    """Every row recomputed: eight times the posterior without any (by one warp of
+    four at a time, beside the tensor cores, 24 times)."""
+    import dataclasses
+
+    import torch
+
+    from paper_2602_10729_gb300 import boute as bt
+    w = wl.scaled(dataclasses.replace(wl.WORKLOADS[4], d=8), N=32768, B=1, n=400)
+    hp = host_problem(w)
+    t = lambda a, dt=torch.float64: torch.as_tensor(np.ascontiguousarray(a), dtype=dt, device="cuda")
+    X, Y, Xc = t(hp.X), t(hp.Y), t(hp.Xc, torch.float32)
+    bt.boute_standardize(Y, Y)
+    mean = torch.empty((1, 2, w.N), dtype=torch.float32, device="cuda")
+    var = torch.empty_like(mean)
+    gp = bt.boute_gp_create(1, w.n, w.d, 2)
+    us = []
+    for f in (0.4, 2.0):
+        bt.boute_gp_fit(gp, X, Y, t(hp.ls * f), t(hp.s2), t(hp.noise))
+        assert bt.boute_gp_status(gp) == 0
+        us.append(_graph_us(lambda: bt.boute_gp_posterior(gp, Xc, w.N, mean, var), 4))
+    gp.free()
+    assert us[1] < 14 * us[0], us
 
 
 def test_three_objectives_monte_carlo_and_box_decomposition():
@@ -342,8 +406,8 @@ def test_per_objective_hyperparameters():
                                             ((0.1, 1.5), (1e-5, 1e-6))])
 def test_ill_conditioned_means(ls_range, noise):
     """Longer lengthscales or smaller noise: sum_j |K*_j alpha_j| reaches 270
-    to 590 times the mean's scale. Rows beyond 256 times take the fp64 path;
-    mean and variance meet 1e-5 everywhere."""
+    to 590 times the mean's scale. Rows beyond 224 times are recomputed in pairs of
+    floats; mean and variance meet 1e-5 everywhere."""
     rng = np.random.default_rng(8)
     hp = rand_problem(9, 70, 5, 2, 333)
     hp.ls[0] = rng.uniform(*ls_range, (2, 5))

@@ -436,6 +436,21 @@ __global__ void __launch_bounds__(kFcThreads, 1) fitc_kernel(
   // this CTA's block rows I = ra + Pr i, each with the columns J = rb + Pc j <= I
   const int lrows = ra < nb ? ((nb - 1 - ra) >> sr) + 1 : 0;
   auto row_count = [&](int I) { return I >= rb ? ((I - rb) >> sc) + 1 : 0; };
+  int nslots = 0;
+  if constexpr (TS) {
+    for (int i = tid; i <= lrows; i += kFcThreads) {
+      int q = 0;
+      for (int e = 0; e < i; ++e) q += row_count(ra + (e << sr));
+      row_first[i] = q;
+    }
+    __syncthreads();
+    nslots = row_first[lrows];
+    for (int i = warp; i < lrows; i += nw)
+      for (int j = lane; j < row_count(ra + (i << sr)); j += 32) {
+        slotI[row_first[i] + j] = (unsigned short)(ra + (i << sr));
+        slotJ[row_first[i] + j] = (unsigned short)(rb + (j << sc));
+      }
+  }
   const double *y = Ys + (size_t)b * n * m + t;
   if (warp == nw - 1) standardize_stats(y, n, m, standardize, lane, ymu, yisd);
   // everything below reads what the set-up kernel wrote
@@ -446,18 +461,6 @@ __global__ void __launch_bounds__(kFcThreads, 1) fitc_kernel(
   bool fits = true;
   auto at = [&](const float *q, int r) { return fc_remote(q, r); };
   if constexpr (TS) {
-    for (int i = tid; i <= lrows; i += kFcThreads) {
-      int q = 0;
-      for (int e = 0; e < i; ++e) q += row_count(ra + (e << sr));
-      row_first[i] = q;
-    }
-    __syncthreads();
-    const int nslots = row_first[lrows];
-    for (int i = warp; i < lrows; i += nw)
-      for (int j = lane; j < row_count(ra + (i << sr)); j += 32) {
-        slotI[row_first[i] + j] = (unsigned short)(ra + (i << sr));
-        slotJ[row_first[i] + j] = (unsigned short)(rb + (j << sc));
-      }
     if (rank == 0 && tid == 0) __stcg(fbad, 0);
     for (int e = tid; e < 32 * lrows; e += kFcThreads) {
       const int i = 32 * (ra + ((e >> 5) << sr)) + (e & 31);

@@ -732,7 +732,8 @@ __global__ void __launch_bounds__(kFcThreads, 1) fitc_kernel(
         sh = s_;
         sl += ol + e;
       }
-      const float r = i < n ? (yv[i] - sh) + (ylo[i] - sl) : 0.f;
+      // (the lanes' sl may differ in the last bit: every CTA gets the first lane's)
+      const float r = __shfl_sync(half, i < n ? (yv[i] - sh) + (ylo[i] - sl) : 0.f, 0, 16);
       if (hl < C) fc_store1(at(x + i, hl), r);
     }
     sync();

@@ -757,6 +757,36 @@ def _median_us(f, reps=15):
     return float(np.median(out))
 
 
+@pytest.mark.parametrize("n,d,seed,b", [(360, 9, 28, 1), (512, 16, 3, 12), (100, 6, 1, 0)])
+def test_fit_does_not_depend_on_the_cluster_size(n, d, seed, b):
+    """A problem fitted alone (16 CTAs, or a CTA per block row) and 24 times in a batch (one
+    to four CTAs): the same sums in the same order, so the same means to the last bit, also
+    where the lanes that send a residual round it differently (the first two)."""
+    import torch
+
+    from paper_2602_10729_gb300 import boute as bt
+    from perf import cases
+    B = 4 if b < 4 else 32
+    p = cases._problem(dict(B=B, n=n, d=d, m=2), seed)
+    Xc = cases._candidates(dict(B=B, N=1000, d=d), seed, d)
+
+    def means(k):
+        t = lambda a: a[b:b + 1].expand(k, *a.shape[1:]).contiguous()
+        Ys = torch.empty_like(t(p["Y"]))
+        bt.boute_standardize(t(p["Y"]), Ys)
+        gp = bt.boute_gp_create(k, n, d, 2)
+        mean = torch.empty((k, 2, 1000), dtype=torch.float32, device="cuda")
+        var = torch.empty_like(mean)
+        bt.boute_gp_fit(gp, t(p["X"]), Ys, t(p["ls"]), t(p["s2"]), t(p["noise"]))
+        bt.boute_gp_posterior(gp, t(Xc), 1000, mean, var)
+        assert bt.boute_gp_status(gp) == 0
+        gp.free()
+        return mean, var
+
+    (mean, var), (mean1, var1) = means(24), means(1)
+    assert torch.equal(mean, mean1.expand_as(mean)) and torch.equal(var, var1.expand_as(var))
+
+
 @pytest.mark.parametrize("n", [256, 512])
 def test_fit_of_problem_objectives_beyond_the_held_clusters(n):
     """15 clusters of 8 fit the device, though 16 of them have no more CTAs than it has

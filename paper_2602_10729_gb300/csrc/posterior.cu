@@ -1190,9 +1190,11 @@ int launch_dp(const Gp *gp, const float *Xc, const float *kst, long long N, floa
 // chunk is stored as a 32 KB fp32 image ([128 x 64], st_off32), which the
 // posterior brings in with one bulk copy and splits into its fp16 operand
 // parts. The training points' side input is staged in shared memory. It needs
-// the set-up's side input (not the fit's results) and the candidates.
+// the set-up's side input (not the fit's results) and the candidates. Two blocks an SM at
+// least: with 82 registers the composite kernel's pairs had an SM to a block of 512 threads
+// at d = 13 .. 16 (n = 128, d = 16, N = 2^17: step 199 -> 173 us; rows held singly 192).
 template <int DP, int KERN>
-__global__ void __launch_bounds__(Layout<DP>::kBld * 32) kstar_kernel(
+__global__ void __launch_bounds__(Layout<DP>::kBld * 32, 2) kstar_kernel(
     const float *Xc, const float *xt, long long N, int d, int m, int n, int tiles_per_problem,
     int nxt, float *kst) {
   // rows in pairs, RPT apart, C columns of each half per thread, as the fused builders

@@ -602,9 +602,23 @@ void boute_engine_free(boute_engine *e) {
 //   d = 6: n = 160 143 : 141 at 140 MiB, 199 : 192 at 260; n = 384 226 : 219 at 140
 //   up to 64 observations the fit is too short to hide it: d = 12, n = 64 206 : 197 at 190
 //     MiB, 266 : 247 at 260
-static bool kstar_worth(const Gp &g, long long N) {
-  const size_t line = g.DP > 16 ? 512 : g.n > 64 && g.n <= 448 && g.DP > 8 ? 256 : 128;
+//   the composite kernel, whose values cost more to build: n = 128, d = 8 230 : 249 at 256
+//     MiB, 331 : 342 at 390; d = 16 285 : 328 at 256, 519 : 585 at 512; n = 256, d = 16 492 :
+//     550 at 512; n = 512, d = 16 438 : 498 at 256
+static bool kstar_worth(const Gp &g, long long N, bool composite) {
+  const size_t line = g.DP > 16 || composite                  ? 512
+                      : g.n > 64 && g.n <= 448 && g.DP > 8 ? 256
+                                                              : 128;
   return kstar_floats(&g, N) * sizeof(float) <= line << 20;
+}
+
+// The engine's K* buffer, for its largest n, where that is worth it.
+static int kstar_alloc(boute_engine *e, bool composite) {
+  Gp cap = e->gp->g;
+  cap.n = e->ncap;
+  cap.plan = make_post_plan(e->ncap, cap.plan.S_in);
+  if (e->kst || !kstar_worth(cap, e->N, composite)) return BOUTE_OK;
+  return dalloc(&e->kst, kstar_floats(&cap, e->N));
 }
 
 // The selection runs inside the acquisition kernel for 2-objective
@@ -676,8 +690,7 @@ int boute_engine_create(int B, int n, int d, int m, long long N, int mode, int S
       r = BOUTE_ERR_CUDA;
     }
   }
-  if (r == BOUTE_OK && kstar_worth(e->gp->g, N))
-    r |= dalloc(&e->kst, kstar_floats(&e->gp->g, N));
+  if (r == BOUTE_OK) r |= kstar_alloc(e, false);
   if (r == BOUTE_OK &&
       (cudaStreamCreateWithFlags(&e->side, cudaStreamNonBlocking) != cudaSuccess ||
        cudaStreamCreateWithFlags(&e->side2, cudaStreamNonBlocking) != cudaSuccess ||
@@ -755,7 +768,9 @@ static int engine_run(boute_engine *e, const double *X, const double *Y, const d
   // K* beside the fit (not in serialised timing, where the posterior builds it, nor
   // while the K* kernel cannot hold the side input of the engine's present n)
   const float *kst =
-      serial || !kstar_fits(&e->gp->g) || !kstar_worth(e->gp->g, e->N) ? nullptr : e->kst;
+      serial || !kstar_fits(&e->gp->g) || !kstar_worth(e->gp->g, e->N, e->gp->g.kern)
+          ? nullptr
+          : e->kst;
   // The graph has one root, the fit's set-up: the front stage (which needs
   // the raw outcomes only) and K* (which needs the set-up's side input) fork
   // after it and run beside the fit (one root launches sooner than two).
@@ -1151,6 +1166,8 @@ int boute_engine_set_kernel(boute_engine *e, int d_tau, const double *params) {
   if (!e) return BOUTE_ERR_INVALID_ARG;
   const int r = boute_gp_set_kernel(e->gp, d_tau, params);
   engine_drop_graphs(e);  // the step's kernel choices change
+  // (without memory for it K* is built inside the posterior)
+  if (r == BOUTE_OK && params && kstar_alloc(e, true) != BOUTE_OK) cudaGetLastError();
   return r;
 }
 

@@ -220,18 +220,25 @@ def test_engine_where_the_side_input_passes_shared_memory(n, d, comp):
                                           (128, 16, 532443, False), (64, 16, 389083, False),
                                           (160, 7, 129627, False), (128, 24, 600000, False),
                                           (512, 12, 48603, False)])
-def test_kstar_beside_the_fit_where_it_is_faster(n, d, N, beside):
+@pytest.mark.parametrize("comp", [False, True])
+def test_kstar_beside_the_fit_where_it_is_faster(n, d, N, beside, comp):
     """A step with K* beside the fit launches one kernel more (its own), as one with few
-    candidates does: up to 512 MiB of K* from 17 dimensions on, 256 with 9 to 16 and 65 to
-    448 observations, else 128."""
+    candidates does: up to 512 MiB of K* from 17 dimensions on and with the composite kernel,
+    256 with 9 to 16 and 65 to 448 observations, else 128."""
     import torch
 
     from paper_2602_10729_gb300 import boute as bt
     hp = rand_problem(31, n, d, 2, 1, ls=0.2 * np.sqrt(d))
     t = lambda a: torch.as_tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")
+    mib = (N + 127) // 128 * 2 * ((n + 63) // 64) / 32
+    beside = mib <= 512 if comp else beside
     count = []
     for cands in (20000, N):
         e = bt.Engine(1, n, d, 2, cands, bt.BOUTE_ACQ_EHVI2D, 0, 4)
+        if comp:  # (set while the engine holds fewer observations than it was made for)
+            bt.boute_engine_set_n(e, 5)
+            bt.boute_engine_set_kernel(e, d // 2, np.full((1, 2, 3 + d - d // 2), 0.1))
+            bt.boute_engine_set_n(e, n)
         Xc = torch.rand((1, cands, d), device="cuda")
         idx = torch.empty((1, 4), dtype=torch.int64, device="cuda")
         val = torch.empty((1, 4), dtype=torch.float32, device="cuda")

@@ -1005,9 +1005,11 @@ static int launch_fit_impl(Gp *gp, const double *X, const double *Ys, int standa
   const int sms = num_sms();
   // side-input blocks: as many as leave one block per SM (K blocks first), 2 .. 16
   const int nprep = std::max(2, std::min(16, sms / BM - nkt));
-  // early triggers only when every block of the grid is resident at once (8
-  // set-up blocks per SM beside the fit's blocks; one fit block per SM), so
-  // that waiting successors can never hold resources a later block needs
+  // The set-up lets the fit launch from its first instruction on where its whole grid is
+  // resident at once with room to spare (8 blocks an SM, on all but one SM per
+  // problem-objective). The fit's CTAs, a whole SM each, come only when every set-up block
+  // has started, so they never hold what a later block needs, however many they are; with
+  // several waves of set-up blocks they would only wait on SMs that the last wave could use.
   const long long setup_blocks = (long long)(nkt + nprep) * BM;
   const int setup_early = setup_blocks <= 8LL * (sms - BM) ? 1 : 0;
   auto setup = [&](auto kern) {

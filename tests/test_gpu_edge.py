@@ -100,26 +100,15 @@ def test_cached_chunks_over_many_tiles(n, d, comp):
     """More than 512 observations (a second group of output blocks takes the
     first one's K* chunks from the cache) and enough candidates that every CTA
     works through several tiles: runs of cached chunks at the end of one tile
-    meet the chunks built for the next. Sampled candidates, POST_REL of the
-    prior variance as everywhere."""
+    meet the chunks built for the next. Sampled candidates."""
     import dataclasses
 
     base = wl.scaled(dataclasses.replace(wl.WORKLOADS[2], d=d), N=60011, n=n)
-    w = wl.composite(base) if comp else base
-    hp = host_problem(w)
+    hp = host_problem(wl.composite(base) if comp else base)
     g = gpu_pipeline(hp)
     assert g["status"] == 0
-    fp = oracle_fit(hp, 0)
-    at = np.unique(np.r_[np.arange(0, 60011, 233), 60010])
-    mean, var = opl.posterior(fp, hp.Xc[0][at])
-    for t in range(w.m):
-        prior = np.full(len(at), hp.s2[0][t])
-        if comp:
-            kern = (hp.d_tau, hp.kc[0][t])
-            prior = np.array([oracle.kernel(c, c, hp.ls[0][t], hp.s2[0][t], kern)
-                              for c in hp.Xc[0][at].astype(np.float64)])
-        check_var(g["var"][0, t, at], var[:, t], prior.max())
-        assert np.abs(g["mean"][0, t, at] - mean[:, t]).max() <= 4 * POST_REL * np.sqrt(prior.max())
+    check_posterior_at(hp, np.unique(np.r_[np.arange(0, 60011, 233), 60010]), g["mean"][0],
+                       g["var"][0])
 
 
 @pytest.mark.parametrize("d", [1, 3, 8, 9, 13, 17, 25, 32])

@@ -560,7 +560,8 @@ def test_invalid_arguments_raise():
 
 # Sizes around a warp of points; every point on the front; ties and signed zeros.
 @pytest.mark.parametrize("kind", ["random", "antichain", "ties"])
-@pytest.mark.parametrize("n,m", [(1, 2), (31, 3), (32, 2), (33, 3), (130, 4), (513, 2), (257, 3)])
+@pytest.mark.parametrize("n,m", [(1, 2), (31, 3), (32, 2), (33, 3), (130, 4), (513, 2), (257, 3),
+                                 (2048, 3)])
 def test_front_and_boxes_edges(n, m, kind):
     import torch
 

@@ -308,15 +308,16 @@ size_t topk_scratch_bytes(int B, long long N, int k) {
   return 2 * (size_t)B * g1 * std::max(k, 32) * sizeof(unsigned long long) + 16;
 }
 
-// The last level's block for len entries: the fewest threads that hold them and k maxima,
-// whose barriers are cheaper and of whose blocks more run at once (N = 1024, k = 32, 1000
-// problems: 8 us with 128 threads, 35 with 1024; N = 4096, k = 8, one problem: 3.9 with
-// 256, 5.5).
+// The last level's block for len entries: the fewest threads that hold them and twice k (with
+// fewer the k-th of their maxima leaves most entries to the second search: N = 8192, k = 512
+// 20 us with 512, 17 with 1024), whose barriers are cheaper and of whose blocks more run at
+// once (N = 1024, k = 32, 1000 problems: 8 us with 128 threads, 35 with 1024; N = 4096,
+// k = 8, one problem: 3.9 with 256, 5.5).
 template <class Go>
 static void final_threads(long long len, int k, Go go) {
-  if (len <= 128 * kR && k <= 128) go(std::integral_constant<int, 128>{});
-  else if (len <= 256 * kR && k <= 256) go(std::integral_constant<int, 256>{});
-  else if (len <= 512 * kR && k <= 512) go(std::integral_constant<int, 512>{});
+  if (len <= 128 * kR && k <= 64) go(std::integral_constant<int, 128>{});
+  else if (len <= 256 * kR && k <= 128) go(std::integral_constant<int, 256>{});
+  else if (len <= 512 * kR && k <= 256) go(std::integral_constant<int, 512>{});
   else go(std::integral_constant<int, kFinThreads>{});
 }
 

@@ -452,9 +452,9 @@ def test_topk_levels_and_k_range(N, k):
 
 # blocks of 128 to 1024 threads at their edges, one level and two, scores mostly equal:
 # fewer others than k, as many, more, none
-@pytest.mark.parametrize("N,k", [(2048, 128), (2048, 129), (2049, 100), (4096, 256), (4097, 32),
-                                 (8192, 512), (8193, 512), (8192, 513), (16384, 7), (20_000, 40),
-                                 (300_000, 64), (300_000, 700), (60, 60)])
+@pytest.mark.parametrize("N,k", [(2048, 64), (2048, 65), (2049, 60), (4096, 128), (4096, 129),
+                                 (4097, 32), (8192, 256), (8193, 256), (8192, 257), (8192, 1024),
+                                 (16384, 7), (20_000, 40), (300_000, 64), (300_000, 700), (60, 60)])
 def test_topk_mostly_equal_scores(N, k):
     import torch
 
